@@ -454,7 +454,12 @@ _STATES = {"epoch": _Engine, "split": _Engine, "blocks": _Engine, "step": _Engin
 
 
 def prepare(case, seed):
-    return _STATES[case["kind"]](case, seed)
+    # A pool initialises its memory on a stream of its own: nothing may still be reading what the
+    # allocator hands it, and its first user may come from any stream.
+    torch.cuda.synchronize()
+    state = _STATES[case["kind"]](case, seed)
+    torch.cuda.synchronize()
+    return state
 
 
 def run(state):
