@@ -139,6 +139,16 @@ def _ok(rc, what):
         raise B.KVError(rc, what)
 
 
+_STREAM = []
+
+
+def _compute():
+    """The engine's compute stream: epochs follow one another on it, whichever pool they belong to."""
+    if not _STREAM:
+        _STREAM.append(torch.cuda.Stream())
+    return _STREAM[0]
+
+
 def _partition(arch, layers, heads, blocks, q_heads=None, head_dim=1, block_tokens=16, ring=16):
     if arch == "gqa":
         return W.gqa(layers, q_heads or 4 * heads, heads, head_dim, block_tokens, blocks, ring)
@@ -244,7 +254,8 @@ class _Engine:
         self.m = min(int(case.get("promote", 0) * n), k // 2) if step else 0
         # handles for as many epochs as a long-running measurement makes (they are never reused)
         tags = n + 64 + (k * min(60_000, (1 << 27) // k) if step else 0)
-        self.pool = p = B.Pool(parts, tags, staging_bytes=staging, max_promote=max(4096, self.m + 16), host_meta=step)
+        self.pool = p = B.Pool(parts, tags, staging_bytes=staging, max_promote=max(4096, self.m + 16),
+                               host_meta=step, stream=_compute())
         for ring in p.rings:
             ring.zero_()
         bases = np.concatenate([[0], np.cumsum([q.n_entries for q in parts])])[:-1].tolist()
@@ -368,7 +379,7 @@ class _Static:
         score, state = self.arrays[self.at % TRACES]
         self.at += 1
         _ok(B.kv_select_victims_static(score, state, score.numel(), self.k, self.victims, self.status,
-                                       torch.cuda.current_stream()), "kv_select_victims_static")
+                                       _compute()), "kv_select_victims_static")
         return {"victims": self.victims, "status": self.status}
 
 
@@ -379,7 +390,8 @@ class _Hash:
         g = torch.Generator(device="cuda").manual_seed(seed)
         part = _partition(case["arch"], case["layers"], case["heads"], case["blocks"], case["q_heads"], case["head_dim"],
                           case["block_tokens"])
-        self.pool = B.Pool([part], part.n_entries, staging_bytes=part.entry_bytes + 4096, max_promote=64, host_meta=False)
+        self.pool = B.Pool([part], part.n_entries, staging_bytes=part.entry_bytes + 4096, max_promote=64,
+                           host_meta=False, stream=_compute())
         blocks = part.n_layers * part.blocks_per_layer
         slab = self.pool.slabs[0].view(torch.int64).view(blocks, -1)
         for lo in range(0, blocks, 1 << 14):
@@ -413,7 +425,8 @@ class _Prefetch:
         n = layers * heads * nb
         self.case = case
         part = _partition("gqa" if heads > 1 else "mqa", layers, heads, nb, ring=int(n * case["away"]) + 64)
-        self.pool = p = B.Pool([part], n + 64, staging_bytes=8 << 20, max_promote=4096, host_meta=False)
+        self.pool = p = B.Pool([part], n + 64, staging_bytes=8 << 20, max_promote=4096, host_meta=False,
+                               stream=_compute())
         pairs = torch.randint(0, 16, (n + 16,), dtype=torch.uint8, device="cuda", generator=g)
         # block handles were given out in (layer, block, head) order; a sequence owns scattered blocks
         perm = torch.randperm(nb, device="cuda", generator=g)
