@@ -475,7 +475,7 @@ int32_t kv_select_victim_blocks(kv_pool* pool, uint64_t k_blocks, uint32_t* d_vi
  * that has given all device memory to its own pools, or code that runs where
  * cudaMalloc is off limits, has no workspace to hand to kv_pool_create.  This
  * call needs none: it takes the score and state arrays directly and keeps its
- * scratch (histograms, scalars, per-tile counts; about 58 KB) in a fixed array
+ * scratch (histograms, scalars, per-tile counts; about 140 KB) in a fixed array
  * inside the library, which every GPU that loads the library holds until the
  * process exits.  It calls no allocating routine.
  *   d_score  (device) f32[n]  eviction scores, as kv_epoch_score writes them
@@ -489,9 +489,9 @@ int32_t kv_select_victim_blocks(kv_pool* pool, uint64_t k_blocks, uint32_t* d_vi
  *     KV_ERR_K_TOO_LARGE; pointers must be 16-byte aligned;
  *   - the first call on each device looks up the array's device address (with
  *     that device current); make that first call before any stream capture;
- *   - all calls on a device share the one array, which is cleared at the start of
- *     each call: two calls whose GPU work overlaps (different streams, no
- *     ordering between them) race and give wrong results.  Order them. */
+ *   - all calls on a device share the one array: two calls whose GPU work overlaps
+ *     (different streams, no ordering between them) race and give wrong results.
+ *     Order them. */
 int32_t kv_select_victims_static(const float* d_score, const uint8_t* d_state, uint64_t n,
                                  uint64_t k, uint32_t* d_victims, uint32_t* d_status,
                                  kv_stream_t stream);

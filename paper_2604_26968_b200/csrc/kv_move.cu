@@ -141,13 +141,16 @@ __global__ void init_scalars_kernel(uint64_t* hits, uint64_t* misses, float* P, 
   for (uint32_t i = t; i < kMaxWindow * 32; i += blockDim.x) ws.blend->win[i] = 0;
   if (t == 0) { ws.blend->head = 0; ws.blend->pad = 0; }
   for (uint32_t b = t; b < 3 * kHistBins; b += blockDim.x) ws.hist[b] = 0;
+  for (uint32_t w = t; w < 2 * sizeof(SelectTurn) / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(ws.turns)[w] = 0;
+  for (uint64_t w = t; w < ws.table_words; w += blockDim.x) ws.table[w] = 0;
   if (t < 4) ws.part_counts[t] = 0;
   if (t == 0) {
     *ws.status = 0;
     ws.sel->prefix = 0; ws.sel->tau = 0; ws.sel->k_rem = 0; ws.sel->need_eq = 0;
-    ws.sel->bar_arrive = 0; ws.sel->bar_done = 0; ws.sel->update_ticket = 0; ws.sel->hint_last = 0;
-    ws.sel->hint_valid = 0; ws.sel->hint_tau = 0; ws.sel->hint_n = 0; ws.sel->below = 0;
+    ws.sel->serial = 0; ws.sel->update_ticket = 0; ws.sel->hint_last = 0;
+    ws.sel->hint_valid = 0; ws.sel->hint_tau = 0; ws.sel->hint_n = 0;
     ws.sel->hint_shift = 11; ws.sel->hint_resid = 0;
+    for (int q = 0; q < 3; ++q) ws.sel->bound[q] = 0;
     ws.sel->n_select = 0; ws.sel->n_hint_hit = 0; ws.sel->n_hint_miss = 0; ws.sel->n_reread = 0;
   }
 }

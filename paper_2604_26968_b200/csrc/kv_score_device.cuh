@@ -310,14 +310,14 @@ __device__ __forceinline__ void commit_predictor(const Predictor& pd, unsigned p
   pd.delta[2 * p + 1] = 0;
 }
 
-// Four consecutive entries (a 16-byte vector of each array) through entry_step,
+// Four consecutive entries (a 16-byte vector of each array) through the entry step,
 // in two halves so that a caller can have the next vector's loads in flight
 // while it finishes this one.  v indexes vectors.  The touch counts are read from
 // L2: other blocks' atomics made them.
 struct EntryVec {
   float4 e, d;
   uint4 t, le;
-  uchar4 pr, st;
+  uint32_t pr4, st4;   // pair and state bytes
 };
 
 __device__ __forceinline__ EntryVec entry_load4(const EntryState& st, uint64_t v, int policy) {
@@ -325,8 +325,8 @@ __device__ __forceinline__ EntryVec entry_load4(const EntryState& st, uint64_t v
   x.e = reinterpret_cast<const float4*>(st.ema)[v];
   x.d = reinterpret_cast<const float4*>(st.decay)[v];
   x.t = __ldcg(reinterpret_cast<const uint4*>(st.touch) + v);
-  x.pr = reinterpret_cast<const uchar4*>(st.pair)[v];
-  x.st = reinterpret_cast<const uchar4*>(st.state)[v];
+  x.pr4 = reinterpret_cast<const uint32_t*>(st.pair)[v];
+  x.st4 = reinterpret_cast<const uint32_t*>(st.state)[v];
   x.le = make_uint4(0, 0, 0, 0);
   if (policy == 2) x.le = reinterpret_cast<const uint4*>(st.last_epoch)[v];  // only LRU reads it
   return x;
@@ -338,19 +338,19 @@ __device__ __forceinline__ EntryVec entry_load4(const EntryState& st, uint64_t v
 template <bool kPlain = false>
 __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, EntryVec& x, const float* sP,
                                               int policy, uint32_t epoch, const HeadWeights& hw, float4& sc) {
-  float4 w = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
-  if (!kPlain && hw.on) {
-    w.x = head_weight(hw, 4 * v + 0);
-    w.y = head_weight(hw, 4 * v + 1);
-    w.z = head_weight(hw, 4 * v + 2);
-    w.w = head_weight(hw, 4 * v + 3);
+  float e[4] = {x.e.x, x.e.y, x.e.z, x.e.w}, s[4];
+  const float d[4] = {x.d.x, x.d.y, x.d.z, x.d.w};
+  const uint32_t t[4] = {x.t.x, x.t.y, x.t.z, x.t.w}, le[4] = {x.le.x, x.le.y, x.le.z, x.le.w};
+  const bool all_resident = x.st4 == KV_STATE_RESIDENT * 0x01010101u;   // nearly always
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float w = 1.0f;
+    if (!kPlain && hw.on) w = head_weight(hw, 4 * v + j);
+    entry_step(e[j], d[j], t[j], x.pr4 >> (8 * j), all_resident ? KV_STATE_RESIDENT : (x.st4 >> (8 * j)) & 0xFFu, sP,
+               kPlain ? 0 : policy, le[j], epoch, w, s[j]);
   }
-  const int pol = kPlain ? 0 : policy;
-  entry_step(x.e.x, x.d.x, x.t.x, x.pr.x, x.st.x, sP, pol, x.le.x, epoch, w.x, sc.x);
-  entry_step(x.e.y, x.d.y, x.t.y, x.pr.y, x.st.y, sP, pol, x.le.y, epoch, w.y, sc.y);
-  entry_step(x.e.z, x.d.z, x.t.z, x.pr.z, x.st.z, sP, pol, x.le.z, epoch, w.z, sc.z);
-  entry_step(x.e.w, x.d.w, x.t.w, x.pr.w, x.st.w, sP, pol, x.le.w, epoch, w.w, sc.w);
-  reinterpret_cast<float4*>(st.ema)[v] = x.e;
+  sc = make_float4(s[0], s[1], s[2], s[3]);
+  reinterpret_cast<float4*>(st.ema)[v] = make_float4(e[0], e[1], e[2], e[3]);
   reinterpret_cast<float4*>(st.score)[v] = sc;
   // touch counts of FREE entries are always zero (events on them are refused)
   if (x.t.x | x.t.y | x.t.z | x.t.w) {

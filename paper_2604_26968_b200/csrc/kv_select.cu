@@ -10,15 +10,9 @@
 // key == tau.  Nothing waits on another block: each phase is its own launch.
 #include <mutex>
 
-#include "kvtier_internal.cuh"
+#include "kv_select_device.cuh"
 
 namespace kvt {
-
-__device__ __forceinline__ uint32_t score_key(float s) {
-  uint32_t b = __float_as_uint(s);
-  if (b == 0x80000000u) b = 0u;  // -0.0 orders with +0.0
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
 
 template <int PASS> struct Digit;
 template <> struct Digit<0> { static constexpr uint32_t shift = 21, bits = 11, fixed_mask = 0u; };
@@ -426,25 +420,27 @@ namespace {
 
 constexpr uint64_t kStaticMaxEntries = 1ull << 22;  // 4,194,304 entries
 constexpr uint64_t kStaticMaxTiles = kStaticMaxEntries / kvt::kTileEntries + 2;
-// layout (bytes): [0, 24576) histograms | [24576, 24832) scalars | [24832, 25088) status |
-//                 [25088, +tiles*8) tile counts | then tile offsets
-constexpr uint64_t kOffHist = 0;
-constexpr uint64_t kOffSel = 3 * kvt::kHistBins * 4;
-constexpr uint64_t kOffStatus = kOffSel + 256;
-static_assert(sizeof(kvt::SelectScalars) <= 256, "the scalars have 256 bytes of the built-in scratch");
-constexpr uint64_t kOffTileCounts = kOffStatus + 256;
-constexpr uint64_t kOffTileOffsets = kOffTileCounts + ((kStaticMaxTiles * 8 + 255) / 256) * 256;
-constexpr uint64_t kStaticScratchBytes = kOffTileOffsets + ((kStaticMaxTiles * 8 + 255) / 256) * 256;
+// What the array holds, in this order.  All of it starts as zeros; every selection leaves the
+// histograms zero again (the persistent one clears the set that the next one uses).
+struct StaticScratch {
+  uint32_t hist[3 * kvt::kHistBins];
+  kvt::SelectTurn turns[2];
+  kvt::SelectScalars sel;
+  uint32_t status[4];
+  uint2 tile_counts[kStaticMaxTiles];
+  uint2 tile_offsets[kStaticMaxTiles];
+  unsigned long long table[kStaticMaxEntries / 4096 + 1024];
+};
 
-static __device__ __align__(256) unsigned char g_select_scratch[kStaticScratchBytes];
+static __device__ __align__(256) unsigned char g_select_scratch[sizeof(StaticScratch)];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mutex;
-unsigned char* g_scratch_addr[kMaxDevices] = {nullptr};
+StaticScratch* g_scratch_addr[kMaxDevices] = {nullptr};
 
 // The array's name is only a stand-in on the host; the address a kernel can use
 // comes from the runtime, once per device, with that device current.
-cudaError_t static_scratch(unsigned char** out) {
+cudaError_t static_scratch(StaticScratch** out) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -454,7 +450,7 @@ cudaError_t static_scratch(unsigned char** out) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_select_scratch);
     if (e != cudaSuccess) return e;
-    g_scratch_addr[dev] = static_cast<unsigned char*>(p);
+    g_scratch_addr[dev] = static_cast<StaticScratch*>(p);
   }
   *out = g_scratch_addr[dev];
   return cudaSuccess;
@@ -472,19 +468,20 @@ extern "C" int32_t kv_select_victims_static(const float* d_score, const uint8_t*
     return KV_ERR_INVALID_ARG;
   if (k == 0) return KV_OK;
   if (!d_victims || (reinterpret_cast<uintptr_t>(d_victims) & 15u)) return KV_ERR_INVALID_ARG;
-  unsigned char* base = nullptr;
-  if (static_scratch(&base) != cudaSuccess) return KV_ERR_CUDA;
+  StaticScratch* scratch = nullptr;
+  if (static_scratch(&scratch) != cudaSuccess) return KV_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The array keeps whatever the previous call left: start the histograms and the
-  // status word from zero (the scalars are reset by the first kernel of the pass).
-  if (cudaMemsetAsync(base + kOffHist, 0, kOffTileCounts, s) != cudaSuccess) return KV_ERR_CUDA;
   kvt::Workspace ws{};
-  ws.hist = reinterpret_cast<uint32_t*>(base + kOffHist);
-  ws.sel = reinterpret_cast<kvt::SelectScalars*>(base + kOffSel);
-  ws.status = d_status ? d_status : reinterpret_cast<uint32_t*>(base + kOffStatus);
-  ws.tile_counts = reinterpret_cast<uint2*>(base + kOffTileCounts);
-  ws.tile_offsets = reinterpret_cast<uint2*>(base + kOffTileOffsets);
+  ws.hist = scratch->hist;
+  ws.sel = &scratch->sel;
+  ws.status = d_status ? d_status : scratch->status;
+  ws.tile_counts = scratch->tile_counts;
+  ws.tile_offsets = scratch->tile_offsets;
   ws.n_tiles = (uint32_t)kStaticMaxTiles;
+  ws.turns = scratch->turns;
+  ws.table = scratch->table;
+  ws.table_words = sizeof(scratch->table) / sizeof(scratch->table[0]);
+  ws.keep_hint = false;   // the next call may be about other scores altogether
   kvt::EntryState st{};
   st.score = const_cast<float*>(d_score);   // selection only reads score and state
   st.state = const_cast<uint8_t*>(d_state);

@@ -142,11 +142,12 @@ constexpr uint32_t kPrefetchWindowCap = 65535;      // default cap on a window, 
 struct Layout {
   uint64_t head_imp, head_mult, head_w;
   uint64_t pf_span, pf_win, pf_counts;
-  uint64_t delta, hist, sel, status, blend, block_score, block_state, block_victims, part_counts, tile_counts, tile_offsets, free_list, slot_list[kListBufs];
+  uint64_t delta, hist, sel, status, blend, block_score, block_state, block_victims, part_counts, tile_counts, tile_offsets, turns, table, free_list, slot_list[kListBufs];
   uint64_t ring[4][6];
   uint64_t dev_total;
   uint64_t h_list[kListBufs], h_counts, h_status, h_sel_stats, host_total;
   uint32_t n_tiles;
+  uint64_t table_words;
 };
 
 struct Derived {
@@ -227,6 +228,9 @@ void make_layout(const kv_pool_desc* d, const Derived& g, Layout* L) {
   L->part_counts = take(4 * 8);
   L->tile_counts = take((uint64_t)L->n_tiles * 8);
   L->tile_offsets = take((uint64_t)L->n_tiles * 8);
+  L->turns = take(2 * sizeof(SelectTurn));
+  L->table_words = select_table_words(g.N);   // (a pool has no more blocks than entries)
+  L->table = take(L->table_words * 8);
   L->free_list = take((g.N + 4096) * 4);   // (the selection's note scratch is addressed by whole chunks of 4,096)
   for (int b = 0; b < kListBufs; ++b) L->slot_list[b] = take(d->max_promote * 4);
   for (int q = 0; q < g.n_parts; ++q) {
@@ -528,6 +532,9 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
   p->ws.free_list = reinterpret_cast<uint32_t*>(w + L.free_list);
   for (int b = 0; b < kListBufs; ++b) p->ws.slot_list[b] = reinterpret_cast<uint32_t*>(w + L.slot_list[b]);
   p->ws.n_tiles = L.n_tiles;
+  p->ws.turns = reinterpret_cast<SelectTurn*>(w + L.turns);
+  p->ws.table = reinterpret_cast<unsigned long long*>(w + L.table);
+  p->ws.table_words = L.table_words;
   uint8_t* hw = static_cast<uint8_t*>(desc->h_workspace);
   for (int b = 0; b < kListBufs; ++b) p->h_list[b] = reinterpret_cast<uint32_t*>(hw + L.h_list[b]);
   p->h_counts = reinterpret_cast<uint64_t*>(hw + L.h_counts);

@@ -87,27 +87,34 @@ struct SelectScalars {
   uint32_t tau;           // key of the k-th smallest entry
   unsigned long long k_rem;    // rank still to resolve inside the current bucket
   unsigned long long need_eq;  // how many entries with key == tau are taken
-  unsigned int bar_arrive;     // grid barrier of the persistent selection: arrivals
-  unsigned int bar_done;       // ... and CTAs that have left (the last one resets both)
+  uint32_t serial;             // number of the last persistent selection
   unsigned int update_ticket;  // blocks of the entry pass that have finished (the last one commits)
   unsigned int hint_valid;     // the persistent selection left a usable hint
   uint32_t hint_tau;           // where the next persistent selection centres its bracket ...
   uint32_t hint_last;          // (tau of the last one)
   unsigned long long hint_n;   // ... and the number of keys it ran over
-  unsigned long long below;    // keys below the bracket (accumulated per launch, cleared inside it)
   unsigned long long phase_ns[16]; // %globaltimer at the phase boundaries of the last persistent selection (CTA 0)
   // how the persistent selections went so far (kv_selection_stats)
   unsigned int n_select;       // selections run
   unsigned int n_hint_hit;     // ... whose hint's bracket held rank k
   unsigned int n_hint_miss;    // ... whose hint's bracket did not
   unsigned int n_reread;       // CTAs (over all selections) that had to re-read their keys although the hint held
-  // persistent selection on a pool of several partitions: (below tau, equal to tau) counts of
-  // the entries before partition boundary q + 1 inside the slice of the CTA that holds it
-  uint2 bsplit[3];
+  // persistent selection on a pool of several partitions: launch number | victims before
+  // partition boundary q + 1, written by the CTA that holds it
+  unsigned long long bound[3];
   // width of the next selection's bracket: its 2,048 bins are 2^hint_shift keys wide (7..11);
   // hint_resid is a slowly decaying maximum of how far tau landed from where the hint put it
   uint32_t hint_shift;
   uint32_t hint_resid;
+};
+
+// What the CTAs of one persistent selection share while it runs.  Two of these are used in turn:
+// a launch finds its own zeroed and clears the next launch's.
+struct SelectTurn {
+  unsigned int bar;             // arrivals at the grid barrier
+  unsigned int pad;
+  unsigned long long below;     // keys below the bracket
+  uint32_t hist[4][kHistBins];  // the bracket's bins, then its last bin's keys or the radix select's digits
 };
 
 // Sliding window of per-epoch (pair, hit) counts for the confidence-weighted
@@ -173,7 +180,7 @@ struct Workspace {
   uint8_t* block_state;     // [blocks] RESIDENT iff every head of the block is
   uint32_t* block_victims;  // [blocks] selected global block indices
   unsigned long long* delta;   // [32] per-epoch (pair, hit) counts: index pair*2+hit
-  uint32_t* hist;              // [3][kHistBins]
+  uint32_t* hist;              // [3][kHistBins], zero between selections
   SelectScalars* sel;
   uint32_t* status;            // device status word
   uint2* tile_counts;          // [n_tiles] (less, equal) or (free, 0)
@@ -182,6 +189,11 @@ struct Workspace {
   uint32_t* slot_list[8];      // [max_promote] promote lists (ring slots), used in turn
   unsigned long long* part_counts;  // [4] victims per partition
   uint32_t n_tiles;
+  // persistent selection
+  SelectTurn* turns;                // [2], used in turn
+  unsigned long long* table;        // [table_words] counts per chunk, tagged with the launch's number
+  uint64_t table_words;
+  bool keep_hint = true;            // selections start from the threshold of the one before
   // One of the state arrays kept in the persisting part of the L2 (kv_set_l2_residency):
   // the scoring kernels are launched with this access-policy window.  bytes == 0: none.
   const void* l2_base = nullptr;
@@ -257,6 +269,9 @@ struct PartCounts {
   unsigned long long* d_counts = nullptr;   // [4]
   unsigned long long* h_counts = nullptr;   // [4] device-visible address of pinned host memory
 };
+// Words of the persistent selection's table of counts for n entries: one per chunk of 4,096 entries
+// of every CTA, the last row's pieces counted as chunks (at most 1,024 CTAs).
+inline uint64_t select_table_words(uint64_t n) { return n / 4096 + 1024; }
 // variant 1 = one persistent cooperative launch (falls back to 0 where the device cannot run
 // it or the slices are too long), 0 = one launch per phase of the radix select
 cudaError_t launch_select(const EntryState& st, uint64_t k, uint32_t* d_victims, const Workspace& ws,
