@@ -6,14 +6,14 @@
 namespace kvt {
 
 // ---- event reduction ---------------------------------------------------------
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kEventThreads, kEventBlocksPerSm)
 event_reduce_kernel(const uint32_t* __restrict__ ev_entry, const uint8_t* __restrict__ ev_hit,
                     uint64_t n_events, const uint8_t* __restrict__ pair,
                     uint32_t* __restrict__ touch, uint64_t n,
                     unsigned long long* __restrict__ delta, uint32_t* __restrict__ status) {
-  __shared__ uint32_t s_cnt[16 * kThreads];   // [pair][thread]: events | hits << 16
-  for (uint32_t i = threadIdx.x; i < 16 * kThreads; i += kThreads) s_cnt[i] = 0;
-  __syncthreads();
+  __shared__ uint32_t s_cnt[16 * kEventThreads];   // [pair][thread]: events | hits << 16
+#pragma unroll
+  for (uint32_t i = 0; i < 16; ++i) s_cnt[i * kEventThreads + threadIdx.x] = 0;   // (the thread's own words)
   const uint32_t bad = reduce_events(ev_entry, ev_hit, n_events, pair, touch, n,
                                      (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
                                      (uint64_t)gridDim.x * blockDim.x, s_cnt, delta);
@@ -23,9 +23,9 @@ event_reduce_kernel(const uint32_t* __restrict__ ev_entry, const uint8_t* __rest
 cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events,
                                 const EntryState& st, const Workspace& ws, cudaStream_t s) {
   if (n_events == 0) return cudaSuccess;
-  uint64_t blocks = (n_events / 4 + kThreads - 1) / kThreads;
+  uint64_t blocks = (n_events / 4 + kEventThreads - 1) / kEventThreads;
   if (blocks == 0) blocks = 1;
-  const uint64_t cap = (uint64_t)sm_count() * 4;  // measured: 4 blocks per SM beat 8 and 2
+  const uint64_t cap = (uint64_t)sm_count() * kEventBlocksPerSm;
   if (blocks > cap) blocks = cap;
   const uint8_t* pair = st.pair;
   uint32_t* touch = st.touch;
@@ -34,7 +34,7 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   uint32_t* status = ws.status;
   void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &n, &delta, &status};
   const cudaError_t e = launch_scoring_kernel((const void*)event_reduce_kernel, dim3((unsigned)blocks),
-                                              dim3(kThreads), args, 0, s, false, ws);
+                                              dim3(kEventThreads), args, 0, s, false, ws);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -50,10 +50,10 @@ entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights h
   __shared__ float sP[16];
   __shared__ bool s_last;
   const int policy = pd.policy;
+  PairStep step;
   if (threadIdx.x < 16) {
-    unsigned long long h, m, wh, wm;
-    const float P = posterior(pd, threadIdx.x, h, m);
-    sP[threadIdx.x] = reuse_estimate(pd, threadIdx.x, P, h, m, wh, wm);
+    step = pair_step(pd, threadIdx.x);
+    sP[threadIdx.x] = step.estimate;
   }
   __syncthreads();
   const uint64_t n4 = st.n / 4;
@@ -83,7 +83,7 @@ entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights h
   }
   __syncthreads();
   if (s_last && threadIdx.x < 16) {
-    commit_predictor(pd, threadIdx.x);
+    commit_predictor(pd, threadIdx.x, step);
     if (threadIdx.x == 0) *pd.ticket = 0;
   }
 }

@@ -12,8 +12,8 @@ namespace kvt {
 
 // ---- event reduction ---------------------------------------------------------
 // Each event adds one to the (pair, hit) counter of its entry's pair -- the
-// alpha += 1 / beta += 1 update of the Bayesian reuse section -- and one to the
-// entry's touch count.  Counters are integers, so the order of the additions
+// alpha += 1 / beta += 1 update of the Bayesian reuse section -- and one to
+// the entry's touch count.  Counters are integers, so the order of the additions
 // does not matter.
 //
 // Pair counters: every thread owns 16 packed counters in shared memory (one per
@@ -32,14 +32,20 @@ namespace kvt {
 // Traces in which a touched block reports all its heads hand every thread four
 // consecutive entries (an aligned group of four ids): one 4-byte load then
 // fetches their pairs and FREE bits, and two atomics count the four touches.
-constexpr uint32_t kEventVecs = 2;          // 4-event vectors a thread has in flight per iteration
+// Those two go out from neighbouring lanes of one instruction, so that a 32-byte
+// sector of counts is visited once and not twice.
+//
+// What bounds it: the latency of two dependent scattered reads (event, pair byte) and
+// the rate of the atomics.  The next vectors' events are on their way while the current
+// ones' pair bytes are fetched.
+constexpr uint32_t kEventThreads = 512;
+constexpr uint32_t kEventBlocksPerSm = 2;
+constexpr uint32_t kEventVecs = 2;          // 4-event vectors a thread handles per iteration
 constexpr uint32_t kEventFlushIters = 4096; // iterations between flushes: 8 events each, below 2^16
 
 struct EventVec {
-  uint32_t id[4];
-  uint32_t hit4;   // bit 8j+7 set: event j carried a hit flag
-  uint32_t pr4;    // byte j: pair byte of event j's entry (bit 7 = FREE or out of range)
-  bool valid, run; // vector inside the trace; ids are an aligned run of four inside the pool
+  uint4 id;
+  uint32_t hit;    // byte j: hit flag of event j
 };
 
 // bit 7 of every non-zero byte
@@ -56,8 +62,8 @@ __device__ __forceinline__ void touch_add(uint32_t* __restrict__ touch, uint32_t
     atomicAdd(&touch[i], 1u);   // last entry of an odd-length array (i is even, inc_pair is 1)
 }
 
-// The calling block's share of the events.  s_cnt: kThreads * 16 words of shared
-// memory, zero on entry; on return word [p * blockDim.x + t] holds thread t's
+// The calling block's share of the events.  s_cnt: kEventThreads * 16 words of shared
+// memory, zero on entry; word [p * kEventThreads + t] holds thread t's
 // counts for pair p (events | hits << 16) since the last flush.  delta: the 32
 // global epoch counters (index 2 * pair + hit).  Returns the KV_DEV_* bits of
 // refused events.  Every thread of the block must call it.
@@ -71,8 +77,9 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* __restrict__ e
   const uint64_t iters = (n4 + stride * kEventVecs - 1) / (stride * kEventVecs);  // same for every thread
   // ids are 32-bit, so the bound is too (an id can never reach 2^32 - 1 = "no entry")
   const uint32_t n32 = n > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)n;
+  const uint32_t lane = threadIdx.x & 31u;
   uint32_t* my = s_cnt + threadIdx.x;
-  const uint32_t col = blockDim.x;
+  constexpr uint32_t col = kEventThreads;
   bool bad_id = false, not_resident = false;
 
   // adds the block's columns to the global counters and clears them; the 32 sums
@@ -80,20 +87,18 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* __restrict__ e
   auto flush = [&]() {
     __shared__ uint32_t s_tot[32];
     __syncthreads();
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = blockDim.x >> 5;
-    for (uint32_t p = warp; p < 16; p += n_warps) {
+    const uint32_t warp = threadIdx.x >> 5;
+    for (uint32_t p = warp; p < 16; p += kEventThreads / 32) {
       uint32_t ev = 0, hi = 0;
-      for (uint32_t t = lane; t < col; t += 32) {
-        const uint32_t c = s_cnt[p * col + t];
-        s_cnt[p * col + t] = 0;
+#pragma unroll
+      for (uint32_t t = 0; t < col; t += 32) {
+        const uint32_t c = s_cnt[p * col + t + lane];
+        s_cnt[p * col + t + lane] = 0;
         ev += c & 0xFFFFu;
         hi += c >> 16;
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        ev += __shfl_xor_sync(0xFFFFFFFFu, ev, o);
-        hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-      }
+      ev = __reduce_add_sync(0xFFFFFFFFu, ev);
+      hi = __reduce_add_sync(0xFFFFFFFFu, hi);
       if (lane == 0) {
         s_tot[2 * p + 1] = hi;
         s_tot[2 * p] = ev - hi;
@@ -106,70 +111,83 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* __restrict__ e
   };
   // counts event j of a vector (pair byte and hit bit already extracted)
   auto count = [&](uint32_t prj, uint32_t hitbit) { my[(prj & 15u) * col] += 1u + (hitbit << 16); };
-
-  for (uint64_t it = 0; it < iters; ++it) {
-    EventVec x[kEventVecs];
-#pragma unroll
-    for (uint32_t u = 0; u < kEventVecs; ++u) {  // all event loads first
-      const uint64_t v = (it * kEventVecs + u) * stride + gtid;
-      x[u].valid = v < n4;
-      uint4 id4 = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);  // past the end: out of range
-      uint32_t h4 = 0;
-      if (x[u].valid) {
-        id4 = reinterpret_cast<const uint4*>(ev_entry)[v];
-        h4 = reinterpret_cast<const uint32_t*>(ev_hit)[v];
-      }
-      x[u].id[0] = id4.x; x[u].id[1] = id4.y; x[u].id[2] = id4.z; x[u].id[3] = id4.w;
-      x[u].hit4 = nonzero_bytes(h4);
-      x[u].run = !(id4.x & 3u) && id4.y == id4.x + 1u && id4.z == id4.x + 2u && id4.w == id4.x + 3u &&
-                 id4.w < n32;
-    }
-#pragma unroll
-    for (uint32_t u = 0; u < kEventVecs; ++u) {  // then all gathers, before any is used
-      if (x[u].run) {
-        x[u].pr4 = *reinterpret_cast<const uint32_t*>(pair + x[u].id[0]);
-      } else {
-        uint32_t pr4 = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          pr4 |= (uint32_t)(x[u].id[j] < n32 ? pair[x[u].id[j]] : (uint8_t)kPairFree) << (8 * j);
-        x[u].pr4 = pr4;
-      }
-    }
+  auto load = [&](uint64_t it, EventVec x[kEventVecs]) {
 #pragma unroll
     for (uint32_t u = 0; u < kEventVecs; ++u) {
-      const uint32_t pr4 = x[u].pr4, hit4 = x[u].hit4;
-      if (x[u].run && !(pr4 & 0x80808080u)) {
-        // four resident entries in a row: two atomics, four counts
-        unsigned long long* t2 = reinterpret_cast<unsigned long long*>(touch + x[u].id[0]);
-        atomicAdd(t2, 0x100000001ull);
-        atomicAdd(t2 + 1, 0x100000001ull);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) count(pr4 >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);
-        continue;
+      const uint64_t v = (it * kEventVecs + u) * stride + gtid;
+      x[u].id = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);  // past the end: no entry
+      x[u].hit = 0;
+      if (v < n4) {
+        x[u].id = __ldcs(reinterpret_cast<const uint4*>(ev_entry) + v);
+        x[u].hit = __ldcs(reinterpret_cast<const uint32_t*>(ev_hit) + v);
       }
-      if (!x[u].valid) continue;
-      bool ok[4];
+    }
+  };
+
+  EventVec nxt[kEventVecs];
+  if (iters) load(0, nxt);
+  for (uint64_t it = 0; it < iters; ++it) {
+    EventVec cur[kEventVecs];
+    bool run[kEventVecs];       // ids are an aligned run of four inside the pool
+    uint32_t pr4[kEventVecs];   // byte j: pair byte of event j's entry (bit 7 = FREE or out of range)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool in = x[u].id[j] < n32;
-        ok[j] = !((pr4 >> (8 * j)) & kPairFree);   // (out of range gathered nothing: FREE)
-        bad_id |= !in;
-        not_resident |= in && !ok[j];
+    for (uint32_t u = 0; u < kEventVecs; ++u) cur[u] = nxt[u];
+#pragma unroll
+    for (uint32_t u = 0; u < kEventVecs; ++u) {  // all gathers before any is used
+      const uint32_t id[4] = {cur[u].id.x, cur[u].id.y, cur[u].id.z, cur[u].id.w};
+      run[u] = !(id[0] & 3u) && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u && id[3] < n32;
+      if (run[u]) {
+        pr4[u] = *reinterpret_cast<const uint32_t*>(pair + id[0]);
+      } else {
+        uint32_t w = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w |= (uint32_t)(id[j] < n32 ? pair[id[j]] : (uint8_t)kPairFree) << (8 * j);
+        pr4[u] = w;
       }
+    }
+    if (it + 1 < iters) load(it + 1, nxt);
 #pragma unroll
-      for (int j = 0; j < 4; j += 2) {
-        const uint32_t i0 = x[u].id[j], i1 = x[u].id[j + 1];
-        if (ok[j] && ok[j + 1] && i1 == i0 + 1u && !(i0 & 1u)) {
-          atomicAdd(reinterpret_cast<unsigned long long*>(touch + i0), 0x100000001ull);
-        } else {
-          if (ok[j]) touch_add(touch, i0, n32, (i0 & 1u) ? (1ull << 32) : 1ull);
-          if (ok[j + 1]) touch_add(touch, i1, n32, (i1 & 1u) ? (1ull << 32) : 1ull);
+    for (uint32_t u = 0; u < kEventVecs; ++u) {
+      const uint32_t id[4] = {cur[u].id.x, cur[u].id.y, cur[u].id.z, cur[u].id.w};
+      const uint32_t pr = pr4[u], hit4 = nonzero_bytes(cur[u].hit);
+      const bool whole = run[u] && !(pr & 0x80808080u);   // four resident entries in a row
+      const uint32_t m = __ballot_sync(0xFFFFFFFFu, whole);
+      if (m) {
+#pragma unroll
+        for (uint32_t half = 0; half < 2; ++half) {   // 16 vectors' pairs of atomics per instruction
+          const uint32_t src = 16u * half + (lane >> 1);
+          const uint32_t i0 = __shfl_sync(0xFFFFFFFFu, id[0], src);
+          if ((m >> src) & 1u)
+            atomicAdd(reinterpret_cast<unsigned long long*>(touch + i0) + (lane & 1u), 0x100000001ull);
         }
       }
+      if (whole) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (ok[j]) count(pr4 >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);
+        for (int j = 0; j < 4; ++j) count(pr >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);
+      } else if ((it * kEventVecs + u) * stride + gtid < n4) {
+        bool ok[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool in = id[j] < n32;
+          ok[j] = !((pr >> (8 * j)) & kPairFree);   // (out of range gathered nothing: FREE)
+          bad_id |= !in;
+          not_resident |= in && !ok[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j += 2) {
+          const uint32_t i0 = id[j], i1 = id[j + 1];
+          if (ok[j] && ok[j + 1] && i1 == i0 + 1u && !(i0 & 1u)) {
+            atomicAdd(reinterpret_cast<unsigned long long*>(touch + i0), 0x100000001ull);
+          } else {
+            if (ok[j]) touch_add(touch, i0, n32, (i0 & 1u) ? (1ull << 32) : 1ull);
+            if (ok[j + 1]) touch_add(touch, i1, n32, (i1 & 1u) ? (1ull << 32) : 1ull);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (ok[j]) count(pr >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);
+      }
+      __syncwarp();
     }
     if ((it + 1) % kEventFlushIters == 0) flush();   // (uniform over the block)
   }
@@ -286,25 +304,39 @@ __device__ __forceinline__ float posterior(const Predictor& pd, unsigned p, unsi
   return __fdiv_rn(a, __fadd_rn(a, b));
 }
 
-// End of an epoch, run by lanes 0..15 of one warp (p = lane) once every block
-// has read the counters: folds the epoch's counts into the totals, publishes P
-// and the estimate, advances the blend's window and clears the counts.
-__device__ __forceinline__ void commit_predictor(const Predictor& pd, unsigned p) {
-  unsigned long long h, m, wh, wm;
-  const float P = posterior(pd, p, h, m);
-  const float est = reuse_estimate(pd, p, P, h, m, wh, wm);
-  pd.hits[p] = h;
-  pd.misses[p] = m;
-  pd.P[p] = P;
-  pd.blend->estimate[p] = est;
-  const uint32_t head = pd.blend->head;
-  __syncwarp(0xFFFFu);  // all 16 lanes have read the head and the expiring window slot
+// What a scoring pass makes of one pair's counters: formed at its start by every block, and
+// stored at its end by one of them (from here, without reading the counters again).
+struct PairStep {
+  unsigned long long h, m, wh, wm;   // totals and window sums with this epoch's counts
+  unsigned long long d0, d1;         // this epoch's counts
+  float P, estimate;
+  uint32_t head;                     // window slot that this epoch takes
+};
+
+__device__ __forceinline__ PairStep pair_step(const Predictor& pd, unsigned p) {
+  PairStep x;
+  x.P = posterior(pd, p, x.h, x.m);
+  x.estimate = reuse_estimate(pd, p, x.P, x.h, x.m, x.wh, x.wm);
+  x.d0 = __ldcg(&pd.delta[2 * p]);
+  x.d1 = __ldcg(&pd.delta[2 * p + 1]);
+  x.head = pd.window ? pd.blend->head : 0u;
+  return x;
+}
+
+// End of an epoch, p = 0..15, once every block has read the counters: folds the epoch's
+// counts into the totals, publishes P and the estimate, advances the blend's window and
+// clears the counts.
+__device__ __forceinline__ void commit_predictor(const Predictor& pd, unsigned p, const PairStep& x) {
+  pd.hits[p] = x.h;
+  pd.misses[p] = x.m;
+  pd.P[p] = x.P;
+  pd.blend->estimate[p] = x.estimate;
   if (pd.window > 0) {   // this epoch's counts replace the oldest slot of the window
-    pd.blend->win[head * 32 + 2 * p] = __ldcg(&pd.delta[2 * p]);
-    pd.blend->win[head * 32 + 2 * p + 1] = __ldcg(&pd.delta[2 * p + 1]);
-    pd.blend->wsum[2 * p] = wm;
-    pd.blend->wsum[2 * p + 1] = wh;
-    if (p == 0) pd.blend->head = (head + 1) % pd.window;
+    pd.blend->win[x.head * 32 + 2 * p] = x.d0;
+    pd.blend->win[x.head * 32 + 2 * p + 1] = x.d1;
+    pd.blend->wsum[2 * p] = x.wm;
+    pd.blend->wsum[2 * p + 1] = x.wh;
+    if (p == 0) pd.blend->head = (x.head + 1) % pd.window;
   }
   pd.delta[2 * p] = 0;
   pd.delta[2 * p + 1] = 0;

@@ -206,6 +206,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   __shared__ uint2 s_rowtot[kPMaxRows];               // (below, equal) of a row over all CTAs ...
   __shared__ uint2 s_colpre[kPMaxRows];               // ... and over the CTAs before this one
   __shared__ float sP[16];
+  __shared__ PairStep s_pair[FUSED ? 16 : 1];
   const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t G = gridDim.x, g = blockIdx.x;
@@ -269,9 +270,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     // reuse estimates from the totals plus this epoch's counts (final: the event
     // reduction is an earlier launch)
     if (t < 16) {
-      unsigned long long h, m, wh, wm;
-      const float P = posterior(a.pd, t, h, m);
-      sP[t] = reuse_estimate(a.pd, t, P, h, m, wh, wm);
+      s_pair[t] = pair_step(a.pd, t);
+      sP[t] = s_pair[t].estimate;
     }
   }
   for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
@@ -304,6 +304,17 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     else if (my_spill) my_spill[at - a.note_cap] = note;   // (a dense slice: the rest goes to L2)
   };
   auto note_get = [&](uint32_t at) { return at < a.note_cap ? my_note[at] : __ldcg(my_spill + (at - a.note_cap)); };
+  // The histograms and the table were written a pass ago and have left the L2 since: fetch their
+  // lines while the last rows are worked on (a miss inside an exchange cost 1-4 us).
+  auto warm_lines = [&]() {
+    constexpr uint32_t kTurnLines = (sizeof(SelectTurn) + 127u) / 128u;
+    const uint32_t lines = kTurnLines + (n_rows * G * 8u + 127u) / 128u;
+    for (uint32_t l = t * G + g; l < lines; l += kPThreads * G) {
+      const char* p = l < kTurnLines ? reinterpret_cast<const char*>(turn) + 128u * l
+                                     : reinterpret_cast<const char*>(a.table) + 128u * (l - kTurnLines);
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    }
+  };
   // (row r, the thread's four scores): the below bits, and a note for each key inside the bracket
   auto classify = [&](uint32_t r, const float s[4]) {
     if (lane == 0) my_nstart[r] = n_noted;
@@ -361,10 +372,13 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
           }
         }
       }
+      if (r + 2u == n_rows || n_rows == 1u) warm_lines();
       classify(r, s);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-  } else if (hint) {
+  } else if (!hint) {
+    warm_lines();
+  } else {
     // (two rows' loads in flight)
     float4 sc[2];
     uint32_t st4[2];
@@ -377,6 +391,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     };
     load(0, 0);
     load(1, 1);
+    warm_lines();
     for (uint32_t r = 0; r < n_rows; r += 2) {
 #pragma unroll
       for (uint32_t u = 0; u < 2; ++u) {
@@ -620,7 +635,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     if constexpr (FUSED) {
       // every CTA has long formed its estimates: the epoch's counts can be folded in (here, where
       // the CTA waits for the others anyway)
-      if (g == 0 && t >= kPThreads - 32u && lane < 16u) commit_predictor(a.pd, lane);
+      if (g == 0 && t >= kPThreads - 32u && lane < 16u) commit_predictor(a.pd, lane, s_pair[lane]);
     }
     for (uint32_t r = warp; r < n_rows; r += kPWarps) {
       uint32_t tl = 0, te = 0, pl = 0, pe = 0;
