@@ -142,7 +142,6 @@ __global__ void init_scalars_kernel(uint64_t* hits, uint64_t* misses, float* P, 
   if (t == 0) { ws.blend->head = 0; ws.blend->pad = 0; }
   for (uint32_t b = t; b < 3 * kHistBins; b += blockDim.x) ws.hist[b] = 0;
   for (uint32_t w = t; w < 2 * sizeof(SelectTurn) / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(ws.turns)[w] = 0;
-  for (uint64_t w = t; w < ws.table_words; w += blockDim.x) ws.table[w] = 0;
   if (t < 4) ws.part_counts[t] = 0;
   if (t == 0) {
     *ws.status = 0;

@@ -429,7 +429,7 @@ struct StaticScratch {
   uint32_t status[4];
   uint2 tile_counts[kStaticMaxTiles];
   uint2 tile_offsets[kStaticMaxTiles];
-  unsigned long long table[kStaticMaxEntries / 4096 + 1024];
+  uint32_t table[kStaticMaxEntries / 4096 + 1024];
 };
 
 static __device__ __align__(256) unsigned char g_select_scratch[sizeof(StaticScratch)];

@@ -29,10 +29,11 @@
 //
 // What bounds it: phase A streams 22-30 B an entry from HBM; B to D are three exchanges
 // between all CTAs (two histograms, one table of counts) of ~2.5 us each, latency of L2
-// and of the block barriers around them.  The first two exchanges are grid barriers (a
-// counter that every CTA increments and polls); the third has no barrier of its own:
-// the table's words carry the launch's number, and a reader polls the words it needs.
-// A cooperative launch guarantees that all CTAs are resident, so every wait ends; all
+// and of the block barriers around them.  An exchange is a grid barrier (a counter that
+// every CTA increments and one of its threads polls).  (Tried for the third one: no
+// barrier, every reader polls the table's words for the launch's number.  With 148 CTAs
+// the polls of a thousand words each crowd out the stores they wait for: 5.0 us where
+// barrier and one reading take 2.5.)  A cooperative launch guarantees that all CTAs are resident, so every wait ends; all
 // are bounded nevertheless, and a CTA that gives up sets KV_DEV_WAIT_EXPIRED and leaves
 // (every other CTA then runs into the same limit).  Barrier and histograms come in two
 // sets used in turn; a launch clears the set of the next one.  The launch's number, which
@@ -79,7 +80,7 @@ struct PArgs {
   uint32_t* victims;
   SelectScalars* sel;
   SelectTurn* turns;      // [2] barrier and histograms of this launch (zero on entry) and of the next
-  unsigned long long* table;   // [n_rows][G] counts of every chunk, tagged with the launch's number
+  uint32_t* table;        // [n_rows][G] counts of every chunk
   uint32_t use_hint;      // 0: plain radix select whatever an earlier selection left
   uint32_t* status;
   uint32_t n_full;        // full rows: chunks of 4,096 entries
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   // lines while the last rows are worked on (a miss inside an exchange cost 1-4 us).
   auto warm_lines = [&]() {
     constexpr uint32_t kTurnLines = (sizeof(SelectTurn) + 127u) / 128u;
-    const uint32_t lines = kTurnLines + (n_rows * G * 8u + 127u) / 128u;
+    const uint32_t lines = kTurnLines + (n_rows * G * 4u + 127u) / 128u;
     for (uint32_t l = t * G + g; l < lines; l += kPThreads * G) {
       const char* p = l < kTurnLines ? reinterpret_cast<const char*>(turn) + 128u * l
                                      : reinterpret_cast<const char*>(a.table) + 128u * (l - kTurnLines);
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     }
   }
   stamp(1);
-  // (number 0 marks an unused word of the table; the turns alternate across the wrap too)
+  // (number 0 marks a word never written; the turns alternate across the wrap too)
   auto end_turn = [&]() { a.sel->serial = tag == 0xFFFFFFFFu ? 1u : tag; };
   uint32_t nbar = 0;        // grid barriers passed
   bool ok = true, hint_hit = false;
@@ -629,31 +630,32 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     if (t < n_rows) {
       const uint4 v = reinterpret_cast<const uint4*>(s_wtot)[t];
       const uint32_t sum = v.x + v.y + v.z + v.w;   // at most 4,096 in either half
-      publish_word(&a.table[t * G + g], tag, (sum & 0xFFFFu) | (sum >> 16) << 13);
+      a.table[t * G + g] = (sum & 0xFFFFu) | (sum >> 16) << 13;
     }
+    grid_arrive(bar);
     stamp(5);
     if constexpr (FUSED) {
       // every CTA has long formed its estimates: the epoch's counts can be folded in (here, where
       // the CTA waits for the others anyway)
       if (g == 0 && t >= kPThreads - 32u && lane < 16u) commit_predictor(a.pd, lane, s_pair[lane]);
     }
+    ok = grid_wait(bar, ++nbar * G);
+    stamp(6);
+    if (!ok) goto fail;
     for (uint32_t r = warp; r < n_rows; r += kPWarps) {
       uint32_t tl = 0, te = 0, pl = 0, pe = 0;
       for (uint32_t c0 = 0; c0 < G; c0 += 160u) {
-        unsigned long long v[5];   // (loads in flight together; a word that is not there yet is polled)
+        uint32_t v[5];   // (loads in flight together)
 #pragma unroll
         for (uint32_t u = 0; u < 5u; ++u) {
           const uint32_t c = c0 + 32u * u + lane;
-          v[u] = c < G ? peek_word(&a.table[r * G + c]) : (unsigned long long)tag << 32;
+          v[u] = c < G ? __ldcg(&a.table[r * G + c]) : 0u;
         }
 #pragma unroll
         for (uint32_t u = 0; u < 5u; ++u) {
-          const uint32_t c = c0 + 32u * u + lane;
-          uint32_t x = (uint32_t)v[u];
-          if ((uint32_t)(v[u] >> 32) != tag) x = await_word(&a.table[r * G + c], tag, ok);
-          const uint32_t l = x & 0x1FFFu, e = x >> 13;
+          const uint32_t l = v[u] & 0x1FFFu, e = v[u] >> 13;
           tl += l; te += e;
-          if (c < g) { pl += l; pe += e; }
+          if (c0 + 32u * u + lane < g) { pl += l; pe += e; }
         }
       }
       tl = __reduce_add_sync(0xFFFFFFFFu, tl);
@@ -662,9 +664,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       pe = __reduce_add_sync(0xFFFFFFFFu, pe);
       if (lane == 0) { s_rowtot[r] = make_uint2(tl, te); s_colpre[r] = make_uint2(pl, pe); }
     }
-    ok = __syncthreads_and(ok) != 0;
-    stamp(6);
-    if (!ok) goto fail;
+    __syncthreads();
     // ---- phase D: where this CTA's chunks start, and the ordered write ----
     // Lane r of every warp: what the pool holds before this CTA's chunk of row r (and of row r + 32).
     uint32_t all_l, all_e, rl0, re0, rl1 = 0, re1 = 0;
@@ -742,7 +742,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         }
         if (!ok) atomicOr(a.status, KV_DEV_WAIT_EXPIRED);
       }
-      end_turn();   // (every CTA has published its counts, so every CTA has read the number)
+      end_turn();   // (every CTA has read the number long ago)
       a.sel->tau = tau;
       a.sel->need_eq = need_eq;
       a.sel->n_select += 1;

@@ -230,7 +230,7 @@ void make_layout(const kv_pool_desc* d, const Derived& g, Layout* L) {
   L->tile_offsets = take((uint64_t)L->n_tiles * 8);
   L->turns = take(2 * sizeof(SelectTurn));
   L->table_words = select_table_words(g.N);   // (a pool has no more blocks than entries)
-  L->table = take(L->table_words * 8);
+  L->table = take(L->table_words * 4);
   L->free_list = take((g.N + 4096) * 4);   // (the selection's note scratch is addressed by whole chunks of 4,096)
   for (int b = 0; b < kListBufs; ++b) L->slot_list[b] = take(d->max_promote * 4);
   for (int q = 0; q < g.n_parts; ++q) {
@@ -533,7 +533,7 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
   for (int b = 0; b < kListBufs; ++b) p->ws.slot_list[b] = reinterpret_cast<uint32_t*>(w + L.slot_list[b]);
   p->ws.n_tiles = L.n_tiles;
   p->ws.turns = reinterpret_cast<SelectTurn*>(w + L.turns);
-  p->ws.table = reinterpret_cast<unsigned long long*>(w + L.table);
+  p->ws.table = reinterpret_cast<uint32_t*>(w + L.table);
   p->ws.table_words = L.table_words;
   uint8_t* hw = static_cast<uint8_t*>(desc->h_workspace);
   for (int b = 0; b < kListBufs; ++b) p->h_list[b] = reinterpret_cast<uint32_t*>(hw + L.h_list[b]);

@@ -191,7 +191,7 @@ struct Workspace {
   uint32_t n_tiles;
   // persistent selection
   SelectTurn* turns;                // [2], used in turn
-  unsigned long long* table;        // [table_words] counts per chunk, tagged with the launch's number
+  uint32_t* table;                  // [table_words] counts per chunk
   uint64_t table_words;
   bool keep_hint = true;            // selections start from the threshold of the one before
   // One of the state arrays kept in the persisting part of the L2 (kv_set_l2_residency):
