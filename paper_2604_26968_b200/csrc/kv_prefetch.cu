@@ -13,11 +13,13 @@
 // head), the ring slot of every block of the sequence's block table at distance < w[l]
 // that sits in the host tier.
 //
-// The list is an ordered compaction of at most distance x layers x heads candidates.
-// Two launches over the same chunks: the first counts the qualifying candidates of each
-// chunk, the second sums the counts before its chunk and writes.  No block waits on
-// another; the block table is read coalesced, d_loc by gather (both passes; the second
-// finds it in L2).
+// The list is an ordered compaction of at most distance x layers x heads candidates, in one
+// launch: a block counts the qualifying candidates of its chunk, publishes the count, adds up
+// the counts of the blocks before it as they appear, and writes.  A block waits only for blocks
+// of lower index (bounded: one that gives up sets KV_DEV_WAIT_EXPIRED and leaves, and so do the
+// blocks behind it).  A call is latency: window, table and d_loc are three dependent reads of
+// about 0.7 us, the counts one more; a second launch for the writing cost as much again
+// (8 lists of 256 x 80 x 8 candidates: 110 -> 56 us).
 #include "kvtier_internal.cuh"
 
 namespace kvt {
@@ -44,6 +46,7 @@ __global__ void prefetch_window_kernel(float* __restrict__ span, uint32_t* __res
                                        const float* __restrict__ x, float d, float tokens, int mode,
                                        uint32_t layers, float block_tokens, uint32_t w_max,
                                        uint32_t* __restrict__ status) {
+  launch_dependents_and_wait();
   int bad = 0;
   if (mode == 0)
     for (uint32_t l = threadIdx.x; l < layers; l += blockDim.x) bad |= !span_ok(x[l]);
@@ -70,104 +73,171 @@ struct ListArgs {
   const uint32_t* loc;     // [n_tags]
   unsigned long long* out;
   unsigned long long* count;
-  uint32_t* chunk_counts;  // [gridDim.x]
+  unsigned long long* words;    // [gridDim.x] launch number << 32 | count of the chunk
+  uint32_t* serial;             // number of the last launch
+  uint32_t* status;
   unsigned long long n_items;   // candidates the host can bound: distances x L x H
-  unsigned long long chunk;     // candidates per block, a multiple of kPfThreads
+  unsigned long long chunk;     // candidates per block, a multiple of kPfTile
   unsigned long long pos0, max_out, n_tags;
   uint32_t layers, heads;
   int dir;
+  int vector;              // table rows are aligned vectors of four handles
 };
 
-// Ring slot of candidate i if it qualifies; candidates are numbered (distance, layer, head).
-__device__ __forceinline__ bool candidate(const ListArgs& a, unsigned long long i, uint32_t row,
-                                          uint32_t* slot) {
-  const unsigned long long dist = i / row;
-  const uint32_t r = (uint32_t)(i - dist * row);
-  if (dist >= __ldg(a.win + r / a.heads)) return false;
-  const unsigned long long pb = a.dir > 0 ? a.pos0 + dist : a.pos0 - dist;
-  const uint32_t t = __ldg(a.table + pb * row + r);
-  if (t >= a.n_tags) return false;
-  const uint32_t where = __ldg(a.loc + t);
-  if (where == KV_NONE || !(where & KV_LOC_HOST)) return false;
-  *slot = where & ~KV_LOC_HOST;
-  return true;
+constexpr uint32_t kPfPerThread = 4;                        // consecutive candidates of a thread
+constexpr uint32_t kPfTile = kPfThreads * kPfPerThread;
+constexpr uint32_t kPfWinCache = 1024;                      // layers whose windows a block keeps in shared memory
+constexpr uint32_t kPfSpins = 1u << 22;
+
+// Bits of the thread's four candidates i0 .. i0+3 that qualify, and their ring slots; candidates
+// are numbered (distance, layer, head).  Index: the type that holds every candidate's number.
+template <typename Index>
+__device__ __forceinline__ uint32_t candidates(const ListArgs& a, Index i0, Index end, uint32_t row,
+                                               const uint32_t* s_win, uint32_t s_wmax,
+                                               uint32_t slot[kPfPerThread]) {
+  if (i0 >= end) return 0u;
+  Index dist = i0 / (Index)row;
+  uint32_t r = (uint32_t)(i0 - dist * (Index)row), t[kPfPerThread], m = 0;
+  // (all reads go to the L2: the kernel ahead may have written any of the arrays while this
+  // block was already set up)
+  if (a.vector) {   // rows of a multiple of four handles: the four are one aligned vector
+    const unsigned long long pb = a.dir > 0 ? a.pos0 + dist : a.pos0 - dist;
+    uint4 v = make_uint4(KV_NONE, KV_NONE, KV_NONE, KV_NONE);
+    if (dist < (Index)s_wmax) v = __ldcg(reinterpret_cast<const uint4*>(a.table + pb * row + r));
+    t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+#pragma unroll
+    for (uint32_t u = 0; u < kPfPerThread; ++u) {
+      const uint32_t layer = (r + u) / a.heads;
+      const uint32_t w = layer < kPfWinCache ? s_win[layer] : __ldcg(a.win + layer);
+      if (dist >= (Index)w) t[u] = KV_NONE;
+    }
+  } else {
+#pragma unroll
+    for (uint32_t u = 0; u < kPfPerThread; ++u) {
+      const uint32_t layer = r / a.heads;
+      const uint32_t w = layer < kPfWinCache ? s_win[layer] : __ldcg(a.win + layer);
+      t[u] = KV_NONE;
+      if (i0 + (Index)u < end && dist < (Index)w) {
+        const unsigned long long pb = a.dir > 0 ? a.pos0 + dist : a.pos0 - dist;
+        t[u] = __ldcg(a.table + pb * row + r);
+      }
+      if (++r == row) { r = 0; ++dist; }
+    }
+  }
+#pragma unroll
+  for (uint32_t u = 0; u < kPfPerThread; ++u) {
+    slot[u] = KV_NONE;
+    if (t[u] < a.n_tags) slot[u] = __ldcg(a.loc + t[u]);   // (KV_NONE is never a handle)
+  }
+#pragma unroll
+  for (uint32_t u = 0; u < kPfPerThread; ++u) {
+    m |= (uint32_t)(slot[u] != KV_NONE && (slot[u] & KV_LOC_HOST)) << u;
+    slot[u] &= ~KV_LOC_HOST;
+  }
+  return m;
 }
 
-template <bool kWrite>
+template <typename Index>
 __global__ void __launch_bounds__(kPfThreads) prefetch_list_kernel(const ListArgs a) {
-  __shared__ unsigned long long s_red[kPfThreads / 32];
+  __shared__ uint32_t s_win[kPfWinCache];
+  __shared__ unsigned long long s_before[kPfThreads / 32];
   __shared__ uint32_t s_warp[kPfThreads / 32];
   __shared__ uint32_t s_wmax;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t row = a.layers * a.heads;
+  launch_dependents_and_wait();
+  const uint32_t tag = *a.serial + 1u;
 
   // the widest window bounds the distances any layer wants
   if (tid == 0) s_wmax = 0;
   __syncthreads();
   uint32_t wm = 0;
-  for (uint32_t l = tid; l < a.layers; l += kPfThreads) wm = max(wm, __ldg(a.win + l));
-  for (int o = 16; o > 0; o >>= 1) wm = max(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
+  for (uint32_t l = tid; l < a.layers; l += kPfThreads) {
+    const uint32_t w = __ldcg(a.win + l);
+    if (l < kPfWinCache) s_win[l] = w;
+    wm = max(wm, w);
+  }
+  wm = __reduce_max_sync(0xFFFFFFFFu, wm);
   if (lane == 0 && wm) atomicMax(&s_wmax, wm);
   __syncthreads();
-  const unsigned long long limit = min(a.n_items, (unsigned long long)s_wmax * row);
-  const unsigned long long c0 = (unsigned long long)blockIdx.x * a.chunk;
-  const unsigned long long c1 = min(c0 + a.chunk, limit);
+  const Index limit = (Index)min(a.n_items, (unsigned long long)s_wmax * row);
+  const Index c0 = (Index)blockIdx.x * (Index)a.chunk;
+  const Index c1 = (Index)min((unsigned long long)c0 + a.chunk, (unsigned long long)limit);   // (c0 >= c1: nothing)
 
-  if (!kWrite) {
-    uint32_t n = 0, slot;
-    for (unsigned long long i = c0 + tid; i < c1; i += kPfThreads) n += candidate(a, i, row, &slot);
-    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xFFFFFFFFu, n, o);
-    if (lane == 0) s_warp[warp] = n;
-    __syncthreads();
+  uint32_t n = 0, m = 0, slot[kPfPerThread];   // m, slot: the last tile's, all there is of a one-tile chunk
+  for (Index i = c0 + (Index)(tid * kPfPerThread), at = c0; at < c1; i += kPfTile, at += kPfTile) {
+    m = candidates<Index>(a, i, c1, row, s_win, s_wmax, slot);
+    n += (uint32_t)__popc(m);
+  }
+  n = __reduce_add_sync(0xFFFFFFFFu, n);
+  if (lane == 0) s_warp[warp] = n;
+  __syncthreads();
+  uint32_t mine = 0;
+#pragma unroll
+  for (int w = 0; w < kPfThreads / 32; ++w) mine += s_warp[w];
+  if (tid == 0)
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(a.words + blockIdx.x),
+                 "l"((unsigned long long)tag << 32 | mine)
+                 : "memory");
+
+  // candidates that qualify before this chunk
+  unsigned long long before = 0;
+  bool ok = true;
+  for (uint32_t b = tid; b < blockIdx.x; b += kPfThreads) {
+    unsigned long long v = 0;
+    uint32_t it = 0;
+    do {
+      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(a.words + b) : "memory");
+    } while ((uint32_t)(v >> 32) != tag && ++it < kPfSpins);
+    ok = ok && (uint32_t)(v >> 32) == tag;
+    before += (uint32_t)v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+  if (lane == 0) s_before[warp] = before;
+  ok = __syncthreads_and(ok) != 0;
+  if (!ok) {
     if (tid == 0) {
-      uint32_t s = 0;
-      for (int w = 0; w < kPfThreads / 32; ++w) s += s_warp[w];
-      a.chunk_counts[blockIdx.x] = s;
+      atomicOr(a.status, KV_DEV_WAIT_EXPIRED);
+      if (blockIdx.x == gridDim.x - 1) *a.serial = tag;
     }
     return;
   }
-
-  // candidates that qualify before this chunk (and, in block 0, in all chunks)
-  unsigned long long before = 0, all = 0;
-  for (uint32_t b = tid; b < gridDim.x; b += kPfThreads) {
-    const uint32_t c = a.chunk_counts[b];
-    all += c;
-    if (b < blockIdx.x) before += c;
-  }
-  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
-  if (lane == 0) s_red[warp] = before;
-  __syncthreads();
   unsigned long long offset = 0;
-  for (int w = 0; w < kPfThreads / 32; ++w) offset += s_red[w];
-  if (blockIdx.x == 0) {
-    __syncthreads();
-    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xFFFFFFFFu, all, o);
-    if (lane == 0) s_red[warp] = all;
-    __syncthreads();
-    if (tid == 0) {
-      unsigned long long s = 0;
-      for (int w = 0; w < kPfThreads / 32; ++w) s += s_red[w];
-      *a.count = s;
-    }
+#pragma unroll
+  for (int w = 0; w < kPfThreads / 32; ++w) offset += s_before[w];
+  if (blockIdx.x == gridDim.x - 1 && tid == 0) {
+    *a.count = offset + mine;
+    *a.serial = tag;   // (every block has published its count, so every block has read the number)
   }
 
-  for (unsigned long long base = c0; base < c1; base += kPfThreads) {   // block-uniform trip count
-    const unsigned long long i = base + tid;
-    uint32_t slot = 0;
-    const bool q = i < c1 && candidate(a, i, row, &slot);
-    const uint32_t m = __ballot_sync(0xFFFFFFFFu, q);
+  const bool one_tile = c0 < c1 && c1 - c0 <= (Index)kPfTile;
+  for (Index i = c0 + (Index)(tid * kPfPerThread), at = c0; at < c1; i += kPfTile, at += kPfTile) {
+    if (!one_tile) m = candidates<Index>(a, i, c1, row, s_win, s_wmax, slot);
+    uint32_t incl = (uint32_t)__popc(m);
+    const uint32_t own = incl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
     __syncthreads();                       // s_warp of the tile before has been read
-    if (lane == 0) s_warp[warp] = __popc(m);
+    if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
     uint32_t ahead = 0, total = 0;
+#pragma unroll
     for (int w = 0; w < kPfThreads / 32; ++w) {
       const uint32_t c = s_warp[w];
       if (w < (int)warp) ahead += c;
       total += c;
     }
-    if (q) {
-      const unsigned long long at = offset + ahead + __popc(m & ((1u << lane) - 1u));
-      if (at < a.max_out) a.out[at] = slot;
+    unsigned long long p = offset + ahead + (incl - own);
+#pragma unroll
+    for (uint32_t u = 0; u < kPfPerThread; ++u) {
+      if ((m >> u) & 1u) {
+        if (p < a.max_out) a.out[p] = slot[u];
+        ++p;
+      }
     }
     offset += total;
   }
@@ -177,23 +247,23 @@ __global__ void __launch_bounds__(kPfThreads) prefetch_list_kernel(const ListArg
 
 cudaError_t launch_prefetch_window(const PrefetchState& pf, int q, int mode, const float* x, float decay,
                                    float tokens, const Workspace& ws, cudaStream_t s) {
-  prefetch_window_kernel<<<1, 128, 0, s>>>(pf.span + pf.off[q], pf.win + pf.off[q], x, decay, tokens, mode,
-                                           pf.layers[q], (float)pf.block_tokens[q], pf.w_max[q], ws.status);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_overlapped(prefetch_window_kernel, 1u, 128u, s, pf.span + pf.off[q], pf.win + pf.off[q], x, decay,
+                           tokens, mode, pf.layers[q], (float)pf.block_tokens[q], pf.w_max[q], ws.status);
 }
 
 cudaError_t launch_prefetch_list(const PrefetchState& pf, int q, const uint32_t* table, uint64_t n_pos,
                                  uint64_t pos0, int dir, const uint32_t* loc, uint64_t n_tags,
                                  unsigned long long* out, uint64_t max_out, unsigned long long* count,
-                                 cudaStream_t s) {
+                                 const Workspace& ws, cudaStream_t s) {
   ListArgs a;
   a.table = table;
   a.win = pf.win + pf.off[q];
   a.loc = loc;
   a.out = out;
   a.count = count;
-  a.chunk_counts = pf.chunk_counts;
+  a.words = pf.words;
+  a.serial = pf.serial;
+  a.status = ws.status;
   a.layers = pf.layers[q];
   a.heads = pf.heads[q];
   a.dir = dir;
@@ -204,16 +274,20 @@ cudaError_t launch_prefetch_list(const PrefetchState& pf, int q, const uint32_t*
   uint64_t dists = n_pos == 0 ? 0 : (dir > 0 ? n_pos - pos0 : pos0 + 1);
   if (dists > pf.w_max[q]) dists = pf.w_max[q];
   a.n_items = dists * a.layers * a.heads;
-  uint64_t chunk = (a.n_items + kPrefetchChunks - 1) / kPrefetchChunks;
-  chunk = (chunk + kPfThreads - 1) / kPfThreads * kPfThreads;
-  if (chunk < 4 * kPfThreads) chunk = 4 * kPfThreads;
+  a.vector = (a.layers * a.heads) % 4 == 0 && (reinterpret_cast<uintptr_t>(table) & 15u) == 0;
+  // One tile of 1,024 candidates per block while two blocks per SM hold them all; beyond that
+  // blocks take several (and evaluate their candidates twice, the second time from the caches).
+  uint64_t most = (uint64_t)sm_count() * 2;
+  if (most > kPrefetchChunks) most = kPrefetchChunks;
+  uint64_t chunk = (a.n_items + most - 1) / most;
+  chunk = (chunk + kPfTile - 1) / kPfTile * kPfTile;
+  if (chunk == 0) chunk = kPfTile;
   a.chunk = chunk;
   uint64_t blocks = (a.n_items + chunk - 1) / chunk;
   if (blocks == 0) blocks = 1;
-  prefetch_list_kernel<false><<<(unsigned)blocks, kPfThreads, 0, s>>>(a);
-  prefetch_list_kernel<true><<<(unsigned)blocks, kPfThreads, 0, s>>>(a);
-  count_launches(2);
-  return cudaGetLastError();
+  // 32-bit numbers divide in a fifth of the instructions
+  if (a.n_items < 0x7FFFFFFFull) return launch_overlapped(prefetch_list_kernel<uint32_t>, (unsigned)blocks, kPfThreads, s, a);
+  return launch_overlapped(prefetch_list_kernel<unsigned long long>, (unsigned)blocks, kPfThreads, s, a);
 }
 
 }  // namespace kvt

@@ -220,7 +220,7 @@ void make_layout(const kv_pool_desc* d, const Derived& g, Layout* L) {
     for (int q = 0; q < g.n_parts; ++q) layers += g.layers[q];
     L->pf_span = take(layers * 4);
     L->pf_win = take(layers * 4);
-    L->pf_counts = take(kPrefetchChunks * 4);
+    L->pf_counts = take(kPrefetchChunks * 8 + 8);
   }
   L->block_score = take(g.n_blocks * 4);
   L->block_state = take(g.n_blocks);
@@ -610,7 +610,8 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
     PrefetchState& pf = p->prefetch;
     pf.span = reinterpret_cast<float*>(w + L.pf_span);
     pf.win = reinterpret_cast<uint32_t*>(w + L.pf_win);
-    pf.chunk_counts = reinterpret_cast<uint32_t*>(w + L.pf_counts);
+    pf.words = reinterpret_cast<unsigned long long*>(w + L.pf_counts);
+    pf.serial = reinterpret_cast<uint32_t*>(pf.words + kPrefetchChunks);
     uint32_t o = 0;
     for (int q = 0; q < 4; ++q) {
       const bool in = q < g.n_parts;
@@ -663,6 +664,7 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
     e = launch_init(p->st, desc->d_hits, desc->d_misses, desc->d_P, p0, desc->d_loc, desc->n_tags,
                     p->geom, p->n_parts, p->ws, S(stream));
     if (e == cudaSuccess) e = launch_head_init(p->head, p->n_head_imp, p->n_head_w, S(stream));
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->prefetch.words, 0, kPrefetchChunks * 8 + 8, S(stream));
     for (int q = 0; q < g.n_parts && e == cudaSuccess; ++q)
       e = launch_prefetch_window(p->prefetch, q, 1, nullptr, 0.0f, kPrefetchSpanTokens, p->ws, S(stream));
   }
@@ -782,7 +784,7 @@ int32_t kv_prefetch_list(kv_pool* p, int32_t q, const uint32_t* d_table, uint64_
   if (rc != KV_OK) return rc;
   KV_CUDA(p, launch_prefetch_list(p->prefetch, q, d_table, n_pos, pos0, direction, p->desc.d_loc, p->desc.n_tags,
                                   reinterpret_cast<unsigned long long*>(d_out_slots), max_out,
-                                  reinterpret_cast<unsigned long long*>(d_out_count), S(stream)));
+                                  reinterpret_cast<unsigned long long*>(d_out_count), p->ws, S(stream)));
   return KV_OK;
 }
 

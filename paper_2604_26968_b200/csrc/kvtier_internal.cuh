@@ -168,7 +168,8 @@ constexpr uint32_t kPrefetchChunks = 1024;   // most blocks of one prefetch-list
 struct PrefetchState {
   float* span;             // [layers] per partition, partition q at off[q]
   uint32_t* win;           // same layout
-  uint32_t* chunk_counts;  // [kPrefetchChunks] scratch of the list kernels
+  unsigned long long* words;   // [kPrefetchChunks] scratch of the list kernel: counts tagged with the launch's number
+  uint32_t* serial;            // number of the last list launch
   uint32_t off[4], layers[4], heads[4];
   uint32_t block_tokens[4];
   uint32_t w_max[4];       // cap on the window, blocks
@@ -231,6 +232,31 @@ inline cudaError_t launch_scoring_kernel(const void* fn, dim3 grid, dim3 block, 
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+// A kernel launched with launch_overlapped may be set up while the kernel ahead of it in the
+// stream is still finishing (programmatic dependent launch): it calls this before it touches
+// memory, which waits until everything ahead of it is complete and visible, and lets the
+// kernel behind it be set up in turn.
+__device__ __forceinline__ void launch_dependents_and_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, cudaStream_t s,
+                                     Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  count_launches(1);
+  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 // ---- kv_score.cu ----
 cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events,
                                 const EntryState& st, const Workspace& ws, cudaStream_t s);
@@ -255,7 +281,7 @@ cudaError_t launch_prefetch_window(const PrefetchState& pf, int q, int mode, con
 cudaError_t launch_prefetch_list(const PrefetchState& pf, int q, const uint32_t* table, uint64_t n_pos,
                                  uint64_t pos0, int dir, const uint32_t* loc, uint64_t n_tags,
                                  unsigned long long* out, uint64_t max_out, unsigned long long* count,
-                                 cudaStream_t s);
+                                 const Workspace& ws, cudaStream_t s);
 // empties the sliding window of the blend (the estimates stay as they are)
 cudaError_t launch_blend_reset(const Workspace& ws, cudaStream_t s);
 
