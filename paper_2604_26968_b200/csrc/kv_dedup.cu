@@ -10,10 +10,19 @@
 //                         the SHA-256 compression function of FIPS 180-4.  The
 //                         work is integer arithmetic (about 25 instructions per
 //                         byte), not memory traffic: a thread reads its 64 bytes as
-//                         four 16-byte loads and then spends ~1,600 instructions on
-//                         them.  Shifts and logic operations fill the integer pipe, so
-//                         the additions are issued as multiply-adds, which run on the
-//                         FMA pipe beside it (861 -> 1,025 GB/s on 8 KB entries).
+//                         four 16-byte loads, a block ahead, and spends ~1,700
+//                         instructions on them.  Shifts and logic operations fill the
+//                         integer pipe, so the additions are issued as multiply-adds,
+//                         which run on the FMA pipe beside it (861 -> 1,025 GB/s on
+//                         8 KB entries).  What then bounds it is the 1,040 shifts,
+//                         rotations and logic operations a block (half rate): 2,363
+//                         cycles a warp and block with four warps on a scheduler.
+//                         Loading a block ahead with one address for its four
+//                         pieces, and 256 bytes into the L2 eight blocks ahead, took
+//                         a lone warp per scheduler from 307 to 190 us on 8 KB.  A message is a serial chain, so a call of a
+//                         few messages per thread slot of the GPU leaves some
+//                         schedulers with one warp more than others; warps then work
+//                         in slices and exchange chains through a queue (below).
 //   dedup_insert_kernel / dedup_resolve_kernel
 //                         an open-addressing table of list positions, probed from
 //                         the first 8 bytes of the digest (a SHA-256 digest is as
@@ -88,70 +97,226 @@ __device__ __forceinline__ uint64_t hash_chunk_offset(const PartGeom& g, uint64_
   return ((lb * g.n_chunks + c) * g.heads + head) * (uint64_t)g.chunk_bytes;
 }
 
+// Chains in turn.  A warp's 32 messages are one chain of up to 131,072 dependent blocks.  Where
+// there are between 2 and ~10 chains per scheduler, an integer number of them per scheduler cannot
+// be even: 2,458 chains on 592 schedulers are 4 on most and 5 on some, and the call takes as long
+// as 5.  So the grid holds an even number of warps, each works on a chain for one slice (a seventh
+// of the longest message), leaves the intermediate hash value in the place of the digest, queues the
+// chain and takes the one that has waited longest: all chains advance at one rate and the call ends
+// everywhere at about the same time (78,643 entries of 8 KB: 788 us
+// without the queue, 661 with it; 120,000: 1,084 and 991; 786,432: 6,331 and 6,303).  The exchange takes a
+// few microseconds of latency; the warps of a scheduler make theirs at different times (a warp's first
+// slice has any length), so that the others keep it busy meanwhile.
+// Places in the queue are given out by two counters (a compare-and-swap loop on them took 0.9 ms a
+// slice: all warps come at the same time).  A warp that finishes its chain takes a place without
+// having queued one, and so may have to wait for another's slice to end; when all chains are
+// finished, those that wait leave.
+struct HashCounters {
+  unsigned int head;       // places taken beyond the first n_warps
+  unsigned int tail;       // chains queued again
+  unsigned int finished;   // chains finished
+  unsigned int pad;
+};
+struct HashQueue {
+  HashCounters* counters = nullptr;    // (nullptr: no queue)
+  unsigned long long* ring = nullptr;  // bit 63 | next block << 32 | chain; zero until written
+  uint32_t n_chains = 0, n_warps = 0, slice_blocks = 0;
+};
+constexpr uint32_t kHashThreads = 128;
+constexpr uint32_t kHashBlocksPerSm = 5;
+constexpr uint32_t kHashSlices = 7;
+constexpr uint32_t kHashStep = 4;          // blocks between two looks at the pace of the others
+constexpr uint32_t kHashSpins = 1u << 22;
+
 // digests[j] = SHA-256 of the image of entry ids[j] (ids == nullptr: entry j).
 // Chunk sizes are multiples of 16 bytes (a pool with others is refused), so a 16-byte piece
 // of the image never straddles the K and V chunks.
-__global__ void __launch_bounds__(128)
+template <bool QUEUE>
+__global__ void __launch_bounds__(QUEUE ? kHashThreads * kHashBlocksPerSm : kHashThreads, QUEUE ? 1 : kHashBlocksPerSm)
 hash_entries_kernel(const HashGeom hg, const uint32_t* __restrict__ ids, uint64_t m,
-                    uint8_t* __restrict__ digests, uint32_t* __restrict__ status, uint32_t one) {
-  const uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m) return;
-  const uint64_t id = ids ? ids[j] : j;
-  int q = -1;
-  for (int i = 0; i < hg.n_parts; ++i)
-    if (id >= hg.part[i].base && id < hg.part[i].base + hg.part[i].n) q = i;
-  if (q < 0) {
-    atomicOr(status, KV_DEV_BAD_INDEX);
-    return;
-  }
-  const PartGeom& g = hg.part[q];
-  const uint64_t local = id - g.base;
-  const uint8_t* ck = g.slab + hash_chunk_offset(g, local, 0);
-  const uint8_t* cv = g.n_chunks > 1 ? g.slab + hash_chunk_offset(g, local, 1) : ck;
-  const uint32_t cb = g.chunk_bytes, eb = g.entry_bytes;
-  auto piece = [&](uint32_t off) -> uint4 {   // 16 bytes of the image at byte offset off
-    const uint8_t* p = off < cb ? ck + off : cv + (off - cb);
-    return __ldg(reinterpret_cast<const uint4*>(p));
+                    uint8_t* digests, uint32_t* __restrict__ status, uint32_t one, const HashQueue queue) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint64_t chain = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  uint32_t b0 = 0;   // the chain's next block
+  // Blocks done by each of the CTA's warps, for fairness: left alone, a scheduler favours some of
+  // its warps up to threefold, and the chains that meet the others are late at the end.
+  __shared__ volatile uint32_t s_pace[4 * kHashBlocksPerSm];
+  constexpr uint32_t kAway = 0x7FFFFFFFu;   // pace of a warp without a chain
+  const uint32_t warp = threadIdx.x >> 5, n_warps_cta = blockDim.x >> 5;
+  uint32_t pace = 0;
+  auto slowest = [&]() {   // the least pace among the warps of this warp's scheduler
+    const uint32_t w = (warp & 3u) + 4u * lane;
+    return __reduce_min_sync(0xFFFFFFFFu, w < n_warps_cta ? s_pace[w] : kAway);
   };
-  uint32_t st[8] = {0x6a09e667u, 0xbb67ae85u, 0x3c6ef372u, 0xa54ff53au,
-                    0x510e527fu, 0x9b05688cu, 0x1f83d9abu, 0x5be0cd19u};
-  uint32_t w[16];
-  const uint32_t full = eb / 64;
-  for (uint32_t b = 0; b < full; ++b) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint4 v = piece(b * 64 + u * 16);
-      w[4 * u + 0] = be32(v.x); w[4 * u + 1] = be32(v.y); w[4 * u + 2] = be32(v.z); w[4 * u + 3] = be32(v.w);
+  if (QUEUE) {
+    if (lane == 0) s_pace[warp] = 0;
+    __syncthreads();
+  }
+  uint32_t slice_len = 0xFFFFFFFFu;
+  if (QUEUE) slice_len = 1u + ((uint32_t)chain * 2654435761u >> 8) % queue.slice_blocks;
+  while (chain * 32u < m) {
+    const uint64_t j = chain * 32u + lane;
+    int q = -1;
+    uint64_t id = 0;
+    if (j < m) {
+      id = ids ? ids[j] : j;
+      for (int i = 0; i < hg.n_parts; ++i)
+        if (id >= hg.part[i].base && id < hg.part[i].base + hg.part[i].n) q = i;
+      if (q < 0 && b0 == 0) atomicOr(status, KV_DEV_BAD_INDEX);
     }
-    sha256_block(st, w, one);
-  }
-  // last block: what is left of the image (0, 16, 32 or 48 bytes), the 1 bit, zeros, the length in bits
-  const uint32_t rem = eb - full * 64;
+    const PartGeom& g = hg.part[q < 0 ? 0 : q];
+    const uint64_t local = q < 0 ? 0 : id - g.base;
+    const uint8_t* ck = g.slab + hash_chunk_offset(g, local, 0);
+    const uint8_t* cv = g.n_chunks > 1 ? g.slab + hash_chunk_offset(g, local, 1) : ck;
+    const uint32_t cb = g.chunk_bytes, eb = g.entry_bytes;
+    const uint32_t full = eb / 64u;                                 // whole blocks of the image ...
+    const uint32_t n_blocks = q < 0 ? 0u : full + 1u;               // ... and one with the padding
+    const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, n_blocks);
+    const uint32_t b1 = slice_len < longest - b0 ? b0 + slice_len : longest;
+    uint4* const out = reinterpret_cast<uint4*>(digests + j * 32);
+    uint32_t st[8] = {0x6a09e667u, 0xbb67ae85u, 0x3c6ef372u, 0xa54ff53au,
+                      0x510e527fu, 0x9b05688cu, 0x1f83d9abu, 0x5be0cd19u};
+    if (b0 != 0 && n_blocks > b0) {   // where another warp left off
+      const uint4 x = __ldcg(out), y = __ldcg(out + 1);
+      st[0] = x.x; st[1] = x.y; st[2] = x.z; st[3] = x.w;
+      st[4] = y.x; st[5] = y.y; st[6] = y.z; st[7] = y.w;
+    }
+    // Blocks that do not straddle the chunks: one address per block, K's up to block k_blocks.
+    const bool even = (cb & 63u) == 0u;
+    const uint32_t k_blocks = g.n_chunks > 1 ? cb / 64u : full;
+    const uint8_t* const v_from = cv - (uint64_t)k_blocks * 64u;   // block b >= k_blocks lies at v_from + 64 * b
+    uint4 v[4];
+    auto load = [&](uint32_t b) {   // the image's 16-byte pieces of block b (zeros past its end)
+      if (even && b < full) {
+        const uint4* p = reinterpret_cast<const uint4*>((b < k_blocks ? ck : v_from) + (uint64_t)b * 64u);
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if ((uint32_t)u * 16 < rem) v = piece(full * 64 + u * 16);
-    w[4 * u + 0] = be32(v.x); w[4 * u + 1] = be32(v.y); w[4 * u + 2] = be32(v.z); w[4 * u + 3] = be32(v.w);
-  }
+        for (uint32_t u = 0; u < 4; ++u)   // (volatile: issued here, ahead of the compression)
+          asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[u].x), "=r"(v[u].y), "=r"(v[u].z), "=r"(v[u].w) : "l"(p + u));
+      } else {
 #pragma unroll
-  for (int i = 0; i < 16; ++i)
-    if ((uint32_t)i * 4 == rem) w[i] = 0x80000000u;
-  w[14] = (uint32_t)(((uint64_t)eb * 8) >> 32);   // rem <= 48: the length always fits this block
-  w[15] = (uint32_t)((uint64_t)eb * 8);
-  sha256_block(st, w, one);
-  uint4* out = reinterpret_cast<uint4*>(digests + j * 32);
-  out[0] = make_uint4(be32(st[0]), be32(st[1]), be32(st[2]), be32(st[3]));
-  out[1] = make_uint4(be32(st[4]), be32(st[5]), be32(st[6]), be32(st[7]));
+        for (uint32_t u = 0; u < 4; ++u) {
+          const uint32_t off = b * 64u + u * 16u;
+          v[u] = make_uint4(0, 0, 0, 0);
+          if (off < eb) v[u] = __ldg(reinterpret_cast<const uint4*>(off < cb ? ck + off : cv + (off - cb)));
+        }
+      }
+    };
+    const uint32_t b_end = b1 < n_blocks ? b1 : n_blocks;
+    if (b0 < b_end) load(b0);
+    for (uint32_t at = b0; at < b1; at += kHashStep) {
+      const uint32_t step_end = QUEUE && at + kHashStep < b_end ? at + kHashStep : b_end;
+      for (uint32_t b = at; b < step_end; ++b) {
+        uint32_t w[16];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          w[4 * u + 0] = be32(v[u].x); w[4 * u + 1] = be32(v[u].y); w[4 * u + 2] = be32(v[u].z); w[4 * u + 3] = be32(v[u].w);
+        }
+        if (b == full) {
+          // what was left of the image (0, 16, 32 or 48 bytes), the 1 bit, zeros, the length in bits
+          const uint32_t rem = eb - full * 64u;
+#pragma unroll
+          for (int i = 0; i < 16; i += 4)
+            if ((uint32_t)i * 4u == rem) w[i] = 0x80000000u;
+          w[14] = (uint32_t)(((uint64_t)eb * 8) >> 32);   // rem <= 48: the length always fits this block
+          w[15] = (uint32_t)((uint64_t)eb * 8);
+        }
+        if (b + 1u < b_end) load(b + 1u);   // (in flight during the compression)
+        if ((b & 3u) == 0u && even) {       // ... and on its way into the L2: 256 bytes, eight blocks on
+          const uint32_t ahead = b + 8u;
+          if (ahead + 4u <= k_blocks || (ahead >= k_blocks && ahead + 4u <= full)) {
+            const uint8_t* p = (ahead < k_blocks ? ck : v_from) + (uint64_t)ahead * 64u;
+            asm volatile("prefetch.global.L2 [%0];\n\tprefetch.global.L2 [%0 + 128];" ::"l"(p));
+          }
+        }
+        sha256_block(st, w, one);
+      }
+      if (!QUEUE) break;
+      pace += kHashStep;
+      if (lane == 0) s_pace[warp] = pace;
+      for (int i = 0; i < 8 && pace > slowest() + kHashStep; ++i) __nanosleep(400);
+    }
+    const bool done = b1 == longest;
+    if (b0 < n_blocks) {   // (a message that ended in an earlier slice has its digest)
+      const bool fin = b1 >= n_blocks;   // this lane's message is complete (others of the chain may be longer)
+      out[0] = fin ? make_uint4(be32(st[0]), be32(st[1]), be32(st[2]), be32(st[3])) : make_uint4(st[0], st[1], st[2], st[3]);
+      out[1] = fin ? make_uint4(be32(st[4]), be32(st[5]), be32(st[6]), be32(st[7])) : make_uint4(st[4], st[5], st[6], st[7]);
+    }
+    if (!QUEUE) return;
+    __syncwarp();
+    unsigned long long word = ~0ull;   // the next chain and its next block, ~0: none
+    if (lane == 0) {
+      if (!done) {   // queue the chain (the lanes' values first)
+        __threadfence();
+        const unsigned int p = atomicAdd(&queue.counters->tail, 1u);
+        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(queue.ring + p),
+                     "l"(1ull << 63 | (unsigned long long)b1 << 32 | (uint32_t)chain)
+                     : "memory");
+      } else {
+        atomicAdd(&queue.counters->finished, 1u);
+      }
+      s_pace[warp] = kAway;
+      const unsigned int pos = queue.n_warps + atomicAdd(&queue.counters->head, 1u);
+      if (pos < queue.n_chains) {
+        word = pos;
+      } else {
+        const unsigned long long* at = queue.ring + (pos - queue.n_chains);
+        for (uint32_t it = 0;; ++it) {
+          unsigned long long w;
+          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(at) : "memory");
+          if (w >> 63) { word = w; break; }
+          if (*reinterpret_cast<volatile unsigned int*>(&queue.counters->finished) == queue.n_chains) break;
+          if (it == kHashSpins) { atomicOr(status, KV_DEV_WAIT_EXPIRED); break; }
+          __nanosleep(256);
+        }
+      }
+    }
+    word = __shfl_sync(0xFFFFFFFFu, word, 0);
+    if (word == ~0ull) return;
+    chain = (uint32_t)word;
+    b0 = (uint32_t)(word >> 32) & 0x7FFFFFFFu;
+    slice_len = queue.slice_blocks;
+    const uint32_t least = slowest();   // (a warp that was away comes back beside the slowest)
+    if (least != kAway && least > pace) pace = least;
+  }
 }
 
 cudaError_t launch_hash_entries(const PartGeom* parts, int n_parts, const uint32_t* ids, uint64_t m,
-                                uint8_t* digests, const Workspace& ws, cudaStream_t s) {
+                                uint8_t* digests, uint64_t n_entries, const Workspace& ws, cudaStream_t s) {
   if (m == 0) return cudaSuccess;
   HashGeom hg;
-  for (int q = 0; q < 4; ++q) hg.part[q] = parts[q < n_parts ? q : 0];
+  uint32_t longest = 0;
+  for (int q = 0; q < 4; ++q) {
+    hg.part[q] = parts[q < n_parts ? q : 0];
+    const uint32_t b = hg.part[q].entry_bytes / 64u + 1u;
+    if (b > longest) longest = b;
+  }
   hg.n_parts = n_parts;
-  const uint64_t blocks = (m + 127) / 128;
-  hash_entries_kernel<<<(unsigned)blocks, 128, 0, s>>>(hg, ids, m, digests, ws.status, 1u);
+  uint64_t blocks = (m + kHashThreads - 1) / kHashThreads;
+  HashQueue queue;
+  // The queue pays where an uneven split costs: two chains per scheduler (one block of four warps
+  // per SM each) or more.  With fewer a scheduler's single warp is bound by its own latency, and a
+  // second chain beside it is nearly free.  Its ring lies in the scratch of promotions and
+  // admissions, which is idle here.
+  const uint64_t per_sm = (uint64_t)sm_count(), chains = (m + 31) / 32;
+  uint64_t depth = blocks / per_sm;
+  if (depth > kHashBlocksPerSm) depth = kHashBlocksPerSm;
+  const uint64_t words = 2 + chains * kHashSlices;   // 64-bit words: counters and ring
+  if (depth >= 2 && blocks > depth * per_sm && words * 2 <= n_entries && chains < (1ull << 31)) {
+    unsigned long long* base = reinterpret_cast<unsigned long long*>(ws.free_list);
+    const cudaError_t e = cudaMemsetAsync(base, 0, words * 8, s);
+    if (e != cudaSuccess) return e;
+    queue.counters = reinterpret_cast<HashCounters*>(base);
+    queue.ring = base + 2;
+    queue.n_chains = (uint32_t)chains;
+    queue.slice_blocks = (longest + kHashSlices - 1) / kHashSlices;
+    blocks = depth * per_sm;
+    queue.n_warps = (uint32_t)(blocks * (kHashThreads / 32));
+  }
+  // (with the queue one CTA per SM holds all of the SM's warps, which then see each other's pace)
+  if (queue.counters)
+    hash_entries_kernel<true><<<(unsigned)per_sm, kHashThreads * (unsigned)depth, 0, s>>>(hg, ids, m, digests, ws.status, 1u, queue);
+  else
+    hash_entries_kernel<false><<<(unsigned)blocks, kHashThreads, 0, s>>>(hg, ids, m, digests, ws.status, 1u, queue);
   count_launches(1);
   return cudaGetLastError();
 }

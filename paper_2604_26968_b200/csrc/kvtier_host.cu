@@ -1169,7 +1169,7 @@ int32_t kv_hash_entries(kv_pool* p, const uint32_t* d_ids, uint64_t m, uint8_t* 
   if (m == 0) return KV_OK;
   if (!d_digests || !aligned16(d_digests) || (d_ids && !aligned16(d_ids))) return KV_ERR_INVALID_ARG;
   if (!d_ids && m > p->stats.n_entries) return KV_ERR_INVALID_ARG;
-  KV_CUDA(p, launch_hash_entries(p->geom, p->n_parts, d_ids, m, d_digests, p->ws, S(stream)));
+  KV_CUDA(p, launch_hash_entries(p->geom, p->n_parts, d_ids, m, d_digests, p->stats.n_entries, p->ws, S(stream)));
   return KV_OK;
 }
 
