@@ -7,17 +7,12 @@
 // used here is w * (s_0 + ... + s_{H-1}) over the block's KV-head entries, summed
 // in head order with every binary32 operation rounded once, w = query heads per
 // KV-head entry; a block is a candidate only while all its heads are RESIDENT.
-// Selection itself is the same radix select as for entries, run on the
-// per-block arrays.
+// Selection itself is the same as for entries; the persistent form (kv_select_persist.cu)
+// sums the heads' scores itself and, on a pool of one partition, writes the entries.  The
+// kernels here serve the other cases.
 #include "kvtier_internal.cuh"
 
 namespace kvt {
-
-__device__ __forceinline__ int block_partition(const BlockGeom& bg, uint64_t gb) {
-  int q = 0;
-  while (q + 1 < bg.n_parts && gb >= bg.block_base[q + 1]) ++q;
-  return q;
-}
 
 __global__ void __launch_bounds__(kThreads)
 block_aggregate_kernel(const float* __restrict__ score, const uint8_t* __restrict__ state,
@@ -77,21 +72,29 @@ cudaError_t launch_select_blocks(const EntryState& st, const BlockGeom& bg, uint
                                  uint32_t* d_victims, const Workspace& ws, cudaStream_t s,
                                  unsigned long long* h_entry_counts) {
   const uint64_t n_blocks = bg.block_base[bg.n_parts];
-  block_aggregate_kernel<<<grid_for(n_blocks), kThreads, 0, s>>>(st.score, st.state, bg, ws.block_score,
-                                                                 ws.block_state);
-  count_launches(1);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  EntryState bs{};
-  bs.score = ws.block_score;
-  bs.state = ws.block_state;
-  bs.n = n_blocks;
   PartCounts pc;   // the selected blocks per partition, a by-product of the selection
   for (int q = 0; q <= 4; ++q) pc.base[q] = bg.block_base[q < bg.n_parts ? q : bg.n_parts];
   pc.n_parts = bg.n_parts;
   pc.d_counts = ws.part_counts;
-  e = launch_select(bs, k_blocks, ws.block_victims, ws, s, 1, &pc);
-  if (e != cudaSuccess) return e;
+  const bool one = bg.n_parts == 1;
+  if (one) pc.h_counts = h_entry_counts;
+  bool used = false;
+  cudaError_t e = launch_select_persistent(st, k_blocks, one ? d_victims : ws.block_victims, ws, s, &used, nullptr, &pc, &bg);
+  if (e != cudaSuccess || (used && one)) return e;
+  if (!used) {
+    block_aggregate_kernel<<<grid_for(n_blocks), kThreads, 0, s>>>(st.score, st.state, bg, ws.block_score,
+                                                                   ws.block_state);
+    count_launches(1);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    EntryState bs{};
+    bs.score = ws.block_score;
+    bs.state = ws.block_state;
+    bs.n = n_blocks;
+    pc.h_counts = nullptr;
+    e = launch_select(bs, k_blocks, ws.block_victims, ws, s, 0, &pc);
+    if (e != cudaSuccess) return e;
+  }
   block_expand_kernel<<<grid_for(k_blocks), kThreads, 0, s>>>(ws.block_victims, k_blocks, bg, ws.part_counts,
                                                               d_victims, h_entry_counts);
   count_launches(1);

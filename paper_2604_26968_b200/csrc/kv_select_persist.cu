@@ -45,6 +45,12 @@
 // inputs streamed through shared-memory stages by asynchronous copies.  The event
 // reduction stays a launch of its own ahead of it: its scattered gathers and atomics ran
 // 2.5x slower inside this kernel when that was tried.
+//
+// And it exists for paged blocks (BLOCKS = true): an "entry" is then a block, whose score is
+// the weighted sum over its heads, formed here from the entries' scores; on a pool of one
+// partition the ordered write puts out the ids of all the block's entries.  (A kernel that
+// wrote the blocks' scores ahead of this one and one that expanded the blocks behind it took
+// 9.2 and 5.2 us of a 64.5 us pass over 393,216 blocks of 8 heads.)
 #include <mutex>
 
 #include "kv_score_device.cuh"
@@ -73,7 +79,7 @@ constexpr uint32_t kStages = 2;                         // rows in flight ahead 
 constexpr uint32_t kNoteCapMin = 128;                   // notes a warp keeps in shared memory, at least (the rest spills)
 
 struct PArgs {
-  const float* score;
+  const float* score;     // of the entries, whatever is selected
   const uint8_t* state;
   unsigned long long n;
   unsigned long long k;
@@ -92,6 +98,8 @@ struct PArgs {
   PartCounts pc;          // partitions of the pool (the victims per partition are a by-product)
   uint32_t* spill;        // global scratch for the notes beyond note_cap: spill_stride words per warp (nullptr: none)
   uint32_t spill_stride;
+  BlockGeom bg;           // block form: the pool's paged blocks ...
+  uint32_t expand;        // ... and, on a pool of one partition, entries per block (0: victims are block indices)
   // the scoring pass of the fused form
   EntryState st;
   Predictor pd;
@@ -185,8 +193,84 @@ struct PendingBin {
   }
 };
 
+// Scores of the four paged blocks b0 .. b0+3 (those below b1): the weighted sum over the block's
+// heads, added in head order with every operation rounded once; resident bit j: all heads of
+// block b0 + j are RESIDENT (the others score +inf).
+__device__ __forceinline__ uint32_t block_scores4(const PArgs& a, unsigned long long b0, unsigned long long b1,
+                                                  float s[4]) {
+  const BlockGeom& bg = a.bg;
+  uint32_t resident = 0;
+  const int q0 = block_partition(bg, b0 < b1 ? b0 : 0);
+  const uint32_t H0 = bg.heads[q0];
+  const unsigned long long f0 = bg.entry_base[q0] + (b0 - bg.block_base[q0]) * H0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) s[j] = __int_as_float(0x7F800000);
+  if (b0 + 4u <= b1 && b0 + 4u <= bg.block_base[q0 + 1] && (f0 & 3u) == 0u && ((H0 & 3u) == 0u || H0 <= 2u)) {
+    // the four blocks' entries are aligned vectors
+    const float4* sc = reinterpret_cast<const float4*>(a.score + f0);
+    const uint32_t* st = reinterpret_cast<const uint32_t*>(a.state + f0);
+    constexpr uint32_t kAll = KV_STATE_RESIDENT * 0x01010101u;
+    float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    bool all[4] = {true, true, true, true};
+    if ((H0 & 3u) == 0u) {
+      const uint32_t per = H0 / 4u;   // vectors per block
+#pragma unroll 2
+      for (uint32_t v = 0; v < per; ++v) {
+        float4 x[4];
+        uint32_t y[4];
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) { x[j] = __ldg(sc + j * per + v); y[j] = __ldg(st + j * per + v); }
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) {
+          sum[j] = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum[j], x[j].x), x[j].y), x[j].z), x[j].w);
+          all[j] = all[j] && y[j] == kAll;
+        }
+      }
+    } else {
+      const float4 x = __ldg(sc);
+      const uint32_t y = __ldg(st);
+      if (H0 == 1u) {
+        sum[0] = __fadd_rn(0.0f, x.x); sum[1] = __fadd_rn(0.0f, x.y);
+        sum[2] = __fadd_rn(0.0f, x.z); sum[3] = __fadd_rn(0.0f, x.w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) all[j] = ((y >> (8 * j)) & 0xFFu) == KV_STATE_RESIDENT;
+      } else {
+        const float4 z = __ldg(sc + 1);
+        const uint32_t w = __ldg(st + 1);
+        sum[0] = __fadd_rn(__fadd_rn(0.0f, x.x), x.y); sum[1] = __fadd_rn(__fadd_rn(0.0f, x.z), x.w);
+        sum[2] = __fadd_rn(__fadd_rn(0.0f, z.x), z.y); sum[3] = __fadd_rn(__fadd_rn(0.0f, z.z), z.w);
+        all[0] = (y & 0xFFFFu) == (kAll & 0xFFFFu); all[1] = (y >> 16) == (kAll >> 16);
+        all[2] = (w & 0xFFFFu) == (kAll & 0xFFFFu); all[3] = (w >> 16) == (kAll >> 16);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (all[j]) { s[j] = __fmul_rn(bg.weight[q0], sum[j]); resident |= 1u << j; }
+    return resident;
+  }
+  for (uint32_t j = 0; j < 4; ++j) {   // other head counts, partition boundaries, the ragged end
+    const unsigned long long gb = b0 + j;
+    if (gb >= b1) break;
+    const int q = block_partition(bg, gb);
+    const uint32_t H = bg.heads[q];
+    const unsigned long long first = bg.entry_base[q] + (gb - bg.block_base[q]) * H;
+    bool all = true;
+    float sum = 0.0f;
+    for (uint32_t h = 0; h < H; ++h) {
+      all = all && a.state[first + h] == KV_STATE_RESIDENT;
+      sum = __fadd_rn(sum, a.score[first + h]);
+    }
+    if (all) {
+      const float x = __fmul_rn(bg.weight[q], sum);
+      if (j == 0u) s[0] = x; else if (j == 1u) s[1] = x; else if (j == 2u) s[2] = x; else s[3] = x;
+      resident |= 1u << j;
+    }
+  }
+  return resident;
+}
+
 // PLAIN (fused form only): the policy is the Bayesian product and no partition is weighted.
-template <bool FUSED, bool PLAIN>
+template <bool FUSED, bool PLAIN, bool BLOCKS>
 __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const PArgs a) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
   const uint32_t n_words = a.n_rows * 128u;           // bitmap words: 128 per row
@@ -380,26 +464,28 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   } else if (!hint) {
     warm_lines();
   } else {
-    // (two rows' loads in flight)
-    float4 sc[2];
-    uint32_t st4[2];
+    constexpr uint32_t kInFlight = BLOCKS ? 1 : 4;   // rows whose loads are in flight
+    float4 sc[kInFlight];
+    uint32_t st4[kInFlight];
     auto load = [&](uint32_t r, uint32_t u) {
       const unsigned long long i0 = row_base(r) + 4u * t;
-      if (r < n_rows && i0 + 4u <= row_end(r)) {
+      if (!BLOCKS && r < n_rows && i0 + 4u <= row_end(r)) {
         sc[u] = __ldcg(reinterpret_cast<const float4*>(a.score + i0));
         st4[u] = __ldcg(reinterpret_cast<const uint32_t*>(a.state + i0));
       }
     };
-    load(0, 0);
-    load(1, 1);
-    warm_lines();
-    for (uint32_t r = 0; r < n_rows; r += 2) {
 #pragma unroll
-      for (uint32_t u = 0; u < 2; ++u) {
+    for (uint32_t u = 0; u < kInFlight; ++u) load(u, u);
+    warm_lines();
+    for (uint32_t r = 0; r < n_rows; r += kInFlight) {
+#pragma unroll
+      for (uint32_t u = 0; u < kInFlight; ++u) {
         if (r + u < n_rows) {
           const unsigned long long i0 = row_base(r + u) + 4u * t, i1 = row_end(r + u);
           float s[4] = {inf, inf, inf, inf};
-          if (i0 + 4u <= i1) {
+          if (BLOCKS) {
+            (void)block_scores4(a, i0, i1, s);
+          } else if (i0 + 4u <= i1) {
             s[0] = (st4[u] & 0xFFu) == KV_STATE_RESIDENT ? sc[u].x : inf;
             s[1] = ((st4[u] >> 8) & 0xFFu) == KV_STATE_RESIDENT ? sc[u].y : inf;
             s[2] = ((st4[u] >> 16) & 0xFFu) == KV_STATE_RESIDENT ? sc[u].z : inf;
@@ -409,7 +495,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
             for (int j = 0; j < 4; ++j)
               if (i0 + j < i1 && a.state[i0 + j] == KV_STATE_RESIDENT) s[j] = a.score[i0 + j];
           }
-          load(r + u + 2, u);
+          load(r + u + kInFlight, u);
           classify(r + u, s);
         }
       }
@@ -473,7 +559,12 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     // RESIDENT give kKeyExcluded
     auto load_keys = [&](uint32_t r, uint32_t key[4]) {
       const unsigned long long i0 = row_base(r) + 4u * t, i1 = row_end(r);
-      if (i0 + 4u <= i1) {
+      if (BLOCKS) {
+        float s[4];
+        const uint32_t resident = block_scores4(a, i0, i1, s);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) key[j] = (resident >> j) & 1u ? score_key(s[j]) : kKeyExcluded;
+      } else if (i0 + 4u <= i1) {
         const float4 sc = __ldcg(reinterpret_cast<const float4*>(a.score + i0));
         const uint32_t st4 = __ldcg(reinterpret_cast<const uint32_t*>(a.state + i0));
         key[0] = (st4 & 0xFFu) == KV_STATE_RESIDENT ? score_key(sc.x) : kKeyExcluded;
@@ -688,6 +779,17 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     }
     const uint32_t eq_room = need_eq > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)need_eq;
     const unsigned long long got = (unsigned long long)all_l + (all_e < eq_room ? all_e : eq_room);
+    // (block form, one partition: the entries of block gb, the pos-th of the selected ones)
+    auto write_block = [&](uint32_t pos, uint32_t gb) {
+      const uint32_t H = a.expand, first = gb * H;
+      uint32_t* const out = a.victims + (unsigned long long)pos * H;
+      if ((H & 3u) == 0u) {
+        for (uint32_t h = 0; h < H; h += 4u)
+          *reinterpret_cast<uint4*>(out + h) = make_uint4(first + h, first + h + 1u, first + h + 2u, first + h + 3u);
+      } else {
+        for (uint32_t h = 0; h < H; ++h) out[h] = first + h;
+      }
+    };
     // With L entries below tau and E entries equal to tau before it in id order, an entry below
     // tau goes to L + min(E, need_eq) and an entry equal to tau, taken while E < need_eq, to L + E.
     for (uint32_t rd = 0; rd < n_rounds; ++rd) {
@@ -716,13 +818,16 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       while (bits) {
         const uint32_t b = (uint32_t)__ffs(bits) - 1u;
         bits &= bits - 1u;
+        uint32_t pos = L + (E < eq_room ? E : eq_room);
         if ((be >> b) & 1u) {
-          if (E < eq_room && L + E < a.k) a.victims[L + E] = id0 + b;
+          if (E >= eq_room) pos = 0xFFFFFFFFu;
           ++E;
         } else {
-          const uint32_t pos = L + (E < eq_room ? E : eq_room);
-          if (pos < a.k) a.victims[pos] = id0 + b;
           ++L;
+        }
+        if (pos < a.k) {
+          if (BLOCKS && a.expand) write_block(pos, id0 + b);
+          else a.victims[pos] = id0 + b;
         }
       }
     }
@@ -741,6 +846,9 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
           prev = upto;
         }
         if (!ok) atomicOr(a.status, KV_DEV_WAIT_EXPIRED);
+      } else if (BLOCKS && a.expand && a.pc.h_counts) {   // what a demotion will want to know
+        a.pc.h_counts[0] = got * a.expand;
+        for (int q = 1; q < 4; ++q) a.pc.h_counts[q] = 0;
       }
       end_turn();   // (every CTA has read the number long ago)
       a.sel->tau = tau;
@@ -809,8 +917,9 @@ inline size_t persist_smem(uint32_t n_rows, uint32_t note_cap, uint32_t stage_wo
 // bitmaps; *used = false (and nothing launched) otherwise.
 cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t* d_victims,
                                      const Workspace& ws, cudaStream_t s, bool* used, const FusedScore* fs,
-                                     const PartCounts* pc) {
+                                     const PartCounts* pc, const BlockGeom* bg) {
   *used = false;
+  const uint64_t n = bg ? bg->block_base[bg->n_parts] : st.n;   // what is selected from
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaGetLastError();
   if (dev < 0 || dev >= kPMaxDevices) return cudaSuccess;
@@ -823,8 +932,8 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
       cudaDeviceGetAttribute(&d.n_sm, cudaDevAttrMultiProcessorCount, dev);
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      void* fns[3] = {(void*)select_persistent_kernel<false, false>, (void*)select_persistent_kernel<true, false>,
-                      (void*)select_persistent_kernel<true, true>};
+      void* fns[4] = {(void*)select_persistent_kernel<false, false, false>, (void*)select_persistent_kernel<true, false, false>,
+                      (void*)select_persistent_kernel<true, true, false>, (void*)select_persistent_kernel<false, false, true>};
       cudaError_t e = cudaSuccess;
       size_t fixed = 0;
       for (void* fn : fns) {
@@ -849,21 +958,21 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   }
   if (pd.state != 1) return cudaSuccess;
   // One CTA per SM, but none with less than 1,024 entries (more CTAs only make the exchanges wider).
-  uint64_t ctas = (st.n + kPChunk / 4 - 1) / (kPChunk / 4);
+  uint64_t ctas = (n + kPChunk / 4 - 1) / (kPChunk / 4);
   if (ctas > (uint64_t)pd.n_sm) ctas = (uint64_t)pd.n_sm;
   if (ctas > kPThreads) ctas = kPThreads;
   const uint32_t G = ctas ? (uint32_t)ctas : 1u;
   PArgs a;
   const uint64_t row = (uint64_t)G * kPChunk;
-  a.n_full = (uint32_t)(st.n / row);
-  const uint64_t rest = st.n - a.n_full * row;
+  a.n_full = (uint32_t)(n / row);
+  const uint64_t rest = n - a.n_full * row;
   a.last_len = (uint32_t)((rest + G * 128ull - 1) / (G * 128ull) * 128ull);
   a.n_rows = a.n_full + (rest ? 1u : 0u);
   if (a.n_rows > kPMaxRows) return cudaSuccess;   // more than the bitmaps hold: the multi-launch selection runs
   if ((uint64_t)a.n_rows * G > ws.table_words) return cudaSuccess;
   a.score = st.score;
   a.state = st.state;
-  a.n = st.n;
+  a.n = n;
   a.k = k;
   a.victims = d_victims;
   a.sel = ws.sel;
@@ -887,6 +996,8 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   // n_rows * 4,096 * G is at most N + 4,096 * G, and every warp keeps at least 128 notes itself)
   a.spill = ws.free_list;
   a.spill_stride = a.n_rows * 128u > cap ? a.n_rows * 128u - cap : 0u;
+  a.bg = bg ? *bg : BlockGeom{};
+  a.expand = bg && bg->n_parts == 1 ? bg->heads[0] : 0u;
   a.st = st;
   a.pd = Predictor{};
   a.hw = HeadWeights{};
@@ -899,8 +1010,10 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   }
   void* args[] = {&a};
   const bool plain = fs && fs->opt.policy == 0 && fs->hw.on == 0;
-  void* fn = !fs ? (void*)select_persistent_kernel<false, false>
-                 : plain ? (void*)select_persistent_kernel<true, true> : (void*)select_persistent_kernel<true, false>;
+  void* fn = bg ? (void*)select_persistent_kernel<false, false, true>
+             : !fs ? (void*)select_persistent_kernel<false, false, false>
+                   : plain ? (void*)select_persistent_kernel<true, true, false>
+                           : (void*)select_persistent_kernel<true, false, false>;
   cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, true, ws);
   if (e != cudaSuccess) return e;
   count_launches(1);

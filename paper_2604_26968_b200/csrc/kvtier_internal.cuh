@@ -145,6 +145,12 @@ struct BlockGeom {
   int n_parts;
 };
 
+__device__ __forceinline__ int block_partition(const BlockGeom& bg, uint64_t gb) {
+  int q = 0;
+  while (q + 1 < bg.n_parts && gb >= bg.block_base[q + 1]) ++q;
+  return q;
+}
+
 // Head-granular importance (head-granular eviction section): per partition a
 // [layer][query head] importance matrix, [layer][KV head] multipliers and the
 // resulting [layer][KV head] score weights, each partition's block at its offset.
@@ -317,7 +323,8 @@ struct FusedScore {
 };
 cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t* d_victims,
                                      const Workspace& ws, cudaStream_t s, bool* used,
-                                     const FusedScore* fs = nullptr, const PartCounts* pc = nullptr);
+                                     const FusedScore* fs = nullptr, const PartCounts* pc = nullptr,
+                                     const BlockGeom* bg = nullptr);   // bg: from paged blocks
 // kv_blocks.cu: k_blocks lowest blocks by weighted aggregate score; writes all their entries
 // (ascending) to d_victims, the per-partition block counts to ws.part_counts and the
 // per-partition ENTRY counts to h_entry_counts (host memory the device can write; may be nullptr)
