@@ -45,7 +45,8 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
 // read and written with 16-byte (for the byte arrays 4-byte) accesses.  The last
 // block to finish folds the epoch's counts into the totals, clears them and
 // publishes P; by then every block has read them.
-__global__ void __launch_bounds__(kThreads, 4)
+constexpr int kUpdateBlocksPerSm = 4;
+__global__ void __launch_bounds__(kThreads, kUpdateBlocksPerSm)
 entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights hw, uint32_t epoch) {
   __shared__ float sP[16];
   __shared__ bool s_last;
@@ -105,7 +106,7 @@ cudaError_t launch_entry_update(const EntryState& st, uint64_t* hits, uint64_t* 
                                 const ScoreOptions& opt, const HeadWeights& hw, cudaStream_t s) {
   uint64_t blocks = (st.n / 4 + kThreads - 1) / kThreads;
   if (blocks == 0) blocks = 1;
-  const uint64_t cap = (uint64_t)sm_count() * 8;
+  const uint64_t cap = (uint64_t)sm_count() * kUpdateBlocksPerSm;   // (one wave: a second one forms the posteriors again)
   if (blocks > cap) blocks = cap;
   const Predictor pd{hits,       misses,    P,          alpha0, beta0, ws.delta, &ws.sel->update_ticket,
                      opt.policy, opt.kappa, opt.window, ws.blend};

@@ -227,6 +227,32 @@ __device__ __forceinline__ float head_weight(const HeadWeights& hw, uint64_t i) 
   return __ldg(&hw.w[hw.w_off[q] + layer * hw.heads[q] + head]);
 }
 
+// The weights of entries i0 .. i0+3: two divisions for the vector (they were the entry pass's
+// largest share of instructions), then steps along the table.
+__device__ __forceinline__ void head_weights4(const HeadWeights& hw, uint64_t i0, float w[4]) {
+  int q = 0;
+  while (q + 1 < hw.n_parts && i0 >= hw.base[q + 1]) ++q;
+  if (q + 1 < hw.n_parts && i0 + 3u >= hw.base[q + 1]) {   // a partition boundary inside the vector
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = head_weight(hw, i0 + j);
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) w[j] = 1.0f;
+  if (!((hw.on >> q) & 1u)) return;
+  const uint32_t local = (uint32_t)(i0 - hw.base[q]), per_layer = hw.per_layer[q], heads = hw.heads[q];
+  const uint32_t layer = local / per_layer;
+  uint32_t in_layer = local - layer * per_layer, head = in_layer % heads;
+  const float* row = hw.w + hw.w_off[q] + layer * heads;
+  const float* const end = hw.w + hw.w_off[q] + hw.layers[q] * heads;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (row < end) w[j] = __ldg(row + head);   // (a vector at the pool's end may reach past the last layer)
+    if (++head == heads) head = 0;
+    if (++in_layer == per_layer) { in_layer = 0; row += heads; }   // (a layer is a multiple of heads: head is 0)
+  }
+}
+
 // ---- per-entry step -----------------------------------------------------------
 // One step of the per-entry EMA, then the eviction score of the chosen policy:
 // 0 = reuse estimate x EMA importance, 1 = EMA only, 2 = LRU (epoch of the last
@@ -374,13 +400,12 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
   const float d[4] = {x.d.x, x.d.y, x.d.z, x.d.w};
   const uint32_t t[4] = {x.t.x, x.t.y, x.t.z, x.t.w}, le[4] = {x.le.x, x.le.y, x.le.z, x.le.w};
   const bool all_resident = x.st4 == KV_STATE_RESIDENT * 0x01010101u;   // nearly always
+  float w[4] = {1.0f, 1.0f, 1.0f, 1.0f};
+  if (!kPlain && hw.on) head_weights4(hw, 4 * v, w);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float w = 1.0f;
-    if (!kPlain && hw.on) w = head_weight(hw, 4 * v + j);
+  for (int j = 0; j < 4; ++j)
     entry_step(e[j], d[j], t[j], x.pr4 >> (8 * j), all_resident ? KV_STATE_RESIDENT : (x.st4 >> (8 * j)) & 0xFFu, sP,
-               kPlain ? 0 : policy, le[j], epoch, w, s[j]);
-  }
+               kPlain ? 0 : policy, le[j], epoch, w[j], s[j]);
   sc = make_float4(s[0], s[1], s[2], s[3]);
   reinterpret_cast<float4*>(st.ema)[v] = make_float4(e[0], e[1], e[2], e[3]);
   reinterpret_cast<float4*>(st.score)[v] = sc;
