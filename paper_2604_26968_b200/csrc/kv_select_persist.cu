@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       long long guess = (long long)tau + step;
       if (guess < 0) guess = 0;
       if (guess > 0xFFFFFFFEll) guess = 0xFFFFFFFEll;
-      // ... and the bracket is as wide as the hints have been off lately: eight times a slowly
+      // ... and the bracket is as wide as the hints have been off lately: five to ten times a slowly
       // decaying maximum of |tau - hinted tau|, full width again after a miss (a narrow
       // bracket means fewer keys to note; a miss costs three passes over the keys)
       uint32_t resid = a.sel->hint_resid, new_shift = kBracketShiftMax;
@@ -871,7 +871,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         resid -= resid >> 2;
         if (off > resid) resid = off;
         new_shift = kBracketShiftMin;
-        while (new_shift < kBracketShiftMax && (1ull << (new_shift + 10u)) < 8ull * resid) ++new_shift;
+        while (new_shift < kBracketShiftMax && (1ull << (new_shift + 10u)) < 5ull * resid) ++new_shift;
       } else {
         resid = 1u << 18;
       }
