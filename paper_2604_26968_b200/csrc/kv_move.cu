@@ -48,7 +48,7 @@ admit_kernel(const PartGeom g, const EntryState st, uint32_t* __restrict__ loc,
        piece += warps) {
     const uint64_t j = piece / ppe;
     const uint32_t r = (uint32_t)(piece - j * ppe);
-    const uint32_t f = free_ids[first + j];
+    const uint32_t f = free_ids[j];
     if ((uint64_t)f < g.base || (uint64_t)f >= g.base + g.n) {
       if (lane == 0) atomicOr(status, KV_DEV_BAD_INDEX);
       continue;

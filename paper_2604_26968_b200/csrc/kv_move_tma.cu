@@ -105,15 +105,19 @@ struct MoveArgs {
   uint64_t meta_offset;    // pack: where the kv_slot_meta records go (~0 = none)
   uint32_t* status;
   uint32_t mode;           // pack only: kMoveAll, kMoveMetaOnly or kMoveCopyOnly
+  uint32_t* free_out;      // pack: the victims' ids again, in order (nullptr: none): the free slots they leave
+  uint8_t* host_meta;      // pack: where the device sees the pinned kv_slot_meta records (nullptr: none)
 };
 
-// Metadata of one demoted entry (ring slot mirror, block table, slot state).
-__device__ __forceinline__ void demote_meta(const MoveArgs& a, uint64_t j, uint32_t v) {
+// Metadata of one demoted entry (ring slot mirror, block table, slot state); its record is left
+// in rec.
+__device__ __forceinline__ void demote_meta(const MoveArgs& a, uint64_t j, uint32_t v, uint32_t rec[6]) {
   const PartGeom& g = a.g;
   const EntryState& st = a.st;
   const uint32_t t = st.tag[v];
   if (st.state[v] != KV_STATE_RESIDENT || t == KV_NONE) {
     atomicOr(a.status, KV_DEV_VICTIM_NOT_RESIDENT);
+    rec[0] = KV_NONE;
     return;
   }
   const uint32_t slot = (uint32_t)((a.ring_start + j) % g.ring_slots);
@@ -132,15 +136,12 @@ __device__ __forceinline__ void demote_meta(const MoveArgs& a, uint64_t j, uint3
   st.pair[v] = (uint8_t)(pr | kPairFree);
   st.tag[v] = KV_NONE;
   st.touch[v] = 0;
-  if (a.meta_offset != ~0ull) {
-    uint32_t* rec = reinterpret_cast<uint32_t*>(a.staging + a.meta_offset + j * kMetaBytes);
-    rec[0] = t;
-    rec[1] = le;
-    rec[2] = __float_as_uint(em);
-    rec[3] = __float_as_uint(de);
-    rec[4] = pr;
-    rec[5] = g.epoch_now;
-  }
+  rec[0] = t;
+  rec[1] = le;
+  rec[2] = __float_as_uint(em);
+  rec[3] = __float_as_uint(de);
+  rec[4] = pr;
+  rec[5] = g.epoch_now;
 }
 
 // Metadata of one promoted entry: restored as it was when demoted (with lazy decay on,
@@ -184,29 +185,60 @@ move_tma_kernel(const MoveArgs a) {
 
   if (warp == 1) {
     // ---- metadata warp: one lane per entry ----
-    for (uint64_t j = e0 + lane; j < e1; j += 32) {
-      const uint32_t id = a.ids[j];
-      if ((uint64_t)id < g.base || (uint64_t)id >= g.base + g.n) {
-        atomicOr(a.status, KV_DEV_BAD_INDEX);
-        continue;
-      }
-      if (PACK) {
-        if (a.mode == kMoveCopyOnly) {
-          // the entry's metadata moved earlier: the record for the host mirror comes from the ring mirror
-          if (a.meta_offset != ~0ull) {
+    if constexpr (PACK) {
+      // The records for the pinned mirror leave in whole lines: 32 of them are put next to each
+      // other in shared memory and go straight over the host link, 128 bytes a store.  (A copy of
+      // staged records behind every chunk's payload copy cost a transfer of its own, 9 us of the
+      // copy stream and 3 us of the host's time.)
+      __shared__ uint32_t s_rec[32 * 6];
+      const bool records = a.host_meta != nullptr || a.meta_offset != ~0ull;
+      if (a.mode == kMoveCopyOnly && (a.host_meta || !records)) return;   // moved earlier
+      for (uint64_t jb = e0; jb < e1; jb += 32) {
+        const uint64_t j = jb + lane;
+        uint32_t rec[6] = {KV_NONE, 0, 0, 0, 0, 0};
+        if (j < e1) {
+          const uint32_t id = a.ids[j];
+          if (a.free_out) a.free_out[j] = id;
+          if ((uint64_t)id < g.base || (uint64_t)id >= g.base + g.n) {
+            atomicOr(a.status, KV_DEV_BAD_INDEX);
+          } else if (a.mode == kMoveCopyOnly) {
+            // the entry's metadata moved earlier: the staged record comes from the ring mirror
             const uint32_t slot = (uint32_t)((a.ring_start + j) % g.ring_slots);
-            uint32_t* rec = reinterpret_cast<uint32_t*>(a.staging + a.meta_offset + j * kMetaBytes);
             rec[0] = g.r_tag[slot];
             rec[1] = g.r_last_epoch[slot];
             rec[2] = __float_as_uint(g.r_ema[slot]);
             rec[3] = __float_as_uint(g.r_decay[slot]);
             rec[4] = g.r_pair[slot];
             rec[5] = g.r_depoch[slot];
+          } else {
+            demote_meta(a, j, id, rec);
           }
+        }
+        if (!records) continue;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) s_rec[lane * 6 + i] = rec[i];
+        __syncwarp();
+        const uint32_t n_words = (uint32_t)(e1 - jb < 32 ? e1 - jb : 32) * 6u;
+        if (a.host_meta) {
+          for (uint32_t w = lane; w < n_words; w += 32u) {
+            const uint32_t r = w / 6u;
+            const uint64_t slot = (a.ring_start + jb + r) % g.ring_slots;
+            if (s_rec[r * 6u] != KV_NONE)
+              reinterpret_cast<uint32_t*>(a.host_meta + slot * kMetaBytes)[w - r * 6u] = s_rec[w];
+          }
+        } else {
+          uint32_t* out = reinterpret_cast<uint32_t*>(a.staging + a.meta_offset + jb * kMetaBytes);
+          for (uint32_t w = lane; w < n_words; w += 32u) out[w] = s_rec[w];
+        }
+        __syncwarp();
+      }
+    } else {
+      for (uint64_t j = e0 + lane; j < e1; j += 32) {
+        const uint32_t id = a.ids[j];
+        if ((uint64_t)id < g.base || (uint64_t)id >= g.base + g.n) {
+          atomicOr(a.status, KV_DEV_BAD_INDEX);
           continue;
         }
-        demote_meta(a, j, id);
-      } else {
         const uint32_t slot = a.slots[j];
         if (slot >= g.ring_slots) {
           atomicOr(a.status, KV_DEV_BAD_INDEX);
@@ -346,7 +378,7 @@ cudaError_t launch_gather_promote(const PartGeom& g, const EntryState& st, uint3
                                   const uint32_t* free_ids, uint64_t count, const uint8_t* ring_dev,
                                   const Workspace& ws, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
-  MoveArgs a{g, st, loc, free_ids, slots, count, 0, nullptr, ~0ull, ws.status, kMoveAll};
+  MoveArgs a{g, st, loc, free_ids, slots, count, 0, nullptr, ~0ull, ws.status, kMoveAll, nullptr, nullptr};
   const uint64_t pieces = count * ((g.chunk_bytes + kGatherPiece - 1) / kGatherPiece) * g.n_chunks;
   uint64_t blocks = (pieces * 32 + kGatherThreads - 1) / kGatherThreads;
   // 32 blocks keep 512 KB of reads in flight, several round trips' worth of the host link; more
@@ -385,9 +417,10 @@ static cudaError_t launch_move(const MoveArgs& a, cudaStream_t s) {
 
 cudaError_t launch_pack_tma(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* victims,
                             uint64_t count, uint64_t ring_start, uint8_t* staging, uint64_t meta_offset,
-                            const Workspace& ws, cudaStream_t s, uint32_t mode) {
+                            const Workspace& ws, cudaStream_t s, uint32_t mode, uint32_t* free_out,
+                            uint8_t* host_meta) {
   if (count == 0) return cudaSuccess;
-  MoveArgs a{g, st, loc, victims, nullptr, count, ring_start, staging, meta_offset, ws.status, mode};
+  MoveArgs a{g, st, loc, victims, nullptr, count, ring_start, staging, meta_offset, ws.status, mode, free_out, host_meta};
   return launch_move<true>(a, s);
 }
 
@@ -395,7 +428,8 @@ cudaError_t launch_unpack_tma(const PartGeom& g, const EntryState& st, uint32_t*
                               const uint32_t* free_ids, uint64_t count, const uint8_t* staging,
                               const Workspace& ws, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
-  MoveArgs a{g, st, loc, free_ids, slots, count, 0, const_cast<uint8_t*>(staging), ~0ull, ws.status, kMoveAll};
+  MoveArgs a{g, st, loc, free_ids, slots, count, 0, const_cast<uint8_t*>(staging), ~0ull, ws.status, kMoveAll,
+             nullptr, nullptr};
   return launch_move<false>(a, s);
 }
 

@@ -71,6 +71,12 @@ struct PartHost {
   uint8_t* h_ring = nullptr;
   uint8_t* h_meta = nullptr;
   const uint8_t* ring_dev = nullptr;   // where the device sees h_ring (nullptr: it cannot)
+  uint8_t* meta_dev = nullptr;         // ... and h_meta
+  // The partition's free slots, ascending, as far as the host knows where they are listed: the
+  // victims of a demotion that found the partition full, less those filled again since (always
+  // the lowest).  They lie in the list scratch from place base + free_off on.
+  bool free_known = false;
+  uint64_t free_off = 0;
 };
 
 }  // namespace
@@ -100,7 +106,8 @@ struct kv_pool {
   cudaEvent_t ev_h2d_done;
   bool h2d_valid = false;
   bool events_made = false;
-  int demote_turn = 0, promote_turn = 0, list_turn = 0;
+  int demote_turn = 0, list_turn = 0;
+  bool list_used[kListBufs] = {};
   int last_cuda_error = 0;
   ScoreOptions score_opt;   // eviction policy and confidence blend
   uint64_t gather_run_bytes = 1u << 20;    // promote lists whose runs average less go through the gather kernel
@@ -278,6 +285,11 @@ void scoring_pass_enqueued(kv_pool* p, uint32_t epoch) {
   for (int q = 0; q < p->n_parts; ++q) p->geom[q].epoch_now = epoch;
 }
 
+// The list scratch is about to be used for something else: what it said of free slots is gone.
+void forget_free_lists(kv_pool* p) {
+  for (int q = 0; q < p->n_parts; ++q) p->host[q].free_known = false;
+}
+
 // every event object the pool owns (the timing events apart)
 std::vector<cudaEvent_t*> all_events(kv_pool* p) {
   std::vector<cudaEvent_t*> evs;
@@ -345,13 +357,15 @@ int32_t enqueue_pack_chunk(kv_pool* p, int q, uint64_t c0, uint64_t cnt) {
   const int b = p->demote_turn;
   p->demote_turn ^= 1;
   KV_CUDA(p, cudaStreamWaitEvent(compute, p->ev_staging_free[b], 0));
-  const uint64_t meta_off = h.h_meta ? align_up(cnt * eb, 16) : ~0ull;
+  const bool staged_meta = h.h_meta && !h.meta_dev;
+  const uint64_t meta_off = staged_meta ? align_up(cnt * eb, 16) : ~0ull;
   const uint64_t slot0 = (pd.cursor0[q] + c0) % R;
   const uint32_t* victims = pd.victims + pd.off[q] + c0;
   {
     TimedScope ts(p, 0, cnt * eb, compute);
     KV_CUDA(p, launch_pack_tma(g, p->st, p->desc.d_loc, victims, cnt, slot0, p->staging[b], meta_off, p->ws,
-                               compute, pd.meta_done ? 2u : 0u));
+                               compute, pd.meta_done ? 2u : 0u,
+                               !pd.meta_done && h.free_known ? p->ws.free_list + g.base + c0 : nullptr, h.meta_dev));
   }
   KV_CUDA(p, cudaEventRecord(p->ev_ready[b], compute));
   KV_CUDA(p, cudaStreamWaitEvent(copy, p->ev_ready[b], 0));
@@ -360,7 +374,7 @@ int32_t enqueue_pack_chunk(kv_pool* p, int q, uint64_t c0, uint64_t cnt) {
   if (cnt > first)
     KV_CUDA(p, cudaMemcpyAsync(h.h_ring, p->staging[b] + first * eb, (cnt - first) * eb,
                                cudaMemcpyDeviceToHost, copy));
-  if (h.h_meta) {
+  if (staged_meta) {
     const uint64_t mb = sizeof(kv_slot_meta);
     KV_CUDA(p, cudaMemcpyAsync(h.h_meta + slot0 * mb, p->staging[b] + meta_off, first * mb,
                                cudaMemcpyDeviceToHost, copy));
@@ -581,6 +595,9 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
       void* dp = nullptr;
       if (ph.h_ring && cudaHostGetDevicePointer(&dp, ph.h_ring, 0) == cudaSuccess) ph.ring_dev = static_cast<const uint8_t*>(dp);
       else (void)cudaGetLastError();
+      dp = nullptr;
+      if (ph.h_meta && cudaHostGetDevicePointer(&dp, ph.h_meta, 0) == cudaSuccess) ph.meta_dev = static_cast<uint8_t*>(dp);
+      else (void)cudaGetLastError();
     }
   }
   {
@@ -794,6 +811,7 @@ int32_t kv_select_victims(kv_pool* p, uint64_t k, uint32_t* d_victims, kv_stream
   if (k > p->stats.n_entries - p->stats.n_free) return KV_ERR_K_TOO_LARGE;
   if (k == 0) return KV_OK;
   if (!d_victims || !aligned16(d_victims)) return KV_ERR_INVALID_ARG;
+  forget_free_lists(p);
   KV_CUDA(p, launch_select(p->st, k, d_victims, p->ws, S(stream), p->select_variant, &p->pc));
   return counts_to_host(p, S(stream));
 }
@@ -813,6 +831,7 @@ int32_t kv_epoch_score_select(kv_pool* p, uint32_t epoch, const uint32_t* d_ev_e
   if (k > 0 && p->select_variant != 0) {
     const FusedScore fs{p->desc.d_hits, p->desc.d_misses, p->desc.d_P, p->desc.alpha0,
                         p->desc.beta0,  epoch,            p->score_opt,  p->head};
+    forget_free_lists(p);
     KV_CUDA(p, launch_select_persistent(p->st, k, d_victims, p->ws, S(stream), &used, &fs, &p->pc));
   }
   if (used) {
@@ -832,6 +851,7 @@ int32_t kv_select_victim_blocks(kv_pool* p, uint64_t k_blocks, uint32_t* d_victi
   if (k_blocks > p->bgeom.block_base[p->n_parts]) return KV_ERR_K_TOO_LARGE;
   if (k_blocks == 0) return KV_OK;
   if (!d_victims || !aligned16(d_victims)) return KV_ERR_INVALID_ARG;
+  forget_free_lists(p);
   KV_CUDA(p, launch_select_blocks(p->st, p->bgeom, k_blocks, d_victims, p->ws, S(stream), p->pc.h_counts));
   if (p->n_parts == 1) {
     if (h_n_victims) *h_n_victims = k_blocks * p->bgeom.heads[0];
@@ -931,12 +951,21 @@ int32_t kv_demote_counted(kv_pool* p, const uint32_t* d_victims, uint64_t m, con
     pd.cursor0[q] = q < p->n_parts ? p->host[q].cursor : 0;
     off += kq[q];
   }
+  // A partition that is full now has exactly these victims as its free slots afterwards: the packing
+  // lists them, and no kernel has to look for them.
+  for (int q = 0; q < p->n_parts; ++q) {
+    if (kq[q] == 0) continue;
+    p->host[q].free_known = p->host[q].n_free == 0;
+    p->host[q].free_off = 0;
+  }
   if (pd.meta_done) {
     // metadata of every victim now (slots become FREE, block table and ring mirror are updated);
     // the payload follows chunk by chunk
     for (int q = 0; q < p->n_parts; ++q)
       KV_CUDA(p, launch_pack_tma(p->geom[q], p->st, p->desc.d_loc, d_victims + pd.off[q], kq[q],
-                                 pd.cursor0[q], p->staging[0], ~0ull, p->ws, compute, 1u));
+                                 pd.cursor0[q], p->staging[0], ~0ull, p->ws, compute, 1u,
+                                 p->host[q].free_known ? p->ws.free_list + p->geom[q].base : nullptr,
+                                 p->host[q].meta_dev));
   }
   pd.active = true;
   // host mirror of the rings: slot assignment is fixed here; overwritten live slots are dropped
@@ -995,7 +1024,7 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
   p->list_turn = (p->list_turn + 1) % kListBufs;
   auto restore = [&]() { for (uint64_t j = 0; j < m; ++j) h.live[h_slots[j]] = 1; };
   // the list given kListBufs calls ago must have left this pinned buffer: normally long done
-  cudaError_t e = cudaEventQuery(p->ev_list_copied[li]);
+  cudaError_t e = p->list_used[li] ? cudaEventQuery(p->ev_list_copied[li]) : cudaSuccess;
   if (e == cudaErrorNotReady) {
     (void)cudaGetLastError();
     p->stats.host_waits += 1;
@@ -1031,10 +1060,14 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(p->ws.slot_list[li], p->h_list[li], m * 4, cudaMemcpyHostToDevice, copy);
   if (e == cudaSuccess) e = cudaEventRecord(p->ev_list_copied[li], copy);
+  p->list_used[li] = true;
   // this partition's free slots, ascending, in the partition's own stretch of the list scratch
-  if (e == cudaSuccess) e = launch_free_list(p->st, g.base, g.base + g.n, m, p->ws, compute, g.base);
+  if (e == cudaSuccess && !h.free_known) {
+    e = launch_free_list(p->st, g.base, g.base + g.n, m, p->ws, compute, g.base);
+    h.free_off = 0;
+  }
   if (e != cudaSuccess) { restore(); return cuda_fail(p, e); }
-  const uint32_t* free_ids = p->ws.free_list + g.base;
+  const uint32_t* free_ids = p->ws.free_list + g.base + h.free_off;
   // With P entries promoted into the partition since the pending demotion began, chunk [c0, c0+cnt)
   // fills FREE slots number P+c0 .. P+c0+cnt-1 of the free set as it was right after that demotion.
   // Any of those that the demotion freed is among its first P+c0+cnt victims of the partition (victims
@@ -1100,6 +1133,7 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
   for (uint64_t j = 0; j < m; ++j) h.live[h_slots[j]] = 0;
   h.n_live -= m;
   h.n_free -= m;
+  h.free_off += m;
   p->stats.n_free -= m;
   p->stats.promoted += m;
   p->stats.bytes_promoted += m * eb;
@@ -1115,14 +1149,19 @@ int32_t kv_admit(kv_pool* p, uint32_t epoch, float decay, const uint8_t* d_new_p
   if (n_free == 0) return KV_OK;
   if (!d_new_pairs || n_new_pairs < n_free) return KV_ERR_INVALID_ARG;
   if (p->next_tag + n_free > p->desc.n_tags) return KV_ERR_TAGS_EXHAUSTED;
-  KV_CUDA(p, launch_free_list(p->st, 0, p->st.n, n_free, p->ws, S(stream)));
+  bool known = true;
+  for (int q = 0; q < p->n_parts; ++q) known = known && (p->host[q].n_free == 0 || p->host[q].free_known);
+  if (!known) KV_CUDA(p, launch_free_list(p->st, 0, p->st.n, n_free, p->ws, S(stream)));
   uint64_t first = 0;
   for (int q = 0; q < p->n_parts; ++q) {
-    const uint64_t cnt = p->host[q].n_free;
-    KV_CUDA(p, launch_admit(p->geom[q], p->st, p->desc.d_loc, p->ws.free_list, first, cnt, p->next_tag,
+    PartHost& h = p->host[q];
+    const uint64_t cnt = h.n_free;
+    const uint32_t* free_ids = p->ws.free_list + (known ? p->geom[q].base + h.free_off : first);
+    KV_CUDA(p, launch_admit(p->geom[q], p->st, p->desc.d_loc, free_ids, first, cnt, p->next_tag,
                             d_new_pairs, epoch, decay, fill_pattern, p->ws, S(stream)));
     first += cnt;
-    p->host[q].n_free = 0;
+    h.n_free = 0;
+    h.free_known = false;
   }
   p->next_tag += n_free;
   p->stats.admitted += n_free;
@@ -1169,6 +1208,7 @@ int32_t kv_hash_entries(kv_pool* p, const uint32_t* d_ids, uint64_t m, uint8_t* 
   if (m == 0) return KV_OK;
   if (!d_digests || !aligned16(d_digests) || (d_ids && !aligned16(d_ids))) return KV_ERR_INVALID_ARG;
   if (!d_ids && m > p->stats.n_entries) return KV_ERR_INVALID_ARG;
+  forget_free_lists(p);
   KV_CUDA(p, launch_hash_entries(p->geom, p->n_parts, d_ids, m, d_digests, p->stats.n_entries, p->ws, S(stream)));
   return KV_OK;
 }

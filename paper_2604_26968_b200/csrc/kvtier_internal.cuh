@@ -352,13 +352,16 @@ cudaError_t launch_init(const EntryState& st, uint64_t* hits, uint64_t* misses, 
                         uint32_t* loc, uint64_t n_tags, const PartGeom* parts, int n_parts,
                         const Workspace& ws, cudaStream_t s);
 // ---- kv_move_tma.cu: gather (demotion) and scatter (promotion) on the bulk asynchronous copy engine ----
-// pack: victims[0 .. count) of one partition into staging (images back to back) followed, at
-// meta_offset, by kv_slot_meta records; also moves the metadata.
+// pack: victims[0 .. count) of one partition into staging (images back to back); also moves the
+// metadata.  The kv_slot_meta records go straight to the pinned mirror (host_meta: the address at
+// which the device sees it), or behind the images at meta_offset (~0: none).  free_out: receives
+// the victims' ids, i.e. the slots they leave, in order.
 // mode: 0 = metadata and payload, 1 = metadata only (staging unused), 2 = payload only
 // (the metadata moved earlier; host-mirror records are rebuilt from the ring mirror)
 cudaError_t launch_pack_tma(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* victims,
                             uint64_t count, uint64_t ring_start, uint8_t* staging, uint64_t meta_offset,
-                            const Workspace& ws, cudaStream_t s, uint32_t mode = 0);
+                            const Workspace& ws, cudaStream_t s, uint32_t mode = 0, uint32_t* free_out = nullptr,
+                            uint8_t* host_meta = nullptr);
 // unpack: staging images [0, count) into the listed free slots of the partition
 cudaError_t launch_unpack_tma(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* slots,
                               const uint32_t* free_ids, uint64_t count, const uint8_t* staging,
@@ -368,7 +371,7 @@ cudaError_t launch_unpack_tma(const PartGeom& g, const EntryState& st, uint32_t*
 cudaError_t launch_gather_promote(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* slots,
                                   const uint32_t* free_ids, uint64_t count, const uint8_t* ring_dev,
                                   const Workspace& ws, cudaStream_t s);
-// admits free_list[first .. first+count) of one partition
+// admits free_ids[0 .. count) of one partition, which are the pool's free slots number first ...
 cudaError_t launch_admit(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* free_ids,
                          uint64_t first, uint64_t count, uint64_t first_tag, const uint8_t* new_pairs,
                          uint32_t epoch, float decay, int fill_pattern, const Workspace& ws,
