@@ -18,9 +18,9 @@ __device__ __forceinline__ bool head_value_ok(float v) {
 }
 
 // One thread per (layer, KV head) of the partition.
-__global__ void head_update_kernel(float* __restrict__ imp, float* __restrict__ mult, float* __restrict__ w,
-                                   const float* __restrict__ src, float d, uint32_t layers, uint32_t q_heads,
-                                   uint32_t heads, int mode, uint32_t* __restrict__ status) {
+__global__ void head_update_kernel(float* imp, float* mult, float* w, const float* src, float d, uint32_t layers,
+                                   uint32_t q_heads, uint32_t heads, int mode, uint32_t* status) {
+  wait_for_kernel_ahead();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= layers * heads) return;
   const uint32_t l = i / heads, h = i % heads;
@@ -65,11 +65,8 @@ __global__ void head_init_kernel(float* imp, float* mult, float* w, uint32_t n_i
 cudaError_t launch_head_update(const HeadWeights& hw, int q, int mode, const float* src, float decay,
                                const Workspace& ws, cudaStream_t s) {
   const uint32_t n = hw.layers[q] * hw.heads[q];
-  head_update_kernel<<<(n + 127) / 128, 128, 0, s>>>(hw.imp + hw.imp_off[q], hw.mult + hw.w_off[q],
-                                                     hw.w + hw.w_off[q], src, decay, hw.layers[q],
-                                                     hw.q_heads[q], hw.heads[q], mode, ws.status);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_overlapped(head_update_kernel, (n + 127) / 128, 128u, s, hw.imp + hw.imp_off[q], hw.mult + hw.w_off[q],
+                           hw.w + hw.w_off[q], src, decay, hw.layers[q], hw.q_heads[q], hw.heads[q], mode, ws.status);
 }
 
 cudaError_t launch_head_init(const HeadWeights& hw, uint32_t n_imp, uint32_t n_w, cudaStream_t s) {

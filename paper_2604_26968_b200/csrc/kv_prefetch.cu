@@ -42,11 +42,11 @@ __device__ __forceinline__ uint32_t window_of(float span, float block_tokens, ui
 
 // One block.  mode 0: EMA step with observations x; mode 1: every span = tokens.
 // A bad observation anywhere leaves the whole partition as it was.
-__global__ void prefetch_window_kernel(float* __restrict__ span, uint32_t* __restrict__ win,
-                                       const float* __restrict__ x, float d, float tokens, int mode,
+__global__ void prefetch_window_kernel(float* span, uint32_t* win,
+                                       const float* x, float d, float tokens, int mode,
                                        uint32_t layers, float block_tokens, uint32_t w_max,
                                        uint32_t* __restrict__ status) {
-  launch_dependents_and_wait();
+  wait_for_kernel_ahead();
   int bad = 0;
   if (mode == 0)
     for (uint32_t l = threadIdx.x; l < layers; l += blockDim.x) bad |= !span_ok(x[l]);
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kPfThreads) prefetch_list_kernel(const ListArg
   __shared__ uint32_t s_wmax;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t row = a.layers * a.heads;
-  launch_dependents_and_wait();
+  wait_for_kernel_ahead();
   const uint32_t tag = *a.serial + 1u;
 
   // the widest window bounds the distances any layer wants

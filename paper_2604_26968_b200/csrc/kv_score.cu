@@ -7,18 +7,21 @@ namespace kvt {
 
 // ---- event reduction ---------------------------------------------------------
 __global__ void __launch_bounds__(kEventThreads, kEventBlocksPerSm)
-event_reduce_kernel(const uint32_t* __restrict__ ev_entry, const uint8_t* __restrict__ ev_hit,
-                    uint64_t n_events, const uint8_t* __restrict__ pair,
-                    uint32_t* __restrict__ touch, uint64_t n,
-                    unsigned long long* __restrict__ delta, uint32_t* __restrict__ status) {
+event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events, const uint8_t* pair,
+                    uint32_t* touch, uint64_t n, unsigned long long* delta, uint32_t* status) {
   __shared__ uint32_t s_cnt[16 * kEventThreads];   // [pair][thread]: events | hits << 16
 #pragma unroll
   for (uint32_t i = 0; i < 16; ++i) s_cnt[i * kEventThreads + threadIdx.x] = 0;   // (the thread's own words)
+  wait_for_kernel_ahead();
   const uint32_t bad = reduce_events(ev_entry, ev_hit, n_events, pair, touch, n,
                                      (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
                                      (uint64_t)gridDim.x * blockDim.x, s_cnt, delta);
   if (bad) atomicOr(status, bad);
 }
+
+// Set up while the kernel ahead finishes, up to this many events: 1.4 M events behind a selection gain
+// 2 us that way (46.4 -> 44.1 a pass), 3.3 M still gain, 15.3 M lose 3 us (188.5 -> 191.4).
+constexpr uint64_t kEventOverlapMax = 8ull << 20;
 
 cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events,
                                 const EntryState& st, const Workspace& ws, cudaStream_t s) {
@@ -34,7 +37,8 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   uint32_t* status = ws.status;
   void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &n, &delta, &status};
   const cudaError_t e = launch_scoring_kernel((const void*)event_reduce_kernel, dim3((unsigned)blocks),
-                                              dim3(kEventThreads), args, 0, s, false, ws);
+                                              dim3(kEventThreads), args, 0, s, false, ws,
+                                              n_events <= kEventOverlapMax);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -51,6 +55,7 @@ entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights h
   __shared__ float sP[16];
   __shared__ bool s_last;
   const int policy = pd.policy;
+  wait_for_kernel_ahead();
   PairStep step;
   if (threadIdx.x < 16) {
     step = pair_step(pd, threadIdx.x);

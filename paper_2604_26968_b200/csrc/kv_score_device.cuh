@@ -53,7 +53,7 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
   return (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
 }
 
-__device__ __forceinline__ void touch_add(uint32_t* __restrict__ touch, uint32_t i, uint32_t n32,
+__device__ __forceinline__ void touch_add(uint32_t* touch, uint32_t i, uint32_t n32,
                                           unsigned long long inc_pair) {
   // inc_pair: what to add to the aligned pair that contains entry i
   if ((i | 1u) < n32)
@@ -67,12 +67,10 @@ __device__ __forceinline__ void touch_add(uint32_t* __restrict__ touch, uint32_t
 // counts for pair p (events | hits << 16) since the last flush.  delta: the 32
 // global epoch counters (index 2 * pair + hit).  Returns the KV_DEV_* bits of
 // refused events.  Every thread of the block must call it.
-__device__ __forceinline__ uint32_t reduce_events(const uint32_t* __restrict__ ev_entry,
-                                                  const uint8_t* __restrict__ ev_hit, uint64_t n_events,
-                                                  const uint8_t* __restrict__ pair,
-                                                  uint32_t* __restrict__ touch, uint64_t n, uint64_t gtid,
-                                                  uint64_t stride, uint32_t* s_cnt,
-                                                  unsigned long long* __restrict__ delta) {
+__device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, const uint8_t* ev_hit,
+                                                  uint64_t n_events, const uint8_t* pair, uint32_t* touch, uint64_t n,
+                                                  uint64_t gtid, uint64_t stride, uint32_t* s_cnt,
+                                                  unsigned long long* delta) {
   const uint64_t n4 = n_events / 4;
   const uint64_t iters = (n4 + stride * kEventVecs - 1) / (stride * kEventVecs);  // same for every thread
   // ids are 32-bit, so the bound is too (an id can never reach 2^32 - 1 = "no entry")
@@ -137,7 +135,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* __restrict__ e
       const uint32_t id[4] = {cur[u].id.x, cur[u].id.y, cur[u].id.z, cur[u].id.w};
       run[u] = !(id[0] & 3u) && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u && id[3] < n32;
       if (run[u]) {
-        pr4[u] = *reinterpret_cast<const uint32_t*>(pair + id[0]);
+        pr4[u] = *reinterpret_cast<const uint32_t*>(pair + id[0]);   // (through the L1: neighbouring blocks share sectors)
       } else {
         uint32_t w = 0;
 #pragma unroll
@@ -198,14 +196,14 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* __restrict__ e
   if (gtid < 3) {
     const uint64_t e = n4 * 4 + gtid;
     if (e < n_events) {
-      const uint32_t i = ev_entry[e];
+      const uint32_t i = __ldcs(ev_entry + e);
       const uint32_t pr = i < n32 ? pair[i] : kPairFree;
       if (i >= n32) {
         bad |= KV_DEV_EVENT_BAD_ID;
       } else if (pr & kPairFree) {
         bad |= KV_DEV_EVENT_NOT_RESIDENT;
       } else {
-        count(pr, ev_hit[e] != 0);
+        count(pr, __ldcs(ev_hit + e) != 0);
         touch_add(touch, i, n32, (i & 1u) ? (1ull << 32) : 1ull);
       }
     }
@@ -224,7 +222,7 @@ __device__ __forceinline__ float head_weight(const HeadWeights& hw, uint64_t i) 
   if (!((hw.on >> q) & 1u)) return 1.0f;
   const uint32_t local = (uint32_t)(i - hw.base[q]);
   const uint32_t layer = local / hw.per_layer[q], head = local % hw.heads[q];
-  return __ldg(&hw.w[hw.w_off[q] + layer * hw.heads[q] + head]);
+  return hw.w[hw.w_off[q] + layer * hw.heads[q] + head];
 }
 
 // The weights of entries i0 .. i0+3: two divisions for the vector (they were the entry pass's
@@ -247,7 +245,7 @@ __device__ __forceinline__ void head_weights4(const HeadWeights& hw, uint64_t i0
   const float* const end = hw.w + hw.w_off[q] + hw.layers[q] * heads;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    if (row < end) w[j] = __ldg(row + head);   // (a vector at the pool's end may reach past the last layer)
+    if (row < end) w[j] = row[head];   // (a vector at the pool's end may reach past the last layer)
     if (++head == heads) head = 0;
     if (++in_layer == per_layer) { in_layer = 0; row += heads; }   // (a layer is a multiple of heads: head is 0)
   }

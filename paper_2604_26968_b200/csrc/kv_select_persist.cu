@@ -75,6 +75,7 @@ static_assert(kBracketShiftMax <= kKeptKeyBits && kPMaxRows <= 64, "a kept note 
 // for the LRU policy, last_epoch (4,096 words each), pair and state bytes (1,024 words each)
 constexpr uint32_t kStageWords = 3u * kPChunk + 2u * kPThreads;
 constexpr uint32_t kStageWordsLru = kStageWords + kPChunk;
+constexpr uint64_t kPAlone = 2 * kPChunk;
 constexpr uint32_t kStages = 2;                         // rows in flight ahead of the one being finished
 constexpr uint32_t kNoteCapMin = 128;                   // notes a warp keeps in shared memory, at least (the rest spills)
 
@@ -146,15 +147,22 @@ __device__ __forceinline__ uint32_t await_word(const unsigned long long* p, uint
   return 0;
 }
 
-// Finds the bin of a global histogram (nbins <= 2048, a power of two) that contains rank
-// k_rem (1-based): (bin, ranks before the bin) to every thread; bin is 0xFFFFFFFF when k_rem
-// exceeds the histogram's total.  A block barrier must lie between two calls.
-__device__ __forceinline__ void pick_bin(const uint32_t* __restrict__ hist, uint32_t nbins,
+// Finds the bin of a histogram (nbins <= 2048, a power of two) that contains rank k_rem (1-based):
+// (bin, ranks before the bin) to every thread; bin is 0xFFFFFFFF when k_rem exceeds the
+// histogram's total.  With local the histogram is the block's own s_hist, which is complete (a
+// block barrier lies behind the last addition) and is cleared.  A block barrier must lie between
+// two calls.
+__device__ __forceinline__ void pick_bin(const uint32_t* hist, bool local, uint32_t* s_hist, uint32_t nbins,
                                          unsigned long long k_rem, uint32_t* s_warp, uint32_t* s_pick,
                                          uint32_t& bin, uint32_t& before_bin) {
   const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
   uint2 c = make_uint2(0u, 0u);
-  if (2u * t < nbins) c = __ldcg(reinterpret_cast<const uint2*>(hist) + t);
+  if (local) {
+    c = reinterpret_cast<const uint2*>(s_hist)[t];   // (bins from nbins on are empty)
+    reinterpret_cast<uint2*>(s_hist)[t] = make_uint2(0u, 0u);
+  } else if (2u * t < nbins) {
+    c = __ldcg(reinterpret_cast<const uint2*>(hist) + t);
+  }
   const uint32_t v = c.x + c.y;
   const uint32_t incl = warp_scan_incl(v, lane);
   if (lane == 31u) s_warp[warp] = incl;
@@ -219,7 +227,7 @@ __device__ __forceinline__ uint32_t block_scores4(const PArgs& a, unsigned long 
         float4 x[4];
         uint32_t y[4];
 #pragma unroll
-        for (uint32_t j = 0; j < 4; ++j) { x[j] = __ldg(sc + j * per + v); y[j] = __ldg(st + j * per + v); }
+        for (uint32_t j = 0; j < 4; ++j) { x[j] = sc[j * per + v]; y[j] = st[j * per + v]; }
 #pragma unroll
         for (uint32_t j = 0; j < 4; ++j) {
           sum[j] = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum[j], x[j].x), x[j].y), x[j].z), x[j].w);
@@ -227,16 +235,16 @@ __device__ __forceinline__ uint32_t block_scores4(const PArgs& a, unsigned long 
         }
       }
     } else {
-      const float4 x = __ldg(sc);
-      const uint32_t y = __ldg(st);
+      const float4 x = sc[0];
+      const uint32_t y = st[0];
       if (H0 == 1u) {
         sum[0] = __fadd_rn(0.0f, x.x); sum[1] = __fadd_rn(0.0f, x.y);
         sum[2] = __fadd_rn(0.0f, x.z); sum[3] = __fadd_rn(0.0f, x.w);
 #pragma unroll
         for (int j = 0; j < 4; ++j) all[j] = ((y >> (8 * j)) & 0xFFu) == KV_STATE_RESIDENT;
       } else {
-        const float4 z = __ldg(sc + 1);
-        const uint32_t w = __ldg(st + 1);
+        const float4 z = sc[1];
+        const uint32_t w = st[1];
         sum[0] = __fadd_rn(__fadd_rn(0.0f, x.x), x.y); sum[1] = __fadd_rn(__fadd_rn(0.0f, x.z), x.w);
         sum[2] = __fadd_rn(__fadd_rn(0.0f, z.x), z.y); sum[3] = __fadd_rn(__fadd_rn(0.0f, z.z), z.w);
         all[0] = (y & 0xFFFFu) == (kAll & 0xFFFFu); all[1] = (y >> 16) == (kAll >> 16);
@@ -295,6 +303,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t G = gridDim.x, g = blockIdx.x;
+  const bool alone = G == 1u;   // one CTA: nothing is exchanged
   const uint32_t n_rows = a.n_rows;
   auto row_base = [&](uint32_t r) -> unsigned long long {
     return r < a.n_full ? ((unsigned long long)r * G + g) * kPChunk
@@ -317,6 +326,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     (void)i;
 #endif
   };
+  wait_for_kernel_ahead();   // (a cooperative launch never starts early: nothing to wait for)
   stamp(0);
 
   // ---- prologue: the first rows' loads go out before anything else ----
@@ -515,13 +525,15 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       if (n_below) atomicAdd(&s_below, n_below);
     }
     __syncthreads();
-    if (hint) {
-      add_pair(turn->hist[0] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
-      if (t == 0 && s_below) atomicAdd(&turn->below, (unsigned long long)s_below);
+    if (!alone) {
+      if (hint) {
+        add_pair(turn->hist[0] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
+        if (t == 0 && s_below) atomicAdd(&turn->below, (unsigned long long)s_below);
+      }
+      grid_arrive(bar);
+      for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
+      ok = grid_wait(bar, ++nbar * G);
     }
-    grid_arrive(bar);
-    for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
-    ok = grid_wait(bar, ++nbar * G);
     stamp(2);
     if (!ok) goto fail;
   }
@@ -532,18 +544,21 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     uint32_t bin = 0, before = 0, tau = 0;
     unsigned long long k_rem = a.k;
     bool found = true;
-    auto send_hist = [&](uint32_t* g_hist, uint32_t nbins) {
+    // The CTA's histogram joins the others' in histogram h; false if the wait ran out.
+    auto exchange_hist = [&](uint32_t h, uint32_t nbins) {
       __syncthreads();
-      if (2u * t < nbins) add_pair(g_hist + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
+      if (alone) return true;
+      if (2u * t < nbins) add_pair(turn->hist[h] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
       grid_arrive(bar);
       for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
+      return grid_wait(bar, ++nbar * G);
     };
     bool use_notes = false;
     uint32_t bin_k = 0;
     if (hint) {
-      const unsigned long long below = __ldcg(&turn->below);
+      const unsigned long long below = alone ? s_below : __ldcg(&turn->below);
       const bool above = a.k > below;
-      pick_bin(turn->hist[0], kHistBins, above ? a.k - below : 1ull, s_warp, s_pick, bin, before);
+      pick_bin(turn->hist[0], alone, s_hist, kHistBins, above ? a.k - below : 1ull, s_warp, s_pick, bin, before);
       hint_hit = above && bin != 0xFFFFFFFFu;
       use_notes = hint_hit && __syncthreads_or(notes_lost) == 0;
       if (hint_hit) {
@@ -636,11 +651,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       p2.flush(s_hist);
       __syncwarp();
       stamp(8);
-      send_hist(turn->hist[1], n_bins);
-      ok = grid_wait(bar, ++nbar * G);
+      ok = exchange_hist(1, n_bins);
       stamp(3);
       if (!ok) goto fail;
-      pick_bin(turn->hist[1], n_bins, k_rem, s_warp, s_pick, bin, before);
+      pick_bin(turn->hist[1], alone, s_hist, n_bins, k_rem, s_warp, s_pick, bin, before);
       found = bin != 0xFFFFFFFFu;
       k_rem -= before;
       const uint32_t tau_low = found ? bin : 0u;
@@ -669,11 +683,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
           }
         });
         p2.flush(s_hist);
-        send_hist(turn->hist[h], 1u << top);
-        ok = grid_wait(bar, ++nbar * G);
+        ok = exchange_hist(h, 1u << top);
         if (digit == 1) stamp(3);
         if (!ok) goto fail;
-        pick_bin(turn->hist[h], 1u << top, k_rem, s_warp, s_pick, bin, before);
+        pick_bin(turn->hist[h], alone, s_hist, 1u << top, k_rem, s_warp, s_pick, bin, before);
         ++h;
         found = found && bin != 0xFFFFFFFFu;
         k_rem -= before;
@@ -721,19 +734,24 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     if (t < n_rows) {
       const uint4 v = reinterpret_cast<const uint4*>(s_wtot)[t];
       const uint32_t sum = v.x + v.y + v.z + v.w;   // at most 4,096 in either half
-      a.table[t * G + g] = (sum & 0xFFFFu) | (sum >> 16) << 13;
+      if (alone) {
+        s_rowtot[t] = make_uint2(sum & 0xFFFFu, sum >> 16);
+        s_colpre[t] = make_uint2(0u, 0u);
+      } else {
+        a.table[t * G + g] = (sum & 0xFFFFu) | (sum >> 16) << 13;
+      }
     }
-    grid_arrive(bar);
+    if (!alone) grid_arrive(bar);
     stamp(5);
     if constexpr (FUSED) {
       // every CTA has long formed its estimates: the epoch's counts can be folded in (here, where
       // the CTA waits for the others anyway)
       if (g == 0 && t >= kPThreads - 32u && lane < 16u) commit_predictor(a.pd, lane, s_pair[lane]);
     }
-    ok = grid_wait(bar, ++nbar * G);
+    if (!alone) ok = grid_wait(bar, ++nbar * G);
     stamp(6);
     if (!ok) goto fail;
-    for (uint32_t r = warp; r < n_rows; r += kPWarps) {
+    for (uint32_t r = warp; r < n_rows && !alone; r += kPWarps) {
       uint32_t tl = 0, te = 0, pl = 0, pe = 0;
       for (uint32_t c0 = 0; c0 < G; c0 += 160u) {
         uint32_t v[5];   // (loads in flight together)
@@ -957,8 +975,9 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
     pd = d;
   }
   if (pd.state != 1) return cudaSuccess;
-  // One CTA per SM, but none with less than 1,024 entries (more CTAs only make the exchanges wider).
-  uint64_t ctas = (n + kPChunk / 4 - 1) / (kPChunk / 4);
+  // One CTA per SM, but none with less than 1,024 entries (more CTAs only make the exchanges wider);
+  // up to kPAlone entries one CTA, which exchanges nothing and needs no cooperative launch.
+  uint64_t ctas = n <= kPAlone ? 1 : (n + kPChunk / 4 - 1) / (kPChunk / 4);
   if (ctas > (uint64_t)pd.n_sm) ctas = (uint64_t)pd.n_sm;
   if (ctas > kPThreads) ctas = kPThreads;
   const uint32_t G = ctas ? (uint32_t)ctas : 1u;
@@ -1014,7 +1033,7 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
              : !fs ? (void*)select_persistent_kernel<false, false, false>
                    : plain ? (void*)select_persistent_kernel<true, true, false>
                            : (void*)select_persistent_kernel<true, false, false>;
-  cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, true, ws);
+  cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, G > 1, ws);
   if (e != cudaSuccess) return e;
   count_launches(1);
   *used = true;

@@ -211,7 +211,8 @@ struct Workspace {
 // Launches fn (kernel taking the arguments in args) with the workspace's L2 window, if it has
 // one, as a launch attribute; cooperative launches carry that attribute too.
 inline cudaError_t launch_scoring_kernel(const void* fn, dim3 grid, dim3 block, void** args, size_t smem,
-                                         cudaStream_t s, bool cooperative, const Workspace& ws) {
+                                         cudaStream_t s, bool cooperative, const Workspace& ws,
+                                         bool overlap = true) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -222,6 +223,10 @@ inline cudaError_t launch_scoring_kernel(const void* fn, dim3 grid, dim3 block, 
   if (cooperative) {
     attr[n].id = cudaLaunchAttributeCooperative;
     attr[n].val.cooperative = 1;
+    ++n;
+  } else if (overlap) {   // (see wait_for_kernel_ahead)
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
     ++n;
   }
   if (ws.l2_bytes) {
@@ -238,13 +243,15 @@ inline cudaError_t launch_scoring_kernel(const void* fn, dim3 grid, dim3 block, 
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-// A kernel launched with launch_overlapped may be set up while the kernel ahead of it in the
-// stream is still finishing (programmatic dependent launch): it calls this before it touches
-// memory, which waits until everything ahead of it is complete and visible, and lets the
-// kernel behind it be set up in turn.
-__device__ __forceinline__ void launch_dependents_and_wait() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// A kernel launched with launch_overlapped (or launch_scoring_kernel, if not cooperative) may be
+// set up while the kernel ahead of it in the stream is still finishing (programmatic dependent
+// launch).  It calls this before it touches memory, which waits until everything ahead of it is
+// complete and visible, and then lets the kernel behind it be set up in turn.  Such a kernel reads
+// nothing through the read-only (non-coherent) path: the kernel ahead may have written it while this
+// one was already resident.  About 1 us per kernel of a chain.
+__device__ __forceinline__ void wait_for_kernel_ahead() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename... Params, typename... Args>
