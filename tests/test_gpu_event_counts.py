@@ -11,7 +11,7 @@ from paper_2604_26968_b200 import workloads as W
 pytestmark = pytest.mark.gpu
 
 BLOCK = 512 * 4                # events of one block's vectors
-GRID = BLOCK * 296             # events of one vector for every thread of the grid
+GRID = BLOCK * 296             # events of one vector for every thread of the grid (over 8 of them: part is dealt out by demand)
 
 
 def trace(style, n, n_events, r):
@@ -25,7 +25,7 @@ def trace(style, n, n_events, r):
 
 
 @pytest.mark.parametrize("style", ["single", "hot", "runs", "broken"])
-@pytest.mark.parametrize("n_events", [1, 3, 4, 7, 128, BLOCK - 4, BLOCK, BLOCK + 5, GRID - 1, GRID + 4, 3 * GRID + 1234])
+@pytest.mark.parametrize("n_events", [1, 3, 4, 7, 128, BLOCK - 4, BLOCK, BLOCK + 5, GRID - 1, GRID + 4, 3 * GRID + 1234, 9 * GRID + 6, 21 * GRID - 2])
 def test_counts(style, n_events):
     import torch
     parts = [W.gqa(3, 6, 3, 16, 8, 7001, 16, "entry")]      # 63,009 entries
