@@ -78,8 +78,7 @@ entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights h
   const uint64_t i = n4 * 4 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < st.n) {
     float sc;
-    uint32_t s1;
-    entry_update1(st, i, sP, policy, epoch, hw, sc, s1);
+    entry_update1(st, i, sP, policy, epoch, hw, sc);
   }
   // commit by the last block to finish
   __syncthreads();

@@ -257,10 +257,11 @@ __device__ __forceinline__ void head_weights4(const HeadWeights& hw, uint64_t i0
 // touch, this epoch's touches included) -- the three policies the paper compares.
 // w: weight of the entry's (layer, head), which the two importance-based policies
 // multiply in (1 = unweighted; x * 1 is exact).
+// pair: the entry's pair byte, whose bit 7 says FREE (the state byte is not read: one byte in 22).
 __device__ __forceinline__ void entry_step(float& ema, float decay, uint32_t touch, uint32_t pair,
-                                           uint32_t state, const float* sP, int policy,
+                                           const float* sP, int policy,
                                            uint32_t last_epoch, uint32_t epoch, float w, float& score) {
-  if (state == KV_STATE_RESIDENT) {
+  if (!(pair & kPairFree)) {
     const float x = __uint2float_rn(touch);
     const float t1 = __fmul_rn(decay, ema);
     const float t2 = __fsub_rn(1.0f, decay);
@@ -373,7 +374,7 @@ __device__ __forceinline__ void commit_predictor(const Predictor& pd, unsigned p
 struct EntryVec {
   float4 e, d;
   uint4 t, le;
-  uint32_t pr4, st4;   // pair and state bytes
+  uint32_t pr4;        // pair bytes
 };
 
 __device__ __forceinline__ EntryVec entry_load4(const EntryState& st, uint64_t v, int policy) {
@@ -382,7 +383,6 @@ __device__ __forceinline__ EntryVec entry_load4(const EntryState& st, uint64_t v
   x.d = reinterpret_cast<const float4*>(st.decay)[v];
   x.t = __ldcg(reinterpret_cast<const uint4*>(st.touch) + v);
   x.pr4 = reinterpret_cast<const uint32_t*>(st.pair)[v];
-  x.st4 = reinterpret_cast<const uint32_t*>(st.state)[v];
   x.le = make_uint4(0, 0, 0, 0);
   if (policy == 2) x.le = reinterpret_cast<const uint4*>(st.last_epoch)[v];  // only LRU reads it
   return x;
@@ -397,12 +397,13 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
   float e[4] = {x.e.x, x.e.y, x.e.z, x.e.w}, s[4];
   const float d[4] = {x.d.x, x.d.y, x.d.z, x.d.w};
   const uint32_t t[4] = {x.t.x, x.t.y, x.t.z, x.t.w}, le[4] = {x.le.x, x.le.y, x.le.z, x.le.w};
-  const bool all_resident = x.st4 == KV_STATE_RESIDENT * 0x01010101u;   // nearly always
+  // (nearly always all four are RESIDENT: one test then serves them)
+  const uint32_t free4 = x.pr4 & (kPairFree * 0x01010101u);
   float w[4] = {1.0f, 1.0f, 1.0f, 1.0f};
   if (!kPlain && hw.on) head_weights4(hw, 4 * v, w);
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    entry_step(e[j], d[j], t[j], x.pr4 >> (8 * j), all_resident ? KV_STATE_RESIDENT : (x.st4 >> (8 * j)) & 0xFFu, sP,
+    entry_step(e[j], d[j], t[j], free4 ? (x.pr4 >> (8 * j)) & 0xFFu : (x.pr4 >> (8 * j)) & 15u, sP,
                kPlain ? 0 : policy, le[j], epoch, w[j], s[j]);
   sc = make_float4(s[0], s[1], s[2], s[3]);
   reinterpret_cast<float4*>(st.ema)[v] = make_float4(e[0], e[1], e[2], e[3]);
@@ -423,14 +424,11 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
 
 // The same for one entry (ragged ends).
 __device__ __forceinline__ void entry_update1(const EntryState& st, uint64_t i, const float* sP, int policy,
-                                              uint32_t epoch, const HeadWeights& hw, float& sc,
-                                              uint32_t& state1) {
+                                              uint32_t epoch, const HeadWeights& hw, float& sc) {
   float e = st.ema[i];
   const uint32_t t = __ldcg(&st.touch[i]);
-  state1 = st.state[i];
   const float w = hw.on ? head_weight(hw, i) : 1.0f;
-  entry_step(e, st.decay[i], t, st.pair[i], state1, sP, policy, policy == 2 ? st.last_epoch[i] : 0u, epoch, w,
-             sc);
+  entry_step(e, st.decay[i], t, st.pair[i], sP, policy, policy == 2 ? st.last_epoch[i] : 0u, epoch, w, sc);
   st.ema[i] = e;
   st.score[i] = sc;
   if (t) {

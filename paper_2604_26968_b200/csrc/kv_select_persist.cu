@@ -72,8 +72,8 @@ constexpr uint32_t kNoteKeyBits = 22, kKeptKeyBits = 11;
 static_assert(kBracketShiftMax + 11 <= kNoteKeyBits && kNoteKeyBits + 7 <= 32, "a note holds any key of the bracket");
 static_assert(kBracketShiftMax <= kKeptKeyBits && kPMaxRows <= 64, "a kept note holds any key of a bin, and its row");
 // Fused form: the entry pass's inputs of one row in shared memory -- ema, decay, touch and,
-// for the LRU policy, last_epoch (4,096 words each), pair and state bytes (1,024 words each)
-constexpr uint32_t kStageWords = 3u * kPChunk + 2u * kPThreads;
+// for the LRU policy, last_epoch (4,096 words each), pair bytes (1,024 words)
+constexpr uint32_t kStageWords = 3u * kPChunk + kPThreads;
 constexpr uint32_t kStageWordsLru = kStageWords + kPChunk;
 constexpr uint64_t kPAlone = 2 * kPChunk;
 constexpr uint32_t kStages = 2;                         // rows in flight ahead of the one being finished
@@ -341,7 +341,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kPChunk), "l"(a.st.decay + i0) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 8u * kPChunk), "l"(a.st.touch + i0) : "memory");
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d1), "l"(a.st.pair + i0) : "memory");
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d1 + 4u * kPThreads), "l"(a.st.state + i0) : "memory");
         if (!PLAIN && a.pd.policy == 2) {
           const uint32_t d2 = (uint32_t)__cvta_generic_to_shared(dst + kStageWords + 4u * t);
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d2), "l"(a.st.last_epoch + i0) : "memory");
@@ -450,7 +449,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         cur.d = *reinterpret_cast<const float4*>(src + kPChunk + 4u * t);
         cur.t = *reinterpret_cast<const uint4*>(src + 2u * kPChunk + 4u * t);
         cur.pr4 = src[3u * kPChunk + t];
-        cur.st4 = src[3u * kPChunk + kPThreads + t];
         cur.le = make_uint4(0, 0, 0, 0);
         if (!PLAIN && policy == 2) cur.le = *reinterpret_cast<const uint4*>(src + kStageWords + 4u * t);
         issue(r + kStages);
@@ -461,10 +459,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         issue(r + kStages);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {   // the pool's ragged end
-          if (i0 + j < i1) {
-            uint32_t s1;
-            entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, s[j], s1);
-          }
+          if (i0 + j < i1) entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, s[j]);
         }
       }
       if (r + 2u == n_rows || n_rows == 1u) warm_lines();
