@@ -236,7 +236,7 @@ def kv_entry_bytes(model: kv_model_desc, block_tokens: int) -> int:
 
 
 def _stream_ptr(s):
-    return C.c_void_p(s.cuda_stream if s is not None else 0)
+    return s.cuda_stream if s is not None else 0   # (the argument types make it a pointer)
 
 
 def kv_dedup_table_slots(m: int) -> int:
@@ -489,8 +489,7 @@ class Pool:
 
     def kv_promote(self, partition, h_slots, batch_bytes):
         h_slots = np.ascontiguousarray(h_slots, dtype=np.uint64)
-        return self.lib.kv_promote(self._h, partition, h_slots.ctypes.data_as(C.c_void_p) if h_slots.size else None,
-                                   h_slots.size, int(batch_bytes), _stream_ptr(self.compute),
+        return self.lib.kv_promote(self._h, partition, h_slots.ctypes.data if h_slots.size else None, h_slots.size, int(batch_bytes), _stream_ptr(self.compute),
                                    _stream_ptr(self.copy_h2d))
 
     def kv_admit(self, epoch, decay, d_new_pairs, fill_pattern=True):

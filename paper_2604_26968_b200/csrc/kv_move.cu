@@ -35,10 +35,10 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long x) {
 }
 
 __global__ void __launch_bounds__(kThreads)
-admit_kernel(const PartGeom g, const EntryState st, uint32_t* __restrict__ loc,
-             const uint32_t* __restrict__ free_ids, uint64_t first, uint64_t count, uint64_t first_tag,
-             const uint8_t* __restrict__ new_pairs, uint32_t epoch, float decay, int fill_pattern,
-             uint32_t* __restrict__ status) {
+admit_kernel(const PartGeom g, const EntryState st, uint32_t* loc, const uint32_t* free_ids, uint64_t first,
+             uint64_t count, uint64_t first_tag, const uint8_t* new_pairs, uint32_t epoch, float decay,
+             int fill_pattern, uint32_t* status) {
+  wait_for_kernel_ahead();
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t ppc = (g.chunk_bytes + kPieceBytes - 1) / kPieceBytes;
   const uint32_t ppe = fill_pattern ? ppc * g.n_chunks : 1u;
@@ -97,10 +97,8 @@ cudaError_t launch_admit(const PartGeom& g, const EntryState& st, uint32_t* loc,
                          cudaStream_t s) {
   if (count == 0) return cudaSuccess;
   const uint64_t pieces = count * (fill_pattern ? pieces_per_entry(g) : 1);
-  admit_kernel<<<move_grid(pieces), kThreads, 0, s>>>(g, st, loc, free_ids, first, count, first_tag,
-                                                      new_pairs, epoch, decay, fill_pattern, ws.status);
-  count_launches(1);
-  return cudaGetLastError();
+  return launch_overlapped(admit_kernel, move_grid(pieces), (unsigned)kThreads, s, g, st, loc, free_ids, first, count,
+                           first_tag, new_pairs, epoch, decay, fill_pattern, ws.status);
 }
 
 // ---- initialisation ---------------------------------------------------------------

@@ -109,6 +109,13 @@ struct MoveArgs {
   uint8_t* host_meta;      // pack: where the device sees the pinned kv_slot_meta records (nullptr: none)
 };
 
+// A short promote list travels with the launch itself: no copy to the device, no buffer to wait
+// for (they took 8 us of the host's time and 1 us of the copy stream's per call).
+struct ListedMoveArgs {
+  MoveArgs a;
+  uint32_t slots[kInlineSlots];
+};
+
 // Metadata of one demoted entry (ring slot mirror, block table, slot state); its record is left
 // in rec.
 __device__ __forceinline__ void demote_meta(const MoveArgs& a, uint64_t j, uint32_t v, uint32_t rec[6]) {
@@ -170,9 +177,9 @@ __device__ __forceinline__ void promote_meta(const MoveArgs& a, uint32_t f, uint
 
 // PACK = true: slab -> staging (entry images back to back).  PACK = false: staging -> slab.
 // Each CTA owns a contiguous range of entries [e0, e1).
-template <bool PACK>
-__global__ void __launch_bounds__(kMoveThreads)
-move_tma_kernel(const MoveArgs a) {
+// slot_of(j): ring slot of the j-th entry (unpack only).
+template <bool PACK, typename SlotOf>
+__device__ __forceinline__ void move_entries(const MoveArgs& a, SlotOf slot_of) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t bars[kStages];
   const PartGeom& g = a.g;
@@ -239,7 +246,7 @@ move_tma_kernel(const MoveArgs a) {
           atomicOr(a.status, KV_DEV_BAD_INDEX);
           continue;
         }
-        const uint32_t slot = a.slots[j];
+        const uint32_t slot = slot_of(j);
         if (slot >= g.ring_slots) {
           atomicOr(a.status, KV_DEV_BAD_INDEX);
           continue;
@@ -326,6 +333,16 @@ move_tma_kernel(const MoveArgs a) {
   }
 }
 
+template <bool PACK>
+__global__ void __launch_bounds__(kMoveThreads) move_tma_kernel(const MoveArgs a) {
+  if constexpr (PACK) wait_for_kernel_ahead();
+  move_entries<PACK>(a, [&](uint64_t j) { return a.slots[j]; });
+}
+
+__global__ void __launch_bounds__(kMoveThreads) unpack_listed_kernel(const __grid_constant__ ListedMoveArgs l) {
+  move_entries<false>(l.a, [&](uint64_t j) { return l.slots[j]; });
+}
+
 // ---- promotion of scattered host entries --------------------------------------------
 // A prefetch list ordered by token position names, for every block, its layers one after
 // the other; in the host ring only a block's heads are neighbours, its layers lie a whole
@@ -337,8 +354,8 @@ move_tma_kernel(const MoveArgs a) {
 constexpr uint32_t kGatherPiece = 2048;   // 32 lanes x 4 x 16 bytes
 constexpr uint32_t kGatherThreads = 256;
 
-__global__ void __launch_bounds__(kGatherThreads)
-gather_promote_kernel(const MoveArgs a, const uint8_t* __restrict__ ring) {
+template <typename SlotOf>
+__device__ __forceinline__ void gather_entries(const MoveArgs& a, const uint8_t* __restrict__ ring, SlotOf slot_of) {
   const PartGeom& g = a.g;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t ppc = (g.chunk_bytes + kGatherPiece - 1) / kGatherPiece;  // pieces per chunk
@@ -351,7 +368,7 @@ gather_promote_kernel(const MoveArgs a, const uint8_t* __restrict__ ring) {
     const uint32_t c = r / ppc;
     const uint32_t in_chunk = (r - c * ppc) * kGatherPiece;
     const uint32_t f = a.ids[j];
-    const uint32_t slot = a.slots[j];
+    const uint32_t slot = slot_of(j);
     if ((uint64_t)f < g.base || (uint64_t)f >= g.base + g.n || slot >= g.ring_slots) {
       if (lane == 0 && r == 0) atomicOr(a.status, KV_DEV_BAD_INDEX);
       continue;
@@ -374,11 +391,26 @@ gather_promote_kernel(const MoveArgs a, const uint8_t* __restrict__ ring) {
   }
 }
 
+__global__ void __launch_bounds__(kGatherThreads)
+gather_promote_kernel(const MoveArgs a, const uint8_t* __restrict__ ring) {
+  gather_entries(a, ring, [&](uint64_t j) { return a.slots[j]; });
+}
+
+__global__ void __launch_bounds__(kGatherThreads)
+gather_listed_kernel(const __grid_constant__ ListedMoveArgs l, const uint8_t* __restrict__ ring) {
+  gather_entries(l.a, ring, [&](uint64_t j) { return l.slots[j]; });
+}
+
+static void list_slots(ListedMoveArgs& l, const uint64_t* h_slots, uint64_t count) {
+  for (uint64_t j = 0; j < count; ++j) l.slots[j] = (uint32_t)h_slots[j];
+}
+
 cudaError_t launch_gather_promote(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* slots,
-                                  const uint32_t* free_ids, uint64_t count, const uint8_t* ring_dev,
-                                  const Workspace& ws, cudaStream_t s) {
+                                  const uint64_t* h_slots, const uint32_t* free_ids, uint64_t count,
+                                  const uint8_t* ring_dev, const Workspace& ws, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
-  MoveArgs a{g, st, loc, free_ids, slots, count, 0, nullptr, ~0ull, ws.status, kMoveAll, nullptr, nullptr};
+  ListedMoveArgs l;
+  l.a = MoveArgs{g, st, loc, free_ids, slots, count, 0, nullptr, ~0ull, ws.status, kMoveAll, nullptr, nullptr};
   const uint64_t pieces = count * ((g.chunk_bytes + kGatherPiece - 1) / kGatherPiece) * g.n_chunks;
   uint64_t blocks = (pieces * 32 + kGatherThreads - 1) / kGatherThreads;
   // 32 blocks keep 512 KB of reads in flight, several round trips' worth of the host link; more
@@ -386,7 +418,13 @@ cudaError_t launch_gather_promote(const PartGeom& g, const EntryState& st, uint3
   // (measured: both directions together carry ~63 GB/s whatever the split)
   const uint64_t cap = 32;
   if (blocks > cap) blocks = cap;
-  gather_promote_kernel<<<(unsigned)(blocks ? blocks : 1), kGatherThreads, 0, s>>>(a, ring_dev);
+  if (blocks == 0) blocks = 1;
+  if (h_slots) {
+    list_slots(l, h_slots, count);
+    gather_listed_kernel<<<(unsigned)blocks, kGatherThreads, 0, s>>>(l, ring_dev);
+  } else {
+    gather_promote_kernel<<<(unsigned)blocks, kGatherThreads, 0, s>>>(l.a, ring_dev);
+  }
   count_launches(1);
   return cudaGetLastError();
 }
@@ -397,20 +435,26 @@ static unsigned tma_grid(uint64_t count) {
   return (unsigned)(blocks ? blocks : 1);
 }
 
-template <bool PACK>
-static cudaError_t launch_move(const MoveArgs& a, cudaStream_t s) {
-  // the opt-in for the shared memory belongs to a device: once per device ordinal
-  static std::atomic<bool> configured[64];
-  const size_t smem = (size_t)kStages * kStageBytes;
+// the opt-in for the shared memory belongs to a device: once per device ordinal
+template <typename Kernel>
+static cudaError_t opt_in(Kernel kernel, std::atomic<bool> (&configured)[64]) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaGetLastError();
-  if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(move_tma_kernel<PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
-  }
-  move_tma_kernel<PACK><<<tma_grid(a.count), kMoveThreads, smem, s>>>(a);
+  if (dev >= 0 && dev < 64 && configured[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(kStages * kStageBytes));
+  if (e == cudaSuccess && dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
+  return e;
+}
+
+template <bool PACK>
+static cudaError_t launch_move(const MoveArgs& a, cudaStream_t s) {
+  static std::atomic<bool> configured[64];
+  const cudaError_t e = opt_in(move_tma_kernel<PACK>, configured);
+  if (e != cudaSuccess) return e;
+  if constexpr (PACK)
+    return launch_overlapped_smem(move_tma_kernel<PACK>, tma_grid(a.count), kMoveThreads, kStages * kStageBytes, s, a);
+  move_tma_kernel<PACK><<<tma_grid(a.count), kMoveThreads, kStages * kStageBytes, s>>>(a);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -425,12 +469,20 @@ cudaError_t launch_pack_tma(const PartGeom& g, const EntryState& st, uint32_t* l
 }
 
 cudaError_t launch_unpack_tma(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* slots,
-                              const uint32_t* free_ids, uint64_t count, const uint8_t* staging,
-                              const Workspace& ws, cudaStream_t s) {
+                              const uint64_t* h_slots, const uint32_t* free_ids, uint64_t count,
+                              const uint8_t* staging, const Workspace& ws, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
-  MoveArgs a{g, st, loc, free_ids, slots, count, 0, const_cast<uint8_t*>(staging), ~0ull, ws.status, kMoveAll,
-             nullptr, nullptr};
-  return launch_move<false>(a, s);
+  ListedMoveArgs l;
+  l.a = MoveArgs{g, st, loc, free_ids, slots, count, 0, const_cast<uint8_t*>(staging), ~0ull, ws.status, kMoveAll,
+                 nullptr, nullptr};
+  if (!h_slots) return launch_move<false>(l.a, s);
+  static std::atomic<bool> configured[64];
+  const cudaError_t e = opt_in(unpack_listed_kernel, configured);
+  if (e != cudaSuccess) return e;
+  list_slots(l, h_slots, count);
+  unpack_listed_kernel<<<tma_grid(count), kMoveThreads, kStages * kStageBytes, s>>>(l);
+  count_launches(1);
+  return cudaGetLastError();
 }
 
 }  // namespace kvt

@@ -1020,11 +1020,12 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
     if (rcj != KV_OK) { for (uint64_t j2 = 0; j2 < m; ++j2) h.live[h_slots[j2]] = 1; return rcj; }
   }
   const uint64_t per = batch_bytes / eb;
+  const bool listed = m <= kInlineSlots;   // the list travels in the launches' arguments
   const int li = p->list_turn;
-  p->list_turn = (p->list_turn + 1) % kListBufs;
+  if (!listed) p->list_turn = (p->list_turn + 1) % kListBufs;
   auto restore = [&]() { for (uint64_t j = 0; j < m; ++j) h.live[h_slots[j]] = 1; };
   // the list given kListBufs calls ago must have left this pinned buffer: normally long done
-  cudaError_t e = p->list_used[li] ? cudaEventQuery(p->ev_list_copied[li]) : cudaSuccess;
+  cudaError_t e = !listed && p->list_used[li] ? cudaEventQuery(p->ev_list_copied[li]) : cudaSuccess;
   if (e == cudaErrorNotReady) {
     (void)cudaGetLastError();
     p->stats.host_waits += 1;
@@ -1040,7 +1041,7 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
   bool hits_pending = false, hits_newest = false;
   for (uint64_t j = 0; j < m; ++j) {
     const uint64_t s = h_slots[j];
-    p->h_list[li][j] = (uint32_t)s;
+    if (!listed) p->h_list[li][j] = (uint32_t)s;
     if (q_pending && (s + R - pd.cursor0[q]) % R < pd.kq[q]) hits_pending = true;
     if (p->d2h[q][0].valid && (s + R - p->d2h[q][0].start) % R < p->d2h[q][0].count) hits_newest = true;
   }
@@ -1055,12 +1056,14 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
   if (e == cudaSuccess && hits_newest) e = cudaStreamWaitEvent(copy, p->d2h[q][0].ev, 0);
   if (e == cudaSuccess && !hits_newest && p->d2h[q][1].valid)
     e = cudaStreamWaitEvent(copy, p->d2h[q][1].ev, 0);
-  if (e == cudaSuccess)
-    e = cudaStreamWaitEvent(copy, p->ev_list_free[li], 0);  // older kernels are done reading the device list
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(p->ws.slot_list[li], p->h_list[li], m * 4, cudaMemcpyHostToDevice, copy);
-  if (e == cudaSuccess) e = cudaEventRecord(p->ev_list_copied[li], copy);
-  p->list_used[li] = true;
+  if (!listed) {
+    if (e == cudaSuccess)
+      e = cudaStreamWaitEvent(copy, p->ev_list_free[li], 0);  // older kernels are done reading the device list
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(p->ws.slot_list[li], p->h_list[li], m * 4, cudaMemcpyHostToDevice, copy);
+    if (e == cudaSuccess) e = cudaEventRecord(p->ev_list_copied[li], copy);
+    p->list_used[li] = true;
+  }
   // this partition's free slots, ascending, in the partition's own stretch of the list scratch
   if (e == cudaSuccess && !h.free_known) {
     e = launch_free_list(p->st, g.base, g.base + g.n, m, p->ws, compute, g.base);
@@ -1117,13 +1120,13 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
     if (rc != KV_OK) return rc;
     TimedScope ts(p, gather ? 2 : 1, cnt * eb, copy);
     if (gather)
-      KV_CUDA(p, launch_gather_promote(g, p->st, p->desc.d_loc, p->ws.slot_list[li] + c0, free_ids + c0, cnt,
-                                       h.ring_dev, p->ws, copy));
+      KV_CUDA(p, launch_gather_promote(g, p->st, p->desc.d_loc, p->ws.slot_list[li] + c0, listed ? h_slots + c0 : nullptr,
+                                       free_ids + c0, cnt, h.ring_dev, p->ws, copy));
     else
-      KV_CUDA(p, launch_unpack_tma(g, p->st, p->desc.d_loc, p->ws.slot_list[li] + c0, free_ids + c0, cnt,
-                                   p->staging[2 + ((c0 / per) & 1u)], p->ws, copy));
+      KV_CUDA(p, launch_unpack_tma(g, p->st, p->desc.d_loc, p->ws.slot_list[li] + c0, listed ? h_slots + c0 : nullptr,
+                                   free_ids + c0, cnt, p->staging[2 + ((c0 / per) & 1u)], p->ws, copy));
   }
-  KV_CUDA(p, cudaEventRecord(p->ev_list_free[li], copy));
+  if (!listed) KV_CUDA(p, cudaEventRecord(p->ev_list_free[li], copy));
   KV_CUDA(p, cudaEventRecord(p->ev_h2d_done, copy));
   KV_CUDA(p, cudaEventRecord(p->ev_promoted[q], copy));
   p->promote_open[q] = true;

@@ -255,11 +255,12 @@ __device__ __forceinline__ void wait_for_kernel_ahead() {
 }
 
 template <typename... Params, typename... Args>
-inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, cudaStream_t s,
-                                     Args... args) {
+inline cudaError_t launch_overlapped_smem(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem,
+                                          cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -268,6 +269,12 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, u
   cfg.numAttrs = 1;
   count_launches(1);
   return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, unsigned block, cudaStream_t s,
+                                     Args... args) {
+  return launch_overlapped_smem(kernel, grid, block, 0, s, args...);
 }
 
 // ---- kv_score.cu ----
@@ -369,15 +376,18 @@ cudaError_t launch_pack_tma(const PartGeom& g, const EntryState& st, uint32_t* l
                             uint64_t count, uint64_t ring_start, uint8_t* staging, uint64_t meta_offset,
                             const Workspace& ws, cudaStream_t s, uint32_t mode = 0, uint32_t* free_out = nullptr,
                             uint8_t* host_meta = nullptr);
-// unpack: staging images [0, count) into the listed free slots of the partition
+// Longest promote list that travels in a launch's arguments (2 KB of them).
+constexpr uint32_t kInlineSlots = 512;
+// unpack: staging images [0, count) into the listed free slots of the partition; the ring slots they
+// come from are listed in h_slots (host, count <= kInlineSlots) or, without it, in slots (device)
 cudaError_t launch_unpack_tma(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* slots,
-                              const uint32_t* free_ids, uint64_t count, const uint8_t* staging,
-                              const Workspace& ws, cudaStream_t s);
+                              const uint64_t* h_slots, const uint32_t* free_ids, uint64_t count,
+                              const uint8_t* staging, const Workspace& ws, cudaStream_t s);
 // the same scatter with the entries fetched by the kernel itself from the pinned ring (ring_dev:
 // the address at which the device sees it): for lists of short runs
 cudaError_t launch_gather_promote(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* slots,
-                                  const uint32_t* free_ids, uint64_t count, const uint8_t* ring_dev,
-                                  const Workspace& ws, cudaStream_t s);
+                                  const uint64_t* h_slots, const uint32_t* free_ids, uint64_t count,
+                                  const uint8_t* ring_dev, const Workspace& ws, cudaStream_t s);
 // admits free_ids[0 .. count) of one partition, which are the pool's free slots number first ...
 cudaError_t launch_admit(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* free_ids,
                          uint64_t first, uint64_t count, uint64_t first_tag, const uint8_t* new_pairs,
