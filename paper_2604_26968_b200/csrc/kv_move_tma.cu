@@ -401,6 +401,74 @@ gather_listed_kernel(const __grid_constant__ ListedMoveArgs l, const uint8_t* __
   gather_entries(l.a, ring, [&](uint64_t j) { return l.slots[j]; });
 }
 
+// ---- demotion of a few entries ----------------------------------------------------
+// A small demotion is latency: packing into a staging buffer, a transfer (two where the ring
+// wraps) and the events between them took 41 us for 0.8 MB, of which the link needs 15.  This
+// kernel stores the entries straight into the pinned ring, a warp per piece of up to 2 KB.
+__global__ void __launch_bounds__(kGatherThreads) pack_direct_kernel(const MoveArgs a, uint8_t* ring) {
+  wait_for_kernel_ahead();
+  const PartGeom& g = a.g;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t ppc = (g.chunk_bytes + kGatherPiece - 1) / kGatherPiece;  // pieces per chunk
+  const uint32_t ppe = ppc * g.n_chunks;                                    // pieces per entry
+  const uint64_t total = a.count * ppe;
+  const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t piece = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); piece < total; piece += warps) {
+    const uint64_t j = piece / ppe;
+    const uint32_t r = (uint32_t)(piece - j * ppe);
+    const uint32_t c = r / ppc;
+    const uint32_t in_chunk = (r - c * ppc) * kGatherPiece;
+    const uint32_t id = a.ids[j];
+    if (r == 0 && lane == 0 && a.free_out) a.free_out[j] = id;
+    if ((uint64_t)id < g.base || (uint64_t)id >= g.base + g.n) {
+      if (lane == 0 && r == 0) atomicOr(a.status, KV_DEV_BAD_INDEX);
+      continue;
+    }
+    const uint64_t slot = (a.ring_start + j) % g.ring_slots;
+    const uint32_t len = min(kGatherPiece, g.chunk_bytes - in_chunk);
+    const uint8_t* src = g.slab + slab_chunk_offset(g, (uint64_t)id - g.base, c) + in_chunk;
+    uint8_t* dst = ring + slot * g.entry_bytes + (uint64_t)c * g.chunk_bytes + in_chunk;
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t off = (u * 32 + lane) * 16;
+      if (off < len) v[u] = __ldcs(reinterpret_cast<const uint4*>(src + off));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t off = (u * 32 + lane) * 16;
+      if (off < len) __stcs(reinterpret_cast<uint4*>(dst + off), v[u]);
+    }
+    if (r == 0) {
+      uint32_t rec[6] = {KV_NONE, 0, 0, 0, 0, 0};
+      if (lane == 0) demote_meta(a, j, id, rec);
+      __syncwarp();
+      if (a.host_meta) {   // the record's six words from six lanes
+        uint32_t w = 0;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          const uint32_t x = __shfl_sync(0xFFFFFFFFu, rec[i], 0);
+          if (lane == (uint32_t)i) w = x;
+        }
+        const bool have = __shfl_sync(0xFFFFFFFFu, rec[0], 0) != KV_NONE;
+        if (have && lane < 6u) reinterpret_cast<uint32_t*>(a.host_meta + slot * kMetaBytes)[lane] = w;
+      }
+    }
+  }
+}
+
+cudaError_t launch_pack_direct(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* victims,
+                               uint64_t count, uint64_t ring_start, uint8_t* ring_dev, const Workspace& ws,
+                               cudaStream_t s, uint32_t* free_out, uint8_t* host_meta) {
+  if (count == 0) return cudaSuccess;
+  const MoveArgs a{g, st, loc, victims, nullptr, count, ring_start, nullptr, ~0ull, ws.status, kMoveAll, free_out, host_meta};
+  const uint64_t pieces = count * ((g.chunk_bytes + kGatherPiece - 1) / kGatherPiece) * g.n_chunks;
+  uint64_t blocks = (pieces * 32 + kGatherThreads - 1) / kGatherThreads;
+  const uint64_t cap = (uint64_t)sm_count();
+  if (blocks > cap) blocks = cap;
+  return launch_overlapped(pack_direct_kernel, (unsigned)blocks, kGatherThreads, s, a, ring_dev);
+}
+
 static void list_slots(ListedMoveArgs& l, const uint64_t* h_slots, uint64_t count) {
   for (uint64_t j = 0; j < count; ++j) l.slots[j] = (uint32_t)h_slots[j];
 }

@@ -376,6 +376,11 @@ cudaError_t launch_pack_tma(const PartGeom& g, const EntryState& st, uint32_t* l
                             uint64_t count, uint64_t ring_start, uint8_t* staging, uint64_t meta_offset,
                             const Workspace& ws, cudaStream_t s, uint32_t mode = 0, uint32_t* free_out = nullptr,
                             uint8_t* host_meta = nullptr);
+// pack of a few entries without staging: images (and records) straight into the pinned ring
+// (ring_dev, host_meta: the addresses at which the device sees them)
+cudaError_t launch_pack_direct(const PartGeom& g, const EntryState& st, uint32_t* loc, const uint32_t* victims,
+                               uint64_t count, uint64_t ring_start, uint8_t* ring_dev, const Workspace& ws,
+                               cudaStream_t s, uint32_t* free_out, uint8_t* host_meta);
 // Longest promote list that travels in a launch's arguments (2 KB of them).
 constexpr uint32_t kInlineSlots = 512;
 // unpack: staging images [0, count) into the listed free slots of the partition; the ring slots they

@@ -44,13 +44,14 @@ class Model:
 
 @pytest.mark.parametrize("deferred", [False, True])
 @pytest.mark.parametrize("host_meta", [False, True])
-@pytest.mark.parametrize("seed", [1, 2, 3])
-def test_sequences(seed, deferred, host_meta):
+@pytest.mark.parametrize("seed,batch", [(1, 20 << 10), (2, 20 << 10), (3, 20 << 10), (4, 512 << 10), (5, 512 << 10)])
+def test_sequences(seed, batch, deferred, host_meta):
+    """batch: several staged chunks per demotion, or (one chunk) stores straight into the ring."""
     import torch
     parts = [W.gqa(2, 8, 4, 16, 4, 331, 1500, "entry"), W.mla(3, 32, 32, 4, 517, 1100, "entry")]
     r = np.random.default_rng(seed)
     n = sum(p.n_entries for p in parts)
-    p = B.Pool(parts, 60_000, staging_bytes=64 << 10, max_promote=2048, host_meta=host_meta)
+    p = B.Pool(parts, 60_000, staging_bytes=2 * batch + (64 << 10), max_promote=2048, host_meta=host_meta)
     pairs = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
     torch.cuda.synchronize()
     assert p.kv_set_deferred_packing(deferred) == 0
@@ -67,7 +68,7 @@ def test_sequences(seed, deferred, host_meta):
             d_v = torch.from_numpy(np.concatenate([v, np.zeros(4, np.int64)]).astype(np.int32)).cuda()
             keep.append(d_v)                      # (deferred packing reads it later)
             torch.cuda.synchronize()
-            assert p.kv_demote(d_v, v.size, 20 << 10) == 0
+            assert p.kv_demote(d_v, v.size, batch) == 0
             m.demote(v)
         elif op == "promote":
             q = int(r.integers(0, 2))
@@ -77,7 +78,7 @@ def test_sequences(seed, deferred, host_meta):
                 continue
             start = int(r.integers(0, held.size - count + 1))
             slots = held[start:start + count] if r.random() < 0.5 else r.permutation(held)[:count]
-            assert p.kv_promote(q, slots.astype(np.uint64), 20 << 10) == 0
+            assert p.kv_promote(q, slots.astype(np.uint64), batch) == 0
             m.promote(q, slots)
         elif op == "select":
             resident = int((m.tag >= 0).sum())
