@@ -97,7 +97,7 @@ struct PArgs {
   uint32_t stage_words;   // fused form: words of one stage
   uint32_t scratch_words; // words of notes and stages together (the plain path's key cache)
   PartCounts pc;          // partitions of the pool (the victims per partition are a by-product)
-  uint32_t* spill;        // global scratch for the notes beyond note_cap: spill_stride words per warp (nullptr: none)
+  uint32_t* spill;        // global scratch for the notes beyond note_cap: spill_stride words per warp (nullptr: no hints)
   uint32_t spill_stride;
   BlockGeom bg;           // block form: the pool's paged blocks ...
   uint32_t expand;        // ... and, on a pool of one partition, entries per block (0: victims are block indices)
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const uint32_t tag = a.sel->serial + 1u;            // this launch's number
   SelectTurn* const turn = a.turns + (tag & 1u);
   unsigned int* const bar = &turn->bar;
-  const bool hint = a.use_hint && a.sel->hint_valid != 0 && a.sel->hint_n == a.n;
+  const bool hint = a.use_hint && a.spill && a.sel->hint_valid != 0 && a.sel->hint_n == a.n;
   const uint32_t hint_tau = a.sel->hint_tau;
   // The bracket's width follows how well the hints have been doing: 2,048 bins of 2^bshift keys.
   uint32_t bshift = a.sel->hint_shift;
@@ -392,10 +392,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   PendingBin ph;
   uint32_t* const my_nstart = s_nstart + warp * (n_rows + 1u);
   uint32_t* const my_note = s_note + warp * a.note_cap;
-  uint32_t* const my_spill = a.spill ? a.spill + (unsigned long long)(g * kPWarps + warp) * a.spill_stride : nullptr;
+  uint32_t* const my_spill = a.spill + (unsigned long long)(g * kPWarps + warp) * a.spill_stride;
   auto note_put = [&](uint32_t at, uint32_t note) {
     if (at < a.note_cap) my_note[at] = note;
-    else if (my_spill) my_spill[at - a.note_cap] = note;   // (a dense slice: the rest goes to L2)
+    else my_spill[at - a.note_cap] = note;   // (a dense slice: the rest goes to L2)
   };
   auto note_get = [&](uint32_t at) { return at < a.note_cap ? my_note[at] : __ldcg(my_spill + (at - a.note_cap)); };
   // The histograms and the table were written a pass ago and have left the L2 since: fetch their
@@ -511,7 +511,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   auto end_turn = [&]() { a.sel->serial = tag == 0xFFFFFFFFu ? 1u : tag; };
   uint32_t nbar = 0;        // grid barriers passed
   bool ok = true, hint_hit = false;
-  const bool notes_lost = !my_spill && n_noted > a.note_cap;
   if (FUSED || hint) {
     ph.flush(s_hist);
     n_below = __reduce_add_sync(0xFFFFFFFFu, n_below);
@@ -548,22 +547,17 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
       return grid_wait(bar, ++nbar * G);
     };
-    bool use_notes = false;
     uint32_t bin_k = 0;
     if (hint) {
       const unsigned long long below = alone ? s_below : __ldcg(&turn->below);
       const bool above = a.k > below;
       pick_bin(turn->hist[0], alone, s_hist, kHistBins, above ? a.k - below : 1ull, s_warp, s_pick, bin, before);
       hint_hit = above && bin != 0xFFFFFFFFu;
-      use_notes = hint_hit && __syncthreads_or(notes_lost) == 0;
       if (hint_hit) {
         k_rem = a.k - below - before;
         bin_k = bin;
       }
-      if (t == 0) {
-        if (g == 0) atomicAdd(hint_hit ? &a.sel->n_hint_hit : &a.sel->n_hint_miss, 1u);
-        if (hint_hit && !use_notes) atomicAdd(&a.sel->n_reread, 1u);
-      }
+      if (g == 0 && t == 0) atomicAdd(hint_hit ? &a.sel->n_hint_hit : &a.sel->n_hint_miss, 1u);
     }
     // keys of the thread's vector of row r, from the arrays; entries past the row's end or not
     // RESIDENT give kKeyExcluded
@@ -611,7 +605,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       rows_in_cache = cached_rows;
     };
 
-    if (use_notes) {
+    if (hint_hit) {
       // One pass over the notes: those of the bins before bin_k set their bits, those of bin_k
       // enter the histogram of its single keys and stay (moved to the front of the list).
       const uint32_t n_bins = 1u << bshift;
