@@ -63,13 +63,15 @@ constexpr uint32_t kPWarps = kPThreads / 32;
 constexpr uint32_t kPChunk = kPThreads * 4;             // 4096 entries: one 16-byte vector per thread
 constexpr uint32_t kPMaxRows = 64;                      // rows the bitmaps and tables are sized for
 constexpr uint32_t kBarrierSpins = 1u << 22;
-constexpr uint32_t kBracketShiftMax = 11;               // a bracket bin is at most 2^11 keys wide: the 2,048 bins then
-                                                        // reach 2^21 keys to either side of the hint ...
-constexpr uint32_t kBracketShiftMin = 7;                // ... and at least 2^7 (2^17 keys to either side)
+// The bracket reaches 2^17 .. 2^21 keys to either side of the hint; its bins, at most 2,048, are 2^7 ..
+// 2^11 keys wide.
+constexpr uint32_t kHalfMin = 1u << 17, kHalfMax = 1u << 21;
+constexpr uint32_t kBracketShiftMin = 7, kBracketShiftMax = 11;
+static_assert((2u * kHalfMax) >> kBracketShiftMax <= kHistBins, "the widest bracket has a bin for every key");
 // A note: key - base of the bracket (22 bits), lane (5 bits), position in the lane's vector (2
 // bits).  A kept note: key inside its bin (11 bits), lane, position, row (6 bits).
 constexpr uint32_t kNoteKeyBits = 22, kKeptKeyBits = 11;
-static_assert(kBracketShiftMax + 11 <= kNoteKeyBits && kNoteKeyBits + 7 <= 32, "a note holds any key of the bracket");
+static_assert(2u * kHalfMax <= 1u << kNoteKeyBits && kNoteKeyBits + 7 <= 32, "a note holds any key of the bracket");
 static_assert(kBracketShiftMax <= kKeptKeyBits && kPMaxRows <= 64, "a kept note holds any key of a bin, and its row");
 // Fused form: the entry pass's inputs of one row in shared memory -- ema, decay, touch and,
 // for the LRU policy, last_epoch (4,096 words each), pair bytes (1,024 words)
@@ -305,13 +307,14 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const uint32_t G = gridDim.x, g = blockIdx.x;
   const bool alone = G == 1u;   // one CTA: nothing is exchanged
   const uint32_t n_rows = a.n_rows;
-  auto row_base = [&](uint32_t r) -> unsigned long long {
-    return r < a.n_full ? ((unsigned long long)r * G + g) * kPChunk
-                        : (unsigned long long)a.n_full * G * kPChunk + (unsigned long long)g * a.last_len;
+  // (ids fit 31 bits)
+  const uint32_t n = (uint32_t)a.n;
+  auto row_base = [&](uint32_t r) -> uint32_t {
+    return r < a.n_full ? (r * G + g) * kPChunk : a.n_full * G * kPChunk + g * a.last_len;
   };
-  auto row_end = [&](uint32_t r) -> unsigned long long {   // (may lie below row_base: an empty piece)
-    const unsigned long long e = row_base(r) + (r < a.n_full ? kPChunk : a.last_len);
-    return e < a.n ? e : a.n;
+  auto row_end = [&](uint32_t r) -> uint32_t {   // (may lie below row_base: an empty piece)
+    const uint32_t e = row_base(r) + (r < a.n_full ? kPChunk : a.last_len);
+    return e < n ? e : n;
   };
   // Phase boundaries of CTA 0 for timing studies (compiled in with -DKV_PHASE_STAMPS only: a
   // read of the global timer stalls the thread for a few hundred nanoseconds).
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   // ---- prologue: the first rows' loads go out before anything else ----
   auto issue = [&](uint32_t r) {
     if constexpr (FUSED) {
-      const unsigned long long i0 = row_base(r) + 4u * t;
+      const uint32_t i0 = row_base(r) + 4u * t;
       if (r < n_rows && i0 + 4u <= row_end(r)) {
         uint32_t* dst = s_stage + (r % kStages) * a.stage_words;
         const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(dst + 4u * t);
@@ -358,8 +361,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   unsigned int* const bar = &turn->bar;
   const bool hint = a.use_hint && a.spill && a.sel->hint_valid != 0 && a.sel->hint_n == a.n;
   const uint32_t hint_tau = a.sel->hint_tau;
-  // The bracket's width follows how well the hints have been doing: 2,048 bins of 2^bshift keys.
-  uint32_t bshift = a.sel->hint_shift;
+  uint32_t half = a.sel->hint_half;   // (the bracket's width follows how well the hints have been doing)
   if constexpr (FUSED) {
     // reuse estimates from the totals plus this epoch's counts (final: the event
     // reduction is an earlier launch)
@@ -373,17 +375,17 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   for (uint32_t w = g * kPThreads + t; w < sizeof(SelectTurn) / 4u; w += G * kPThreads)
     reinterpret_cast<uint32_t*>(a.turns + ((tag & 1u) ^ 1u))[w] = 0;
   if (t == 0) s_below = 0;
-  bshift = bshift < kBracketShiftMin ? kBracketShiftMin : (bshift > kBracketShiftMax ? kBracketShiftMax : bshift);
-  const uint32_t bbits = bshift + 11u;                  // log2 of the bracket's width in keys
-  // The bracket [base0, base0 + 2^bbits) stays between the keys of -inf and of +inf, so that its
+  half = half < kHalfMin ? kHalfMin : (half > kHalfMax ? kHalfMax : half);
+  uint32_t bshift = kBracketShiftMin;                   // bins are 2^bshift keys wide
+  while ((2u * half - 1u) >> bshift >= kHistBins) ++bshift;
+  // The bracket [base0, base0 + 2 * half) stays between the keys of -inf and of +inf, so that its
   // ends are floats: comparing scores with them is comparing keys (the key order is the float
   // order, and the two zeros share a key).  An entry that is no candidate scores +inf.
-  const uint32_t bhalf = 1u << (bbits - 1u);
-  const uint32_t base_max = kKeyPosInf - (1u << bbits);
-  uint32_t base0 = hint_tau > bhalf ? hint_tau - bhalf : 0u;
+  const uint32_t base_max = kKeyPosInf - 2u * half;
+  uint32_t base0 = hint_tau > half ? hint_tau - half : 0u;
   base0 = base0 < kKeyNegInf ? kKeyNegInf : (base0 > base_max ? base_max : base0);
   const float neg_inf = __int_as_float(0xFF800000);
-  const float lo_f = hint ? key_score(base0) : neg_inf, hi_f = hint ? key_score(base0 + (1u << bbits)) : neg_inf;
+  const float lo_f = hint ? key_score(base0) : neg_inf, hi_f = hint ? key_score(base0 + 2u * half) : neg_inf;
   __syncthreads();
 
   // ---- phase A ----
@@ -440,7 +442,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     const int policy = PLAIN ? 0 : a.pd.policy;
     for (uint32_t r = 0; r < n_rows; ++r) {
       asm volatile("cp.async.wait_group 1;" ::: "memory");   // kStages - 1 newer groups may be pending
-      const unsigned long long i0 = row_base(r) + 4u * t, i1 = row_end(r);
+      const uint32_t i0 = row_base(r) + 4u * t, i1 = row_end(r);
       float s[4] = {inf, inf, inf, inf};
       if (i0 + 4u <= i1) {
         const uint32_t* src = s_stage + (r % kStages) * a.stage_words;
@@ -473,7 +475,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     float4 sc[kInFlight];
     uint32_t st4[kInFlight];
     auto load = [&](uint32_t r, uint32_t u) {
-      const unsigned long long i0 = row_base(r) + 4u * t;
+      const uint32_t i0 = row_base(r) + 4u * t;
       if (!BLOCKS && r < n_rows && i0 + 4u <= row_end(r)) {
         sc[u] = __ldcg(reinterpret_cast<const float4*>(a.score + i0));
         st4[u] = __ldcg(reinterpret_cast<const uint32_t*>(a.state + i0));
@@ -486,7 +488,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
 #pragma unroll
       for (uint32_t u = 0; u < kInFlight; ++u) {
         if (r + u < n_rows) {
-          const unsigned long long i0 = row_base(r + u) + 4u * t, i1 = row_end(r + u);
+          const uint32_t i0 = row_base(r + u) + 4u * t, i1 = row_end(r + u);
           float s[4] = {inf, inf, inf, inf};
           if (BLOCKS) {
             (void)block_scores4(a, i0, i1, s);
@@ -562,7 +564,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     // keys of the thread's vector of row r, from the arrays; entries past the row's end or not
     // RESIDENT give kKeyExcluded
     auto load_keys = [&](uint32_t r, uint32_t key[4]) {
-      const unsigned long long i0 = row_base(r) + 4u * t, i1 = row_end(r);
+      const uint32_t i0 = row_base(r) + 4u * t, i1 = row_end(r);
       if (BLOCKS) {
         float s[4];
         const uint32_t resident = block_scores4(a, i0, i1, s);
@@ -810,11 +812,11 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       ex += (quarter > 0u ? wt.x : 0u) + (quarter > 1u ? wt.y : 0u) + (quarter > 2u ? wt.z : 0u);
       uint32_t L = __shfl_sync(0xFFFFFFFFu, row < 32u ? rl0 : rl1, row & 31u) + (ex & 0xFFFFu);
       uint32_t E = __shfl_sync(0xFFFFFFFFu, row < 32u ? re0 : re1, row & 31u) + (ex >> 16);
-      const uint32_t id0 = (uint32_t)row_base(row) + 32u * (W & 127u);   // (ids fit 32 bits)
+      const uint32_t id0 = row_base(row) + 32u * (W & 127u);
       // a partition boundary at one of this word's entries: the victims before it
       for (uint32_t q = 1; (int)q < a.pc.n_parts; ++q) {
         const uint32_t b = (uint32_t)a.pc.base[q] - id0;
-        if (a.pc.base[q] < a.n && b < 32u && (unsigned long long)id0 + b < row_end(row)) {
+        if (a.pc.base[q] < a.n && b < 32u && id0 + b < row_end(row)) {
           const uint32_t m = (1u << b) - 1u;
           const uint32_t l = L + (uint32_t)__popc(bl & m), e = E + (uint32_t)__popc(be & m);
           publish_word(&a.sel->bound[q - 1], tag, l + (e < eq_room ? e : eq_room));
@@ -869,21 +871,22 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       long long guess = (long long)tau + step;
       if (guess < 0) guess = 0;
       if (guess > 0xFFFFFFFEll) guess = 0xFFFFFFFEll;
-      // ... and the bracket is as wide as the hints have been off lately: five to ten times a slowly
-      // decaying maximum of |tau - hinted tau|, full width again after a miss (a narrow
-      // bracket means fewer keys to note; a miss costs three passes over the keys)
-      uint32_t resid = a.sel->hint_resid, new_shift = kBracketShiftMax;
+      // ... and the bracket is as wide as the hints have been off lately: five times a slowly
+      // decaying maximum of |tau - hinted tau| to either side, full width again after a miss (a
+      // narrow bracket means fewer keys to note; a miss costs three passes over the keys.  Five times
+      // instead of the eight to sixteen of powers of two cost no further miss in 32 pools)
+      uint32_t resid = a.sel->hint_resid, new_half = kHalfMax;
       if (hint_hit) {
         const uint32_t off = tau > hint_tau ? tau - hint_tau : hint_tau - tau;
         resid -= resid >> 2;
         if (off > resid) resid = off;
-        new_shift = kBracketShiftMin;
-        while (new_shift < kBracketShiftMax && (1ull << (new_shift + 10u)) < 5ull * resid) ++new_shift;
+        new_half = resid < kHalfMax / 5u ? 5u * resid : kHalfMax;
+        if (new_half < kHalfMin) new_half = kHalfMin;
       } else {
         resid = 1u << 18;
       }
       a.sel->hint_resid = resid;
-      a.sel->hint_shift = new_shift;
+      a.sel->hint_half = new_half;
       a.sel->hint_last = tau;
       a.sel->hint_tau = (uint32_t)guess;
       a.sel->hint_n = a.n;

@@ -102,9 +102,9 @@ struct SelectScalars {
   // persistent selection on a pool of several partitions: launch number | victims before
   // partition boundary q + 1, written by the CTA that holds it
   unsigned long long bound[3];
-  // width of the next selection's bracket: its 2,048 bins are 2^hint_shift keys wide (7..11);
-  // hint_resid is a slowly decaying maximum of how far tau landed from where the hint put it
-  uint32_t hint_shift;
+  // how far the next selection's bracket reaches to either side of the hint, in keys; hint_resid is a
+  // slowly decaying maximum of how far tau landed from where the hint put it
+  uint32_t hint_half;
   uint32_t hint_resid;
 };
 
