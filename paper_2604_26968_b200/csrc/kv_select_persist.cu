@@ -824,6 +824,18 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       }
       if (!found) continue;
       uint32_t bits = (E >= eq_room) ? bl : (bl | be);
+      const uint32_t p0 = L + (E < eq_room ? E : eq_room);
+      // Where the warp has no entry equal to tau that is taken (nearly everywhere), a victim is a bit
+      // and a place: half the work of the general loop below (18.8 M entries 182.5 -> 181.0 us a
+      // pass, 0.9 M entries 28.7 -> 28.3).
+      if (!BLOCKS && __all_sync(0xFFFFFFFFu, (be == 0u || E >= eq_room) && p0 + (uint32_t)__popc(bits) <= (uint32_t)a.k)) {
+        uint32_t* out = a.victims + p0;
+        while (bits) {
+          *out++ = id0 + (uint32_t)__ffs(bits) - 1u;
+          bits &= bits - 1u;
+        }
+        continue;
+      }
       while (bits) {
         const uint32_t b = (uint32_t)__ffs(bits) - 1u;
         bits &= bits - 1u;
