@@ -293,7 +293,8 @@ int32_t kv_epoch_score_select(kv_pool* pool, uint32_t epoch, const uint32_t* d_e
 /* Demotes the m entries listed in d_victims (device, ascending distinct ids of
  * RESIDENT entries, as kv_select_victims writes them): packs their K/V (or MLA)
  * chunks into the staging buffers in chunks of at most batch_bytes on `compute`,
- * and copies each chunk to the partition's host ring on `copy`.  The j-th victim
+ * and copies each chunk to the partition's host ring on `copy` (at most 1 MiB in one
+ * batch: a kernel on `compute` stores them straight into the ring).  The j-th victim
  * of a partition takes ring slot (cursor + j) mod ring_slots; a live slot that
  * is overwritten is dropped (d_loc of its tag becomes KV_NONE).  Each victim's
  * slot becomes FREE, its tag KV_NONE, and d_loc[tag] = KV_LOC_HOST | slot.
@@ -578,8 +579,8 @@ int32_t kv_set_select_variant(kv_pool* pool, int32_t variant);
  * a hint (the threshold of the selection before it): a hit means one short pass after
  * the scoring pass finished it, a miss that the keys were read again (two or three
  * passes); reread_ctas counts thread blocks that read their keys again although the
- * hint held (more keys near the threshold than they could note).  Blocks the host
- * until `stream` has drained. */
+ * hint held: always 0 now, what a block cannot note in shared memory goes to a scratch.
+ * Blocks the host until `stream` has drained. */
 typedef struct {
   uint64_t selections, hint_hits, hint_misses, reread_ctas;
 } kv_select_stats;
