@@ -185,24 +185,6 @@ __device__ __forceinline__ void pick_bin(const uint32_t* hist, bool local, uint3
   before_bin = s_pick[1];
 }
 
-// A histogram count that waits in the thread while the bin stays the same: entries with equal
-// scores come in runs, and atomics of many threads on one hot bin serialise.
-struct PendingBin {
-  uint32_t bin = 0, cnt = 0;
-  __device__ __forceinline__ void add(uint32_t* s_hist, uint32_t b) {
-    if (b != bin) {
-      if (cnt) atomicAdd(&s_hist[bin], cnt);
-      bin = b;
-      cnt = 0;
-    }
-    ++cnt;
-  }
-  __device__ __forceinline__ void flush(uint32_t* s_hist) {
-    if (cnt) atomicAdd(&s_hist[bin], cnt);
-    cnt = 0;
-  }
-};
-
 // Scores of the four paged blocks b0 .. b0+3 (those below b1): the weighted sum over the block's
 // heads, added in head order with every operation rounded once; resident bit j: all heads of
 // block b0 + j are RESIDENT (the others score +inf).
@@ -391,7 +373,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   // ---- phase A ----
   uint32_t n_noted = 0;     // notes of this warp
   uint32_t n_below = 0;     // keys of this thread below the bracket
-  PendingBin ph;
   uint32_t* const my_nstart = s_nstart + warp * (n_rows + 1u);
   uint32_t* const my_note = s_note + warp * a.note_cap;
   uint32_t* const my_spill = a.spill + (unsigned long long)(g * kPWarps + warp) * a.spill_stride;
@@ -430,7 +411,9 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       for (int q = 0; q < 4; ++q) {
         if (in[q]) {
           const uint32_t d = score_key(s[q]) - base0;
-          ph.add(s_hist, d >> bshift);
+          // (additions of 1 to one bin are merged by the hardware: collecting a thread's equal bins in a
+          // register first cost 0.7 of 42.1 us at 3.1 M entries, 1.7 of 20.4 in the plain radix select)
+          atomicAdd(&s_hist[d >> bshift], 1u);
           note_put(n_noted + (uint32_t)__popc(wi[q] & lt), d | lane << kNoteKeyBits | (uint32_t)q << (kNoteKeyBits + 5));
         }
         n_noted += (uint32_t)__popc(wi[q]);
@@ -514,7 +497,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   uint32_t nbar = 0;        // grid barriers passed
   bool ok = true, hint_hit = false;
   if (FUSED || hint) {
-    ph.flush(s_hist);
     n_below = __reduce_add_sync(0xFFFFFFFFu, n_below);
     if (lane == 0) {
       my_nstart[n_rows] = n_noted;
@@ -611,7 +593,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       // One pass over the notes: those of the bins before bin_k set their bits, those of bin_k
       // enter the histogram of its single keys and stay (moved to the front of the list).
       const uint32_t n_bins = 1u << bshift;
-      PendingBin p2;
       uint32_t row = 0, row_ends = my_nstart[1];   // row of this lane's note (its places ascend)
       uint32_t n_kept = 0;
       for (uint32_t p0 = 0; p0 < n_noted; p0 += 128u) {
@@ -633,13 +614,12 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
           const uint32_t m = __ballot_sync(0xFFFFFFFFu, keep);
           if (keep) {
             const uint32_t low = d & (n_bins - 1u);
-            p2.add(s_hist, low);
+            atomicAdd(&s_hist[low], 1u);
             note_put(n_kept + (uint32_t)__popc(m & lt), low | at << kKeptKeyBits | row << (kKeptKeyBits + 7));
           }
           n_kept += (uint32_t)__popc(m);
         }
       }
-      p2.flush(s_hist);
       __syncwarp();
       stamp(8);
       ok = exchange_hist(1, n_bins);
@@ -665,15 +645,13 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       for (int digit = 0; digit < 3; ++digit) {
         const uint32_t shift = digit == 0 ? 21u : digit == 1 ? 10u : 0u, top = digit == 2 ? 10u : 11u;
         __syncthreads();   // (the notes are dead: their space becomes the key cache)
-        PendingBin p2;
         for_keys([&](uint32_t, const uint32_t key[4]) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const uint32_t d = (key[q] - base) >> shift;
-            if (key[q] != kKeyExcluded && key[q] >= base && (digit == 0 || (d >> top) == 0u)) p2.add(s_hist, d);
+            if (key[q] != kKeyExcluded && key[q] >= base && (digit == 0 || (d >> top) == 0u)) atomicAdd(&s_hist[d], 1u);
           }
         });
-        p2.flush(s_hist);
         ok = exchange_hist(h, 1u << top);
         if (digit == 1) stamp(3);
         if (!ok) goto fail;
