@@ -19,10 +19,11 @@
 //                         cycles a warp and block with four warps on a scheduler.
 //                         Loading a block ahead with one address for its four
 //                         pieces, and 256 bytes into the L2 eight blocks ahead, took
-//                         a lone warp per scheduler from 307 to 190 us on 8 KB.  A message is a serial chain, so a call of a
-//                         few messages per thread slot of the GPU leaves some
-//                         schedulers with one warp more than others; warps then work
-//                         in slices and exchange chains through a queue (below).
+//                         a lone warp per scheduler from 307 to 190 us on 8 KB.
+//                         A message is a serial chain, so a call of a few messages
+//                         per thread slot of the GPU leaves some schedulers with one
+//                         warp more than others; warps then work in slices and
+//                         exchange chains through a queue (below).
 //   dedup_insert_kernel / dedup_resolve_kernel
 //                         an open-addressing table of list positions, probed from
 //                         the first 8 bytes of the digest (a SHA-256 digest is as
@@ -103,10 +104,10 @@ __device__ __forceinline__ uint64_t hash_chunk_offset(const PartGeom& g, uint64_
 // as 5.  So the grid holds an even number of warps, each works on a chain for one slice (a seventh
 // of the longest message), leaves the intermediate hash value in the place of the digest, queues the
 // chain and takes the one that has waited longest: all chains advance at one rate and the call ends
-// everywhere at about the same time (78,643 entries of 8 KB: 788 us
-// without the queue, 661 with it; 120,000: 1,084 and 991; 786,432: 6,331 and 6,303).  The exchange takes a
-// few microseconds of latency; the warps of a scheduler make theirs at different times (a warp's first
-// slice has any length), so that the others keep it busy meanwhile.
+// everywhere at about the same time (78,643 entries of 8 KB: 788 us without the queue, 661 with it;
+// 120,000: 1,084 and 991; 786,432: 6,331 and 6,303).  The exchange takes a few microseconds of
+// latency; the warps of a scheduler make theirs at different times (a warp's first slice has any
+// length), so that the others keep it busy meanwhile.
 // Places in the queue are given out by two counters (a compare-and-swap loop on them took 0.9 ms a
 // slice: all warps come at the same time).  A warp that finishes its chain takes a place without
 // having queued one, and so may have to wait for another's slice to end; when all chains are

@@ -32,13 +32,16 @@
 // and of the block barriers around them.  An exchange is a grid barrier (a counter that
 // every CTA increments and one of its threads polls).  (Tried for the third one: no
 // barrier, every reader polls the table's words for the launch's number.  With 148 CTAs
-// the polls of a thousand words each crowd out the stores they wait for: 5.0 us where
-// barrier and one reading take 2.5.)  A cooperative launch guarantees that all CTAs are resident, so every wait ends; all
-// are bounded nevertheless, and a CTA that gives up sets KV_DEV_WAIT_EXPIRED and leaves
-// (every other CTA then runs into the same limit).  Barrier and histograms come in two
-// sets used in turn; a launch clears the set of the next one.  The launch's number, which
-// also says whose turn it is, lives in device memory, so that a captured launch can be
-// replayed.
+// the polls of a thousand words each crowd out the stores they wait for: 5.0 us
+// where barrier and one reading take 2.5.)  A cooperative launch guarantees that all CTAs
+// are resident, so every wait ends; all are bounded nevertheless, and a CTA that gives up
+// sets KV_DEV_WAIT_EXPIRED and leaves (every other CTA then runs into the same limit).
+// Barrier and histograms come in two sets used in turn; a launch clears the set of the
+// next one.  The launch's number, which also says whose turn it is, lives in device
+// memory, so that a captured launch can be replayed.
+// Measured, a pass with the event reduction, against notes per thread and whole chunks
+// only: 4,096 entries 32.5 -> 13.5 us, 0.9 M 40.3 -> 27.4, 3.1 M 59.9 -> 41.3, 18.8 M
+// 206 -> 180.
 //
 // The same kernel also exists fused with the per-entry scoring pass (FUSED = true):
 // every CTA first updates the entries of its own rows (posterior, EMA, score), their
