@@ -37,6 +37,7 @@
 // The round constants and the initial hash value are the ones FIPS 180-4 defines
 // (the first 32 bits of the fractional parts of the cube roots of the first 64
 // primes, and of the square roots of the first 8).
+#include "kv_hash_queue.h"
 #include "kvtier_internal.cuh"
 
 namespace kvt {
@@ -111,7 +112,8 @@ __device__ __forceinline__ uint64_t hash_chunk_offset(const PartGeom& g, uint64_
 // Places in the queue are given out by two counters (a compare-and-swap loop on them took 0.9 ms a
 // slice: all warps come at the same time).  A warp that finishes its chain takes a place without
 // having queued one, and so may have to wait for another's slice to end; when all chains are
-// finished, those that wait leave.
+// finished, those that wait leave.  Every warp takes a last place that nothing comes to: one behind
+// the ring's end is not looked at.
 struct HashCounters {
   unsigned int head;       // places taken beyond the first n_warps
   unsigned int tail;       // chains queued again
@@ -120,12 +122,11 @@ struct HashCounters {
 };
 struct HashQueue {
   HashCounters* counters = nullptr;    // (nullptr: no queue)
-  unsigned long long* ring = nullptr;  // bit 63 | next block << 32 | chain; zero until written
-  uint32_t n_chains = 0, n_warps = 0, slice_blocks = 0;
+  unsigned long long* ring = nullptr;  // [shape.ring_places], zero until written
+  HashShape shape;
 };
 constexpr uint32_t kHashThreads = 128;
 constexpr uint32_t kHashBlocksPerSm = 5;
-constexpr uint32_t kHashSlices = 7;
 constexpr uint32_t kHashStep = 4;          // blocks between two looks at the pace of the others
 constexpr uint32_t kHashSpins = 1u << 22;
 
@@ -154,7 +155,7 @@ hash_entries_kernel(const HashGeom hg, const uint32_t* __restrict__ ids, uint64_
     __syncthreads();
   }
   uint32_t slice_len = 0xFFFFFFFFu;
-  if (QUEUE) slice_len = 1u + ((uint32_t)chain * 2654435761u >> 8) % queue.slice_blocks;
+  if (QUEUE) slice_len = hash_first_slice(queue.shape, (uint32_t)chain);
   while (chain * 32u < m) {
     const uint64_t j = chain * 32u + lane;
     int q = -1;
@@ -249,33 +250,38 @@ hash_entries_kernel(const HashGeom hg, const uint32_t* __restrict__ ids, uint64_
       if (!done) {   // queue the chain (the lanes' values first)
         __threadfence();
         const unsigned int p = atomicAdd(&queue.counters->tail, 1u);
-        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(queue.ring + p),
-                     "l"(1ull << 63 | (unsigned long long)b1 << 32 | (uint32_t)chain)
-                     : "memory");
+        if (p < queue.shape.ring_places)
+          asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(queue.ring + p), "l"(hash_word((uint32_t)chain, b1)) : "memory");
+        else
+          atomicOr(status, KV_DEV_BAD_INDEX);   // (more slices than there are)
       } else {
         atomicAdd(&queue.counters->finished, 1u);
       }
       s_pace[warp] = kAway;
-      const unsigned int pos = queue.n_warps + atomicAdd(&queue.counters->head, 1u);
-      if (pos < queue.n_chains) {
-        word = pos;
-      } else {
-        const unsigned long long* at = queue.ring + (pos - queue.n_chains);
+      uint32_t at;
+      const HashPlace place = hash_place(queue.shape, queue.shape.n_warps + atomicAdd(&queue.counters->head, 1u), at);
+      if (place == kHashChain) {
+        word = at;
+      } else if (place == kHashRing) {
         for (uint32_t it = 0;; ++it) {
           unsigned long long w;
-          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(at) : "memory");
-          if (w >> 63) { word = w; break; }
-          if (*reinterpret_cast<volatile unsigned int*>(&queue.counters->finished) == queue.n_chains) break;
+          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(queue.ring + at) : "memory");
+          if (w != 0) {
+            if (hash_word_good(queue.shape, w)) word = w; else atomicOr(status, KV_DEV_BAD_INDEX);
+            break;
+          }
+          if (*reinterpret_cast<volatile unsigned int*>(&queue.counters->finished) >= queue.shape.n_chains) break;
           if (it == kHashSpins) { atomicOr(status, KV_DEV_WAIT_EXPIRED); break; }
           __nanosleep(256);
         }
       }
     }
     word = __shfl_sync(0xFFFFFFFFu, word, 0);
+    __syncwarp();   // (the lanes read the values behind lane 0's acquire)
     if (word == ~0ull) return;
-    chain = (uint32_t)word;
-    b0 = (uint32_t)(word >> 32) & 0x7FFFFFFFu;
-    slice_len = queue.slice_blocks;
+    chain = hash_word_chain(word);
+    b0 = hash_word_block(word);
+    slice_len = queue.shape.slice_blocks;
     const uint32_t least = slowest();   // (a warp that was away comes back beside the slowest)
     if (least != kAway && least > pace) pace = least;
   }
@@ -302,16 +308,14 @@ cudaError_t launch_hash_entries(const PartGeom* parts, int n_parts, const uint32
   uint64_t depth = blocks / per_sm;
   if (depth > kHashBlocksPerSm) depth = kHashBlocksPerSm;
   const uint64_t words = 2 + chains * kHashSlices;   // 64-bit words: counters and ring
-  if (depth >= 2 && blocks > depth * per_sm && words * 2 <= n_entries && chains < (1ull << 31)) {
+  if (depth >= 2 && blocks > depth * per_sm && words * 2 <= n_entries && chains * kHashSlices < (1ull << 31)) {
     unsigned long long* base = reinterpret_cast<unsigned long long*>(ws.free_list);
     const cudaError_t e = cudaMemsetAsync(base, 0, words * 8, s);
     if (e != cudaSuccess) return e;
     queue.counters = reinterpret_cast<HashCounters*>(base);
     queue.ring = base + 2;
-    queue.n_chains = (uint32_t)chains;
-    queue.slice_blocks = (longest + kHashSlices - 1) / kHashSlices;
     blocks = depth * per_sm;
-    queue.n_warps = (uint32_t)(blocks * (kHashThreads / 32));
+    queue.shape = hash_shape((uint32_t)chains, (uint32_t)(blocks * (kHashThreads / 32)), longest);
   }
   // (with the queue one CTA per SM holds all of the SM's warps, which then see each other's pace)
   if (queue.counters)

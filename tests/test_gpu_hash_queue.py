@@ -51,3 +51,36 @@ def test_digests(m, mixed):
             assert got[j].tobytes() == hashlib.sha256(img[which[j] - lo].tobytes()).digest(), j
     assert p.kv_device_status() == 0
     p.close()
+
+
+def test_lists_of_falling_length_on_one_pool(monkeypatch):
+    """The queue's memory is as an earlier, longer call left it, and before the first call as the
+    caller handed it over (here: ones in every bit).  Images of 8 KB: chains are queued again so
+    often that the places that warps take reach beyond the ring."""
+    import torch
+    real = torch.empty
+
+    def ones(*a, **k):
+        t = real(*a, **k)
+        return t.fill_(255) if t.dtype == torch.uint8 else t
+
+    part = W.gqa(2, 8, 2, 128, 16, 30_000, 16, "entry")
+    monkeypatch.setattr(torch, "empty", ones)
+    p = B.Pool([part], part.n_entries + 16, staging_bytes=1 << 16, max_promote=64, host_meta=False)
+    monkeypatch.undo()
+    assert part.entry_bytes == 8192 and p.N == 120_000
+    g = torch.Generator(device="cuda").manual_seed(5)
+    p.slabs[0].copy_(torch.randint(0, 256, (p.slabs[0].numel(),), dtype=torch.uint8, device="cuda", generator=g))
+    raw = p.slabs[0].cpu().numpy().reshape(-1, 2, part.heads, part.entry_bytes // 2)
+    img = np.ascontiguousarray(raw.transpose(0, 2, 1, 3)).reshape(part.n_entries, part.entry_bytes)
+    want = np.frombuffer(b"".join(hashlib.sha256(x).digest() for x in img), np.uint8).reshape(-1, 32)
+    out = torch.zeros((p.N, 32), dtype=torch.uint8, device="cuda")
+    for m in (120_000, 78_643, 60_000, 37_889, 120_000, 37_889):
+        out.zero_()
+        torch.cuda.synchronize()
+        assert p.kv_hash_entries(None, m, out) == 0
+        p.sync()
+        assert np.array_equal(out[:m].cpu().numpy(), want[:m]), m
+        assert not out[m:].any()
+    assert p.kv_device_status() == 0
+    p.close()
