@@ -113,9 +113,11 @@ __device__ __forceinline__ uint64_t hash_chunk_offset(const PartGeom& g, uint64_
 // slice: all warps come at the same time).  A warp that finishes its chain takes a place without
 // having queued one, and so may have to wait for another's slice to end; when all chains are
 // finished, those that wait leave.  Every warp takes a last place that nothing comes to: one behind
-// the ring's end is not looked at.
+// the ring's end is not looked at.  A warp's first chain is a place like any other, taken when its
+// block starts: the warps that run can then finish all chains by themselves, and never wait for a
+// block that other work on the GPU keeps from starting.
 struct HashCounters {
-  unsigned int head;       // places taken beyond the first n_warps
+  unsigned int head;       // places taken
   unsigned int tail;       // chains queued again
   unsigned int finished;   // chains finished
   unsigned int pad;
@@ -150,12 +152,46 @@ hash_entries_kernel(const HashGeom hg, const uint32_t* __restrict__ ids, uint64_
     const uint32_t w = (warp & 3u) + 4u * lane;
     return __reduce_min_sync(0xFFFFFFFFu, w < n_warps_cta ? s_pace[w] : kAway);
   };
-  if (QUEUE) {
-    if (lane == 0) s_pace[warp] = 0;
-    __syncthreads();
-  }
+  // What comes at place pos of the line: the word of a chain, or ~0 if nothing does (lane 0).
+  auto work_at = [&](uint32_t pos) -> unsigned long long {
+    uint32_t at;
+    const HashPlace place = hash_place(queue.shape, pos, at);
+    if (place == kHashChain) return at;
+    if (place == kHashNothing) return ~0ull;
+    for (uint32_t it = 0;; ++it) {
+      unsigned long long w;
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(queue.ring + at) : "memory");
+      if (w != 0) {
+        if (hash_word_good(queue.shape, w)) return w;
+        atomicOr(status, KV_DEV_BAD_INDEX);
+        return ~0ull;
+      }
+      if (*reinterpret_cast<volatile unsigned int*>(&queue.counters->finished) >= queue.shape.n_chains) return ~0ull;
+      if (it == kHashSpins) { atomicOr(status, KV_DEV_WAIT_EXPIRED); return ~0ull; }
+      __nanosleep(256);
+    }
+  };
   uint32_t slice_len = 0xFFFFFFFFu;
-  if (QUEUE) slice_len = hash_first_slice(queue.shape, (uint32_t)chain);
+  // Takes up that chain; false: there is none.
+  auto take_up = [&](unsigned long long word) {
+    word = __shfl_sync(0xFFFFFFFFu, word, 0);
+    __syncwarp();   // (the lanes read the values behind lane 0's acquire)
+    if (word == ~0ull) return false;
+    chain = hash_word_chain(word);
+    b0 = hash_word_block(word);
+    slice_len = queue.shape.slice_blocks;
+    const uint32_t least = slowest();   // (a warp that was away comes back beside the slowest)
+    if (least != kAway && least > pace) pace = least;
+    return true;
+  };
+  if (QUEUE) {
+    __shared__ uint32_t s_first;
+    if (lane == 0) s_pace[warp] = kAway;
+    if (threadIdx.x == 0) s_first = atomicAdd(&queue.counters->head, n_warps_cta);
+    __syncthreads();
+    if (!take_up(lane == 0 ? work_at(s_first + warp) : 0ull)) return;
+    if (b0 == 0) slice_len = hash_first_slice(queue.shape, (uint32_t)chain);
+  }
   while (chain * 32u < m) {
     const uint64_t j = chain * 32u + lane;
     int q = -1;
@@ -258,32 +294,9 @@ hash_entries_kernel(const HashGeom hg, const uint32_t* __restrict__ ids, uint64_
         atomicAdd(&queue.counters->finished, 1u);
       }
       s_pace[warp] = kAway;
-      uint32_t at;
-      const HashPlace place = hash_place(queue.shape, queue.shape.n_warps + atomicAdd(&queue.counters->head, 1u), at);
-      if (place == kHashChain) {
-        word = at;
-      } else if (place == kHashRing) {
-        for (uint32_t it = 0;; ++it) {
-          unsigned long long w;
-          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(queue.ring + at) : "memory");
-          if (w != 0) {
-            if (hash_word_good(queue.shape, w)) word = w; else atomicOr(status, KV_DEV_BAD_INDEX);
-            break;
-          }
-          if (*reinterpret_cast<volatile unsigned int*>(&queue.counters->finished) >= queue.shape.n_chains) break;
-          if (it == kHashSpins) { atomicOr(status, KV_DEV_WAIT_EXPIRED); break; }
-          __nanosleep(256);
-        }
-      }
+      word = work_at(atomicAdd(&queue.counters->head, 1u));
     }
-    word = __shfl_sync(0xFFFFFFFFu, word, 0);
-    __syncwarp();   // (the lanes read the values behind lane 0's acquire)
-    if (word == ~0ull) return;
-    chain = hash_word_chain(word);
-    b0 = hash_word_block(word);
-    slice_len = queue.shape.slice_blocks;
-    const uint32_t least = slowest();   // (a warp that was away comes back beside the slowest)
-    if (least != kAway && least > pace) pace = least;
+    if (!take_up(word)) return;
   }
 }
 
@@ -315,7 +328,7 @@ cudaError_t launch_hash_entries(const PartGeom* parts, int n_parts, const uint32
     queue.counters = reinterpret_cast<HashCounters*>(base);
     queue.ring = base + 2;
     blocks = depth * per_sm;
-    queue.shape = hash_shape((uint32_t)chains, (uint32_t)(blocks * (kHashThreads / 32)), longest);
+    queue.shape = hash_shape((uint32_t)chains, longest);
   }
   // (with the queue one CTA per SM holds all of the SM's warps, which then see each other's pace)
   if (queue.counters)

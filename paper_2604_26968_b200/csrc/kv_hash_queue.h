@@ -16,19 +16,17 @@ constexpr uint32_t kHashSlices = 7;
 
 struct HashShape {
   uint32_t n_chains = 0;
-  uint32_t n_warps = 0;
   uint32_t slice_blocks = 0;   // blocks of a slice: a seventh of the longest message
   uint32_t longest = 0;        // blocks of the longest message
   uint32_t ring_places = 0;    // times that chains can be queued again, all together
 };
 
-// A chain's first slice has 1 to slice_blocks blocks, each further one slice_blocks until the
+// A chain's first slice has 1 to slice_blocks blocks, each further one has slice_blocks until the
 // message ends.  After the first block at most (longest - 1) / slice_blocks, rounded up, slices are
 // left, which is at most kHashSlices: so often is a chain queued again, at most.
-KV_QUEUE_FN HashShape hash_shape(uint32_t n_chains, uint32_t n_warps, uint32_t longest) {
+KV_QUEUE_FN HashShape hash_shape(uint32_t n_chains, uint32_t longest) {
   HashShape s;
   s.n_chains = n_chains;
-  s.n_warps = n_warps;
   s.longest = longest;
   s.slice_blocks = (longest + kHashSlices - 1u) / kHashSlices;
   s.ring_places = n_chains * kHashSlices;

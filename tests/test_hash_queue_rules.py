@@ -1,6 +1,7 @@
 """The rules by which the hash kernel's warps pass chains of messages on, played through on the CPU:
 no place behind the cleared part of the queue's memory is looked at or written, whatever an earlier
-call left there, and every chain is finished, block after block.  Sizes just above a multiple of the
+call left there, every chain is finished, block after block, and no warp waits for a thread block
+that has not started.  Sizes just above a multiple of the
 warps are the ones whose warps take the most places that nothing comes to."""
 import os
 import subprocess
@@ -20,9 +21,13 @@ def sim(tmp_path_factory):
 
 @pytest.mark.parametrize("seed", [1, 2])
 @pytest.mark.parametrize("blocks", [2, 9, 129, 1153])
-@pytest.mark.parametrize("messages,warps", [(37_889, 1184), (60_000, 1776), (78_643, 2368), (120_000, 2960)])
-def test_played_through(sim, messages, warps, blocks, seed):
-    r = subprocess.run([sim, str(messages), str(blocks), str(warps), str(seed)], capture_output=True, text=True, timeout=60)
+@pytest.mark.parametrize("resident", [148, 147, 60, 1])
+@pytest.mark.parametrize("messages,depth", [(37_889, 2), (60_000, 3), (78_643, 4), (120_000, 5)])
+def test_played_through(sim, messages, depth, resident, blocks, seed):
+    """depth: groups of four warps per SM; resident: thread blocks of the 148 that run at a time (other
+    work may hold SMs)."""
+    a = [messages, blocks, 148, 4 * depth, resident, seed]
+    r = subprocess.run([sim, *map(str, a)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout
     most, ring, requeued = map(int, r.stdout.split())
     assert most < ring and requeued <= ring
