@@ -106,10 +106,12 @@ struct kv_pool {
   kv_stats stats;
   uint64_t last_counts[4] = {0, 0, 0, 0};
   cudaEvent_t ev_staging_free[4], ev_ready[4], ev_list_copied[kListBufs], ev_list_free[kListBufs], ev_counts;
-  // copies in flight: the last two demotions per partition (ring slot range + completion event of
-  // their D2H copies) and the last promotion's H2D copies
-  struct D2H { cudaEvent_t ev; uint64_t start = 0, count = 0; bool valid = false; };
-  D2H d2h[4][2];
+  // Writes to the ring in flight, per partition: the last two demotions that went through staging
+  // buffers and transfers (their events on the D2H stream) and the last two that stored into the ring
+  // themselves (theirs on the compute stream).  Of either kind the newer one's event implies all
+  // older ones, but neither kind's implies the other's.  And the last promotion's H2D copies.
+  struct Write { cudaEvent_t ev; uint64_t start = 0, count = 0; bool valid = false; };
+  Write d2h[4][2], direct[4][2];
   cudaEvent_t ev_h2d_done;
   bool h2d_valid = false;
   bool events_made = false;
@@ -301,7 +303,8 @@ void forget_free_lists(kv_pool* p) {
 std::vector<cudaEvent_t*> all_events(kv_pool* p) {
   std::vector<cudaEvent_t*> evs;
   for (int b = 0; b < 4; ++b) { evs.push_back(&p->ev_staging_free[b]); evs.push_back(&p->ev_ready[b]); }
-  for (int q = 0; q < 4; ++q) { evs.push_back(&p->d2h[q][0].ev); evs.push_back(&p->d2h[q][1].ev); }
+  for (int q = 0; q < 4; ++q)
+    for (int i = 0; i < 2; ++i) { evs.push_back(&p->d2h[q][i].ev); evs.push_back(&p->direct[q][i].ev); }
   evs.push_back(&p->ev_h2d_done);
   for (int b = 0; b < kListBufs; ++b) { evs.push_back(&p->ev_list_copied[b]); evs.push_back(&p->ev_list_free[b]); }
   evs.push_back(&p->ev_counts);
@@ -393,6 +396,24 @@ int32_t enqueue_pack_chunk(kv_pool* p, int q, uint64_t c0, uint64_t cnt) {
   return KV_OK;
 }
 
+// Notes that all writes to slots [start, start + count) have now been enqueued on `stream`.
+int32_t note_write(kv_pool* p, kv_pool::Write (&w)[2], uint64_t start, uint64_t count, cudaStream_t stream) {
+  std::swap(w[0], w[1]);   // (the older one's event object is used again)
+  w[0].start = start;
+  w[0].count = count;
+  w[0].valid = true;
+  KV_CUDA(p, cudaEventRecord(w[0].ev, stream));
+  return KV_OK;
+}
+
+// Lets `s` wait for those of the writes w that may reach slots a list or demotion is about: the last
+// one's if they may be among them, else all older ones'.
+int32_t wait_for_writes(kv_pool* p, const kv_pool::Write (&w)[2], bool hits_last, cudaStream_t s) {
+  const kv_pool::Write& x = hits_last && w[0].valid ? w[0] : w[1];
+  if (x.valid) KV_CUDA(p, cudaStreamWaitEvent(s, x.ev, 0));
+  return KV_OK;
+}
+
 // Enqueues pending chunks of the last demotion: of partition q_only until `need` of its
 // victims are packed (the other partitions' chunks stay where they are: every partition has
 // its own ring, so their order among each other is free), or, with q_only < 0, of every
@@ -414,13 +435,8 @@ int32_t drain_pending(kv_pool* p, int q_only, uint64_t need, uint64_t max_chunks
       ++done;
       if (pd.next[q] == pd.kq[q]) {
         // all copies of this partition are enqueued: remember the slots they write and when they end
-        kv_pool::D2H older = p->d2h[q][1];
-        p->d2h[q][1] = p->d2h[q][0];
-        p->d2h[q][0] = older;  // reuse the older record's event object
-        p->d2h[q][0].start = pd.cursor0[q];
-        p->d2h[q][0].count = pd.kq[q];
-        p->d2h[q][0].valid = true;
-        KV_CUDA(p, cudaEventRecord(p->d2h[q][0].ev, pd.copy));
+        const int32_t rcw = note_write(p, p->d2h[q], pd.cursor0[q], pd.kq[q], pd.copy);
+        if (rcw != KV_OK) return rcw;
       }
     }
   }
@@ -438,22 +454,20 @@ int32_t demote_direct(kv_pool* p) {
     if (pd.kq[q] == 0) continue;
     PartHost& h = p->host[q];
     const PartGeom& g = p->geom[q];
-    // slots that an earlier demotion's transfers may still be writing
-    for (kv_pool::D2H& d : p->d2h[q]) {
-      const uint64_t R = g.ring_slots, from = (pd.cursor0[q] + R - d.start) % R;
-      if (d.valid && (from < d.count || R - from < pd.kq[q])) KV_CUDA(p, cudaStreamWaitEvent(pd.compute, d.ev, 0));
-    }
+    // slots that an earlier demotion's transfers may still be writing (direct demotions follow one
+    // another on the compute stream)
+    const kv_pool::Write& last = p->d2h[q][0];
+    const uint64_t R = g.ring_slots, from = (pd.cursor0[q] + R - last.start) % R;
+    int32_t rc = wait_for_writes(p, p->d2h[q], from < last.count || R - from < pd.kq[q], pd.compute);
+    if (rc != KV_OK) return rc;
     {
       TimedScope ts(p, 0, pd.kq[q] * g.entry_bytes, pd.compute);
       KV_CUDA(p, launch_pack_direct(g, p->st, p->desc.d_loc, pd.victims + pd.off[q], pd.kq[q], pd.cursor0[q], h.ring_dev,
                                     p->ws, pd.compute, h.free_known ? p->ws.free_list + g.base : nullptr, h.meta_dev));
     }
-    std::swap(p->d2h[q][0], p->d2h[q][1]);   // (the older record's event object is used again)
-    p->d2h[q][0].start = pd.cursor0[q];
-    p->d2h[q][0].count = pd.kq[q];
-    p->d2h[q][0].valid = true;
-    KV_CUDA(p, cudaEventRecord(p->d2h[q][0].ev, pd.compute));
-    KV_CUDA(p, cudaStreamWaitEvent(pd.copy, p->d2h[q][0].ev, 0));   // (synchronising the copy stream completes a demotion)
+    rc = note_write(p, p->direct[q], pd.cursor0[q], pd.kq[q], pd.compute);
+    if (rc != KV_OK) return rc;
+    KV_CUDA(p, cudaStreamWaitEvent(pd.copy, p->direct[q][0].ev, 0));   // (synchronising the copy stream completes a demotion)
     pd.next[q] = pd.kq[q];
   }
   return KV_OK;
@@ -970,8 +984,6 @@ int32_t kv_demote_counted(kv_pool* p, const uint32_t* d_victims, uint64_t m, con
     per[q] = entries_per_batch(p, q, batch_bytes);
     if (per[q] == 0 || batch_bytes > p->staging_bytes) return KV_ERR_INVALID_ARG;
   }
-  // ring slots written below may have been read by the last promotion's H2D copies
-  if (p->h2d_valid) KV_CUDA(p, cudaStreamWaitEvent(copy, p->ev_h2d_done, 0));
   kv_pool::Pending& pd = p->pending;
   pd.victims = d_victims;
   pd.compute = compute;
@@ -1002,6 +1014,9 @@ int32_t kv_demote_counted(kv_pool* p, const uint32_t* d_victims, uint64_t m, con
     direct = direct && p->host[q].ring_dev && (!p->host[q].h_meta || p->host[q].meta_dev);
   }
   direct = direct && bytes <= kDirectBytes && bytes <= batch_bytes;   // (a caller's smaller batches are kept to)
+  // ring slots written below may have been read by the last promotion's H2D copies (the compute stream
+  // has joined that promotion; a wait on it here would keep the packing from being set up early)
+  if (p->h2d_valid && !direct) KV_CUDA(p, cudaStreamWaitEvent(copy, p->ev_h2d_done, 0));
   if (direct) {
     const int32_t rcd = demote_direct(p);
     if (rcd != KV_OK) return rcd;
@@ -1080,19 +1095,26 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
     e = cudaEventSynchronize(p->ev_list_copied[li]);
   }
   if (e != cudaSuccess) { restore(); return cuda_fail(p, e); }
-  // The H2D copies below may run on another stream than the D2H copies that filled the slots, so the
-  // copy stream has to wait for the demotion(s) whose slot ranges the list touches.  d2h[q][0] is the
+  // What follows may run on another stream than the D2H copies that filled the slots, so the copy
+  // stream has to wait for the demotion(s) whose slot ranges the list touches.  d2h[q][0] is the
   // newest demotion whose copies are all enqueued; a pending (deferred) demotion is newer still and
-  // has no completion event yet.
+  // has no completion event yet.  A list of short runs (a position-ordered prefetch: a block's layers
+  // lie far apart in the ring) would cost one DMA set-up per run; the gather kernel fetches such
+  // entries itself.
   const kv_pool::Pending& pd = p->pending;
   const bool q_pending = pd.active && pd.next[q] < pd.kq[q];
-  bool hits_pending = false, hits_newest = false;
+  bool hits_pending = false, hits_newest = false, hits_direct = false;
+  uint64_t n_runs = 0;
+  const kv_pool::Write &newest = p->d2h[q][0], &stored = p->direct[q][0];
   for (uint64_t j = 0; j < m; ++j) {
     const uint64_t s = h_slots[j];
     if (!listed) p->h_list[li][j] = (uint32_t)s;
     if (q_pending && (s + R - pd.cursor0[q]) % R < pd.kq[q]) hits_pending = true;
-    if (p->d2h[q][0].valid && (s + R - p->d2h[q][0].start) % R < p->d2h[q][0].count) hits_newest = true;
+    if (newest.valid && (s + R - newest.start) % R < newest.count) hits_newest = true;
+    if (stored.valid && (s + R - stored.start) % R < stored.count) hits_direct = true;
+    n_runs += (j == 0 || s != h_slots[j - 1] + 1);
   }
+  const bool gather = h.ring_dev && m * eb < n_runs * p->gather_run_bytes;
   if (hits_pending) {
     // enqueue all of that demotion's copies for this partition; its record then becomes d2h[q][0]
     const int32_t rc = drain_pending(p, q, pd.kq[q], ~0ull);
@@ -1101,9 +1123,10 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
   } else if (q_pending) {
     hits_newest = p->d2h[q][0].valid;  // everything older than the pending demotion: wait for the newest recorded
   }
-  if (e == cudaSuccess && hits_newest) e = cudaStreamWaitEvent(copy, p->d2h[q][0].ev, 0);
-  if (e == cudaSuccess && !hits_newest && p->d2h[q][1].valid)
-    e = cudaStreamWaitEvent(copy, p->d2h[q][1].ev, 0);
+  int32_t rcw = wait_for_writes(p, p->d2h[q], hits_newest, copy);
+  // (the kernels wait for the compute stream in any case, transfers run ahead of them)
+  if (rcw == KV_OK && !gather) rcw = wait_for_writes(p, p->direct[q], hits_direct, copy);
+  if (rcw != KV_OK) { restore(); return rcw; }
   if (!listed) {
     if (e == cudaSuccess)
       e = cudaStreamWaitEvent(copy, p->ev_list_free[li], 0);  // older kernels are done reading the device list
@@ -1133,11 +1156,6 @@ int32_t kv_promote(kv_pool* p, int32_t q, const uint64_t* h_slots, uint64_t m, u
     KV_CUDA(p, cudaStreamWaitEvent(copy, p->ev_promote_ready, 0));
     return KV_OK;
   };
-  // A list of short runs (a position-ordered prefetch: a block's layers lie far apart in the
-  // ring) would cost one DMA set-up per run; the gather kernel fetches such entries itself.
-  uint64_t n_runs = 0;
-  for (uint64_t j = 0; j < m; ++j) n_runs += (j == 0 || h_slots[j] != h_slots[j - 1] + 1);
-  const bool gather = h.ring_dev && m * eb < n_runs * p->gather_run_bytes;
   // The transfers AND the scatter kernels go to the copy stream: the compute stream never waits
   // for the host link, and pack kernels of a demotion keep flowing between them.  Transfers run
   // one chunk ahead of the kernels (two staging buffers).
