@@ -490,9 +490,9 @@ int32_t kv_select_victim_blocks(kv_pool* pool, uint64_t k_blocks, uint32_t* d_vi
  *     KV_ERR_K_TOO_LARGE; pointers must be 16-byte aligned;
  *   - the first call on each device looks up the array's device address (with
  *     that device current); make that first call before any stream capture;
- *   - all calls on a device share the one array: two calls whose GPU work overlaps
- *     (different streams, no ordering between them) race and give wrong results.
- *     Order them. */
+ *   - all calls on a device share the one array, which each call clears as far as it
+ *     needs it: two calls whose GPU work overlaps (different streams, no ordering
+ *     between them) race and give wrong results.  Order them. */
 int32_t kv_select_victims_static(const float* d_score, const uint8_t* d_state, uint64_t n,
                                  uint64_t k, uint32_t* d_victims, uint32_t* d_status,
                                  kv_stream_t stream);

@@ -343,6 +343,10 @@ cudaError_t launch_select(const EntryState& st, uint64_t k, uint32_t* d_victims,
     const cudaError_t e = launch_select_persistent(st, k, d_victims, ws, s, &used, nullptr, pc);
     if (e != cudaSuccess || used) return e;
   }
+  if (ws.shared_words) {
+    const cudaError_t e = cudaMemsetAsync(ws.hist, 0, 3 * kHistBins * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+  }
   const unsigned g = hist_grid(st.n);
   select_begin_kernel<<<1, 1, 0, s>>>(ws.sel, k);
   select_hist_kernel<0><<<g, kThreads, 0, s>>>(st.score, st.state, st.n, ws.sel, ws.hist);
@@ -405,6 +409,26 @@ cudaError_t launch_partition_counts(const uint32_t* d_victims, uint64_t m, const
   return cudaGetLastError();
 }
 
+cudaError_t launch_select_static(const float* score, const uint8_t* state, uint64_t n, uint64_t k, uint32_t* d_victims,
+                                 StaticScratch* scratch, uint32_t* status, cudaStream_t s, int variant) {
+  Workspace ws{};
+  ws.hist = scratch->hist;
+  ws.sel = &scratch->sel;
+  ws.status = status ? status : scratch->status;
+  ws.tile_counts = scratch->tile_counts;
+  ws.tile_offsets = scratch->tile_offsets;
+  ws.n_tiles = (uint32_t)kStaticMaxTiles;
+  ws.turns = &scratch->turn;
+  ws.table = scratch->table;
+  ws.table_words = sizeof(scratch->table) / sizeof(scratch->table[0]);
+  ws.shared_words = scratch->words;
+  EntryState st{};
+  st.score = const_cast<float*>(score);   // selection only reads score and state
+  st.state = const_cast<uint8_t*>(state);
+  st.n = n;
+  return launch_select(st, k, d_victims, ws, s, variant);
+}
+
 }  // namespace kvt
 
 // ---- selection without any caller-provided or allocated scratch -------------------
@@ -415,22 +439,11 @@ cudaError_t launch_partition_counts(const uint32_t* d_victims, uint64_t m, const
 // needs -- three digit histograms, a handful of scalars and the per-tile counts
 // of the compaction -- lives in this fixed array, which every GPU that loads the
 // library holds until the process exits.  Its size bounds the problem:
-// kStaticMaxEntries entries.
+// kStaticMaxEntries entries.  Calls that gave up on a wait or ran at the same time leave it in any
+// state; the next one clears what it needs.
 namespace {
 
-constexpr uint64_t kStaticMaxEntries = 1ull << 22;  // 4,194,304 entries
-constexpr uint64_t kStaticMaxTiles = kStaticMaxEntries / kvt::kTileEntries + 2;
-// What the array holds, in this order.  All of it starts as zeros; every selection leaves the
-// histograms zero again (the persistent one clears the set that the next one uses).
-struct StaticScratch {
-  uint32_t hist[3 * kvt::kHistBins];
-  kvt::SelectTurn turns[2];
-  kvt::SelectScalars sel;
-  uint32_t status[4];
-  uint2 tile_counts[kStaticMaxTiles];
-  uint2 tile_offsets[kStaticMaxTiles];
-  uint32_t table[kStaticMaxEntries / 4096 + 1024];
-};
+using kvt::StaticScratch;
 
 static __device__ __align__(256) unsigned char g_select_scratch[sizeof(StaticScratch)];
 
@@ -461,7 +474,7 @@ cudaError_t static_scratch(StaticScratch** out) {
 extern "C" int32_t kv_select_victims_static(const float* d_score, const uint8_t* d_state, uint64_t n,
                                             uint64_t k, uint32_t* d_victims, uint32_t* d_status,
                                             kv_stream_t stream) {
-  if (n == 0 || n > kStaticMaxEntries) return KV_ERR_INVALID_ARG;  // beyond the built-in scratch
+  if (n == 0 || n > kvt::kStaticMaxEntries) return KV_ERR_INVALID_ARG;  // beyond the built-in scratch
   if (k > n) return KV_ERR_K_TOO_LARGE;
   if (!d_score || !d_state || (reinterpret_cast<uintptr_t>(d_score) & 15u) ||
       (reinterpret_cast<uintptr_t>(d_state) & 15u))
@@ -471,21 +484,6 @@ extern "C" int32_t kv_select_victims_static(const float* d_score, const uint8_t*
   StaticScratch* scratch = nullptr;
   if (static_scratch(&scratch) != cudaSuccess) return KV_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  kvt::Workspace ws{};
-  ws.hist = scratch->hist;
-  ws.sel = &scratch->sel;
-  ws.status = d_status ? d_status : scratch->status;
-  ws.tile_counts = scratch->tile_counts;
-  ws.tile_offsets = scratch->tile_offsets;
-  ws.n_tiles = (uint32_t)kStaticMaxTiles;
-  ws.turns = scratch->turns;
-  ws.table = scratch->table;
-  ws.table_words = sizeof(scratch->table) / sizeof(scratch->table[0]);
-  ws.keep_hint = false;   // the next call may be about other scores altogether
-  kvt::EntryState st{};
-  st.score = const_cast<float*>(d_score);   // selection only reads score and state
-  st.state = const_cast<uint8_t*>(d_state);
-  st.n = n;
-  if (kvt::launch_select(st, k, d_victims, ws, s) != cudaSuccess) return KV_ERR_CUDA;
+  if (kvt::launch_select_static(d_score, d_state, n, k, d_victims, scratch, d_status, s) != cudaSuccess) return KV_ERR_CUDA;
   return KV_OK;
 }

@@ -38,7 +38,9 @@
 // sets KV_DEV_WAIT_EXPIRED and leaves (every other CTA then runs into the same limit).
 // Barrier and histograms come in two sets used in turn; a launch clears the set of the
 // next one.  The launch's number, which also says whose turn it is, lives in device
-// memory, so that a captured launch can be replayed.
+// memory, so that a captured launch can be replayed.  The selection without caller's scratch
+// (SHARED = true) cannot rely on the launch before it: it clears its one set itself, while its
+// keys are read (a memset ahead of the launch took 3.0 us of a 21.9 us pass over 1,000,003 entries).
 // Measured, a pass with the event reduction, against notes per thread and whole chunks
 // only: 4,096 entries 32.5 -> 13.5 us, 0.9 M 40.3 -> 27.4, 3.1 M 59.9 -> 41.3, 18.8 M
 // 206 -> 180.
@@ -91,9 +93,9 @@ struct PArgs {
   unsigned long long k;
   uint32_t* victims;
   SelectScalars* sel;
-  SelectTurn* turns;      // [2] barrier and histograms of this launch (zero on entry) and of the next
+  SelectTurn* turns;      // [2] barrier and histograms of this launch (zero on entry) and of the next; shared scratch: [1]
   uint32_t* table;        // [n_rows][G] counts of every chunk
-  uint32_t use_hint;      // 0: plain radix select whatever an earlier selection left
+  unsigned long long* words;   // shared scratch (nullptr: the pool's own): number of the last call, then words of the first CTAs
   uint32_t* status;
   uint32_t n_full;        // full rows: chunks of 4,096 entries
   uint32_t last_len;      // entries of a CTA's piece of the last, shorter row (multiple of 128; 0: no such row)
@@ -265,7 +267,8 @@ __device__ __forceinline__ uint32_t block_scores4(const PArgs& a, unsigned long 
 }
 
 // PLAIN (fused form only): the policy is the Bayesian product and no partition is weighted.
-template <bool FUSED, bool PLAIN, bool BLOCKS>
+// SHARED: on scratch that calls share which know nothing of each other.
+template <bool FUSED, bool PLAIN, bool BLOCKS, bool SHARED>
 __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const PArgs a) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
   const uint32_t n_words = a.n_rows * 128u;           // bitmap words: 128 per row
@@ -341,10 +344,15 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     issue(0);
     issue(1);
   }
-  const uint32_t tag = a.sel->serial + 1u;            // this launch's number
-  SelectTurn* const turn = a.turns + (tag & 1u);
+  // Shared scratch: the first CTAs clear the counters, each says so in its word, with a number higher
+  // than any a call has ever used there, and none adds to a counter before all have said so.  (The
+  // numbers compare equal, so the CTAs of calls that overlap run into the limit instead of finishing
+  // with different ones.)
+  const unsigned long long call = SHARED ? a.words[0] + 1u : 0u;
+  const uint32_t tag = SHARED ? (uint32_t)call : a.sel->serial + 1u;   // this launch's number
+  SelectTurn* const turn = a.turns + (SHARED ? 0u : tag & 1u);
   unsigned int* const bar = &turn->bar;
-  const bool hint = a.use_hint && a.spill && a.sel->hint_valid != 0 && a.sel->hint_n == a.n;
+  const bool hint = !SHARED && a.sel->hint_valid != 0 && a.sel->hint_n == a.n;
   const uint32_t hint_tau = a.sel->hint_tau;
   uint32_t half = a.sel->hint_half;   // (the bracket's width follows how well the hints have been doing)
   if constexpr (FUSED) {
@@ -358,7 +366,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
   for (uint32_t w = t; w < n_words; w += kPThreads) s_be[w] = 0;
   for (uint32_t w = g * kPThreads + t; w < sizeof(SelectTurn) / 4u; w += G * kPThreads)
-    reinterpret_cast<uint32_t*>(a.turns + ((tag & 1u) ^ 1u))[w] = 0;
+    reinterpret_cast<uint32_t*>(a.turns + (SHARED ? 0u : (tag & 1u) ^ 1u))[w] = 0;
   if (t == 0) s_below = 0;
   half = half < kHalfMin ? kHalfMin : (half > kHalfMax ? kHalfMax : half);
   uint32_t bshift = kBracketShiftMin;                   // bins are 2^bshift keys wide
@@ -372,6 +380,21 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const float neg_inf = __int_as_float(0xFF800000);
   const float lo_f = hint ? key_score(base0) : neg_inf, hi_f = hint ? key_score(base0 + 2u * half) : neg_inf;
   __syncthreads();
+  constexpr uint32_t kClearing = (sizeof(SelectTurn) / 4u + kPThreads - 1u) / kPThreads;   // CTAs that clear something
+  static_assert(kClearing <= kSharedCtas, "each of them has a word");
+  if (SHARED && g < kClearing && t == 0)
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(a.words + 1 + g), "l"(call) : "memory");
+  auto cleared = [&]() {   // what this thread knows of it; false if its wait ran out
+    bool said = !SHARED || t >= kClearing || t >= G;
+    if constexpr (SHARED) {
+      for (uint32_t it = 0; it < kBarrierSpins && !said; ++it) {
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(a.words + 1 + t) : "memory");
+        said = v == call;
+      }
+    }
+    return said;
+  };
 
   // ---- phase A ----
   uint32_t n_noted = 0;     // notes of this warp
@@ -496,7 +519,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   }
   stamp(1);
   // (number 0 marks a word never written; the turns alternate across the wrap too)
-  auto end_turn = [&]() { a.sel->serial = tag == 0xFFFFFFFFu ? 1u : tag; };
+  auto end_turn = [&]() {
+    if (SHARED) atomicMax(a.words, call);
+    else a.sel->serial = tag == 0xFFFFFFFFu ? 1u : tag;
+  };
   uint32_t nbar = 0;        // grid barriers passed
   bool ok = true, hint_hit = false;
   if (FUSED || hint) {
@@ -526,8 +552,12 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     unsigned long long k_rem = a.k;
     bool found = true;
     // The CTA's histogram joins the others' in histogram h; false if the wait ran out.
-    auto exchange_hist = [&](uint32_t h, uint32_t nbins) {
-      __syncthreads();
+    auto exchange_hist = [&](uint32_t h, uint32_t nbins, bool ready = true) {
+      if constexpr (SHARED) {
+        if (!__syncthreads_and(ready)) return false;
+      } else {
+        __syncthreads();
+      }
       if (alone) return true;
       if (2u * t < nbins) add_pair(turn->hist[h] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
       grid_arrive(bar);
@@ -655,7 +685,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
             if (key[q] != kKeyExcluded && key[q] >= base && (digit == 0 || (d >> top) == 0u)) atomicAdd(&s_hist[d], 1u);
           }
         });
-        ok = exchange_hist(h, 1u << top);
+        ok = exchange_hist(h, 1u << top, digit != 0 || alone || cleared());
         if (digit == 1) stamp(3);
         if (!ok) goto fail;
         pick_bin(turn->hist[h], alone, s_hist, 1u << top, k_rem, s_warp, s_pick, bin, before);
@@ -935,8 +965,9 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
       cudaDeviceGetAttribute(&d.n_sm, cudaDevAttrMultiProcessorCount, dev);
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      void* fns[4] = {(void*)select_persistent_kernel<false, false, false>, (void*)select_persistent_kernel<true, false, false>,
-                      (void*)select_persistent_kernel<true, true, false>, (void*)select_persistent_kernel<false, false, true>};
+      void* fns[5] = {(void*)select_persistent_kernel<false, false, false, false>, (void*)select_persistent_kernel<true, false, false, false>,
+                      (void*)select_persistent_kernel<true, true, false, false>, (void*)select_persistent_kernel<false, false, true, false>,
+                      (void*)select_persistent_kernel<false, false, false, true>};
       cudaError_t e = cudaSuccess;
       size_t fixed = 0;
       for (void* fn : fns) {
@@ -982,7 +1013,7 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   a.sel = ws.sel;
   a.turns = ws.turns;
   a.table = ws.table;
-  a.use_hint = ws.keep_hint ? 1u : 0u;
+  a.words = ws.shared_words;
   a.status = ws.status;
   a.stage_words = fs ? (fs->opt.policy == 2 ? kStageWordsLru : kStageWords) : 0u;
   // Notes: the bracket typically holds 4-15 % of a warp's keys, in some traces several times
@@ -1014,10 +1045,11 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   }
   void* args[] = {&a};
   const bool plain = fs && fs->opt.policy == 0 && fs->hw.on == 0;
-  void* fn = bg ? (void*)select_persistent_kernel<false, false, true>
-             : !fs ? (void*)select_persistent_kernel<false, false, false>
-                   : plain ? (void*)select_persistent_kernel<true, true, false>
-                           : (void*)select_persistent_kernel<true, false, false>;
+  void* fn = bg ? (void*)select_persistent_kernel<false, false, true, false>
+             : ws.shared_words ? (void*)select_persistent_kernel<false, false, false, true>
+             : !fs ? (void*)select_persistent_kernel<false, false, false, false>
+                   : plain ? (void*)select_persistent_kernel<true, true, false, false>
+                           : (void*)select_persistent_kernel<true, false, false, false>;
   cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, G > 1, ws);
   if (e != cudaSuccess) return e;
   count_launches(1);

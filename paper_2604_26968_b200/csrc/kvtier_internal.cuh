@@ -108,8 +108,8 @@ struct SelectScalars {
   uint32_t hint_resid;
 };
 
-// What the CTAs of one persistent selection share while it runs.  Two of these are used in turn:
-// a launch finds its own zeroed and clears the next launch's.
+// What the CTAs of one persistent selection share while it runs.  A pool has two of these, used in
+// turn: a launch finds its own zeroed and clears the next launch's.
 struct SelectTurn {
   unsigned int bar;             // arrivals at the grid barrier
   unsigned int pad;
@@ -200,7 +200,10 @@ struct Workspace {
   SelectTurn* turns;                // [2], used in turn
   uint32_t* table;                  // [table_words] counts per chunk
   uint64_t table_words;
-  bool keep_hint = true;            // selections start from the threshold of the one before
+  // Scratch that calls share which know nothing of each other (nullptr: it is the pool's own): the
+  // number of the last call, then a word for each CTA that clears (up to kSharedCtas).  Each call
+  // clears its set of counters itself, whatever the one before has left.
+  unsigned long long* shared_words = nullptr;
   // One of the state arrays kept in the persisting part of the L2 (kv_set_l2_residency):
   // the scoring kernels are launched with this access-policy window.  bytes == 0: none.
   const void* l2_base = nullptr;
@@ -318,6 +321,23 @@ struct PartCounts {
 // Words of the persistent selection's table of counts for n entries: one per chunk of 4,096 entries
 // of every CTA, the last row's pieces counted as chunks (at most 1,024 CTAs).
 inline uint64_t select_table_words(uint64_t n) { return n / 4096 + 1024; }
+// The scratch of selections for callers that have none to give (kv_select.cu).
+constexpr uint64_t kStaticMaxEntries = 1ull << 22;  // 4,194,304 entries
+constexpr uint64_t kStaticMaxTiles = kStaticMaxEntries / kTileEntries + 2;
+constexpr uint32_t kSharedCtas = 16;
+struct StaticScratch {
+  uint32_t hist[3 * kHistBins];
+  SelectTurn turn;
+  SelectScalars sel;
+  unsigned long long words[1 + kSharedCtas];
+  uint32_t status[4];
+  uint2 tile_counts[kStaticMaxTiles];
+  uint2 tile_offsets[kStaticMaxTiles];
+  uint32_t table[kStaticMaxEntries / 4096 + 1024];
+};
+// n <= kStaticMaxEntries; status may be nullptr
+cudaError_t launch_select_static(const float* score, const uint8_t* state, uint64_t n, uint64_t k, uint32_t* d_victims,
+                                 StaticScratch* scratch, uint32_t* status, cudaStream_t s, int variant = 1);
 // variant 1 = one persistent cooperative launch (falls back to 0 where the device cannot run
 // it or the slices are too long), 0 = one launch per phase of the radix select
 cudaError_t launch_select(const EntryState& st, uint64_t k, uint32_t* d_victims, const Workspace& ws,
