@@ -4,14 +4,22 @@
 
 namespace kvt {
 
-// 32-bit keys whose unsigned order is the order of the scores.  -0.0 orders with +0.0, so the
-// key 0x7FFFFFFF (its own bit pattern's) never occurs.
-constexpr uint32_t kKeyExcluded = 0xFFFFFFFFu;   // key of an entry that is no candidate (a NaN's)
+// 32-bit keys whose unsigned order is the order of the scores; NaNs (a caller's array may hold them)
+// are ordered by their bits, below -inf or above +inf.  -0.0 orders with +0.0, so the key 0x7FFFFFFF
+// (its own bit pattern's) never occurs and stands for an entry that is no candidate.
+constexpr uint32_t kKeyExcluded = 0x7FFFFFFFu;
 constexpr uint32_t kKeyNegInf = 0x007FFFFFu, kKeyPosInf = 0xFF800000u;
 
-__device__ __forceinline__ uint32_t score_key(float s) {
-  const uint32_t b = __float_as_uint(__fadd_rn(s, 0.0f));   // -0.0 + 0.0 = +0.0; every other value is itself
+__device__ __forceinline__ uint32_t key_of_bits(uint32_t b) {
   return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ uint32_t score_key(float s) {
+  const uint32_t b = __float_as_uint(s);
+  return key_of_bits(b == 0x80000000u ? 0u : b);
+}
+// The same, in fewer instructions, of a number or of a NaN that arithmetic gave.
+__device__ __forceinline__ uint32_t number_key(float s) {
+  return key_of_bits(__float_as_uint(__fadd_rn(s, 0.0f)));   // -0.0 + 0.0 = +0.0; every other value is itself
 }
 
 // The score with a given key (keys of -inf .. +inf).

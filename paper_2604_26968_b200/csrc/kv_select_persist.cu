@@ -427,7 +427,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     uint32_t wl[4], wi[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const bool lo = s[q] < lo_f;
+      // (a NaN is neither below nor inside; the scores that this kernel forms are positive ones, which
+      // come behind all numbers, but an array may hold negative ones, which come before)
+      bool lo = s[q] < lo_f;
+      if constexpr (!FUSED && !BLOCKS) lo = lo || __float_as_uint(s[q]) > 0xFF800000u;
       in[q] = s[q] < hi_f && !lo;
       n_below += lo;
       wl[q] = __ballot_sync(0xFFFFFFFFu, lo);
@@ -438,7 +441,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         if (in[q]) {
-          const uint32_t d = score_key(s[q]) - base0;
+          const uint32_t d = number_key(s[q]) - base0;   // (inside the bracket: no NaN)
           // (additions of 1 to one bin are merged by the hardware: collecting a thread's equal bins in a
           // register first cost 0.7 of 42.1 us at 3.1 M entries, 1.7 of 20.4 in the plain radix select)
           atomicAdd(&s_hist[d >> bshift], 1u);
@@ -580,24 +583,26 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     }
     // keys of the thread's vector of row r, from the arrays; entries past the row's end or not
     // RESIDENT give kKeyExcluded
+    // (scores that the kernel forms itself: a NaN has the one bit pattern that arithmetic gives)
+    auto key_of = [](float x) { return FUSED || BLOCKS ? number_key(x) : score_key(x); };
     auto load_keys = [&](uint32_t r, uint32_t key[4]) {
       const uint32_t i0 = row_base(r) + 4u * t, i1 = row_end(r);
       if (BLOCKS) {
         float s[4];
         const uint32_t resident = block_scores4(a, i0, i1, s);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) key[j] = (resident >> j) & 1u ? score_key(s[j]) : kKeyExcluded;
+        for (int j = 0; j < 4; ++j) key[j] = (resident >> j) & 1u ? key_of(s[j]) : kKeyExcluded;
       } else if (i0 + 4u <= i1) {
         const float4 sc = __ldcg(reinterpret_cast<const float4*>(a.score + i0));
         const uint32_t st4 = __ldcg(reinterpret_cast<const uint32_t*>(a.state + i0));
-        key[0] = (st4 & 0xFFu) == KV_STATE_RESIDENT ? score_key(sc.x) : kKeyExcluded;
-        key[1] = ((st4 >> 8) & 0xFFu) == KV_STATE_RESIDENT ? score_key(sc.y) : kKeyExcluded;
-        key[2] = ((st4 >> 16) & 0xFFu) == KV_STATE_RESIDENT ? score_key(sc.z) : kKeyExcluded;
-        key[3] = (st4 >> 24) == KV_STATE_RESIDENT ? score_key(sc.w) : kKeyExcluded;
+        key[0] = (st4 & 0xFFu) == KV_STATE_RESIDENT ? key_of(sc.x) : kKeyExcluded;
+        key[1] = ((st4 >> 8) & 0xFFu) == KV_STATE_RESIDENT ? key_of(sc.y) : kKeyExcluded;
+        key[2] = ((st4 >> 16) & 0xFFu) == KV_STATE_RESIDENT ? key_of(sc.z) : kKeyExcluded;
+        key[3] = (st4 >> 24) == KV_STATE_RESIDENT ? key_of(sc.w) : kKeyExcluded;
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          key[j] = (i0 + j < i1 && a.state[i0 + j] == KV_STATE_RESIDENT) ? score_key(a.score[i0 + j]) : kKeyExcluded;
+          key[j] = (i0 + j < i1 && a.state[i0 + j] == KV_STATE_RESIDENT) ? key_of(a.score[i0 + j]) : kKeyExcluded;
       }
     };
     // A pass over the CTA's keys, rows in order: body(r, key) sees the thread's four keys of row
@@ -702,7 +707,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         uint32_t wl[4], we[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          wl[q] = __ballot_sync(0xFFFFFFFFu, key[q] < tau);
+          wl[q] = __ballot_sync(0xFFFFFFFFu, key[q] < tau && key[q] != kKeyExcluded);
           we[q] = __ballot_sync(0xFFFFFFFFu, key[q] == tau && key[q] != kKeyExcluded);
         }
         if (lane == 0) {

@@ -85,6 +85,69 @@ def test_hinted_selection_rows(n_rows, rest):
     p.close()
 
 
+def expected_by_bits(score, state, k):
+    """Scores ordered by their bits: NaNs with the sign bit lie below -inf, the others above +inf."""
+    b = (score + np.float32(0.0)).view(np.uint32).astype(np.int64)
+    b = np.where(np.isnan(score), score.view(np.uint32), b)
+    key = np.where(b >> 31, 0xFFFFFFFF - b, b + 0x80000000)
+    ids = np.flatnonzero(state != 0)
+    return np.sort(ids[np.argsort(key[ids], kind="stable")[:k]]).astype(np.uint32)
+
+
+def with_nans(n, seed):
+    r = np.random.default_rng(seed)
+    score = draw(n, seed)
+    at = r.permutation(n)
+    bits = score.view(np.uint32)
+    few = max(1, n // 50)
+    for i, special in enumerate((0x7FC00000, 0xFFC00000, 0x7FFFFFFF, 0xFFFFFFFF, 0x7F800000, 0xFF800000, 0x80000000, 0)):
+        bits[at[i * few:(i + 1) * few]] = special
+    return score
+
+
+@pytest.mark.parametrize("n", [1000, 8192, 37 * 1024 + 11, ROW + 999])
+def test_scores_that_are_not_numbers(n):
+    """A caller's array may hold them; they have their places in the order like all others."""
+    import torch
+    state = (np.random.default_rng(n).random(n) > 0.02).astype(np.uint8)
+    score = with_nans(n, 5)
+    resident = int(state.sum())
+    d_score, d_state = torch.from_numpy(score).cuda(), torch.from_numpy(state).cuda()
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    for k in (1, n // 100, n // 10, n // 2, resident - 3, resident):
+        out = torch.full((k + 4,), -1, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        assert B.kv_select_victims_static(d_score, d_state, n, k, out, status, torch.cuda.current_stream()) == 0
+        torch.cuda.synchronize()
+        assert np.array_equal(out[:k].cpu().numpy().view(np.uint32), expected_by_bits(score, state, k)), k
+    assert int(status[0]) == 0
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+def test_scores_that_are_not_numbers_in_a_pool(variant):
+    """The same with thresholds taken from the selection before (variant 1)."""
+    import torch
+    w = W.Workload("rows", [W.gqa(1, 4, 2, 4, 2, 50_003, 16, "entry")], 0.1, 0.0, seed=3)
+    p = B.Pool(w.parts, w.N + 16, staging_bytes=4096, max_promote=64, host_meta=False)
+    pairs = torch.zeros(w.N + 16, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    assert p.kv_set_select_variant(variant) == 0
+    assert p.kv_admit(0, 0.9, pairs, False)[0] == 0
+    p.sync()
+    state = np.ones(w.N, np.uint8)
+    for i, k in enumerate((w.N // 5, w.N // 5 + 7, w.N // 5 + 9, w.N // 100, w.N - 5, w.N)):
+        score = with_nans(w.N, 9 + i // 4)
+        out = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+        p.score[:w.N].copy_(torch.from_numpy(score))
+        torch.cuda.synchronize()
+        assert p.kv_select_victims(k, out) == 0
+        p.sync()
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), expected_by_bits(score, state, k)), (i, k)
+        assert p.kv_device_status() == 0
+    assert variant == 0 or p.kv_selection_stats()["hint_hits"] >= 1
+    p.close()
+
+
 def test_captured_selection_can_be_replayed():
     import torch
     n, k = ROW + 999, 20_000
