@@ -357,7 +357,8 @@ int32_t kv_promote(kv_pool* pool, int32_t partition, const uint64_t* h_host_slot
  * (distance, layer, head): a list kv_promote accepts once it has been brought to the
  * host.  Handles >= n_tags, dropped or never admitted, and blocks already in HBM are
  * skipped.  *d_out_count (device-accessible u64) receives how many qualified; if that
- * exceeds max_out only the first max_out were written.  n_pos == 0 gives count 0.
+ * exceeds max_out only the first max_out were written.  n_pos == 0 gives count 0.  A list
+ * that sets KV_DEV_WAIT_EXPIRED is void.
  * One small launch on `stream`, which first joins the pool's promotions in flight
  * (they write d_loc); call it on the pool's compute stream.  Calls of one pool share a
  * scratch array: do not run two of them concurrently on different streams. */

@@ -17,7 +17,7 @@
 // launch: a block counts the qualifying candidates of its chunk, publishes the count, adds up
 // the counts of the blocks before it as they appear, and writes.  A block waits only for blocks
 // of lower index (bounded: one that gives up sets KV_DEV_WAIT_EXPIRED and leaves, and so do the
-// blocks behind it).  A call is latency: window, table and d_loc are three dependent reads of
+// blocks behind it; the last one then reports an empty list).  A call is latency: window, table and d_loc are three dependent reads of
 // about 0.7 us, the counts one more; a second launch for the writing cost as much again
 // (8 lists of 256 x 80 x 8 candidates: 110 -> 56 us).
 #include "kvtier_internal.cuh"
@@ -199,7 +199,10 @@ __global__ void __launch_bounds__(kPfThreads) prefetch_list_kernel(const ListArg
   if (!ok) {
     if (tid == 0) {
       atomicOr(a.status, KV_DEV_WAIT_EXPIRED);
-      if (blockIdx.x == gridDim.x - 1) *a.serial = tag;
+      if (blockIdx.x == gridDim.x - 1) {
+        *a.count = 0;
+        *a.serial = tag;
+      }
     }
     return;
   }
