@@ -890,6 +890,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         for (int q = 1; q < 4; ++q) a.pc.h_counts[q] = 0;
       }
       end_turn();   // (every CTA has read the number long ago)
+      if constexpr (SHARED) return;   // (nobody comes after it who could use what follows)
       a.sel->tau = tau;
       a.sel->need_eq = need_eq;
       a.sel->n_select += 1;
