@@ -289,13 +289,14 @@ def time_dedup(torch, pool, w, B, reps=3):
             "dedup_unique": int(extra[0].item()), "dedup_status": int(extra[4].item())}
 
 
-def oracle_pool(w):
+def oracle_pool(w, n_epochs):
+    """The workload's pool in the oracle, with handles for n_epochs epochs (each admits at most w.k blocks)."""
     from oracle import kv_oracle as O
     parts = [dict(model=O.Model(p.variant, p.n_layers, p.n_q_heads, p.n_kv_heads, p.head_dim,
                                 p.d_latent, p.d_rope, p.dtype_bits),
                   block_tokens=p.block_tokens, blocks_per_layer=p.blocks_per_layer,
                   ring_slots=p.ring_slots) for p in w.parts]
-    return O, O.OraclePool(parts, w.alpha0, w.beta0, n_tags=w.n_tags, payload=False)
+    return O, O.OraclePool(parts, w.alpha0, w.beta0, n_tags=max(w.n_tags, w.N + n_epochs * w.k), payload=False)
 
 
 def oracle_epochs(w, n_epochs, warm=0):
@@ -303,7 +304,7 @@ def oracle_epochs(w, n_epochs, warm=0):
     bytes) on the workload.  Returns (seconds in score+select, seconds per full
     epoch, epochs timed)."""
     from paper_2604_26968_b200.harness import INITIAL_EPOCH_KEY
-    O, pool = oracle_pool(w)
+    O, pool = oracle_pool(w, warm + n_epochs)
     fresh = np.flatnonzero(pool.state == O.FREE).astype(np.uint32)
     pool.admit(0, w.decay, w.new_pairs(INITIAL_EPOCH_KEY, fresh.size), None)
     t_ss, t_all, done = 0.0, 0.0, 0
