@@ -147,7 +147,8 @@ typedef struct {
   uint32_t* d_touch;      /* touches seen in the current epoch */
   uint32_t* d_last_epoch; /* epoch of the last touch */
   uint8_t* d_pair;        /* 4*block_type + transition_type, 0..15; the library sets bit 7
-                             while the entry is FREE (the value is then meaningless) */
+                             while the entry is FREE (the value is then meaningless, but the
+                             bit is what scoring goes by: leave the bytes of FREE entries alone) */
   uint8_t* d_state;       /* KV_STATE_* */
   uint32_t* d_tag;        /* logical handle of the block in the slot, KV_NONE if FREE */
   float* d_score;         /* eviction score, +inf for FREE entries */
@@ -425,7 +426,9 @@ int32_t kv_set_lazy_decay(kv_pool* pool, int32_t on);
  * ids; NULL = entries 0..m-1): the entry's K chunk followed by its V chunk, or its
  * single MLA chunk, exactly the bytes kv_demote would send to the host ring.  The
  * entries need not be RESIDENT (a FREE slot's bytes are whatever was left there).
- * An id >= N sets KV_DEV_BAD_INDEX and leaves its digest unwritten. */
+ * An id >= N sets KV_DEV_BAD_INDEX and leaves its digest unwritten.  While the call runs
+ * d_digests holds intermediate values, and it uses the pool's scratch: like every call
+ * on a pool it belongs on the pool's compute stream. */
 int32_t kv_hash_entries(kv_pool* pool, const uint32_t* d_ids, uint64_t m, uint8_t* d_digests,
                         kv_stream_t stream);
 
@@ -579,8 +582,8 @@ int32_t kv_set_select_variant(kv_pool* pool, int32_t variant);
 /* Measurement aid: how the pool's persistent selections went so far.  Each starts from
  * a hint (the threshold of the selection before it): a hit means one short pass after
  * the scoring pass finished it, a miss that the keys were read again (two or three
- * passes); reread_ctas counts thread blocks that read their keys again although the
- * hint held: always 0 now, what a block cannot note in shared memory goes to a scratch.
+ * passes); reread_ctas is reserved and 0 (what a block cannot note in shared memory
+ * goes to a scratch; none reads its keys again while the hint holds).
  * Blocks the host until `stream` has drained. */
 typedef struct {
   uint64_t selections, hint_hits, hint_misses, reread_ctas;

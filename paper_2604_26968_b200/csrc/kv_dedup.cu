@@ -100,7 +100,7 @@ __device__ __forceinline__ uint64_t hash_chunk_offset(const PartGeom& g, uint64_
 }
 
 // Chains in turn.  A warp's 32 messages are one chain of up to 131,072 dependent blocks.  Where
-// there are between 2 and ~10 chains per scheduler, an integer number of them per scheduler cannot
+// the chains are no multiple of the schedulers, an integer number of them per scheduler cannot
 // be even: 2,458 chains on 592 schedulers are 4 on most and 5 on some, and the call takes as long
 // as 5.  So the grid holds an even number of warps, each works on a chain for one slice (a seventh
 // of the longest message), leaves the intermediate hash value in the place of the digest, queues the

@@ -98,7 +98,7 @@ struct SelectScalars {
   unsigned int n_select;       // selections run
   unsigned int n_hint_hit;     // ... whose hint's bracket held rank k
   unsigned int n_hint_miss;    // ... whose hint's bracket did not
-  unsigned int n_reread;       // CTAs (over all selections) that had to re-read their keys although the hint held
+  unsigned int n_reread;       // reserved (kv_selection_stats reports it), 0
   // persistent selection on a pool of several partitions: launch number | victims before
   // partition boundary q + 1, written by the CTA that holds it
   unsigned long long bound[3];

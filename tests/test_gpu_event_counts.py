@@ -11,7 +11,7 @@ from paper_2604_26968_b200 import workloads as W
 pytestmark = pytest.mark.gpu
 
 BLOCK = 512 * 4                # events of one block's vectors
-GRID = BLOCK * 296             # events of one vector for every thread of the grid (over 8 of them: part is dealt out by demand)
+GRID = BLOCK * 296             # events of one vector for every thread of the grid
 
 
 def trace(style, n, n_events, r):

@@ -1,7 +1,7 @@
 """A prefetch list whose last block's wait for the counts before it runs out: the status says so, and
 the count, which the caller's word may hold from an earlier call, says that nothing is listed.  The
 kernel is built with a limit of one look; its last block has nothing of its own to do and looks while
-the first is still reading its part of the table."""
+the first is still reading its part of the table, tile after tile."""
 import ctypes as C
 import os
 import subprocess
@@ -28,12 +28,12 @@ def test_count_of_a_list_that_gave_up(tmp_path):
     lib = C.CDLL(so)
     u64, u32, ptr = C.c_uint64, C.c_uint32, C.c_void_p
     lib.prefetch_list.argtypes = [ptr, ptr, ptr, ptr, u32, u32, u32, ptr, u64, ptr, u64, ptr, u64, ptr, ptr]
-    layers, heads, n_pos = 32, 8, 1184   # 303,104 candidates, a block for each 1,024; the windows are 3 positions wide
+    layers, heads, n_pos = 32, 8, 18_944   # 296 blocks of 16 x 1,024 candidates; the windows hold the first one's
 
     def ints(n, value, dtype=torch.int32):
         return torch.full((n,), value, dtype=dtype, device="cuda")
 
-    win, words, serial, status = ints(layers, 3), ints(1024, 0, torch.int64), ints(4, 0), ints(4, 0)
+    win, words, serial, status = ints(layers, 64), ints(1024, 0, torch.int64), ints(4, 0), ints(4, 0)
     table, n_tags = torch.arange(n_pos * layers * heads, dtype=torch.int32, device="cuda"), n_pos * layers * heads
     loc = (torch.arange(n_tags, device="cuda") + (1 << 31)).to(torch.uint32).view(torch.int32)   # all in the host tier
     out, count = ints(4096, -1, torch.int64), ints(2, 77, torch.int64)

