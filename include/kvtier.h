@@ -144,7 +144,8 @@ typedef struct {
   /* per-entry state, struct of arrays of length N in global id order (device) */
   float* d_ema;           /* EMA access score */
   float* d_decay;         /* EMA decay per entry */
-  uint32_t* d_touch;      /* touches seen in the current epoch */
+  uint32_t* d_touch;      /* touches that kv_epoch_events has counted and no scoring pass has taken up;
+                             else zero, whatever a pass in progress keeps there.  The library's to write */
   uint32_t* d_last_epoch; /* epoch of the last touch */
   uint8_t* d_pair;        /* 4*block_type + transition_type, 0..15; the library sets bit 7
                              while the entry is FREE (the value is then meaningless, but the
@@ -283,7 +284,7 @@ int32_t kv_select_victims(kv_pool* pool, uint64_t k, uint32_t* d_victims, kv_str
  * scores are written once for the caller and never read back, and a launch
  * boundary disappears (two launches in all: the event reduction, then the rest).
  * State, d_victims and the device status word end up exactly as after the two
- * calls.  All arguments are checked before anything is enqueued: on an error
+ * calls.  The trace is read by both launches: leave it alone until the call's work has run.  All arguments are checked before anything is enqueued: on an error
  * (including KV_ERR_K_TOO_LARGE) the epoch has NOT been scored.  k == 0 scores
  * only.  Where the device cannot keep the kernel's whole grid resident at once,
  * the separate kernels run one after the other instead. */
@@ -391,9 +392,10 @@ int32_t kv_set_gather_threshold(kv_pool* pool, uint64_t run_bytes);
  * arrays once more; between the two, and from one epoch to the next, the gigabytes that
  * the block movement sends through the L2 evict them.  With a budget > 0 the scoring
  * kernels (event reduction, entry pass, fused selection) are launched with an access-policy
- * window that keeps ONE array in the persisting part of the L2: the touch counts (4 B per
- * entry) when they fit the budget whole, else the pair bytes (1 B per entry), a fraction
- * of them if even those do not fit.  Measured on a B200 (126 MB L2): 47 MB of touch counts
+ * window that keeps ONE array in the persisting part of the L2: the touch counts when they
+ * fit the budget whole (4 B per entry, or the 2 B per entry that kv_epoch_score_select
+ * counts in its workspace), else the pair bytes (1 B per entry), a fraction of them if even
+ * those do not fit.  Measured on a B200 (126 MB L2): 47 MB of touch counts
  * resident take 20 us off a 150 us pass; 75 MB resident leave too little L2 for the
  * streaming entry pass and cost more than they save, hence the rule.  A budget of 3/8 of
  * the L2 is a good choice.  Results are bit for bit the same.

@@ -22,18 +22,29 @@ namespace kvt {
 // event is a plain read-add-write of the thread's own word: no vote, no atomic.
 // The block adds its columns up once at the end.
 //
-// Touch counts: every update is a 64-bit atomic on the aligned pair of 32-bit
-// counts (touch[2i], touch[2i+1]) -- adding 1, 1 << 32 or both -- so that all
-// atomics on a word have one size.  (A carry out of the low count would need
-// 2^32 touches of one entry in one epoch, where the count wraps anyway.)  The
-// one exception is the last entry of an array of odd length, whose partner
-// would lie outside the array: it takes 32-bit atomics, and only those.
+// Touch counts, in the array that the caller may look at (kv_epoch_events): every update
+// is a 64-bit atomic on the aligned pair of 32-bit counts (touch[2i], touch[2i+1]) --
+// adding 1, 1 << 32 or both -- so that all atomics on a word have one size.  (A carry out
+// of the low count would need 2^32 touches of one entry in one epoch, where the count
+// wraps anyway.)  The one exception is the last entry of an array of odd length, whose
+// partner would lie outside the array: it takes 32-bit atomics, and only those.
+//
+// Touch counts that only the fused scoring pass of the same call reads (PACKED): 64 bits
+// for four entries, nine for each and the sum of the four in the upper 28, so that one
+// atomic counts all events of a vector on the same four entries, and half the bytes are
+// scattered over and then read.  A count that overflows carries into the next field and
+// takes 511 from the sum of the fields, or, the last one, 512, and adds one to the sum
+// kept beside them: the two agree again only after 512 * 2^28 / 513 touches, more than a
+// trace that is counted this way has, so the scoring pass sees of every word whether it is
+// right.  (Atomics that return the word they found would tell the event reduction of every
+// carry, and bytes would do, but they took 37.6 us instead of 28.4 for 15.3 M events, 9.2
+// instead of 6.3 for 0.6 M.)
 //
 // Traces in which a touched block reports all its heads hand every thread four
 // consecutive entries (an aligned group of four ids): one 4-byte load then
-// fetches their pairs and FREE bits, and two atomics count the four touches.
-// Those two go out from neighbouring lanes of one instruction, so that a 32-byte
-// sector of counts is visited once and not twice.
+// fetches their pairs and FREE bits, and one atomic on a packed word, or two on the 32-bit
+// counts, counts the four touches.  Those two go out from neighbouring lanes of one instruction, so
+// that a 32-byte sector of counts is visited once and not twice.
 //
 // What bounds it: the latency of two dependent scattered reads (event, pair byte) and
 // the rate of the atomics.  The next vectors' events are on their way while the current
@@ -62,15 +73,46 @@ __device__ __forceinline__ void touch_add(uint32_t* touch, uint32_t i, uint32_t 
     atomicAdd(&touch[i], 1u);   // last entry of an odd-length array (i is even, inc_pair is 1)
 }
 
+constexpr uint32_t kFieldBits = 9, kFieldMax = (1u << kFieldBits) - 1u, kSumShift = 4u * kFieldBits;
+// Touches of four entries, one byte each (a few of each), as what they add to the entries' packed word.
+__device__ __forceinline__ unsigned long long packed_touches(uint32_t b) {
+  const uint32_t lo = (b & 0xFFu) | (b & 0xFF00u) << 1 | (b & 0xFF0000u) << 2;
+  return ((unsigned long long)(b >> 24) << (3u * kFieldBits) | lo) + ((unsigned long long)__dp4a(b, 0x01010101u, 0u) << kSumShift);
+}
+// The four counts; false if one of them has overflowed.
+__device__ __forceinline__ bool unpack_touches(uint2 w, uint32_t t[4]) {
+  t[0] = w.x & kFieldMax;
+  t[1] = (w.x >> kFieldBits) & kFieldMax;
+  t[2] = (w.x >> (2u * kFieldBits)) & kFieldMax;
+  t[3] = __funnelshift_r(w.x, w.y, 3u * kFieldBits) & kFieldMax;
+  return t[0] + t[1] + t[2] + t[3] == w.y >> (kSumShift - 32u);
+}
+
+// The packed counts w of vector v as its touch counts, in x.t, the 32-bit counts added where they hold
+// anything (hot); both are cleared.  False, and nothing done, if a packed count has overflowed.
+__device__ __forceinline__ bool take_touches(const EntryState& st, uint64_t v, uint2 w, const uint32_t* hot, uint4& sum) {
+  uint32_t t[4];
+  if (!unpack_touches(w, t)) return false;
+  sum = make_uint4(t[0], t[1], t[2], t[3]);
+  if (w.x | w.y) st.packed[v] = 0;
+  if (hot) {
+    const uint4 x = __ldcg(reinterpret_cast<const uint4*>(st.touch) + v);
+    sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+    if (x.x | x.y | x.z | x.w) reinterpret_cast<uint4*>(st.touch)[v] = make_uint4(0, 0, 0, 0);
+  }
+  return true;
+}
+
 // The calling block's share of the events.  s_cnt: kEventThreads * 16 words of shared
 // memory, zero on entry; word [p * kEventThreads + t] holds thread t's
 // counts for pair p (events | hits << 16) since the last flush.  delta: the 32
 // global epoch counters (index 2 * pair + hit).  Returns the KV_DEV_* bits of
 // refused events.  Every thread of the block must call it.
+template <bool PACKED>
 __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, const uint8_t* ev_hit,
-                                                  uint64_t n_events, const uint8_t* pair, uint32_t* touch, uint64_t n,
-                                                  uint64_t gtid, uint64_t stride, uint32_t* s_cnt,
-                                                  unsigned long long* delta) {
+                                                  uint64_t n_events, const uint8_t* pair, uint32_t* touch,
+                                                  unsigned long long* packed, uint64_t n, uint64_t gtid,
+                                                  uint64_t stride, uint32_t* s_cnt, unsigned long long* delta) {
   const uint64_t n4 = n_events / 4;
   const uint64_t iters = (n4 + stride * kEventVecs - 1) / (stride * kEventVecs);  // same for every thread
   // ids are 32-bit, so the bound is too (an id can never reach 2^32 - 1 = "no entry")
@@ -122,34 +164,53 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
     }
   };
 
+  auto ids_of = [](const EventVec& x, uint32_t id[4]) { id[0] = x.id.x; id[1] = x.id.y; id[2] = x.id.z; id[3] = x.id.w; };
+  // Four entries in a row: an aligned group, or (PACKED) one whose words of pair bytes lie inside the array.
+  auto is_run = [&](const uint32_t id[4]) {
+    return (PACKED || !(id[0] & 3u)) && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u &&
+           (PACKED ? id[3] | 3u : id[3]) < n32;
+  };
+  auto gather = [&](const uint32_t id[4], bool run) {   // the vector's pair bytes (bit 7 = FREE or out of range)
+    uint32_t w = 0;
+    if (run) {   // (through the L1: neighbouring blocks share sectors)
+      const uint32_t* p = reinterpret_cast<const uint32_t*>(pair) + (id[0] >> 2);
+      w = p[0];
+      if (PACKED && (id[0] & 3u)) w = __funnelshift_r(w, p[1], 8u * (id[0] & 3u));
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) w |= (uint32_t)(id[j] < n32 ? pair[id[j]] : (uint8_t)kPairFree) << (8 * j);
+    }
+    return w;
+  };
+
   EventVec nxt[kEventVecs];
   if (iters) load(0, nxt);
   for (uint64_t it = 0; it < iters; ++it) {
     EventVec cur[kEventVecs];
-    bool run[kEventVecs];       // ids are an aligned run of four inside the pool
+    bool run[kEventVecs];       // ids are a run of four inside the pool
     uint32_t pr4[kEventVecs];   // byte j: pair byte of event j's entry (bit 7 = FREE or out of range)
 #pragma unroll
     for (uint32_t u = 0; u < kEventVecs; ++u) cur[u] = nxt[u];
 #pragma unroll
     for (uint32_t u = 0; u < kEventVecs; ++u) {  // all gathers before any is used
-      const uint32_t id[4] = {cur[u].id.x, cur[u].id.y, cur[u].id.z, cur[u].id.w};
-      run[u] = !(id[0] & 3u) && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u && id[3] < n32;
-      if (run[u]) {
-        pr4[u] = *reinterpret_cast<const uint32_t*>(pair + id[0]);   // (through the L1: neighbouring blocks share sectors)
-      } else {
-        uint32_t w = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w |= (uint32_t)(id[j] < n32 ? pair[id[j]] : (uint8_t)kPairFree) << (8 * j);
-        pr4[u] = w;
-      }
+      uint32_t id[4];
+      ids_of(cur[u], id);
+      run[u] = is_run(id);
+      pr4[u] = gather(id, run[u]);
     }
     if (it + 1 < iters) load(it + 1, nxt);
 #pragma unroll
     for (uint32_t u = 0; u < kEventVecs; ++u) {
-      const uint32_t id[4] = {cur[u].id.x, cur[u].id.y, cur[u].id.z, cur[u].id.w};
+      uint32_t id[4];
+      ids_of(cur[u], id);
       const uint32_t pr = pr4[u], hit4 = nonzero_bytes(cur[u].hit);
       const bool whole = run[u] && !(pr & 0x80808080u);   // four resident entries in a row
-      const uint32_t m = __ballot_sync(0xFFFFFFFFu, whole);
+      if (PACKED && whole) {
+        const uint32_t r = id[0] & 3u;
+        atomicAdd(packed + (id[0] >> 2), packed_touches(0x01010101u << (8u * r)));
+        if (r) atomicAdd(packed + (id[0] >> 2) + 1u, packed_touches(0x01010101u >> (32u - 8u * r)));
+      }
+      const uint32_t m = PACKED ? 0u : __ballot_sync(0xFFFFFFFFu, whole);
       if (m) {
 #pragma unroll
         for (uint32_t half = 0; half < 2; ++half) {   // 16 vectors' pairs of atomics per instruction
@@ -171,8 +232,18 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
           bad_id |= !in;
           not_resident |= in && !ok[j];
         }
+        if constexpr (PACKED) {   // (the last event on a word adds for those before it)
+          uint32_t inc[4];
 #pragma unroll
-        for (int j = 0; j < 4; j += 2) {
+          for (int j = 0; j < 4; ++j) inc[j] = ok[j] ? 1u << (8u * (id[j] & 3u)) : 0u;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (j < 3 && (id[j] >> 2) == (id[j + 1] >> 2)) inc[j + 1] += inc[j];
+            else if (inc[j]) atomicAdd(packed + (id[j] >> 2), packed_touches(inc[j]));
+          }
+        }
+#pragma unroll
+        for (int j = 0; !PACKED && j < 4; j += 2) {
           const uint32_t i0 = id[j], i1 = id[j + 1];
           if (ok[j] && ok[j + 1] && i1 == i0 + 1u && !(i0 & 1u)) {
             atomicAdd(reinterpret_cast<unsigned long long*>(touch + i0), 0x100000001ull);
@@ -183,8 +254,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (ok[j]) count(pr >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);
-      }
+          if (ok[j]) count(pr >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);      }
       __syncwarp();
     }
     if ((it + 1) % kEventFlushIters == 0) flush();   // (uniform over the block)
@@ -204,7 +274,8 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
         bad |= KV_DEV_EVENT_NOT_RESIDENT;
       } else {
         count(pr, __ldcs(ev_hit + e) != 0);
-        touch_add(touch, i, n32, (i & 1u) ? (1ull << 32) : 1ull);
+        if constexpr (PACKED) atomicAdd(packed + (i >> 2), packed_touches(1u << (8u * (i & 3u))));
+        else touch_add(touch, i, n32, (i & 1u) ? (1ull << 32) : 1ull);
       }
     }
   }
@@ -370,10 +441,12 @@ __device__ __forceinline__ void commit_predictor(const Predictor& pd, unsigned p
 // Four consecutive entries (a 16-byte vector of each array) through the entry step,
 // in two halves so that a caller can have the next vector's loads in flight
 // while it finishes this one.  v indexes vectors.  The touch counts are read from
-// L2: other blocks' atomics made them.
+// L2: other blocks' atomics made them.  PACKED: take_touches has read and cleared them.  hot:
+// where to say that an entry has had too many touches for the packed counts to be tried again.
+constexpr uint32_t kTouchHot = kFieldMax / 2;
 struct EntryVec {
   float4 e, d;
-  uint4 t, le;
+  uint4 t, le;         // t: touch counts
   uint32_t pr4;        // pair bytes
 };
 
@@ -388,12 +461,13 @@ __device__ __forceinline__ EntryVec entry_load4(const EntryState& st, uint64_t v
   return x;
 }
 
-// touch and last_epoch are only written where an entry was touched.  kPlain: the caller
+// The counts and last_epoch are only written where an entry was touched.  kPlain: the caller
 // knows that the policy is the Bayesian product and that no partition is weighted (the
 // policy and weight tests then fold away at compile time).
-template <bool kPlain = false>
+template <bool PACKED, bool kPlain = false>
 __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, EntryVec& x, const float* sP,
-                                              int policy, uint32_t epoch, const HeadWeights& hw, float4& sc) {
+                                              int policy, uint32_t epoch, const HeadWeights& hw, uint32_t* hot,
+                                              float4& sc) {
   float e[4] = {x.e.x, x.e.y, x.e.z, x.e.w}, s[4];
   const float d[4] = {x.d.x, x.d.y, x.d.z, x.d.w};
   const uint32_t t[4] = {x.t.x, x.t.y, x.t.z, x.t.w}, le[4] = {x.le.x, x.le.y, x.le.z, x.le.w};
@@ -410,7 +484,8 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
   reinterpret_cast<float4*>(st.score)[v] = sc;
   // touch counts of FREE entries are always zero (events on them are refused)
   if (x.t.x | x.t.y | x.t.z | x.t.w) {
-    reinterpret_cast<uint4*>(st.touch)[v] = make_uint4(0, 0, 0, 0);
+    if (!PACKED) reinterpret_cast<uint4*>(st.touch)[v] = make_uint4(0, 0, 0, 0);
+    if (hot && max(max(x.t.x, x.t.y), max(x.t.z, x.t.w)) > kTouchHot) *hot = 1u;
     if (x.t.x && x.t.y && x.t.z && x.t.w) {   // a block that reported all its heads: one store
       reinterpret_cast<uint4*>(st.last_epoch)[v] = make_uint4(epoch, epoch, epoch, epoch);
     } else {
@@ -422,19 +497,21 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
   }
 }
 
-// The same for one entry (ragged ends).
+// The same for one entry (ragged ends), which has had t touches beside those of the 32-bit count (if that
+// is to be looked at: wide).
 __device__ __forceinline__ void entry_update1(const EntryState& st, uint64_t i, const float* sP, int policy,
-                                              uint32_t epoch, const HeadWeights& hw, float& sc) {
+                                              uint32_t epoch, const HeadWeights& hw, uint32_t t, bool wide,
+                                              uint32_t* hot, float& sc) {
   float e = st.ema[i];
-  const uint32_t t = __ldcg(&st.touch[i]);
+  const uint32_t tw = wide ? __ldcg(&st.touch[i]) : 0u;
+  t += tw;
   const float w = hw.on ? head_weight(hw, i) : 1.0f;
   entry_step(e, st.decay[i], t, st.pair[i], sP, policy, policy == 2 ? st.last_epoch[i] : 0u, epoch, w, sc);
   st.ema[i] = e;
   st.score[i] = sc;
-  if (t) {
-    st.touch[i] = 0;
-    st.last_epoch[i] = epoch;
-  }
+  if (tw) st.touch[i] = 0;
+  if (hot && t > kTouchHot) *hot = 1u;
+  if (t) st.last_epoch[i] = epoch;
 }
 
 }  // namespace kvt

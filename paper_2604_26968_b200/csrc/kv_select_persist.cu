@@ -45,9 +45,12 @@
 // only: 4,096 entries 32.5 -> 13.5 us, 0.9 M 40.3 -> 27.4, 3.1 M 59.9 -> 41.3, 18.8 M
 // 206 -> 180.
 //
-// The same kernel also exists fused with the per-entry scoring pass (FUSED = true):
+// The same kernel also exists fused with the per-entry scoring pass (kScoring, kScoringPacked):
 // every CTA first updates the entries of its own rows (posterior, EMA, score), their
-// inputs streamed through shared-memory stages by asynchronous copies.  The event
+// inputs streamed through shared-memory stages by asynchronous copies.  The touch counts are
+// the packed ones of reduce_events, two bytes an entry (entry phase of 18.8 M entries 97 -> 83 us,
+// the event reduction ahead of it 40 -> 32; a pass 177 -> 152, of 3.1 M entries 41.1 -> 39.3, of
+// 0.9 M even), or, after a trace that overflowed them, the 32-bit ones (kScoring).  The event
 // reduction stays a launch of its own ahead of it: its scattered gathers and atomics ran
 // 2.5x slower inside this kernel when that was tried.
 //
@@ -78,11 +81,15 @@ static_assert((2u * kHalfMax) >> kBracketShiftMax <= kHistBins, "the widest brac
 constexpr uint32_t kNoteKeyBits = 22, kKeptKeyBits = 11;
 static_assert(2u * kHalfMax <= 1u << kNoteKeyBits && kNoteKeyBits + 7 <= 32, "a note holds any key of the bracket");
 static_assert(kBracketShiftMax <= kKeptKeyBits && kPMaxRows <= 64, "a kept note holds any key of a bin, and its row");
-// Fused form: the entry pass's inputs of one row in shared memory -- ema, decay, touch and,
-// for the LRU policy, last_epoch (4,096 words each), pair bytes (1,024 words)
-constexpr uint32_t kStageWords = 3u * kPChunk + kPThreads;
-constexpr uint32_t kStageWordsLru = kStageWords + kPChunk;
+// Fused form: the entry pass's inputs of one row in shared memory -- ema, decay and, for the LRU
+// policy, last_epoch (4,096 words each), pair bytes (1,024 words), touch counts (4,096 words, or 2,048 packed)
+enum Fusion { kNoScoring, kScoring, kScoringPacked };
+__host__ __device__ constexpr uint32_t stage_words(Fusion f, bool lru) {
+  return 2u * kPChunk + kPThreads + (f == kScoringPacked ? 2u * kPThreads : kPChunk) + (lru ? kPChunk : 0u);
+}
 constexpr uint64_t kPAlone = 2 * kPChunk;
+constexpr uint64_t kPackedMaxEvents = 1ull << 27;       // (reduce_events: no overflow goes unseen)
+constexpr unsigned long long kOverflowed = 1ull << 48;  // in SelectTurn::below
 constexpr uint32_t kStages = 2;                         // rows in flight ahead of the one being finished
 constexpr uint32_t kNoteCapMin = 128;                   // notes a warp keeps in shared memory, at least (the rest spills)
 
@@ -113,6 +120,9 @@ struct PArgs {
   Predictor pd;
   HeadWeights hw;
   uint32_t epoch;
+  const uint32_t* ev_entry;   // the trace that the packed touch counts hold
+  unsigned long long n_events;
+  uint32_t* h_hot;
 };
 
 // The two halves of the bounded grid-wide barrier; work put between them overlaps the wait.
@@ -152,6 +162,12 @@ __device__ __forceinline__ uint32_t await_word(const unsigned long long* p, uint
   }
   ok = false;
   return 0;
+}
+
+// What a CTA adds to SelectTurn::below: its keys below the bracket, bit 31 of them kOverflowed.
+template <bool PACKED>
+__device__ __forceinline__ unsigned long long below_word(uint32_t s_below) {
+  return PACKED ? (s_below & 0x7FFFFFFFu) | (s_below >> 31 ? kOverflowed : 0ull) : s_below;
 }
 
 // Finds the bin of a histogram (nbins <= 2048, a power of two) that contains rank k_rem (1-based):
@@ -268,9 +284,12 @@ __device__ __forceinline__ uint32_t block_scores4(const PArgs& a, unsigned long 
 
 // PLAIN (fused form only): the policy is the Bayesian product and no partition is weighted.
 // SHARED: on scratch that calls share which know nothing of each other.
-template <bool FUSED, bool PLAIN, bool BLOCKS, bool SHARED>
+template <Fusion FUSION, bool PLAIN, bool BLOCKS, bool SHARED>
 __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const PArgs a) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
+  constexpr bool FUSED = FUSION != kNoScoring, PACKED = FUSION == kScoringPacked;
+  // offsets in a stage
+  constexpr uint32_t kAtPair = 2u * kPChunk, kAtTouch = kAtPair + kPThreads, kAtLast = stage_words(FUSION, false);
   const uint32_t n_words = a.n_rows * 128u;           // bitmap words: 128 per row
   // Bitmaps "below tau" and "equal to tau".  While they are filled, word 4*(row*32 + warp) + q
   // holds position q of the 32 lanes' vectors (a ballot); before they are counted they are
@@ -327,13 +346,16 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       if (r < n_rows && i0 + 4u <= row_end(r)) {
         uint32_t* dst = s_stage + (r % kStages) * a.stage_words;
         const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(dst + 4u * t);
-        const uint32_t d1 = (uint32_t)__cvta_generic_to_shared(dst + 3u * kPChunk + t);
+        const uint32_t d1 = (uint32_t)__cvta_generic_to_shared(dst + kAtPair + t);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0), "l"(a.st.ema + i0) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kPChunk), "l"(a.st.decay + i0) : "memory");
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 8u * kPChunk), "l"(a.st.touch + i0) : "memory");
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d1), "l"(a.st.pair + i0) : "memory");
+        if constexpr (PACKED)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d1 + 4u * kPThreads + 4u * t), "l"(a.st.packed + i0 / 4u) : "memory");
+        else
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kAtTouch), "l"(a.st.touch + i0) : "memory");
         if (!PLAIN && a.pd.policy == 2) {
-          const uint32_t d2 = (uint32_t)__cvta_generic_to_shared(dst + kStageWords + 4u * t);
+          const uint32_t d2 = (uint32_t)__cvta_generic_to_shared(dst + kAtLast + 4u * t);
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d2), "l"(a.st.last_epoch + i0) : "memory");
         }
       }
@@ -341,8 +363,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   if constexpr (FUSED) {
-    issue(0);
-    issue(1);
+#pragma unroll
+    for (uint32_t r = 0; r < kStages; ++r) issue(r);
   }
   // Shared scratch: the first CTAs clear the counters, each says so in its word, with a number higher
   // than any a call has ever used there, and none adds to a counter before all have said so.  (The
@@ -356,6 +378,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const uint32_t hint_valid = a.sel->hint_valid, hint_tau = a.sel->hint_tau;
   const unsigned long long hint_n = a.sel->hint_n;
   uint32_t half = a.sel->hint_half;   // (the bracket's width follows how well the hints have been doing)
+  const bool touch_used = PACKED && __ldcg(&a.sel->touch_used) != 0u;
   const bool hint = !SHARED && (a.spill != nullptr) & (hint_valid != 0u) & (hint_n == a.n);
   if constexpr (FUSED) {
     // reuse estimates from the totals plus this epoch's counts (final: the event
@@ -382,6 +405,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const float neg_inf = __int_as_float(0xFF800000);
   const float lo_f = hint ? key_score(base0) : neg_inf, hi_f = hint ? key_score(base0 + 2u * half) : neg_inf;
   __syncthreads();
+  // where to note counts too large for the packed ones (nullptr: the 32-bit counts hold nothing)
+  uint32_t* hot = FUSED && (!PACKED || touch_used) ? &a.sel->touch_hot : nullptr;
   constexpr uint32_t kClearing = (sizeof(SelectTurn) / 4u + kPThreads - 1u) / kPThreads;   // CTAs that clear something
   static_assert(kClearing <= kSharedCtas, "each of them has a word");
   if (SHARED && g < kClearing && t == 0)
@@ -401,6 +426,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   // ---- phase A ----
   uint32_t n_noted = 0;     // notes of this warp
   uint32_t n_below = 0;     // keys of this thread below the bracket
+  bool overflowed = false;  // PACKED: a count of this thread's has
   uint32_t* const my_nstart = s_nstart + warp * (n_rows + 1u);
   uint32_t* const my_note = s_note + warp * a.note_cap;
   uint32_t* const my_spill = a.spill + (unsigned long long)(g * kPWarps + warp) * a.spill_stride;
@@ -455,7 +481,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   if constexpr (FUSED) {
     const int policy = PLAIN ? 0 : a.pd.policy;
     for (uint32_t r = 0; r < n_rows; ++r) {
-      asm volatile("cp.async.wait_group 1;" ::: "memory");   // kStages - 1 newer groups may be pending
+      asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1u) : "memory");   // (that many newer groups may be pending)
       const uint32_t i0 = row_base(r) + 4u * t, i1 = row_end(r);
       float s[4] = {inf, inf, inf, inf};
       if (i0 + 4u <= i1) {
@@ -463,19 +489,32 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         EntryVec cur;
         cur.e = *reinterpret_cast<const float4*>(src + 4u * t);
         cur.d = *reinterpret_cast<const float4*>(src + kPChunk + 4u * t);
-        cur.t = *reinterpret_cast<const uint4*>(src + 2u * kPChunk + 4u * t);
-        cur.pr4 = src[3u * kPChunk + t];
+        cur.pr4 = src[kAtPair + t];
+        uint2 packed = make_uint2(0, 0);
+        if constexpr (PACKED) packed = *reinterpret_cast<const uint2*>(src + kAtTouch + 2u * t);
+        else cur.t = *reinterpret_cast<const uint4*>(src + kAtTouch + 4u * t);
         cur.le = make_uint4(0, 0, 0, 0);
-        if (!PLAIN && policy == 2) cur.le = *reinterpret_cast<const uint4*>(src + kStageWords + 4u * t);
+        if (!PLAIN && policy == 2) cur.le = *reinterpret_cast<const uint4*>(src + kAtLast + 4u * t);
         issue(r + kStages);
-        float4 sc;
-        entry_finish4<PLAIN>(a.st, i0 / 4, cur, sP, policy, a.epoch, a.hw, sc);
-        s[0] = sc.x; s[1] = sc.y; s[2] = sc.z; s[3] = sc.w;
+        if (PACKED && !take_touches(a.st, i0 / 4, packed, hot, cur.t)) {
+          overflowed = true;   // (these entries are left as they are until the trace has been counted again)
+        } else {
+          float4 sc;
+          entry_finish4<PACKED, PLAIN>(a.st, i0 / 4, cur, sP, policy, a.epoch, a.hw, hot, sc);
+          s[0] = sc.x; s[1] = sc.y; s[2] = sc.z; s[3] = sc.w;
+        }
       } else {
         issue(r + kStages);
+        if (i0 < i1) {   // the pool's ragged end
+          uint32_t c[4] = {0, 0, 0, 0};
+          if (PACKED && !unpack_touches(__ldcg(reinterpret_cast<const uint2*>(a.st.packed) + i0 / 4u), c)) {
+            overflowed = true;
+          } else {
+            if constexpr (PACKED) a.st.packed[i0 / 4u] = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {   // the pool's ragged end
-          if (i0 + j < i1) entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, s[j]);
+            for (int j = 0; j < 4; ++j)
+              if (i0 + j < i1) entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, c[j], hot != nullptr, hot, s[j]);
+          }
         }
       }
       if (r + 2u == n_rows || n_rows == 1u) warm_lines();
@@ -529,19 +568,19 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     else a.sel->serial = tag == 0xFFFFFFFFu ? 1u : tag;
   };
   uint32_t nbar = 0;        // grid barriers passed
-  bool ok = true, hint_hit = false;
+  bool ok = true, hint_hit = false, recounted = false;
+  unsigned long long below = 0;   // keys below the bracket, of all CTAs
   if (FUSED || hint) {
     n_below = __reduce_add_sync(0xFFFFFFFFu, n_below);
     if (lane == 0) {
       my_nstart[n_rows] = n_noted;
       if (n_below) atomicAdd(&s_below, n_below);
     }
+    if (PACKED && overflowed) atomicOr(&s_below, 1u << 31);   // (a CTA has fewer entries than that)
     __syncthreads();
     if (!alone) {
-      if (hint) {
-        add_pair(turn->hist[0] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
-        if (t == 0 && s_below) atomicAdd(&turn->below, (unsigned long long)s_below);
-      }
+      if (hint) add_pair(turn->hist[0] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
+      if ((PACKED || hint) && t == 0 && s_below) atomicAdd(&turn->below, below_word<PACKED>(s_below));
       grid_arrive(bar);
       for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
       ok = grid_wait(bar, ++nbar * G);
@@ -549,7 +588,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     stamp(2);
     if (!ok) goto fail;
   }
-
   {
     // ---- phase B: narrow [base, base + 2^shift) around rank k, one histogram per exchange ----
     // Every CTA reads the same global data, so all of them take the same path.
@@ -571,8 +609,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     };
     uint32_t bin_k = 0;
     if (hint) {
-      const unsigned long long below = alone ? s_below : __ldcg(&turn->below);
-      const bool above = a.k > below;
+      below = alone ? below_word<PACKED>(s_below) : __ldcg(&turn->below);   // (in flight together with the histogram)
+      const bool above = a.k > below;   // (false beside kOverflowed)
       pick_bin(turn->hist[0], alone, s_hist, kHistBins, above ? a.k - below : 1ull, s_warp, s_pick, bin, before);
       hint_hit = above && bin != 0xFFFFFFFFu;
       if (hint_hit) {
@@ -580,6 +618,42 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         bin_k = bin;
       }
       if (g == 0 && t == 0) atomicAdd(hint_hit ? &a.sel->n_hint_hit : &a.sel->n_hint_miss, 1u);
+    }
+    if constexpr (PACKED) {
+      // A packed count overflowed somewhere: the trace is counted again, in the 32-bit array, the entries
+      // beside such a count get their scoring step, and the selection starts from the scores.  (Traces like
+      // that are counted in the 32-bit array from the start as soon as the host has heard of it.)
+      if (!hint) below = alone ? below_word<PACKED>(s_below) : __ldcg(&turn->below);
+      recounted = below >= kOverflowed;
+      if (recounted) {
+        hint_hit = false;
+        hot = &a.sel->touch_hot;
+        for (unsigned long long e = g * kPThreads + t; e < a.n_events; e += G * kPThreads) {
+          const uint32_t i = a.ev_entry[e];
+          if (i < n && !(a.st.pair[i] & kPairFree)) atomicAdd(a.st.touch + i, 1u);
+        }
+        for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
+        if (alone) {
+          __syncthreads();
+        } else {
+          grid_arrive(bar);
+          ok = grid_wait(bar, ++nbar * G);
+          if (!ok) goto fail;
+        }
+        for (uint32_t r = 0; r < n_rows; ++r) {
+          const uint32_t i0 = row_base(r) + 4u * t, i1 = row_end(r), v = i0 / 4u;
+          if (i0 >= i1) continue;
+          uint32_t unused[4];
+          const bool done = unpack_touches(__ldcg(reinterpret_cast<const uint2*>(a.st.packed) + v), unused);
+          if (!done) a.st.packed[v] = 0;
+#pragma unroll 1
+          for (uint32_t i = i0; i < i1 && i < i0 + 4u; ++i) {
+            float s;
+            if (done) a.st.touch[i] = 0;
+            else entry_update1(a.st, i, sP, PLAIN ? 0 : a.pd.policy, a.epoch, a.hw, 0u, true, hot, s);
+          }
+        }
+      }
     }
     // keys of the thread's vector of row r, from the arrays; entries past the row's end or not
     // RESIDENT give kKeyExcluded
@@ -755,7 +829,16 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     if constexpr (FUSED) {
       // every CTA has long formed its estimates: the epoch's counts can be folded in (here, where
       // the CTA waits for the others anyway)
-      if (g == 0 && t >= kPThreads - 32u && lane < 16u) commit_predictor(a.pd, lane, s_pair[lane]);
+      if (g == 0 && t >= kPThreads - 32u && lane < 16u) {
+        commit_predictor(a.pd, lane, s_pair[lane]);
+        if (lane == 0u) {
+          a.sel->touch_used = 0;   // (the 32-bit counts have been cleared)
+          if (hot) {
+            if (a.h_hot) *a.h_hot = __ldcg(hot);
+            *hot = 0;
+          }
+        }
+      }
     }
     if (!alone) ok = grid_wait(bar, ++nbar * G);
     stamp(6);
@@ -948,8 +1031,8 @@ PersistDevice g_persist[kPMaxDevices];
 
 // Dynamic shared memory of a launch: two bitmaps, where the warps' notes of each row begin, the
 // notes, and the entry pass's stages.
-inline size_t persist_smem(uint32_t n_rows, uint32_t note_cap, uint32_t stage_words) {
-  return 4u * ((size_t)n_rows * 256u + (n_rows + 1u) * 32u + (size_t)note_cap * kPWarps + (size_t)kStages * stage_words);
+inline size_t persist_smem(uint32_t n_rows, uint32_t note_cap, uint32_t stages_words) {
+  return 4u * ((size_t)n_rows * 256u + (n_rows + 1u) * 32u + (size_t)note_cap * kPWarps + (size_t)stages_words);
 }
 }  // namespace
 
@@ -973,9 +1056,10 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
       cudaDeviceGetAttribute(&d.n_sm, cudaDevAttrMultiProcessorCount, dev);
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      void* fns[5] = {(void*)select_persistent_kernel<false, false, false, false>, (void*)select_persistent_kernel<true, false, false, false>,
-                      (void*)select_persistent_kernel<true, true, false, false>, (void*)select_persistent_kernel<false, false, true, false>,
-                      (void*)select_persistent_kernel<false, false, false, true>};
+      void* fns[7] = {(void*)select_persistent_kernel<kNoScoring, false, false, false>, (void*)select_persistent_kernel<kNoScoring, false, true, false>,
+                      (void*)select_persistent_kernel<kNoScoring, false, false, true>, (void*)select_persistent_kernel<kScoring, false, false, false>,
+                      (void*)select_persistent_kernel<kScoring, true, false, false>, (void*)select_persistent_kernel<kScoringPacked, false, false, false>,
+                      (void*)select_persistent_kernel<kScoringPacked, true, false, false>};
       cudaError_t e = cudaSuccess;
       size_t fixed = 0;
       for (void* fn : fns) {
@@ -985,7 +1069,7 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
       }
       // the most a launch may ask for: everything a block can opt in to beyond the kernels' static share
       const size_t want = (size_t)optin > fixed ? ((size_t)optin - fixed) / 1024 * 1024 : 0;
-      if (want < persist_smem(kPMaxRows, kNoteCapMin, kStageWords)) e = cudaErrorInvalidValue;
+      if (want < persist_smem(kPMaxRows, kNoteCapMin, kStages * stage_words(kScoring, false))) e = cudaErrorInvalidValue;
       d.smem_max = want;
       for (void* fn : fns) {
         int b = 0;
@@ -1023,17 +1107,20 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   a.table = ws.table;
   a.words = ws.shared_words;
   a.status = ws.status;
-  a.stage_words = fs ? (fs->opt.policy == 2 ? kStageWordsLru : kStageWords) : 0u;
+  const Fusion fusion = !fs ? kNoScoring : fs->n_events < kPackedMaxEvents && *fs->hot == 0u ? kScoringPacked : kScoring;
+  const bool lru = fs && fs->opt.policy == 2;
+  a.stage_words = fs ? stage_words(fusion, lru) : 0u;
+  const uint32_t stages_words = kStages * a.stage_words;
   // Notes: the bracket typically holds 4-15 % of a warp's keys, in some traces several times
   // that.  A quarter of them stays in shared memory (what does not fit goes to the global scratch);
   // the form without the entry pass takes room for every key, which the plain path fills.
   uint32_t cap = fs ? a.n_rows * 32u : a.n_rows * 128u;
   if (cap < kNoteCapMin) cap = kNoteCapMin;
-  while (cap > kNoteCapMin && persist_smem(a.n_rows, cap, a.stage_words) > pd.smem_max) cap -= 4;
-  const size_t smem = persist_smem(a.n_rows, cap, a.stage_words);
+  while (cap > kNoteCapMin && persist_smem(a.n_rows, cap, stages_words) > pd.smem_max) cap -= 4;
+  const size_t smem = persist_smem(a.n_rows, cap, stages_words);
   if (smem > pd.smem_max) return cudaSuccess;
   a.note_cap = cap;
-  a.scratch_words = cap * kPWarps + kStages * a.stage_words;
+  a.scratch_words = cap * kPWarps + stages_words;
   a.pc = pc ? *pc : PartCounts{};
   // (scratch of promotions and admissions: idle while a selection runs.  It has N + 4,096 words;
   // n_rows * 4,096 * G is at most N + 4,096 * G, and every warp keeps at least 128 notes itself)
@@ -1044,22 +1131,39 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   a.st = st;
   a.pd = Predictor{};
   a.hw = HeadWeights{};
+  const Workspace lws = fusion == kScoringPacked ? ws.for_packed() : ws;
   a.epoch = 0;
+  a.ev_entry = nullptr;
+  a.n_events = 0;
+  a.h_hot = nullptr;
   if (fs) {
     a.pd = Predictor{fs->hits,       fs->misses,    fs->P,          fs->alpha0, fs->beta0, ws.delta, nullptr,
                      fs->opt.policy, fs->opt.kappa, fs->opt.window, ws.blend};
     a.hw = fs->hw;
     a.epoch = fs->epoch;
+    EntryState ev = st;
+    if (fusion != kScoringPacked) ev.packed = nullptr;
+    const cudaError_t e = launch_event_reduce(fs->ev_entry, fs->ev_hit, fs->n_events, ev, lws, s);
+    if (e != cudaSuccess) return e;
+    a.ev_entry = fs->ev_entry;
+    a.n_events = fs->n_events;
+    a.h_hot = fs->hot_dev;
   }
   void* args[] = {&a};
   const bool plain = fs && fs->opt.policy == 0 && fs->hw.on == 0;
-  void* fn = bg ? (void*)select_persistent_kernel<false, false, true, false>
-             : ws.shared_words ? (void*)select_persistent_kernel<false, false, false, true>
-             : !fs ? (void*)select_persistent_kernel<false, false, false, false>
-                   : plain ? (void*)select_persistent_kernel<true, true, false, false>
-                           : (void*)select_persistent_kernel<true, false, false, false>;
-  cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, G > 1, ws);
-  if (e != cudaSuccess) return e;
+  void* fn = bg ? (void*)select_persistent_kernel<kNoScoring, false, true, false>
+             : ws.shared_words ? (void*)select_persistent_kernel<kNoScoring, false, false, true>
+             : fusion == kNoScoring ? (void*)select_persistent_kernel<kNoScoring, false, false, false>
+             : fusion == kScoring ? (plain ? (void*)select_persistent_kernel<kScoring, true, false, false>
+                                           : (void*)select_persistent_kernel<kScoring, false, false, false>)
+                                  : (plain ? (void*)select_persistent_kernel<kScoringPacked, true, false, false>
+                                           : (void*)select_persistent_kernel<kScoringPacked, false, false, false>);
+  cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, G > 1, lws);
+  if (e != cudaSuccess) {
+    if (fusion == kScoringPacked)   // (nobody takes the packed counts up)
+      (void)cudaMemsetAsync(st.packed, 0, (st.n + 3) / 4 * 8, s);
+    return e;
+  }
   count_launches(1);
   *used = true;
   return cudaSuccess;

@@ -130,6 +130,9 @@ struct kv_pool {
   HeadWeights head{};       // head-granular importance matrices and weights
   uint32_t n_head_imp = 0, n_head_w = 0;
   PrefetchState prefetch{}; // per-layer prefetch windows
+  unsigned long long* packed = nullptr;   // EntryState::packed of the fused scoring pass
+  volatile uint32_t* h_hot = nullptr;  // FusedScore::hot
+  uint32_t* hot_dev = nullptr;
   // a demotion whose later chunks are not enqueued yet (deferred packing)
   struct Pending {
     bool active = false, meta_done = false;
@@ -158,10 +161,10 @@ constexpr uint32_t kPrefetchWindowCap = 65535;      // default cap on a window, 
 struct Layout {
   uint64_t head_imp, head_mult, head_w;
   uint64_t pf_span, pf_win, pf_counts;
-  uint64_t delta, hist, sel, status, blend, block_score, block_state, block_victims, part_counts, tile_counts, tile_offsets, turns, table, free_list, slot_list[kListBufs];
+  uint64_t delta, hist, sel, status, blend, block_score, block_state, block_victims, part_counts, tile_counts, tile_offsets, turns, table, packed, free_list, slot_list[kListBufs];
   uint64_t ring[4][6];
   uint64_t dev_total;
-  uint64_t h_list[kListBufs], h_counts, h_status, h_sel_stats, host_total;
+  uint64_t h_list[kListBufs], h_counts, h_status, h_sel_stats, h_hot, host_total;
   uint32_t n_tiles;
   uint64_t table_words;
 };
@@ -255,6 +258,7 @@ void make_layout(const kv_pool_desc* d, const Derived& g, Layout* L) {
     L->ring[q][4] = take(R);
     L->ring[q][5] = take(R * 4);
   }
+  L->packed = take((g.N + 3) / 4 * 8);
   L->dev_total = o;
   uint64_t h = 0;
   auto htake = [&h](uint64_t bytes) { uint64_t at = h; h = align_up(h + bytes, kAlign); return at; };
@@ -262,6 +266,7 @@ void make_layout(const kv_pool_desc* d, const Derived& g, Layout* L) {
   L->h_counts = htake(4 * 8);
   L->h_status = htake(4);
   L->h_sel_stats = htake(16);
+  L->h_hot = htake(4);
   L->host_total = h;
 }
 
@@ -593,6 +598,7 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
   p->ws.part_counts = reinterpret_cast<unsigned long long*>(w + L.part_counts);
   p->ws.tile_counts = reinterpret_cast<uint2*>(w + L.tile_counts);
   p->ws.tile_offsets = reinterpret_cast<uint2*>(w + L.tile_offsets);
+  p->packed = reinterpret_cast<unsigned long long*>(w + L.packed);
   p->ws.free_list = reinterpret_cast<uint32_t*>(w + L.free_list);
   for (int b = 0; b < kListBufs; ++b) p->ws.slot_list[b] = reinterpret_cast<uint32_t*>(w + L.slot_list[b]);
   p->ws.n_tiles = L.n_tiles;
@@ -614,6 +620,14 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
     for (int q = 0; q < 4; ++q) p->h_counts[q] = 0;
   }
   p->h_sel_stats = reinterpret_cast<uint32_t*>(hw + L.h_sel_stats);
+  {
+    uint32_t* const hot = reinterpret_cast<uint32_t*>(hw + L.h_hot);
+    *hot = 0;
+    p->h_hot = hot;
+    void* dp = nullptr;
+    if (cudaHostGetDevicePointer(&dp, hot, 0) == cudaSuccess) p->hot_dev = static_cast<uint32_t*>(dp);
+    else (void)cudaGetLastError();
+  }
   p->st = EntryState{desc->d_ema, desc->d_decay, desc->d_touch, desc->d_last_epoch, desc->d_pair,
                      desc->d_state, desc->d_tag, desc->d_score, g.N};
 
@@ -732,6 +746,7 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
                     p->geom, p->n_parts, p->ws, S(stream));
     if (e == cudaSuccess) e = launch_head_init(p->head, p->n_head_imp, p->n_head_w, S(stream));
     if (e == cudaSuccess) e = cudaMemsetAsync(p->prefetch.words, 0, kPrefetchChunks * 8 + 8, S(stream));
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->packed, 0, (g.N + 3) / 4 * 8, S(stream));
     for (int q = 0; q < g.n_parts && e == cudaSuccess; ++q)
       e = launch_prefetch_window(p->prefetch, q, 1, nullptr, 0.0f, kPrefetchSpanTokens, p->ws, S(stream));
   }
@@ -875,20 +890,22 @@ int32_t kv_epoch_score_select(kv_pool* p, uint32_t epoch, const uint32_t* d_ev_e
     return KV_ERR_INVALID_ARG;
   if (k > p->stats.n_entries - p->stats.n_free) return KV_ERR_K_TOO_LARGE;
   if (k > 0 && (!d_victims || !aligned16(d_victims))) return KV_ERR_INVALID_ARG;
-  KV_CUDA(p, launch_event_reduce(d_ev_entry, d_ev_hit, n_events, p->st, p->ws, S(stream)));
-  p->stats.events += n_events;
   bool used = false;
   if (k > 0 && p->select_variant != 0) {
     const FusedScore fs{p->desc.d_hits, p->desc.d_misses, p->desc.d_P, p->desc.alpha0,
-                        p->desc.beta0,  epoch,            p->score_opt,  p->head};
+                        p->desc.beta0,  epoch,            p->score_opt,  p->head,
+                        d_ev_entry,     d_ev_hit,         n_events,   p->h_hot,        p->hot_dev};
     forget_free_lists(p);
-    KV_CUDA(p, launch_select_persistent(p->st, k, d_victims, p->ws, S(stream), &used, &fs, &p->pc));
+    EntryState st = p->st;
+    st.packed = p->packed;
+    KV_CUDA(p, launch_select_persistent(st, k, d_victims, p->ws, S(stream), &used, &fs, &p->pc));
   }
   if (used) {
+    p->stats.events += n_events;
     scoring_pass_enqueued(p, epoch);
     return counts_to_host(p, S(stream));
   }
-  const int32_t rc = kv_epoch_update(p, epoch, stream);
+  const int32_t rc = kv_epoch_score(p, epoch, d_ev_entry, d_ev_hit, n_events, stream);
   if (rc != KV_OK || k == 0) return rc;
   return kv_select_victims(p, k, d_victims, stream);
 }
@@ -1347,6 +1364,7 @@ int32_t kv_set_l2_residency(kv_pool* p, uint64_t budget_bytes) {
       p->ws.l2_base = nullptr;
       p->ws.l2_bytes = 0;
       p->ws.l2_ratio = 0.0f;
+      p->ws.l2_packed = nullptr;
       KV_CUDA(p, cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, 0));
     }
     return KV_OK;
@@ -1364,7 +1382,12 @@ int32_t kv_set_l2_residency(kv_pool* p, uint64_t budget_bytes) {
     bytes = pair_bytes < (uint64_t)max_window ? pair_bytes : (uint64_t)max_window;
     set_aside = bytes < budget ? bytes : budget;
   }
+  const uint64_t packed_bytes = (p->st.n + 3) / 4 * 8;
+  const bool packed_fits = packed_bytes <= budget && packed_bytes <= (uint64_t)max_window;   // the packed counts, whole
+  if (packed_fits && set_aside < packed_bytes) set_aside = packed_bytes;
   KV_CUDA(p, cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, (size_t)set_aside));
+  p->ws.l2_packed = packed_fits ? p->packed : nullptr;
+  p->ws.l2_packed_bytes = packed_fits ? (size_t)packed_bytes : 0;
   p->ws.l2_base = base;
   p->ws.l2_bytes = (size_t)bytes;
   p->ws.l2_ratio = set_aside >= bytes ? 1.0f : (float)((double)set_aside / (double)bytes);

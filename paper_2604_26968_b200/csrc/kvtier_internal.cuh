@@ -79,6 +79,9 @@ struct EntryState {
   uint32_t* tag;
   float* score;
   uint64_t n;
+  // Touches that only the fused scoring pass of the same call reads, a word for four entries, zero
+  // between calls (nullptr: touches are counted in `touch`).  See reduce_events in kv_score_device.cuh.
+  unsigned long long* packed = nullptr;
 };
 
 // Small block of device scalars used by selection and compaction.
@@ -106,6 +109,8 @@ struct SelectScalars {
   // slowly decaying maximum of how far tau landed from where the hint put it
   uint32_t hint_half;
   uint32_t hint_resid;
+  uint32_t touch_used;         // `touch` holds something (else it is all zero and need not be read)
+  uint32_t touch_hot;          // ... an entry with more touches than the packed counts are tried again with
 };
 
 // What the CTAs of one persistent selection share while it runs.  A pool has two of these, used in
@@ -113,7 +118,7 @@ struct SelectScalars {
 struct SelectTurn {
   unsigned int bar;             // arrivals at the grid barrier
   unsigned int pad;
-  unsigned long long below;     // keys below the bracket
+  unsigned long long below;     // keys below the bracket (and kOverflowed for CTAs that met an overflowed count)
   uint32_t hist[4][kHistBins];  // the bracket's bins, then its last bin's keys or the radix select's digits
 };
 
@@ -209,6 +214,14 @@ struct Workspace {
   const void* l2_base = nullptr;
   size_t l2_bytes = 0;
   float l2_ratio = 0.0f;
+  // ... or this one, for the launches that count touches in EntryState::packed
+  const void* l2_packed = nullptr;
+  size_t l2_packed_bytes = 0;
+  Workspace for_packed() const {
+    Workspace w = *this;
+    if (l2_packed) { w.l2_base = l2_packed; w.l2_bytes = l2_packed_bytes; w.l2_ratio = 1.0f; }
+    return w;
+  }
 };
 
 // Launches fn (kernel taking the arguments in args) with the workspace's L2 window, if it has
@@ -281,6 +294,7 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, u
 }
 
 // ---- kv_score.cu ----
+// With st.packed the touches go there, for the fused scoring pass.
 cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events,
                                 const EntryState& st, const Workspace& ws, cudaStream_t s);
 // posterior (from hits/misses plus the epoch counters in ws.delta) + EMA + score in one launch;
@@ -344,8 +358,8 @@ cudaError_t launch_select(const EntryState& st, uint64_t k, uint32_t* d_victims,
                           cudaStream_t s, int variant = 1, const PartCounts* pc = nullptr);
 // kv_select_persist.cu: the same selection as one cooperative launch; *used tells
 // whether it was launched (false: the device cannot co-schedule it, nothing was enqueued)
-// With fs the launch also does the entry pass first (posterior, EMA, score; the
-// epoch's events have been reduced by an earlier launch).
+// With fs a launch of the event reduction goes ahead (touches into st.packed), and the launch also
+// does the entry pass first (posterior, EMA, score).
 struct FusedScore {
   uint64_t* hits;
   uint64_t* misses;
@@ -354,6 +368,11 @@ struct FusedScore {
   uint32_t epoch;
   ScoreOptions opt;
   HeadWeights hw;
+  const uint32_t* ev_entry;      // the epoch's trace, whose reduction is launched ahead
+  const uint8_t* ev_hit;
+  uint64_t n_events;
+  const volatile uint32_t* hot;  // host word: not 0 while the packed counts do not hold every entry's touches ...
+  uint32_t* hot_dev;             // ... where the device can write it (nullptr: it cannot)
 };
 cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t* d_victims,
                                      const Workspace& ws, cudaStream_t s, bool* used,
