@@ -171,39 +171,32 @@ __device__ __forceinline__ unsigned long long below_word(uint32_t s_below) {
 }
 
 // Finds the bin of a histogram (nbins <= 2048, a power of two) that contains rank k_rem (1-based):
-// (bin, ranks before the bin) to every thread; bin is 0xFFFFFFFF when k_rem exceeds the
-// histogram's total.  With local the histogram is the block's own s_hist, which is complete (a
-// block barrier lies behind the last addition) and is cleared.  A block barrier must lie between
-// two calls.
-__device__ __forceinline__ void pick_bin(const uint32_t* hist, bool local, uint32_t* s_hist, uint32_t nbins,
-                                         unsigned long long k_rem, uint32_t* s_warp, uint32_t* s_pick,
-                                         uint32_t& bin, uint32_t& before_bin) {
+// (bin, ranks before the bin, ranks in it) to every thread; bin is 0xFFFFFFFF
+// when k_rem exceeds the histogram's total.  s_hist, the block's own histogram, is complete (a block
+// barrier lies behind the last addition) and is cleared; with local it is the one that is looked at.  A
+// block barrier must lie between two calls.
+struct Pick { uint32_t bin, before, count; };
+__device__ __forceinline__ Pick pick_bin(const uint32_t* hist, bool local, uint32_t* s_hist, uint32_t nbins,
+                                         uint32_t k_rem, uint32_t* s_warp, uint4* s_pick) {
   const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5;
-  uint2 c = make_uint2(0u, 0u);
-  if (local) {
-    c = reinterpret_cast<const uint2*>(s_hist)[t];   // (bins from nbins on are empty)
-    reinterpret_cast<uint2*>(s_hist)[t] = make_uint2(0u, 0u);
-  } else if (2u * t < nbins) {
-    c = __ldcg(reinterpret_cast<const uint2*>(hist) + t);
-  }
-  const uint32_t v = c.x + c.y;
-  const uint32_t incl = warp_scan_incl(v, lane);
-  if (lane == 31u) s_warp[warp] = incl;
-  if (t == 0) { s_pick[0] = 0xFFFFFFFFu; s_pick[1] = 0; }
+  const uint2 own = reinterpret_cast<const uint2*>(s_hist)[t];   // (bins from nbins on are empty)
+  reinterpret_cast<uint2*>(s_hist)[t] = make_uint2(0u, 0u);
+  uint2 c = own;
+  if (!local) c = 2u * t < nbins ? __ldcg(reinterpret_cast<const uint2*>(hist) + t) : make_uint2(0u, 0u);
+  const uint32_t v = c.x + c.y, all = __reduce_add_sync(0xFFFFFFFFu, v);
+  if (lane == 0u) s_warp[warp] = all;
+  if (t == 0) *s_pick = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
   __syncthreads();
-  const uint32_t w = s_warp[lane];
-  const uint32_t wincl = warp_scan_incl(w, lane);
-  const uint32_t before = __shfl_sync(0xFFFFFFFFu, wincl - w, warp) + incl - v;
-  if (c.x && (unsigned long long)before < k_rem && k_rem <= (unsigned long long)before + c.x) {
-    s_pick[0] = 2u * t; s_pick[1] = before;
-  }
-  const uint32_t before1 = before + c.x;
-  if (c.y && (unsigned long long)before1 < k_rem && k_rem <= (unsigned long long)before1 + c.y) {
-    s_pick[0] = 2u * t + 1u; s_pick[1] = before1;
+  // (one reduction instead of a second scan, and only the warp that holds the rank looks further)
+  const uint32_t ahead = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? s_warp[lane] : 0u);
+  if (ahead < k_rem && k_rem - ahead <= all) {
+    const uint32_t before = ahead + warp_scan_incl(v, lane) - v, before1 = before + c.x;
+    if (before < k_rem && k_rem - before <= c.x) *s_pick = make_uint4(2u * t, before, c.x, 0u);
+    if (before1 < k_rem && k_rem - before1 <= c.y) *s_pick = make_uint4(2u * t + 1u, before1, c.y, 0u);
   }
   __syncthreads();
-  bin = s_pick[0];
-  before_bin = s_pick[1];
+  const uint4 p = *s_pick;
+  return Pick{p.x, p.y, p.z};
 }
 
 // Scores of the four paged blocks b0 .. b0+3 (those below b1): the weighted sum over the block's
@@ -302,7 +295,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   // once phase A is over, notes and stages together are the key cache of the plain path
   __shared__ __align__(16) uint32_t s_hist[kHistBins];
   __shared__ uint32_t s_warp[32];
-  __shared__ uint32_t s_pick[2];
+  __shared__ uint4 s_pick;
   __shared__ uint32_t s_below;
   __shared__ __align__(16) uint32_t s_wtot[kPMaxRows * 4];   // per 32 bitmap words: below | equal << 16
   __shared__ uint2 s_rowtot[kPMaxRows];               // (below, equal) of a row over all CTAs ...
@@ -582,7 +575,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       if (hint) add_pair(turn->hist[0] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
       if ((PACKED || hint) && t == 0 && s_below) atomicAdd(&turn->below, below_word<PACKED>(s_below));
       grid_arrive(bar);
-      for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
       ok = grid_wait(bar, ++nbar * G);
     }
     stamp(2);
@@ -591,8 +583,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   {
     // ---- phase B: narrow [base, base + 2^shift) around rank k, one histogram per exchange ----
     // Every CTA reads the same global data, so all of them take the same path.
-    uint32_t bin = 0, before = 0, tau = 0;
-    unsigned long long k_rem = a.k;
+    uint32_t tau = 0;
+    uint32_t k_rem = (uint32_t)a.k;   // (k is at most n)
     bool found = true;
     // The CTA's histogram joins the others' in histogram h; false if the wait ran out.
     auto exchange_hist = [&](uint32_t h, uint32_t nbins, bool ready = true) {
@@ -604,18 +596,18 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       if (alone) return true;
       if (2u * t < nbins) add_pair(turn->hist[h] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
       grid_arrive(bar);
-      for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
       return grid_wait(bar, ++nbar * G);
     };
+    Pick pick{0u, 0u, 0u};
     uint32_t bin_k = 0;
     if (hint) {
       below = alone ? below_word<PACKED>(s_below) : __ldcg(&turn->below);   // (in flight together with the histogram)
       const bool above = a.k > below;   // (false beside kOverflowed)
-      pick_bin(turn->hist[0], alone, s_hist, kHistBins, above ? a.k - below : 1ull, s_warp, s_pick, bin, before);
-      hint_hit = above && bin != 0xFFFFFFFFu;
+      pick = pick_bin(turn->hist[0], alone, s_hist, kHistBins, above ? (uint32_t)(a.k - below) : 1u, s_warp, &s_pick);
+      hint_hit = above && pick.bin != 0xFFFFFFFFu;
       if (hint_hit) {
-        k_rem = a.k - below - before;
-        bin_k = bin;
+        k_rem = (uint32_t)(a.k - below) - pick.before;
+        bin_k = pick.bin;
       }
       if (g == 0 && t == 0) atomicAdd(hint_hit ? &a.sel->n_hint_hit : &a.sel->n_hint_miss, 1u);
     }
@@ -632,7 +624,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
           const uint32_t i = a.ev_entry[e];
           if (i < n && !(a.st.pair[i] & kPairFree)) atomicAdd(a.st.touch + i, 1u);
         }
-        for (uint32_t b = t; b < kHistBins; b += kPThreads) s_hist[b] = 0;
         if (alone) {
           __syncthreads();
         } else {
@@ -739,10 +730,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       ok = exchange_hist(1, n_bins);
       stamp(3);
       if (!ok) goto fail;
-      pick_bin(turn->hist[1], alone, s_hist, n_bins, k_rem, s_warp, s_pick, bin, before);
-      found = bin != 0xFFFFFFFFu;
-      k_rem -= before;
-      const uint32_t tau_low = found ? bin : 0u;
+      pick = pick_bin(turn->hist[1], alone, s_hist, n_bins, k_rem, s_warp, &s_pick);
+      found = pick.bin != 0xFFFFFFFFu;
+      k_rem -= pick.before;
+      const uint32_t tau_low = found ? pick.bin : 0u;
       tau = base0 + (bin_k << bshift) + tau_low;
       // phase C from the kept notes: those below tau and equal to it set their bits
       for (uint32_t p = lane; p < n_kept; p += 32u) {
@@ -751,10 +742,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         if (low <= tau_low) atomicOr(low < tau_low ? &s_bl[w] : &s_be[w], 1u << (at & 31u));
       }
     } else {
+      uint32_t base = 0;
       // plain radix select: digits of 11, 11 and 10 bits
       uint32_t h = hint ? 1u : 0u;   // (histogram 0 holds the bracket's counts of this launch)
-      uint32_t base = 0;
-      k_rem = a.k;
+      k_rem = (uint32_t)a.k;
 #pragma unroll 1
       for (int digit = 0; digit < 3; ++digit) {
         const uint32_t shift = digit == 0 ? 21u : digit == 1 ? 10u : 0u, top = digit == 2 ? 10u : 11u;
@@ -769,11 +760,11 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         ok = exchange_hist(h, 1u << top, digit != 0 || alone || cleared());
         if (digit == 1) stamp(3);
         if (!ok) goto fail;
-        pick_bin(turn->hist[h], alone, s_hist, 1u << top, k_rem, s_warp, s_pick, bin, before);
+        pick = pick_bin(turn->hist[h], alone, s_hist, 1u << top, k_rem, s_warp, &s_pick);
         ++h;
-        found = found && bin != 0xFFFFFFFFu;
-        k_rem -= before;
-        base += (bin & (kHistBins - 1u)) << shift;
+        found = found && pick.bin != 0xFFFFFFFFu;
+        k_rem -= pick.before;
+        base += (pick.bin & (kHistBins - 1u)) << shift;
       }
       tau = base;
       // phase C from the keys
@@ -782,7 +773,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           wl[q] = __ballot_sync(0xFFFFFFFFu, key[q] < tau && key[q] != kKeyExcluded);
-          we[q] = __ballot_sync(0xFFFFFFFFu, key[q] == tau && key[q] != kKeyExcluded);
+          const bool in = key[q] == tau && key[q] != kKeyExcluded;
+          we[q] = __ballot_sync(0xFFFFFFFFu, in);
         }
         if (lane == 0) {
           *reinterpret_cast<uint4*>(s_bl + 4u * (r * 32u + warp)) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
@@ -791,40 +783,24 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       });
     }
     stamp(10);
-    const unsigned long long need_eq = k_rem;
     __syncthreads();
 
-    // ---- counts: bitmaps into natural order, population counts per 32 words ----
-    // Thread t owns words t, t + 1024, ...: a row's 128 words belong to four neighbouring warps.
-    const uint32_t n_rounds = (n_words + kPThreads - 1u) / kPThreads;
-    for (uint32_t rd = 0; rd < n_rounds; ++rd) {
-      const uint32_t W = rd * kPThreads + t;
-      uint32_t bl = 0, be = 0;
-      if (W < n_words) {   // (n_words is a multiple of 128: the whole warp)
-        const uint4 x = reinterpret_cast<const uint4*>(s_bl)[W >> 2], y = reinterpret_cast<const uint4*>(s_be)[W >> 2];
-        const uint32_t sh = 8u * (W & 3u);
-        bl = interleave4(x.x >> sh, x.y >> sh, x.z >> sh, x.w >> sh);
-        be = (y.x | y.y | y.z | y.w) ? interleave4(y.x >> sh, y.y >> sh, y.z >> sh, y.w >> sh) : 0u;
-        __syncwarp();
-        s_bl[W] = bl;
-        s_be[W] = be;
-        const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(bl) | (uint32_t)__popc(be) << 16);
-        if (lane == 0) s_wtot[rd * kPWarps + warp] = c;
+    // ---- last exchange: the counts of every chunk, (below | equal << 13), row after row ----
+    for (uint32_t r = warp; r < n_rows; r += kPWarps) {
+      const uint4 x = reinterpret_cast<const uint4*>(s_bl)[32u * r + lane], y = reinterpret_cast<const uint4*>(s_be)[32u * r + lane];
+      const uint32_t l = (uint32_t)(__popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w));
+      const uint32_t e = (uint32_t)(__popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w));
+      const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, l | e << 16);   // at most 4,096 in either half
+      if (lane == 0u) {
+        if (alone) {
+          s_rowtot[r] = make_uint2(sum & 0xFFFFu, sum >> 16);
+          s_colpre[r] = make_uint2(0u, 0u);
+        } else {
+          a.table[r * G + g] = (sum & 0xFFFFu) | (sum >> 16) << 13;
+        }
       }
     }
-    __syncthreads();
-    // ---- third exchange: the counts of every chunk, (below | equal << 13), row after row ----
-    if (t < n_rows) {
-      const uint4 v = reinterpret_cast<const uint4*>(s_wtot)[t];
-      const uint32_t sum = v.x + v.y + v.z + v.w;   // at most 4,096 in either half
-      if (alone) {
-        s_rowtot[t] = make_uint2(sum & 0xFFFFu, sum >> 16);
-        s_colpre[t] = make_uint2(0u, 0u);
-      } else {
-        a.table[t * G + g] = (sum & 0xFFFFu) | (sum >> 16) << 13;
-      }
-    }
-    if (!alone) grid_arrive(bar);
+    if (alone) __syncthreads(); else grid_arrive(bar);
     stamp(5);
     if constexpr (FUSED) {
       // every CTA has long formed its estimates: the epoch's counts can be folded in (here, where
@@ -838,6 +814,24 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
             *hot = 0;
           }
         }
+      }
+    }
+    // (while the others arrive: 3.1 M entries 39.3 -> 38.0 us a pass against doing it before) the bitmaps
+    // into natural order, and population counts per 32 words.  Thread t owns words t, t + 1024, ...: a
+    // row's 128 words belong to four neighbouring warps.
+    const uint32_t n_rounds = (n_words + kPThreads - 1u) / kPThreads;
+    for (uint32_t rd = 0; rd < n_rounds; ++rd) {
+      const uint32_t W = rd * kPThreads + t;
+      if (W < n_words) {   // (n_words is a multiple of 128: the whole warp)
+        const uint4 x = reinterpret_cast<const uint4*>(s_bl)[W >> 2], y = reinterpret_cast<const uint4*>(s_be)[W >> 2];
+        const uint32_t sh = 8u * (W & 3u);
+        const uint32_t bl = interleave4(x.x >> sh, x.y >> sh, x.z >> sh, x.w >> sh);
+        const uint32_t be = (y.x | y.y | y.z | y.w) ? interleave4(y.x >> sh, y.y >> sh, y.z >> sh, y.w >> sh) : 0u;
+        __syncwarp();
+        s_bl[W] = bl;
+        s_be[W] = be;
+        const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(bl) | (uint32_t)__popc(be) << 16);
+        if (lane == 0) s_wtot[rd * kPWarps + warp] = c;
       }
     }
     if (!alone) ok = grid_wait(bar, ++nbar * G);
@@ -866,6 +860,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       if (lane == 0) { s_rowtot[r] = make_uint2(tl, te); s_colpre[r] = make_uint2(pl, pe); }
     }
     __syncthreads();
+    const uint32_t need_eq = k_rem;
     // ---- phase D: where this CTA's chunks start, and the ordered write ----
     // Lane r of every warp: what the pool holds before this CTA's chunk of row r (and of row r + 32).
     uint32_t all_l, all_e, rl0, re0, rl1 = 0, re1 = 0;
@@ -887,7 +882,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         all_e += __shfl_sync(0xFFFFFFFFu, j1, 31);
       }
     }
-    const uint32_t eq_room = need_eq > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)need_eq;
+    const uint32_t eq_room = need_eq;
     const unsigned long long got = (unsigned long long)all_l + (all_e < eq_room ? all_e : eq_room);
     // (block form, one partition: the entries of block gb, the pos-th of the selected ones)
     auto write_block = [&](uint32_t pos, uint32_t gb) {
