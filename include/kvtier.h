@@ -482,7 +482,7 @@ int32_t kv_select_victim_blocks(kv_pool* pool, uint64_t k_blocks, uint32_t* d_vi
  * that has given all device memory to its own pools, or code that runs where
  * cudaMalloc is off limits, has no workspace to hand to kv_pool_create.  This
  * call needs none: it takes the score and state arrays directly and keeps its
- * scratch (histograms, scalars, per-tile counts; about 130 KB) in a fixed array
+ * scratch (histograms, scalars, per-tile counts; about 140 KB) in a fixed array
  * inside the library, which every GPU that loads the library holds until the
  * process exits.  It calls no allocating routine.
  *   d_score  (device) f32[n]  eviction scores, as kv_epoch_score writes them

@@ -421,6 +421,7 @@ cudaError_t launch_select_static(const float* score, const uint8_t* state, uint6
   ws.turns = &scratch->turn;
   ws.table = scratch->table;
   ws.table_words = sizeof(scratch->table) / sizeof(scratch->table[0]);
+  ws.list = scratch->list;
   ws.shared_words = scratch->words;
   EntryState st{};
   st.score = const_cast<float*>(score);   // selection only reads score and state

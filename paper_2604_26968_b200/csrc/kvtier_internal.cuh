@@ -117,7 +117,7 @@ struct SelectScalars {
 // turn: a launch finds its own zeroed and clears the next launch's.
 struct SelectTurn {
   unsigned int bar;             // arrivals at the grid barrier
-  unsigned int pad;
+  unsigned int listed;          // keys in the list
   unsigned long long below;     // keys below the bracket (and kOverflowed for CTAs that met an overflowed count)
   uint32_t hist[4][kHistBins];  // the bracket's bins, then its last bin's keys or the radix select's digits
 };
@@ -204,6 +204,7 @@ struct Workspace {
   // persistent selection
   SelectTurn* turns;                // [2], used in turn
   uint32_t* table;                  // [table_words] counts per chunk
+  unsigned long long* list = nullptr;   // shared scratch: [kListMax] the keys of the last bin, and where they are
   uint64_t table_words;
   // Scratch that calls share which know nothing of each other (nullptr: it is the pool's own): the
   // number of the last call, then a word for each CTA that clears (up to kSharedCtas).  Each call
@@ -339,6 +340,9 @@ inline uint64_t select_table_words(uint64_t n) { return n / 4096 + 1024; }
 constexpr uint64_t kStaticMaxEntries = 1ull << 22;  // 4,194,304 entries
 constexpr uint64_t kStaticMaxTiles = kStaticMaxEntries / kTileEntries + 2;
 constexpr uint32_t kSharedCtas = 16;
+// Keys of one bin that the persistent selection on shared scratch puts on a list which every CTA reads,
+// instead of another exchange: at most these.
+constexpr uint32_t kListMax = 1024;
 struct StaticScratch {
   uint32_t hist[3 * kHistBins];
   SelectTurn turn;
@@ -348,6 +352,7 @@ struct StaticScratch {
   uint2 tile_counts[kStaticMaxTiles];
   uint2 tile_offsets[kStaticMaxTiles];
   uint32_t table[kStaticMaxEntries / 4096 + 1024];
+  unsigned long long list[kListMax];
 };
 // n <= kStaticMaxEntries; status may be nullptr
 cudaError_t launch_select_static(const float* score, const uint8_t* state, uint64_t n, uint64_t k, uint32_t* d_victims,
