@@ -105,10 +105,11 @@ struct SelectScalars {
   // persistent selection on a pool of several partitions: launch number | victims before
   // partition boundary q + 1, written by the CTA that holds it
   unsigned long long bound[3];
-  // how far the next selection's bracket reaches to either side of the hint, in keys; hint_resid is a
-  // slowly decaying maximum of how far tau landed from where the hint put it
+  // how far the next selection's bracket reaches to either side of the hint, in keys; slowly decaying
+  // maxima of how far tau landed from the last one and from where the trend of the last two put it
   uint32_t hint_half;
-  uint32_t hint_resid;
+  uint32_t hint_off_last, hint_off_trend;
+  uint32_t hint_trend;         // where the trend puts the next tau
   uint32_t touch_used;         // `touch` holds something (else it is all zero and need not be read)
   uint32_t touch_hot;          // ... an entry with more touches than the packed counts are tried again with
 };
