@@ -977,6 +977,9 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         for (uint32_t h = 0; h < H; ++h) out[h] = first + h;
       }
     };
+    // (the notes are dead: their space holds a warp's ids on their way out)
+    const uint32_t room = a.scratch_words / kPWarps;
+    uint32_t* const ids = s_note + warp * room;
     // With L entries below tau and E entries equal to tau before it in id order, an entry below
     // tau goes to L + min(E, need_eq) and an entry equal to tau, taken while E < need_eq, to L + E.
     for (uint32_t rd = 0; rd < n_rounds; ++rd) {
@@ -1004,13 +1007,29 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       uint32_t bits = (E >= eq_room) ? bl : (bl | be);
       const uint32_t p0 = L + (E < eq_room ? E : eq_room);
       // Where the warp has no entry equal to tau that is taken (nearly everywhere), a victim is a bit
-      // and a place: half the work of the general loop below (18.8 M entries 182.5 -> 181.0 us a
-      // pass, 0.9 M entries 28.7 -> 28.3).
-      if (!BLOCKS && __all_sync(0xFFFFFFFFu, (be == 0u || E >= eq_room) && p0 + (uint32_t)__popc(bits) <= (uint32_t)a.k)) {
-        uint32_t* out = a.victims + p0;
-        while (bits) {
-          *out++ = id0 + (uint32_t)__ffs(bits) - 1u;
-          bits &= bits - 1u;
+      // and a place: half the work of the general loop below.  The warp's ids are neighbours.  Where they
+      // are many they leave together through shared memory (a store of 32 lanes' next ids touches a dozen
+      // sectors, each of them again for the ids that follow: 3.2 M entries of which 15 % leave, three
+      // calls, 55.0 -> 53.7 us); with 10 % and less the detour costs what it saves (18.8 M entries even,
+      // 1.0 M in the radix select 17.0 -> 17.6).
+      const uint32_t p1 = p0 + (uint32_t)__popc(bits);
+      if (!BLOCKS && __all_sync(0xFFFFFFFFu, (be == 0u || E >= eq_room) && p1 <= (uint32_t)a.k)) {
+        const uint32_t from = __shfl_sync(0xFFFFFFFFu, p0, 0), n_ids = __shfl_sync(0xFFFFFFFFu, p1, 31) - from;
+        if (!SHARED && n_ids > 128u && n_ids <= room) {
+          uint32_t* out = ids + (p0 - from);
+          while (bits) {
+            *out++ = id0 + (uint32_t)__ffs(bits) - 1u;
+            bits &= bits - 1u;
+          }
+          __syncwarp();
+          for (uint32_t i = lane; i < n_ids; i += 32u) a.victims[from + i] = ids[i];
+          __syncwarp();
+        } else {
+          uint32_t* out = a.victims + p0;
+          while (bits) {
+            *out++ = id0 + (uint32_t)__ffs(bits) - 1u;
+            bits &= bits - 1u;
+          }
         }
         continue;
       }
