@@ -679,6 +679,8 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
       hd.q_heads[q] = in ? (uint32_t)g.q_heads[q] : 1u;
       hd.layers[q] = in ? (uint32_t)g.layers[q] : 0u;
       hd.per_layer[q] = in ? (uint32_t)(g.n[q] / g.layers[q]) : 1u;
+      hd.by_layer[q] = Divisor(hd.per_layer[q]);
+      hd.by_heads[q] = Divisor(hd.heads[q]);
       hd.imp_off[q] = io;
       hd.w_off[q] = wo;
       if (in) { io += hd.layers[q] * hd.q_heads[q]; wo += hd.layers[q] * hd.heads[q]; }

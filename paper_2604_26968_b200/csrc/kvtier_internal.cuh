@@ -157,6 +157,23 @@ __device__ __forceinline__ int block_partition(const BlockGeom& bg, uint64_t gb)
   return q;
 }
 
+// Division of numbers below 2^31 by d, as a multiplication: with 2^s the power of two from d on and
+// mul = ceil(2^(31+s) / d), the product exceeds x * 2^(31+s) / d by less than x * 2^s / d < 2^(31+s) / d,
+// too little to reach the next quotient (Granlund and Montgomery, "Division by invariant integers using
+// multiplication", 1994).
+struct Divisor {
+  uint32_t mul = 0, shift = 0;   // mul 0: d is 1
+  Divisor() = default;
+  explicit Divisor(uint32_t d) {
+    if (d < 2u) return;
+    uint32_t s = 0;
+    while ((1ull << s) < d) ++s;
+    mul = (uint32_t)(((1ull << (31u + s)) + d - 1u) / d);
+    shift = s - 1u;
+  }
+  __device__ __forceinline__ uint32_t operator()(uint32_t x) const { return mul ? __umulhi(x, mul) >> shift : x; }
+};
+
 // Head-granular importance (head-granular eviction section): per partition a
 // [layer][query head] importance matrix, [layer][KV head] multipliers and the
 // resulting [layer][KV head] score weights, each partition's block at its offset.
@@ -167,6 +184,7 @@ struct HeadWeights {
   uint64_t base[5];        // first global entry id of each partition; [n_parts] = N
   uint32_t per_layer[4];   // entries per layer: blocks per layer x KV heads
   uint32_t heads[4];       // KV heads (1 for MLA)
+  Divisor by_layer[4], by_heads[4];   // the same, to divide by
   uint32_t q_heads[4];     // tracked query heads per layer (1 for MLA)
   uint32_t layers[4];
   uint32_t imp_off[4], w_off[4];
