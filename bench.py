@@ -49,7 +49,7 @@ PACK_KERNEL_NAME = "move_tma_kernel<true> (pack)"
 # at the pool's full entry count with --tiny-entries (these kernels never touch block payload).
 # None = no capture of the kernels as they stand.  (ncu flushes the caches before every kernel it
 # replays: the figures are those of a cold L2, without what kv_set_l2_residency keeps there.)
-NCU_SCORE_SELECT_TRAFFIC = {5: 527.9e6, 3: 424.4e6}
+NCU_SCORE_SELECT_TRAFFIC = {5: 465.0e6, 3: 352.0e6}
 
 
 def parse():

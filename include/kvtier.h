@@ -144,8 +144,9 @@ typedef struct {
   /* per-entry state, struct of arrays of length N in global id order (device) */
   float* d_ema;           /* EMA access score */
   float* d_decay;         /* EMA decay per entry */
-  uint32_t* d_touch;      /* touches that kv_epoch_events has counted and no scoring pass has taken up;
-                             else zero, whatever a pass in progress keeps there.  The library's to write */
+  uint32_t* d_touch;      /* touches that kv_epoch_events has counted and no scoring pass has taken
+                             up yet, else zero (the library's to write: kv_epoch_score_select
+                             counts in the workspace and looks here only for what that call left) */
   uint32_t* d_last_epoch; /* epoch of the last touch */
   uint8_t* d_pair;        /* 4*block_type + transition_type, 0..15; the library sets bit 7
                              while the entry is FREE (the value is then meaningless, but the
@@ -284,7 +285,8 @@ int32_t kv_select_victims(kv_pool* pool, uint64_t k, uint32_t* d_victims, kv_str
  * scores are written once for the caller and never read back, and a launch
  * boundary disappears (two launches in all: the event reduction, then the rest).
  * State, d_victims and the device status word end up exactly as after the two
- * calls.  The trace is read by both launches: leave it alone until the call's work has run.  All arguments are checked before anything is enqueued: on an error
+ * calls.  The trace is read by both launches: leave it alone until the call's work
+ * has run.  All arguments are checked before anything is enqueued: on an error
  * (including KV_ERR_K_TOO_LARGE) the epoch has NOT been scored.  k == 0 scores
  * only.  Where the device cannot keep the kernel's whole grid resident at once,
  * the separate kernels run one after the other instead. */
