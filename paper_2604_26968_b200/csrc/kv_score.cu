@@ -6,7 +6,7 @@
 namespace kvt {
 
 // ---- event reduction ---------------------------------------------------------
-template <bool PACKED>
+template <bool PACKED, bool DEAL>
 __global__ void __launch_bounds__(kEventThreads, kEventBlocksPerSm)
 event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events, const uint8_t* pair,
                     uint32_t* touch, unsigned long long* packed, uint64_t n, unsigned long long* delta,
@@ -16,7 +16,7 @@ event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_
   for (uint32_t i = 0; i < 16; ++i) s_cnt[i * kEventThreads + threadIdx.x] = 0;   // (the thread's own words)
   wait_for_kernel_ahead();
   if (!PACKED && blockIdx.x == 0 && threadIdx.x == 0) *touch_used = 1u;
-  const uint32_t bad = reduce_events<PACKED>(ev_entry, ev_hit, n_events, pair, touch, packed, n,
+  const uint32_t bad = reduce_events<PACKED, DEAL>(ev_entry, ev_hit, n_events, pair, touch, packed, n,
                                              (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
                                              (uint64_t)gridDim.x * blockDim.x, s_cnt, delta);
   if (bad) atomicOr(status, bad);
@@ -40,7 +40,10 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   unsigned long long* delta = ws.delta;
   uint32_t* status = ws.status;
   void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &packed, &n, &delta, &touch_used, &status};
-  const void* fn = packed ? (const void*)event_reduce_kernel<true> : (const void*)event_reduce_kernel<false>;
+  const bool rounds = n_events / 4 > blocks * kEventThreads * kEventVecs;   // more than one of the grid: see reduce_events
+  const void* fn = !packed ? (const void*)event_reduce_kernel<false, false>
+                 : rounds  ? (const void*)event_reduce_kernel<true, true>
+                           : (const void*)event_reduce_kernel<true, false>;
   const cudaError_t e = launch_scoring_kernel(fn, dim3((unsigned)blocks), dim3(kEventThreads), args, 0, s, false, ws,
                                               n_events <= kEventOverlapMax);
   count_launches(1);

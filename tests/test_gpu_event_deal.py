@@ -1,0 +1,42 @@
+"""Traces of several rounds whose warps' events are dealt out again where vectors are no runs: runs, broken
+runs, single entries, entries out of range and flags of any value mixed in one trace, around a round of
+the whole grid, against the oracle, bit for bit, with the status bits."""
+import numpy as np
+import pytest
+
+from oracle import kv_oracle as O
+from paper_2604_26968_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+ROUND = 512 * 296 * 8          # events of one round of the grid
+
+
+@pytest.mark.parametrize("n_events", [ROUND - 5, ROUND + 4, ROUND + 128 * 7 + 3, 2 * ROUND + 131])
+def test_mixed_trace(n_events):
+    from lockstep import Lockstep
+    w = W.Workload("deal", [W.gqa(3, 6, 3, 16, 8, 7001, 9000, "entry")], 0.05, 0.0, seed=7)      # 63,009 entries
+    ls = Lockstep(w, payload=False, batch_bytes=1 << 20)
+    g, o = ls.gpu, ls.ora
+    r = np.random.default_rng(n_events)
+    starts = r.integers(0, w.N // 4 - 9, -(-n_events // 32)) * 4
+    ev = (starts[:, None] + np.arange(32)[None, :]).reshape(-1)[:n_events]                       # aligned runs ...
+    half = n_events // 2
+    ev[half:] = np.sort(r.integers(0, w.N, n_events - half))                                     # ... and freed slots in order
+    some = r.integers(0, n_events, 3000)
+    ev[some] = r.integers(0, w.N, 3000)
+    hit = r.integers(0, 3, n_events).astype(np.uint8) * 85                                       # any non-zero flag is a hit
+    ev = ev.astype(np.uint32)
+    d_e, d_h, n = g.stage_events(ev, hit)
+    g.check(g.pool.kv_epoch_score_select(0, d_e, d_h, n, w.k, g.victims), "kv_epoch_score_select")
+    assert o.epoch_score(0, ev, hit) == O.OK
+    ls.compare_state(n_events)
+    rc, v = o.select_victims(w.k)
+    assert rc == O.OK and np.array_equal(g.victims[:w.k].cpu().numpy().view(np.uint32), v)
+    ev[:: n_events // 50] = w.N + 3                                                              # refused, and flagged
+    d_e, d_h, n = g.stage_events(ev, hit)
+    g.check(g.pool.kv_epoch_score_select(1, d_e, d_h, n, w.k, g.victims), "kv_epoch_score_select")
+    assert o.epoch_score(1, ev[ev < w.N], hit[ev < w.N]) == O.OK
+    assert g.pool.kv_device_status() == 1          # KV_DEV_EVENT_BAD_ID
+    ls.compare_state((n_events, "refused"))
+    ls.close()
