@@ -103,6 +103,15 @@ __device__ __forceinline__ bool take_touches(const EntryState& st, uint64_t v, u
   return true;
 }
 
+// Four events on entries in a row, all of them in a pool of n: an aligned group, or (PACKED) one whose words
+// of pair bytes lie inside the array.  (From 2^32 - 3 on the sums wrap: the first id has to lie below the
+// last one, or an event that is refused would be taken for the neighbour of the pool's first entries.)
+template <bool PACKED>
+__host__ __device__ __forceinline__ bool is_run(const uint32_t id[4], uint32_t n) {
+  return (PACKED || !(id[0] & 3u)) && id[0] < id[3] && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u &&
+         (PACKED ? id[3] | 3u : id[3]) < n;
+}
+
 // The calling block's share of the events.  s_cnt: kEventThreads * 16 words of shared
 // memory, zero on entry; word [p * kEventThreads + t] holds thread t's
 // counts for pair p (events | hits << 16) since the last flush.  delta: the 32
@@ -165,11 +174,6 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
   };
 
   auto ids_of = [](const EventVec& x, uint32_t id[4]) { id[0] = x.id.x; id[1] = x.id.y; id[2] = x.id.z; id[3] = x.id.w; };
-  // Four entries in a row: an aligned group, or (PACKED) one whose words of pair bytes lie inside the array.
-  auto is_run = [&](const uint32_t id[4]) {
-    return (PACKED || !(id[0] & 3u)) && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u &&
-           (PACKED ? id[3] | 3u : id[3]) < n32;
-  };
   auto gather = [&](const uint32_t id[4], bool run) {   // the vector's pair bytes (bit 7 = FREE or out of range)
     uint32_t w = 0;
     if (run) {   // (through the L1: neighbouring blocks share sectors)
@@ -195,7 +199,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
     for (uint32_t u = 0; u < kEventVecs; ++u) {  // all gathers before any is used
       uint32_t id[4];
       ids_of(cur[u], id);
-      run[u] = is_run(id);
+      run[u] = is_run<PACKED>(id, n32);
       if constexpr (DEAL) {
         // Where vectors are no runs (the slots that an epoch has filled again, in order of their ids), a
         // warp's 128 events are dealt out again, neighbours to neighbouring lanes: a gather or an
