@@ -144,9 +144,9 @@ typedef struct {
   /* per-entry state, struct of arrays of length N in global id order (device) */
   float* d_ema;           /* EMA access score */
   float* d_decay;         /* EMA decay per entry */
-  uint32_t* d_touch;      /* touches that kv_epoch_events has counted and no scoring pass has taken
-                             up yet, else zero (the library's to write: kv_epoch_score_select
-                             counts in the workspace and looks here only for what that call left) */
+  uint32_t* d_touch;      /* touches seen in the current epoch: what kv_epoch_events, or the caller,
+                             has put here since the last scoring pass (the touches of a call's own
+                             trace may be counted in the workspace) */
   uint32_t* d_last_epoch; /* epoch of the last touch */
   uint8_t* d_pair;        /* 4*block_type + transition_type, 0..15; the library sets bit 7
                              while the entry is FREE (the value is then meaningless, but the

@@ -10,12 +10,11 @@ template <bool PACKED, bool DEAL>
 __global__ void __launch_bounds__(kEventThreads, kEventBlocksPerSm)
 event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events, const uint8_t* pair,
                     uint32_t* touch, unsigned long long* packed, uint64_t n, unsigned long long* delta,
-                    uint32_t* touch_used, uint32_t* status) {
+                    uint32_t* status) {
   __shared__ uint32_t s_cnt[16 * kEventThreads];   // [pair][thread]: events | hits << 16
 #pragma unroll
   for (uint32_t i = 0; i < 16; ++i) s_cnt[i * kEventThreads + threadIdx.x] = 0;   // (the thread's own words)
   wait_for_kernel_ahead();
-  if (!PACKED && blockIdx.x == 0 && threadIdx.x == 0) *touch_used = 1u;
   const uint32_t bad = reduce_events<PACKED, DEAL>(ev_entry, ev_hit, n_events, pair, touch, packed, n,
                                              (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
                                              (uint64_t)gridDim.x * blockDim.x, s_cnt, delta);
@@ -34,12 +33,12 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   const uint64_t cap = (uint64_t)sm_count() * kEventBlocksPerSm;
   if (blocks > cap) blocks = cap;
   const uint8_t* pair = st.pair;
-  uint32_t *touch = st.touch, *touch_used = &ws.sel->touch_used;
+  uint32_t* touch = st.touch;
   unsigned long long* packed = st.packed;
   uint64_t n = st.n;
   unsigned long long* delta = ws.delta;
   uint32_t* status = ws.status;
-  void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &packed, &n, &delta, &touch_used, &status};
+  void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &packed, &n, &delta, &status};
   const bool rounds = n_events / 4 > blocks * kEventThreads * kEventVecs;   // more than one of the grid: see reduce_events
   const void* fn = !packed ? (const void*)event_reduce_kernel<false, false>
                  : rounds  ? (const void*)event_reduce_kernel<true, true>
@@ -58,7 +57,7 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
 // publishes P; by then every block has read them.
 constexpr int kUpdateBlocksPerSm = 4;
 __global__ void __launch_bounds__(kThreads, kUpdateBlocksPerSm)
-entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights hw, uint32_t epoch, uint32_t* touch_used) {
+entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights hw, uint32_t epoch) {
   __shared__ float sP[16];
   __shared__ bool s_last;
   const int policy = pd.policy;
@@ -85,7 +84,7 @@ entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights h
   const uint64_t i = n4 * 4 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < st.n) {
     float sc;
-    entry_update1(st, i, sP, policy, epoch, hw, 0u, true, nullptr, sc);
+    entry_update1(st, i, sP, policy, epoch, hw, 0u, nullptr, sc);
   }
   // commit by the last block to finish
   __syncthreads();
@@ -96,10 +95,7 @@ entry_update_kernel(const EntryState st, const Predictor pd, const HeadWeights h
   __syncthreads();
   if (s_last && threadIdx.x < 16) {
     commit_predictor(pd, threadIdx.x, step);
-    if (threadIdx.x == 0) {
-      *pd.ticket = 0;
-      *touch_used = 0;   // (all touch counts are zero now)
-    }
+    if (threadIdx.x == 0) *pd.ticket = 0;
   }
 }
 
@@ -127,8 +123,7 @@ cudaError_t launch_entry_update(const EntryState& st, uint64_t* hits, uint64_t* 
   EntryState st_arg = st;
   Predictor pd_arg = pd;
   HeadWeights hw_arg = hw;
-  uint32_t* touch_used = &ws.sel->touch_used;
-  void* args[] = {&st_arg, &pd_arg, &hw_arg, &epoch, &touch_used};
+  void* args[] = {&st_arg, &pd_arg, &hw_arg, &epoch};
   const cudaError_t e = launch_scoring_kernel((const void*)entry_update_kernel, dim3((unsigned)blocks),
                                               dim3(kThreads), args, 0, s, false, ws);
   count_launches(1);

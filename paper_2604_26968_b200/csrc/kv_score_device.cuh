@@ -32,7 +32,7 @@ namespace kvt {
 // Touch counts that only the fused scoring pass of the same call reads (PACKED): 64 bits
 // for four entries, nine for each and the sum of the four in the upper 28, so that one
 // atomic counts all events of a vector on the same four entries, and half the bytes are
-// scattered over and then read.  A count that overflows carries into the next field and
+// scattered over.  A count that overflows carries into the next field and
 // takes 511 from the sum of the fields, or, the last one, 512, and adds one to the sum
 // kept beside them: the two agree again only after 512 * 2^28 / 513 touches, more than a
 // trace that is counted this way has, so the scoring pass sees of every word whether it is
@@ -88,18 +88,16 @@ __device__ __forceinline__ bool unpack_touches(uint2 w, uint32_t t[4]) {
   return t[0] + t[1] + t[2] + t[3] == w.y >> (kSumShift - 32u);
 }
 
-// The packed counts w of vector v as its touch counts, in x.t, the 32-bit counts added where they hold
-// anything (hot); both are cleared.  False, and nothing done, if a packed count has overflowed.
-__device__ __forceinline__ bool take_touches(const EntryState& st, uint64_t v, uint2 w, const uint32_t* hot, uint4& sum) {
-  uint32_t t[4];
-  if (!unpack_touches(w, t)) return false;
-  sum = make_uint4(t[0], t[1], t[2], t[3]);
+// The packed counts w of vector v are added to its 32-bit counts t, and both are cleared.  False, and nothing
+// done, if a packed count has overflowed.  (The 32-bit counts are looked at in any case: kv_epoch_events or the
+// caller may have left something there.  To have the event reduction look for that took longer, 18.8 M entries
+// 158 us a pass instead of 156.)
+__device__ __forceinline__ bool take_touches(const EntryState& st, uint64_t v, uint2 w, uint4& t) {
+  uint32_t p[4];
+  if (!unpack_touches(w, p)) return false;
   if (w.x | w.y) st.packed[v] = 0;
-  if (hot) {
-    const uint4 x = __ldcg(reinterpret_cast<const uint4*>(st.touch) + v);
-    sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
-    if (x.x | x.y | x.z | x.w) reinterpret_cast<uint4*>(st.touch)[v] = make_uint4(0, 0, 0, 0);
-  }
+  if (t.x | t.y | t.z | t.w) reinterpret_cast<uint4*>(st.touch)[v] = make_uint4(0, 0, 0, 0);
+  t.x += p[0]; t.y += p[1]; t.z += p[2]; t.w += p[3];
   return true;
 }
 
@@ -522,13 +520,12 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
   }
 }
 
-// The same for one entry (ragged ends), which has had t touches beside those of the 32-bit count (if that
-// is to be looked at: wide).
+// The same for one entry (ragged ends), which has had t touches beside those of the 32-bit count.
 __device__ __forceinline__ void entry_update1(const EntryState& st, uint64_t i, const float* sP, int policy,
-                                              uint32_t epoch, const HeadWeights& hw, uint32_t t, bool wide,
+                                              uint32_t epoch, const HeadWeights& hw, uint32_t t,
                                               uint32_t* hot, float& sc) {
   float e = st.ema[i];
-  const uint32_t tw = wide ? __ldcg(&st.touch[i]) : 0u;
+  const uint32_t tw = __ldcg(&st.touch[i]);
   t += tw;
   const float w = hw.on ? head_weight(hw, i) : 1.0f;
   entry_step(e, st.decay[i], t, st.pair[i], sP, policy, policy == 2 ? st.last_epoch[i] : 0u, epoch, w, sc);

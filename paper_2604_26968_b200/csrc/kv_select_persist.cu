@@ -81,11 +81,11 @@ static_assert((2u * kHalfMax) >> kBracketShiftMax <= kHistBins, "the widest brac
 constexpr uint32_t kNoteKeyBits = 22, kKeptKeyBits = 11;
 static_assert(2u * kHalfMax <= 1u << kNoteKeyBits && kNoteKeyBits + 7 <= 32, "a note holds any key of the bracket");
 static_assert(kBracketShiftMax <= kKeptKeyBits && kPMaxRows <= 64, "a kept note holds any key of a bin, and its row");
-// Fused form: the entry pass's inputs of one row in shared memory -- ema, decay and, for the LRU
-// policy, last_epoch (4,096 words each), pair bytes (1,024 words), touch counts (4,096 words, or 2,048 packed)
+// Fused form: the entry pass's inputs of one row in shared memory -- ema, decay, touch counts and, for the
+// LRU policy, last_epoch (4,096 words each), pair bytes (1,024 words), packed touch counts (2,048 words)
 enum Fusion { kNoScoring, kScoring, kScoringPacked };
 __host__ __device__ constexpr uint32_t stage_words(Fusion f, bool lru) {
-  return 2u * kPChunk + kPThreads + (f == kScoringPacked ? 2u * kPThreads : kPChunk) + (lru ? kPChunk : 0u);
+  return 3u * kPChunk + kPThreads + (f == kScoringPacked ? 2u * kPThreads : 0u) + (lru ? kPChunk : 0u);
 }
 constexpr uint64_t kPAlone = 2 * kPChunk;
 constexpr uint64_t kPackedMaxEvents = 1ull << 27;       // (reduce_events: no overflow goes unseen)
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   extern __shared__ __align__(16) uint32_t s_dyn[];
   constexpr bool FUSED = FUSION != kNoScoring, PACKED = FUSION == kScoringPacked;
   // offsets in a stage
-  constexpr uint32_t kAtPair = 2u * kPChunk, kAtTouch = kAtPair + kPThreads, kAtLast = stage_words(FUSION, false);
+  constexpr uint32_t kAtTouch = 2u * kPChunk, kAtPair = 3u * kPChunk, kAtPacked = kAtPair + kPThreads, kAtLast = stage_words(FUSION, false);
   const uint32_t n_words = a.n_rows * 128u;           // bitmap words: 128 per row
   // Bitmaps "below tau" and "equal to tau".  While they are filled, word 4*(row*32 + warp) + q
   // holds position q of the 32 lanes' vectors (a ballot); before they are counted they are
@@ -347,10 +347,9 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0), "l"(a.st.ema + i0) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kPChunk), "l"(a.st.decay + i0) : "memory");
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d1), "l"(a.st.pair + i0) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kAtTouch), "l"(a.st.touch + i0) : "memory");
         if constexpr (PACKED)
           asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d1 + 4u * kPThreads + 4u * t), "l"(a.st.packed + i0 / 4u) : "memory");
-        else
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kAtTouch), "l"(a.st.touch + i0) : "memory");
         if (!PLAIN && a.pd.policy == 2) {
           const uint32_t d2 = (uint32_t)__cvta_generic_to_shared(dst + kAtLast + 4u * t);
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d2), "l"(a.st.last_epoch + i0) : "memory");
@@ -375,7 +374,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const uint32_t hint_valid = a.sel->hint_valid, hint_tau = a.sel->hint_tau;
   const unsigned long long hint_n = a.sel->hint_n;
   uint32_t half = a.sel->hint_half;   // (the bracket's width follows how well the hints have been doing)
-  const bool touch_used = PACKED && __ldcg(&a.sel->touch_used) != 0u;
   const bool hint = !SHARED && (a.spill != nullptr) & (hint_valid != 0u) & (hint_n == a.n);
   if constexpr (FUSED) {
     // reuse estimates from the totals plus this epoch's counts (final: the event
@@ -403,8 +401,8 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const float neg_inf = __int_as_float(0xFF800000);
   const float lo_f = hint ? key_score(base0) : neg_inf, hi_f = hint ? key_score(base0 + 2u * half) : neg_inf;
   __syncthreads();
-  // where to note counts too large for the packed ones (nullptr: the 32-bit counts hold nothing)
-  uint32_t* hot = FUSED && (!PACKED || touch_used) ? &a.sel->touch_hot : nullptr;
+  // where to note counts too large for the packed ones (nullptr: the trace is in the packed ones)
+  uint32_t* hot = FUSED && !PACKED ? &a.sel->touch_hot : nullptr;
   constexpr uint32_t kClearing = (sizeof(SelectTurn) / 4u + kPThreads - 1u) / kPThreads;   // CTAs that clear something
   static_assert(kClearing <= kSharedCtas, "each of them has a word");
   if (SHARED && g < kClearing && t == 0)
@@ -490,12 +488,12 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         cur.d = *reinterpret_cast<const float4*>(src + kPChunk + 4u * t);
         cur.pr4 = src[kAtPair + t];
         uint2 packed = make_uint2(0, 0);
-        if constexpr (PACKED) packed = *reinterpret_cast<const uint2*>(src + kAtTouch + 2u * t);
-        else cur.t = *reinterpret_cast<const uint4*>(src + kAtTouch + 4u * t);
+        if constexpr (PACKED) packed = *reinterpret_cast<const uint2*>(src + kAtPacked + 2u * t);
+        cur.t = *reinterpret_cast<const uint4*>(src + kAtTouch + 4u * t);
         cur.le = make_uint4(0, 0, 0, 0);
         if (!PLAIN && policy == 2) cur.le = *reinterpret_cast<const uint4*>(src + kAtLast + 4u * t);
         issue(r + kStages);
-        if (PACKED && !take_touches(a.st, i0 / 4, packed, hot, cur.t)) {
+        if (PACKED && !take_touches(a.st, i0 / 4, packed, cur.t)) {
           overflowed = true;   // (these entries are left as they are until the trace has been counted again)
         } else {
           float4 sc;
@@ -512,7 +510,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
             if constexpr (PACKED) a.st.packed[i0 / 4u] = 0;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-              if (i0 + j < i1) entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, c[j], hot != nullptr, hot, s[j]);
+              if (i0 + j < i1) entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, c[j], hot, s[j]);
           }
         }
       }
@@ -654,7 +652,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
           for (uint32_t i = i0; i < i1 && i < i0 + 4u; ++i) {
             float s;
             if (done) a.st.touch[i] = 0;
-            else entry_update1(a.st, i, sP, PLAIN ? 0 : a.pd.policy, a.epoch, a.hw, 0u, true, hot, s);
+            else entry_update1(a.st, i, sP, PLAIN ? 0 : a.pd.policy, a.epoch, a.hw, 0u, hot, s);
           }
         }
       }
@@ -835,12 +833,9 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       // the CTA waits for the others anyway)
       if (g == 0 && t >= kPThreads - 32u && lane < 16u) {
         commit_predictor(a.pd, lane, s_pair[lane]);
-        if (lane == 0u) {
-          a.sel->touch_used = 0;   // (the 32-bit counts have been cleared)
-          if (hot) {
-            if (a.h_hot) *a.h_hot = __ldcg(hot);
-            *hot = 0;
-          }
+        if (lane == 0u && hot) {
+          if (a.h_hot) *a.h_hot = __ldcg(hot);
+          *hot = 0;
         }
       }
     }
@@ -1206,8 +1201,11 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   a.list = ws.list;
   a.words = ws.shared_words;
   a.status = ws.status;
-  const Fusion fusion = !fs ? kNoScoring : fs->n_events < kPackedMaxEvents && *fs->hot == 0u ? kScoringPacked : kScoring;
   const bool lru = fs && fs->opt.policy == 2;
+  // (the LRU policy's stages leave no room for the packed counts on pools of more than 41 rows)
+  const bool packed = fs && fs->n_events < kPackedMaxEvents && *fs->hot == 0u &&
+                      persist_smem(a.n_rows, kNoteCapMin, kStages * stage_words(kScoringPacked, lru)) <= pd.smem_max;
+  const Fusion fusion = !fs ? kNoScoring : packed ? kScoringPacked : kScoring;
   a.stage_words = fs ? stage_words(fusion, lru) : 0u;
   const uint32_t stages_words = kStages * a.stage_words;
   // Notes: the bracket typically holds 4-15 % of a warp's keys, in some traces several times

@@ -110,8 +110,7 @@ struct SelectScalars {
   uint32_t hint_half;
   uint32_t hint_off_last, hint_off_trend;
   uint32_t hint_trend;         // where the trend puts the next tau
-  uint32_t touch_used;         // `touch` holds something (else it is all zero and need not be read)
-  uint32_t touch_hot;          // ... an entry with more touches than the packed counts are tried again with
+  uint32_t touch_hot;          // an entry has more touches than the packed counts are tried again with
 };
 
 // What the CTAs of one persistent selection share while it runs.  A pool has two of these, used in
