@@ -147,7 +147,7 @@ __global__ void init_scalars_kernel(uint64_t* hits, uint64_t* misses, float* P, 
     ws.sel->serial = 0; ws.sel->update_ticket = 0; ws.sel->hint_last = 0;
     ws.sel->hint_valid = 0; ws.sel->hint_tau = 0; ws.sel->hint_n = 0;
     ws.sel->hint_half = 0; ws.sel->hint_off_last = 0; ws.sel->hint_off_trend = 0; ws.sel->hint_trend = 0;
-    ws.sel->touch_hot = 0;
+    ws.sel->touch_wide = 0; ws.sel->touch_hot = 0;
     for (int q = 0; q < 3; ++q) ws.sel->bound[q] = 0;
     ws.sel->n_select = 0; ws.sel->n_hint_hit = 0; ws.sel->n_hint_miss = 0; ws.sel->n_reread = 0;
   }

@@ -6,18 +6,21 @@
 namespace kvt {
 
 // ---- event reduction ---------------------------------------------------------
+// PACKED: touches go to the packed counts, or, while the last epochs' have overflowed them (wide), to the others.
 template <bool PACKED, bool DEAL>
 __global__ void __launch_bounds__(kEventThreads, kEventBlocksPerSm)
 event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events, const uint8_t* pair,
                     uint32_t* touch, unsigned long long* packed, uint64_t n, unsigned long long* delta,
-                    uint32_t* status) {
+                    const uint32_t* wide, uint32_t* status) {
   __shared__ uint32_t s_cnt[16 * kEventThreads];   // [pair][thread]: events | hits << 16
 #pragma unroll
   for (uint32_t i = 0; i < 16; ++i) s_cnt[i * kEventThreads + threadIdx.x] = 0;   // (the thread's own words)
   wait_for_kernel_ahead();
-  const uint32_t bad = reduce_events<PACKED, DEAL>(ev_entry, ev_hit, n_events, pair, touch, packed, n,
-                                             (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
-                                             (uint64_t)gridDim.x * blockDim.x, s_cnt, delta);
+  const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+  EventVec first[kEventVecs];   // (together with *wide: one behind the other is a latency more)
+  load_events(ev_entry, ev_hit, n_events / 4, 0, gtid, stride, first);
+  const uint32_t bad = reduce_events<PACKED, DEAL>(PACKED && *wide == 0u, first, ev_entry, ev_hit, n_events, pair, touch,
+                                                   packed, n, gtid, stride, s_cnt, delta);
   if (bad) atomicOr(status, bad);
 }
 
@@ -34,11 +37,12 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   if (blocks > cap) blocks = cap;
   const uint8_t* pair = st.pair;
   uint32_t* touch = st.touch;
+  const uint32_t* wide = &ws.sel->touch_wide;
   unsigned long long* packed = st.packed;
   uint64_t n = st.n;
   unsigned long long* delta = ws.delta;
   uint32_t* status = ws.status;
-  void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &packed, &n, &delta, &status};
+  void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &packed, &n, &delta, &wide, &status};
   const bool rounds = n_events / 4 > blocks * kEventThreads * kEventVecs;   // more than one of the grid: see reduce_events
   const void* fn = !packed ? (const void*)event_reduce_kernel<false, false>
                  : rounds  ? (const void*)event_reduce_kernel<true, true>

@@ -59,6 +59,21 @@ struct EventVec {
   uint32_t hit;    // byte j: hit flag of event j
 };
 
+// The calling thread's vectors of iteration it.
+__device__ __forceinline__ void load_events(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n4, uint64_t it,
+                                            uint64_t gtid, uint64_t stride, EventVec x[kEventVecs]) {
+#pragma unroll
+  for (uint32_t u = 0; u < kEventVecs; ++u) {
+    const uint64_t v = (it * kEventVecs + u) * stride + gtid;
+    x[u].id = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);  // past the end: no entry
+    x[u].hit = 0;
+    if (v < n4) {
+      x[u].id = __ldcs(reinterpret_cast<const uint4*>(ev_entry) + v);
+      x[u].hit = __ldcs(reinterpret_cast<const uint32_t*>(ev_hit) + v);
+    }
+  }
+}
+
 // bit 7 of every non-zero byte
 __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
   return (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
@@ -101,22 +116,23 @@ __device__ __forceinline__ bool take_touches(const EntryState& st, uint64_t v, u
   return true;
 }
 
-// Four events on entries in a row, all of them in a pool of n: an aligned group, or (PACKED) one whose words
+// Four events on entries in a row, all of them in a pool of n: an aligned group, or (packed) one whose words
 // of pair bytes lie inside the array.  (From 2^32 - 3 on the sums wrap: the first id has to lie below the
 // last one, or an event that is refused would be taken for the neighbour of the pool's first entries.)
-template <bool PACKED>
-__host__ __device__ __forceinline__ bool is_run(const uint32_t id[4], uint32_t n) {
-  return (PACKED || !(id[0] & 3u)) && id[0] < id[3] && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u &&
-         (PACKED ? id[3] | 3u : id[3]) < n;
+__host__ __device__ __forceinline__ bool is_run(const uint32_t id[4], uint32_t n, bool packed) {
+  return (packed || !(id[0] & 3u)) && id[0] < id[3] && id[1] == id[0] + 1u && id[2] == id[0] + 2u && id[3] == id[0] + 3u &&
+         (id[3] | 3u) < n;
 }
 
 // The calling block's share of the events.  s_cnt: kEventThreads * 16 words of shared
 // memory, zero on entry; word [p * kEventThreads + t] holds thread t's
 // counts for pair p (events | hits << 16) since the last flush.  delta: the 32
 // global epoch counters (index 2 * pair + hit).  Returns the KV_DEV_* bits of
-// refused events.  Every thread of the block must call it.
+// refused events.  nxt: the thread's first vectors, from load_events.  use_packed (PACKED only): where the
+// touches go; no second template, since a kernel with two copies of this takes longer to fetch (4,096 entries
+// 13.4 -> 13.9 us a pass).  Every thread of the block must call it.
 template <bool PACKED, bool DEAL>
-__device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, const uint8_t* ev_hit,
+__device__ __forceinline__ uint32_t reduce_events(bool use_packed, EventVec nxt[kEventVecs], const uint32_t* ev_entry, const uint8_t* ev_hit,
                                                   uint64_t n_events, const uint8_t* pair, uint32_t* touch,
                                                   unsigned long long* packed, uint64_t n, uint64_t gtid,
                                                   uint64_t stride, uint32_t* s_cnt, unsigned long long* delta) {
@@ -127,6 +143,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t* my = s_cnt + threadIdx.x;
   constexpr uint32_t col = kEventThreads;
+  const bool to_packed = PACKED && use_packed;
   bool bad_id = false, not_resident = false;
 
   // adds the block's columns to the global counters and clears them; the 32 sums
@@ -158,18 +175,6 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
   };
   // counts event j of a vector (pair byte and hit bit already extracted)
   auto count = [&](uint32_t prj, uint32_t hitbit) { my[(prj & 15u) * col] += 1u + (hitbit << 16); };
-  auto load = [&](uint64_t it, EventVec x[kEventVecs]) {
-#pragma unroll
-    for (uint32_t u = 0; u < kEventVecs; ++u) {
-      const uint64_t v = (it * kEventVecs + u) * stride + gtid;
-      x[u].id = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);  // past the end: no entry
-      x[u].hit = 0;
-      if (v < n4) {
-        x[u].id = __ldcs(reinterpret_cast<const uint4*>(ev_entry) + v);
-        x[u].hit = __ldcs(reinterpret_cast<const uint32_t*>(ev_hit) + v);
-      }
-    }
-  };
 
   auto ids_of = [](const EventVec& x, uint32_t id[4]) { id[0] = x.id.x; id[1] = x.id.y; id[2] = x.id.z; id[3] = x.id.w; };
   auto gather = [&](const uint32_t id[4], bool run) {   // the vector's pair bytes (bit 7 = FREE or out of range)
@@ -185,8 +190,6 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
     return w;
   };
 
-  EventVec nxt[kEventVecs];
-  if (iters) load(0, nxt);
   for (uint64_t it = 0; it < iters; ++it) {
     EventVec cur[kEventVecs];
     bool run[kEventVecs];       // ids are a run of four inside the pool
@@ -197,7 +200,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
     for (uint32_t u = 0; u < kEventVecs; ++u) {  // all gathers before any is used
       uint32_t id[4];
       ids_of(cur[u], id);
-      run[u] = is_run<PACKED>(id, n32);
+      run[u] = is_run(id, n32, to_packed);
       if constexpr (DEAL) {
         // Where vectors are no runs (the slots that an epoch has filled again, in order of their ids), a
         // warp's 128 events are dealt out again, neighbours to neighbouring lanes: a gather or an
@@ -220,19 +223,19 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
       }
       pr4[u] = gather(id, run[u]);
     }
-    if (it + 1 < iters) load(it + 1, nxt);
+    if (it + 1 < iters) load_events(ev_entry, ev_hit, n4, it + 1, gtid, stride, nxt);
 #pragma unroll
     for (uint32_t u = 0; u < kEventVecs; ++u) {
       uint32_t id[4];
       ids_of(cur[u], id);
       const uint32_t pr = pr4[u], hit4 = nonzero_bytes(cur[u].hit);
       const bool whole = run[u] && !(pr & 0x80808080u);   // four resident entries in a row
-      if (PACKED && whole) {
+      if (to_packed && whole) {
         const uint32_t r = id[0] & 3u;
         atomicAdd(packed + (id[0] >> 2), packed_touches(0x01010101u << (8u * r)));
         if (r) atomicAdd(packed + (id[0] >> 2) + 1u, packed_touches(0x01010101u >> (32u - 8u * r)));
       }
-      const uint32_t m = PACKED ? 0u : __ballot_sync(0xFFFFFFFFu, whole);
+      const uint32_t m = to_packed ? 0u : __ballot_sync(0xFFFFFFFFu, whole);
       if (m) {
 #pragma unroll
         for (uint32_t half = 0; half < 2; ++half) {   // 16 vectors' pairs of atomics per instruction
@@ -254,7 +257,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
           bad_id |= !in;
           not_resident |= in && !ok[j];
         }
-        if constexpr (PACKED) {   // (the last event on a word adds for those before it)
+        if (to_packed) {   // (the last event on a word adds for those before it)
           uint32_t inc[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) inc[j] = ok[j] ? 1u << (8u * (id[j] & 3u)) : 0u;
@@ -263,20 +266,22 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
             if (j < 3 && (id[j] >> 2) == (id[j + 1] >> 2)) inc[j + 1] += inc[j];
             else if (inc[j]) atomicAdd(packed + (id[j] >> 2), packed_touches(inc[j]));
           }
-        }
+        } else {
 #pragma unroll
-        for (int j = 0; !PACKED && j < 4; j += 2) {
-          const uint32_t i0 = id[j], i1 = id[j + 1];
-          if (ok[j] && ok[j + 1] && i1 == i0 + 1u && !(i0 & 1u)) {
-            atomicAdd(reinterpret_cast<unsigned long long*>(touch + i0), 0x100000001ull);
-          } else {
-            if (ok[j]) touch_add(touch, i0, n32, (i0 & 1u) ? (1ull << 32) : 1ull);
-            if (ok[j + 1]) touch_add(touch, i1, n32, (i1 & 1u) ? (1ull << 32) : 1ull);
+          for (int j = 0; j < 4; j += 2) {
+            const uint32_t i0 = id[j], i1 = id[j + 1];
+            if (ok[j] && ok[j + 1] && i1 == i0 + 1u && !(i0 & 1u)) {
+              atomicAdd(reinterpret_cast<unsigned long long*>(touch + i0), 0x100000001ull);
+            } else {
+              if (ok[j]) touch_add(touch, i0, n32, (i0 & 1u) ? (1ull << 32) : 1ull);
+              if (ok[j + 1]) touch_add(touch, i1, n32, (i1 & 1u) ? (1ull << 32) : 1ull);
+            }
           }
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (ok[j]) count(pr >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);      }
+          if (ok[j]) count(pr >> (8 * j), (hit4 >> (8 * j + 7)) & 1u);
+      }
       __syncwarp();
     }
     if ((it + 1) % kEventFlushIters == 0) flush();   // (uniform over the block)
@@ -296,7 +301,7 @@ __device__ __forceinline__ uint32_t reduce_events(const uint32_t* ev_entry, cons
         bad |= KV_DEV_EVENT_NOT_RESIDENT;
       } else {
         count(pr, __ldcs(ev_hit + e) != 0);
-        if constexpr (PACKED) atomicAdd(packed + (i >> 2), packed_touches(1u << (8u * (i & 3u))));
+        if (to_packed) atomicAdd(packed + (i >> 2), packed_touches(1u << (8u * (i & 3u))));
         else touch_add(touch, i, n32, (i & 1u) ? (1ull << 32) : 1ull);
       }
     }
@@ -465,8 +470,7 @@ __device__ __forceinline__ void commit_predictor(const Predictor& pd, unsigned p
 // in two halves so that a caller can have the next vector's loads in flight
 // while it finishes this one.  v indexes vectors.  The touch counts are read from
 // L2: other blocks' atomics made them.  PACKED: take_touches has read and cleared them.  hot:
-// where to say that an entry has had too many touches for the packed counts to be tried again.
-constexpr uint32_t kTouchHot = kFieldMax / 2;
+// where to say that an entry has had more touches than a packed count holds.
 struct EntryVec {
   float4 e, d;
   uint4 t, le;         // t: touch counts
@@ -508,7 +512,7 @@ __device__ __forceinline__ void entry_finish4(const EntryState& st, uint64_t v, 
   // touch counts of FREE entries are always zero (events on them are refused)
   if (x.t.x | x.t.y | x.t.z | x.t.w) {
     if (!PACKED) reinterpret_cast<uint4*>(st.touch)[v] = make_uint4(0, 0, 0, 0);
-    if (hot && max(max(x.t.x, x.t.y), max(x.t.z, x.t.w)) > kTouchHot) *hot = 1u;
+    if (hot && max(max(x.t.x, x.t.y), max(x.t.z, x.t.w)) > kFieldMax) *hot = 1u;
     if (x.t.x && x.t.y && x.t.z && x.t.w) {   // a block that reported all its heads: one store
       reinterpret_cast<uint4*>(st.last_epoch)[v] = make_uint4(epoch, epoch, epoch, epoch);
     } else {
@@ -532,7 +536,7 @@ __device__ __forceinline__ void entry_update1(const EntryState& st, uint64_t i, 
   st.ema[i] = e;
   st.score[i] = sc;
   if (tw) st.touch[i] = 0;
-  if (hot && t > kTouchHot) *hot = 1u;
+  if (hot && t > kFieldMax) *hot = 1u;
   if (t) st.last_epoch[i] = epoch;
 }
 

@@ -44,12 +44,12 @@
 // Measured, a pass with the event reduction: 4,096 entries 13.1 us, 0.9 M 26.8, 3.1 M 37.2, 18.8 M 149
 // (notes per thread and whole chunks only, 32-bit touch counts: 32.5, 40.3, 59.9, 206).
 //
-// The same kernel also exists fused with the per-entry scoring pass (kScoring, kScoringPacked):
+// The same kernel also exists fused with the per-entry scoring pass (FUSED = true):
 // every CTA first updates the entries of its own rows (posterior, EMA, score), their
 // inputs streamed through shared-memory stages by asynchronous copies.  The touch counts are
-// the packed ones of reduce_events, two bytes an entry (entry phase of 18.8 M entries 97 -> 83 us,
+// the packed ones of reduce_events, two bytes an entry, beside the caller's (entry phase of 18.8 M entries 97 -> 83 us,
 // the event reduction ahead of it 40 -> 32; a pass 177 -> 152, of 3.1 M entries 41.1 -> 39.3, of
-// 0.9 M even), or, after a trace that overflowed them, the 32-bit ones (kScoring).  The event
+// 0.9 M even), or, for a while after a trace that overflowed them, the caller's alone.  The event
 // reduction stays a launch of its own ahead of it: its scattered gathers and atomics run slower
 // beside this kernel's shared memory (11.5 M entries 101 -> 111 us), and for small traces a
 // cooperative launch's own gap of ~3 us takes the place of the one saved (0.9 M 27.3 -> 27.5).
@@ -81,15 +81,18 @@ static_assert((2u * kHalfMax) >> kBracketShiftMax <= kHistBins, "the widest brac
 constexpr uint32_t kNoteKeyBits = 22, kKeptKeyBits = 11;
 static_assert(2u * kHalfMax <= 1u << kNoteKeyBits && kNoteKeyBits + 7 <= 32, "a note holds any key of the bracket");
 static_assert(kBracketShiftMax <= kKeptKeyBits && kPMaxRows <= 64, "a kept note holds any key of a bin, and its row");
-// Fused form: the entry pass's inputs of one row in shared memory -- ema, decay, touch counts and, for the
-// LRU policy, last_epoch (4,096 words each), pair bytes (1,024 words), packed touch counts (2,048 words)
-enum Fusion { kNoScoring, kScoring, kScoringPacked };
-__host__ __device__ constexpr uint32_t stage_words(Fusion f, bool lru) {
-  return 3u * kPChunk + kPThreads + (f == kScoringPacked ? 2u * kPThreads : 0u) + (lru ? kPChunk : 0u);
+// Fused form: the entry pass's inputs of one row in shared memory -- ema, decay and touch counts (4,096 words
+// each), pair bytes (1,024 words), for the LRU policy last_epoch (4,096 words), packed touch counts (2,048 words)
+__host__ __device__ constexpr uint32_t stage_words(bool packed, bool lru) {
+  return 3u * kPChunk + kPThreads + (lru ? kPChunk : 0u) + (packed ? 2u * kPThreads : 0u);
 }
 constexpr uint64_t kPAlone = 2 * kPChunk;
 constexpr uint64_t kPackedMaxEvents = 1ull << 27;       // (reduce_events: no overflow goes unseen)
 constexpr unsigned long long kOverflowed = 1ull << 48;  // in SelectTurn::below
+// Epochs that go on counting in 32 bits after the last one with a count that the packed ones cannot hold.  18.8 M
+// entries: a pass takes 157 us, with 32-bit counts 175, the one that finds such a count out 300.  With 64 no
+// trace that is hot now and then costs more than 32-bit counts for all epochs would (184 without packed ones).
+constexpr uint32_t kWideEpochs = 64;
 constexpr uint32_t kStages = 2;                         // rows in flight ahead of the one being finished
 constexpr uint32_t kNoteCapMin = 128;                   // notes a warp keeps in shared memory, at least (the rest spills)
 
@@ -123,7 +126,6 @@ struct PArgs {
   uint32_t epoch;
   const uint32_t* ev_entry;   // the trace that the packed touch counts hold
   unsigned long long n_events;
-  uint32_t* h_hot;
 };
 
 // The two halves of the bounded grid-wide barrier; work put between them overlaps the wait.
@@ -166,9 +168,9 @@ __device__ __forceinline__ uint32_t await_word(const unsigned long long* p, uint
 }
 
 // What a CTA adds to SelectTurn::below: its keys below the bracket, bit 31 of them kOverflowed.
-template <bool PACKED>
+template <bool FUSED>
 __device__ __forceinline__ unsigned long long below_word(uint32_t s_below) {
-  return PACKED ? (s_below & 0x7FFFFFFFu) | (s_below >> 31 ? kOverflowed : 0ull) : s_below;
+  return FUSED ? (s_below & 0x7FFFFFFFu) | (s_below >> 31 ? kOverflowed : 0ull) : s_below;
 }
 
 // Finds the bin of a histogram (nbins <= 2048, a power of two) that contains rank k_rem (1-based):
@@ -278,12 +280,12 @@ __device__ __forceinline__ uint32_t block_scores4(const PArgs& a, unsigned long 
 
 // PLAIN (fused form only): the policy is the Bayesian product and no partition is weighted.
 // SHARED: on scratch that calls share which know nothing of each other.
-template <Fusion FUSION, bool PLAIN, bool BLOCKS, bool SHARED>
+template <bool FUSED, bool PLAIN, bool BLOCKS, bool SHARED>
 __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const PArgs a) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
-  constexpr bool FUSED = FUSION != kNoScoring, PACKED = FUSION == kScoringPacked;
   // offsets in a stage
-  constexpr uint32_t kAtTouch = 2u * kPChunk, kAtPair = 3u * kPChunk, kAtPacked = kAtPair + kPThreads, kAtLast = stage_words(FUSION, false);
+  constexpr uint32_t kAtTouch = 2u * kPChunk, kAtPair = 3u * kPChunk, kAtLast = kAtPair + kPThreads;
+  const uint32_t at_packed = kAtLast + (!PLAIN && a.pd.policy == 2 ? kPChunk : 0u);
   const uint32_t n_words = a.n_rows * 128u;           // bitmap words: 128 per row
   // Bitmaps "below tau" and "equal to tau".  While they are filled, word 4*(row*32 + warp) + q
   // holds position q of the 32 lanes' vectors (a ballot); before they are counted they are
@@ -337,6 +339,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   stamp(0);
 
   // ---- prologue: the first rows' loads go out before anything else ----
+  bool packed = FUSED && a.st.packed != nullptr;   // the trace is in the packed counts (those are zero otherwise)
   auto issue = [&](uint32_t r) {
     if constexpr (FUSED) {
       const uint32_t i0 = row_base(r) + 4u * t;
@@ -348,8 +351,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kPChunk), "l"(a.st.decay + i0) : "memory");
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d1), "l"(a.st.pair + i0) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d0 + 4u * kAtTouch), "l"(a.st.touch + i0) : "memory");
-        if constexpr (PACKED)
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d1 + 4u * kPThreads + 4u * t), "l"(a.st.packed + i0 / 4u) : "memory");
+        if (packed) {
+          const uint32_t d3 = (uint32_t)__cvta_generic_to_shared(dst + at_packed + 2u * t);
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d3), "l"(a.st.packed + i0 / 4u) : "memory");
+        }
         if (!PLAIN && a.pd.policy == 2) {
           const uint32_t d2 = (uint32_t)__cvta_generic_to_shared(dst + kAtLast + 4u * t);
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d2), "l"(a.st.last_epoch + i0) : "memory");
@@ -374,6 +379,10 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const uint32_t hint_valid = a.sel->hint_valid, hint_tau = a.sel->hint_tau;
   const unsigned long long hint_n = a.sel->hint_n;
   uint32_t half = a.sel->hint_half;   // (the bracket's width follows how well the hints have been doing)
+  const uint32_t wide = packed ? a.sel->touch_wide : 0u;   // (as the event reduction has found it)
+  packed = packed && wide == 0u;
+  // where to note counts that the packed ones could not hold (nullptr: they have been tried)
+  uint32_t* const hot = wide ? &a.sel->touch_hot : nullptr;
   const bool hint = !SHARED && (a.spill != nullptr) & (hint_valid != 0u) & (hint_n == a.n);
   if constexpr (FUSED) {
     // reuse estimates from the totals plus this epoch's counts (final: the event
@@ -401,8 +410,6 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   const float neg_inf = __int_as_float(0xFF800000);
   const float lo_f = hint ? key_score(base0) : neg_inf, hi_f = hint ? key_score(base0 + 2u * half) : neg_inf;
   __syncthreads();
-  // where to note counts too large for the packed ones (nullptr: the trace is in the packed ones)
-  uint32_t* hot = FUSED && !PACKED ? &a.sel->touch_hot : nullptr;
   constexpr uint32_t kClearing = (sizeof(SelectTurn) / 4u + kPThreads - 1u) / kPThreads;   // CTAs that clear something
   static_assert(kClearing <= kSharedCtas, "each of them has a word");
   if (SHARED && g < kClearing && t == 0)
@@ -422,7 +429,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
   // ---- phase A ----
   uint32_t n_noted = 0;     // notes of this warp
   uint32_t n_below = 0;     // keys of this thread below the bracket
-  bool overflowed = false;  // PACKED: a count of this thread's has
+  bool overflowed = false;  // a packed count of this thread's has
   uint32_t* const my_nstart = s_nstart + warp * (n_rows + 1u);
   uint32_t* const my_note = s_note + warp * a.note_cap;
   uint32_t* const my_spill = a.spill + (unsigned long long)(g * kPWarps + warp) * a.spill_stride;
@@ -487,27 +494,27 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         cur.e = *reinterpret_cast<const float4*>(src + 4u * t);
         cur.d = *reinterpret_cast<const float4*>(src + kPChunk + 4u * t);
         cur.pr4 = src[kAtPair + t];
-        uint2 packed = make_uint2(0, 0);
-        if constexpr (PACKED) packed = *reinterpret_cast<const uint2*>(src + kAtPacked + 2u * t);
+        uint2 counts = make_uint2(0, 0);
+        if (packed) counts = *reinterpret_cast<const uint2*>(src + at_packed + 2u * t);
         cur.t = *reinterpret_cast<const uint4*>(src + kAtTouch + 4u * t);
         cur.le = make_uint4(0, 0, 0, 0);
         if (!PLAIN && policy == 2) cur.le = *reinterpret_cast<const uint4*>(src + kAtLast + 4u * t);
         issue(r + kStages);
-        if (PACKED && !take_touches(a.st, i0 / 4, packed, cur.t)) {
+        if (!take_touches(a.st, i0 / 4, counts, cur.t)) {
           overflowed = true;   // (these entries are left as they are until the trace has been counted again)
         } else {
           float4 sc;
-          entry_finish4<PACKED, PLAIN>(a.st, i0 / 4, cur, sP, policy, a.epoch, a.hw, hot, sc);
+          entry_finish4<true, PLAIN>(a.st, i0 / 4, cur, sP, policy, a.epoch, a.hw, hot, sc);
           s[0] = sc.x; s[1] = sc.y; s[2] = sc.z; s[3] = sc.w;
         }
       } else {
         issue(r + kStages);
         if (i0 < i1) {   // the pool's ragged end
           uint32_t c[4] = {0, 0, 0, 0};
-          if (PACKED && !unpack_touches(__ldcg(reinterpret_cast<const uint2*>(a.st.packed) + i0 / 4u), c)) {
+          if (packed && !unpack_touches(__ldcg(reinterpret_cast<const uint2*>(a.st.packed) + i0 / 4u), c)) {
             overflowed = true;
           } else {
-            if constexpr (PACKED) a.st.packed[i0 / 4u] = 0;
+            if (packed) a.st.packed[i0 / 4u] = 0;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
               if (i0 + j < i1) entry_update1(a.st, i0 + j, sP, policy, a.epoch, a.hw, c[j], hot, s[j]);
@@ -573,11 +580,11 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       my_nstart[n_rows] = n_noted;
       if (n_below) atomicAdd(&s_below, n_below);
     }
-    if (PACKED && overflowed) atomicOr(&s_below, 1u << 31);   // (a CTA has fewer entries than that)
+    if (FUSED && overflowed) atomicOr(&s_below, 1u << 31);   // (a CTA has fewer entries than that)
     __syncthreads();
     if (!alone) {
       if (hint) add_pair(turn->hist[0] + 2u * t, reinterpret_cast<const uint2*>(s_hist)[t]);
-      if ((PACKED || hint) && t == 0 && s_below) atomicAdd(&turn->below, below_word<PACKED>(s_below));
+      if (t == 0 && s_below) atomicAdd(&turn->below, below_word<FUSED>(s_below));
       grid_arrive(bar);
       ok = grid_wait(bar, ++nbar * G);
     }
@@ -612,7 +619,7 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
     Pick pick{0u, 0u, 0u, 0u};
     uint32_t bin_k = 0;
     if (hint) {
-      below = alone ? below_word<PACKED>(s_below) : __ldcg(&turn->below);   // (in flight together with the histogram)
+      below = alone ? below_word<FUSED>(s_below) : __ldcg(&turn->below);   // (in flight together with the histogram)
       const bool above = a.k > below;   // (false beside kOverflowed)
       pick = pick_bin(turn->hist[0], alone, s_hist, kHistBins, above ? (uint32_t)(a.k - below) : 1u, s_warp, &s_pick);
       hint_hit = above && pick.bin != 0xFFFFFFFFu;
@@ -622,18 +629,27 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       }
       if (g == 0 && t == 0) atomicAdd(hint_hit ? &a.sel->n_hint_hit : &a.sel->n_hint_miss, 1u);
     }
-    if constexpr (PACKED) {
-      // A packed count overflowed somewhere: the trace is counted again, in the 32-bit array, the entries
-      // beside such a count get their scoring step, and the selection starts from the scores.  (Traces like
-      // that are counted in the 32-bit array from the start as soon as the host has heard of it.)
-      if (!hint) below = alone ? below_word<PACKED>(s_below) : __ldcg(&turn->below);
+    if constexpr (FUSED) {
+      // A packed count overflowed somewhere.  The words that hold one are the only ones that are not zero by
+      // now: the touches of their entries are counted again, in the 32-bit array, these entries get their
+      // scoring step, and the selection starts from the scores.  (kWideEpochs epochs are then counted in the
+      // 32-bit array from the start.)
+      if (!hint) below = alone ? below_word<FUSED>(s_below) : __ldcg(&turn->below);
       recounted = below >= kOverflowed;
       if (recounted) {
         hint_hit = false;
-        hot = &a.sel->touch_hot;
-        for (unsigned long long e = g * kPThreads + t; e < a.n_events; e += G * kPThreads) {
-          const uint32_t i = a.ev_entry[e];
-          if (i < n && !(a.st.pair[i] & kPairFree)) atomicAdd(a.st.touch + i, 1u);
+        constexpr uint32_t kAtOnce = 4;   // (two loads behind one another, four of each in flight)
+        for (unsigned long long e = g * kPThreads + t; e < a.n_events; e += kAtOnce * G * kPThreads) {
+          uint32_t id[kAtOnce];
+          unsigned long long w[kAtOnce];
+#pragma unroll
+          for (uint32_t j = 0; j < kAtOnce; ++j)
+            id[j] = e + j * G * kPThreads < a.n_events ? a.ev_entry[e + j * G * kPThreads] : 0xFFFFFFFFu;
+#pragma unroll
+          for (uint32_t j = 0; j < kAtOnce; ++j) w[j] = id[j] < n ? __ldcg(a.st.packed + id[j] / 4u) : 0ull;
+#pragma unroll
+          for (uint32_t j = 0; j < kAtOnce; ++j)
+            if (w[j] && !(a.st.pair[id[j]] & kPairFree)) atomicAdd(a.st.touch + id[j], 1u);
         }
         if (alone) {
           __syncthreads();
@@ -644,15 +660,12 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
         }
         for (uint32_t r = 0; r < n_rows; ++r) {
           const uint32_t i0 = row_base(r) + 4u * t, i1 = row_end(r), v = i0 / 4u;
-          if (i0 >= i1) continue;
-          uint32_t unused[4];
-          const bool done = unpack_touches(__ldcg(reinterpret_cast<const uint2*>(a.st.packed) + v), unused);
-          if (!done) a.st.packed[v] = 0;
+          if (i0 >= i1 || __ldcg(a.st.packed + v) == 0ull) continue;
+          a.st.packed[v] = 0;
 #pragma unroll 1
           for (uint32_t i = i0; i < i1 && i < i0 + 4u; ++i) {
             float s;
-            if (done) a.st.touch[i] = 0;
-            else entry_update1(a.st, i, sP, PLAIN ? 0 : a.pd.policy, a.epoch, a.hw, 0u, hot, s);
+            entry_update1(a.st, i, sP, PLAIN ? 0 : a.pd.policy, a.epoch, a.hw, 0u, nullptr, s);
           }
         }
       }
@@ -833,9 +846,9 @@ __global__ void __launch_bounds__(kPThreads, 1) select_persistent_kernel(const P
       // the CTA waits for the others anyway)
       if (g == 0 && t >= kPThreads - 32u && lane < 16u) {
         commit_predictor(a.pd, lane, s_pair[lane]);
-        if (lane == 0u && hot) {
-          if (a.h_hot) *a.h_hot = __ldcg(hot);
-          *hot = 0;
+        if (lane == 0u && (wide || recounted)) {
+          a.sel->touch_wide = recounted || __ldcg(hot) ? kWideEpochs : wide - 1u;
+          a.sel->touch_hot = 0;
         }
       }
     }
@@ -1149,10 +1162,9 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
       cudaDeviceGetAttribute(&d.n_sm, cudaDevAttrMultiProcessorCount, dev);
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      void* fns[7] = {(void*)select_persistent_kernel<kNoScoring, false, false, false>, (void*)select_persistent_kernel<kNoScoring, false, true, false>,
-                      (void*)select_persistent_kernel<kNoScoring, false, false, true>, (void*)select_persistent_kernel<kScoring, false, false, false>,
-                      (void*)select_persistent_kernel<kScoring, true, false, false>, (void*)select_persistent_kernel<kScoringPacked, false, false, false>,
-                      (void*)select_persistent_kernel<kScoringPacked, true, false, false>};
+      void* fns[5] = {(void*)select_persistent_kernel<false, false, false, false>, (void*)select_persistent_kernel<true, false, false, false>,
+                      (void*)select_persistent_kernel<true, true, false, false>, (void*)select_persistent_kernel<false, false, true, false>,
+                      (void*)select_persistent_kernel<false, false, false, true>};
       cudaError_t e = cudaSuccess;
       size_t fixed = 0;
       for (void* fn : fns) {
@@ -1162,7 +1174,7 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
       }
       // the most a launch may ask for: everything a block can opt in to beyond the kernels' static share
       const size_t want = (size_t)optin > fixed ? ((size_t)optin - fixed) / 1024 * 1024 : 0;
-      if (want < persist_smem(kPMaxRows, kNoteCapMin, kStages * stage_words(kScoring, false))) e = cudaErrorInvalidValue;
+      if (want < persist_smem(kPMaxRows, kNoteCapMin, kStages * stage_words(true, false))) e = cudaErrorInvalidValue;
       d.smem_max = want;
       for (void* fn : fns) {
         int b = 0;
@@ -1203,10 +1215,9 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   a.status = ws.status;
   const bool lru = fs && fs->opt.policy == 2;
   // (the LRU policy's stages leave no room for the packed counts on pools of more than 41 rows)
-  const bool packed = fs && fs->n_events < kPackedMaxEvents && *fs->hot == 0u &&
-                      persist_smem(a.n_rows, kNoteCapMin, kStages * stage_words(kScoringPacked, lru)) <= pd.smem_max;
-  const Fusion fusion = !fs ? kNoScoring : packed ? kScoringPacked : kScoring;
-  a.stage_words = fs ? stage_words(fusion, lru) : 0u;
+  const bool packed = fs && fs->n_events < kPackedMaxEvents &&
+                      persist_smem(a.n_rows, kNoteCapMin, kStages * stage_words(true, lru)) <= pd.smem_max;
+  a.stage_words = fs ? stage_words(packed, lru) : 0u;
   const uint32_t stages_words = kStages * a.stage_words;
   // Notes: the bracket typically holds 4-15 % of a warp's keys, in some traces several times
   // that.  A quarter of them stays in shared memory (what does not fit goes to the global scratch);
@@ -1226,38 +1237,33 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
   a.bg = bg ? *bg : BlockGeom{};
   a.expand = bg && bg->n_parts == 1 ? bg->heads[0] : 0u;
   a.st = st;
+  if (!packed) a.st.packed = nullptr;
   a.pd = Predictor{};
   a.hw = HeadWeights{};
-  const Workspace lws = fusion == kScoringPacked ? ws.for_packed() : ws;
+  const Workspace lws = packed ? ws.for_packed() : ws;
   a.epoch = 0;
   a.ev_entry = nullptr;
   a.n_events = 0;
-  a.h_hot = nullptr;
   if (fs) {
     a.pd = Predictor{fs->hits,       fs->misses,    fs->P,          fs->alpha0, fs->beta0, ws.delta, nullptr,
                      fs->opt.policy, fs->opt.kappa, fs->opt.window, ws.blend};
     a.hw = fs->hw;
     a.epoch = fs->epoch;
-    EntryState ev = st;
-    if (fusion != kScoringPacked) ev.packed = nullptr;
-    const cudaError_t e = launch_event_reduce(fs->ev_entry, fs->ev_hit, fs->n_events, ev, lws, s);
+    const cudaError_t e = launch_event_reduce(fs->ev_entry, fs->ev_hit, fs->n_events, a.st, lws, s);
     if (e != cudaSuccess) return e;
     a.ev_entry = fs->ev_entry;
     a.n_events = fs->n_events;
-    a.h_hot = fs->hot_dev;
   }
   void* args[] = {&a};
   const bool plain = fs && fs->opt.policy == 0 && fs->hw.on == 0;
-  void* fn = bg ? (void*)select_persistent_kernel<kNoScoring, false, true, false>
-             : ws.shared_words ? (void*)select_persistent_kernel<kNoScoring, false, false, true>
-             : fusion == kNoScoring ? (void*)select_persistent_kernel<kNoScoring, false, false, false>
-             : fusion == kScoring ? (plain ? (void*)select_persistent_kernel<kScoring, true, false, false>
-                                           : (void*)select_persistent_kernel<kScoring, false, false, false>)
-                                  : (plain ? (void*)select_persistent_kernel<kScoringPacked, true, false, false>
-                                           : (void*)select_persistent_kernel<kScoringPacked, false, false, false>);
+  void* fn = bg ? (void*)select_persistent_kernel<false, false, true, false>
+             : ws.shared_words ? (void*)select_persistent_kernel<false, false, false, true>
+             : !fs ? (void*)select_persistent_kernel<false, false, false, false>
+                   : plain ? (void*)select_persistent_kernel<true, true, false, false>
+                           : (void*)select_persistent_kernel<true, false, false, false>;
   cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, G > 1, lws);
   if (e != cudaSuccess) {
-    if (fusion == kScoringPacked)   // (nobody takes the packed counts up)
+    if (packed)   // (nobody takes the packed counts up)
       (void)cudaMemsetAsync(st.packed, 0, (st.n + 3) / 4 * 8, s);
     return e;
   }

@@ -131,8 +131,6 @@ struct kv_pool {
   uint32_t n_head_imp = 0, n_head_w = 0;
   PrefetchState prefetch{}; // per-layer prefetch windows
   unsigned long long* packed = nullptr;   // EntryState::packed of the fused scoring pass
-  volatile uint32_t* h_hot = nullptr;  // FusedScore::hot
-  uint32_t* hot_dev = nullptr;
   // a demotion whose later chunks are not enqueued yet (deferred packing)
   struct Pending {
     bool active = false, meta_done = false;
@@ -164,7 +162,7 @@ struct Layout {
   uint64_t delta, hist, sel, status, blend, block_score, block_state, block_victims, part_counts, tile_counts, tile_offsets, turns, table, packed, free_list, slot_list[kListBufs];
   uint64_t ring[4][6];
   uint64_t dev_total;
-  uint64_t h_list[kListBufs], h_counts, h_status, h_sel_stats, h_hot, host_total;
+  uint64_t h_list[kListBufs], h_counts, h_status, h_sel_stats, host_total;
   uint32_t n_tiles;
   uint64_t table_words;
 };
@@ -266,7 +264,6 @@ void make_layout(const kv_pool_desc* d, const Derived& g, Layout* L) {
   L->h_counts = htake(4 * 8);
   L->h_status = htake(4);
   L->h_sel_stats = htake(16);
-  L->h_hot = htake(4);
   L->host_total = h;
 }
 
@@ -620,14 +617,6 @@ int32_t kv_pool_create(const kv_pool_desc* desc, kv_stream_t stream, kv_pool** o
     for (int q = 0; q < 4; ++q) p->h_counts[q] = 0;
   }
   p->h_sel_stats = reinterpret_cast<uint32_t*>(hw + L.h_sel_stats);
-  {
-    uint32_t* const hot = reinterpret_cast<uint32_t*>(hw + L.h_hot);
-    *hot = 0;
-    p->h_hot = hot;
-    void* dp = nullptr;
-    if (cudaHostGetDevicePointer(&dp, hot, 0) == cudaSuccess) p->hot_dev = static_cast<uint32_t*>(dp);
-    else (void)cudaGetLastError();
-  }
   p->st = EntryState{desc->d_ema, desc->d_decay, desc->d_touch, desc->d_last_epoch, desc->d_pair,
                      desc->d_state, desc->d_tag, desc->d_score, g.N};
 
@@ -896,7 +885,7 @@ int32_t kv_epoch_score_select(kv_pool* p, uint32_t epoch, const uint32_t* d_ev_e
   if (k > 0 && p->select_variant != 0) {
     const FusedScore fs{p->desc.d_hits, p->desc.d_misses, p->desc.d_P, p->desc.alpha0,
                         p->desc.beta0,  epoch,            p->score_opt,  p->head,
-                        d_ev_entry,     d_ev_hit,         n_events,   p->h_hot,        p->hot_dev};
+                        d_ev_entry,     d_ev_hit,         n_events};
     forget_free_lists(p);
     EntryState st = p->st;
     st.packed = p->packed;

@@ -110,7 +110,8 @@ struct SelectScalars {
   uint32_t hint_half;
   uint32_t hint_off_last, hint_off_trend;
   uint32_t hint_trend;         // where the trend puts the next tau
-  uint32_t touch_hot;          // an entry has more touches than the packed counts are tried again with
+  uint32_t touch_wide;         // so many epochs to come of the fused pass count their touches in `touch` ...
+  uint32_t touch_hot;          // ... and one of them has met an entry with more than a packed count holds
 };
 
 // What the CTAs of one persistent selection share while it runs.  A pool has two of these, used in
@@ -394,8 +395,6 @@ struct FusedScore {
   const uint32_t* ev_entry;      // the epoch's trace, whose reduction is launched ahead
   const uint8_t* ev_hit;
   uint64_t n_events;
-  const volatile uint32_t* hot;  // host word: not 0 while the packed counts do not hold every entry's touches ...
-  uint32_t* hot_dev;             // ... where the device can write it (nullptr: it cannot)
 };
 cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t* d_victims,
                                      const Workspace& ws, cudaStream_t s, bool* used,

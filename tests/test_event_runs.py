@@ -14,7 +14,7 @@ template <bool PACKED> bool wrong(uint32_t n, uint32_t start, uint32_t last_step
   // a run reads the words of four pair bytes that hold its first and its last entry
   const unsigned long long end = ((unsigned long long)start + 3u) / 4u * 4u + 4u;
   const bool want = last_step == 3u && (PACKED || start % 4u == 0u) && end <= n;
-  if (kvt::is_run<PACKED>(id, n) == want) return false;
+  if (kvt::is_run(id, n, PACKED) == want) return false;
   std::printf("packed %d, pool of %u, start %u, last step %u: %d\n", (int)PACKED, n, start, last_step, (int)!want);
   return true;
 }
