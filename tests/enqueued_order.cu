@@ -210,8 +210,12 @@ cudaError_t launch_select(const EntryState& st, uint64_t, uint32_t*, const Works
   return cudaSuccess;
 }
 cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t* v, const Workspace& ws, cudaStream_t s, bool* used,
-                                     const FusedScore*, const PartCounts* pc, const BlockGeom*) {
+                                     const FusedScore* fs, const PartCounts* pc, const BlockGeom*) {
   *used = true;
+  if (fs) {
+    whole_pool(op(s, "events"), st, true);
+    whole_pool(op(s, "entry pass"), st, true);
+  }
   return launch_select(st, k, v, ws, s, 1, pc);
 }
 cudaError_t launch_select_blocks(const EntryState& st, const BlockGeom&, uint64_t k, uint32_t* v, const Workspace& ws, cudaStream_t s, unsigned long long*) {
@@ -373,8 +377,12 @@ int main(int argc, char** argv) {
         check(kv_hash_entries(p, nullptr, n, (uint8_t*)d.d_loc, compute), "kv_hash_entries");
       } else if (rng() % 2) {
         check(kv_admit(p, ++epoch, 0.9f, pairs.data(), pairs.size(), 0, nullptr, compute), "kv_admit");
-      } else {
+      } else if (rng() % 2) {
         check(kv_epoch_score(p, ++epoch, nullptr, nullptr, 0, compute), "kv_epoch_score");
+      } else {
+        const uint64_t resident = ids(0, true).size() + ids(1, true).size();
+        check(kv_epoch_score_select(p, ++epoch, nullptr, nullptr, 0, resident ? 1 + rng() % resident : 0, (uint32_t*)d.d_score, compute),
+              "kv_epoch_score_select");
       }
     }
   }
