@@ -287,8 +287,9 @@ int32_t kv_select_victims(kv_pool* pool, uint64_t k, uint32_t* d_victims, kv_str
  * State, d_victims and the device status word end up exactly as after the two
  * calls.  The trace is read by both launches: leave it alone until the call's work
  * has run.  All arguments are checked before anything is enqueued: on an error
- * (including KV_ERR_K_TOO_LARGE) the epoch has NOT been scored.  k == 0 scores
- * only.  Where the device cannot keep the kernel's whole grid resident at once,
+ * (including KV_ERR_K_TOO_LARGE) the epoch has NOT been scored.  (KV_ERR_CUDA from
+ * the second launch leaves the events counted, as kv_epoch_events does, for
+ * kv_epoch_update to take up.)  k == 0 scores only.  Where the device cannot keep the kernel's whole grid resident at once,
  * the separate kernels run one after the other instead. */
 int32_t kv_epoch_score_select(kv_pool* pool, uint32_t epoch, const uint32_t* d_ev_entry,
                               const uint8_t* d_ev_hit, uint64_t n_events, uint64_t k,

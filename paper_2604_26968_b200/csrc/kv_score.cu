@@ -53,6 +53,28 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The touches of a trace whose packed counts nobody takes up, in the 32-bit ones (where they are already while
+// *wide says so).
+__global__ void __launch_bounds__(kThreads)
+event_recount_kernel(const uint32_t* ev_entry, uint64_t n_events, const uint8_t* pair, uint32_t* touch, uint64_t n,
+                     const uint32_t* wide) {
+  if (*wide) return;
+  for (uint64_t e = (uint64_t)blockIdx.x * kThreads + threadIdx.x; e < n_events; e += (uint64_t)gridDim.x * kThreads) {
+    const uint32_t i = ev_entry[e];
+    if (i < n && !(pair[i] & kPairFree)) atomicAdd(touch + i, 1u);
+  }
+}
+
+cudaError_t launch_event_recount(const uint32_t* ev_entry, uint64_t n_events, const EntryState& st, const Workspace& ws,
+                                 cudaStream_t s) {
+  if (n_events == 0) return cudaSuccess;
+  const uint64_t blocks = (n_events + kThreads - 1) / kThreads, cap = (uint64_t)sm_count() * 8;
+  event_recount_kernel<<<(unsigned)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(ev_entry, n_events, st.pair, st.touch,
+                                                                                   st.n, &ws.sel->touch_wide);
+  count_launches(1);
+  return cudaMemsetAsync(st.packed, 0, (st.n + 3) / 4 * 8, s);
+}
+
 // ---- entry pass ----------------------------------------------------------------------
 // Every block forms the 16 posteriors itself (32 counters, read-only here), then
 // streams its share of the entries: four per thread and iteration, every array

@@ -1263,8 +1263,7 @@ cudaError_t launch_select_persistent(const EntryState& st, uint64_t k, uint32_t*
                            : (void*)select_persistent_kernel<true, false, false, false>;
   cudaError_t e = launch_scoring_kernel(fn, dim3(G), dim3(kPThreads), args, smem, s, G > 1, lws);
   if (e != cudaSuccess) {
-    if (packed)   // (nobody takes the packed counts up)
-      (void)cudaMemsetAsync(st.packed, 0, (st.n + 3) / 4 * 8, s);
+    if (packed) (void)launch_event_recount(fs->ev_entry, fs->n_events, a.st, ws, s);
     return e;
   }
   count_launches(1);

@@ -317,6 +317,10 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), unsigned grid, u
 // With st.packed the touches go there, for the fused scoring pass.
 cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events,
                                 const EntryState& st, const Workspace& ws, cudaStream_t s);
+// Behind a launch_event_reduce into st.packed whose scoring pass could not be launched: the touches go where
+// kv_epoch_events leaves them, beside the epoch counters, which hold the trace already.
+cudaError_t launch_event_recount(const uint32_t* ev_entry, uint64_t n_events, const EntryState& st, const Workspace& ws,
+                                 cudaStream_t s);
 // posterior (from hits/misses plus the epoch counters in ws.delta) + EMA + score in one launch;
 // folds ws.delta into hits/misses, clears it and writes P
 cudaError_t launch_entry_update(const EntryState& st, uint64_t* hits, uint64_t* misses, float* P,
