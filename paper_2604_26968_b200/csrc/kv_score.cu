@@ -7,7 +7,7 @@ namespace kvt {
 
 // ---- event reduction ---------------------------------------------------------
 // PACKED: touches go to the packed counts, or, while the last epochs' have overflowed them (wide), to the others.
-template <bool PACKED, bool DEAL>
+template <bool PACKED>
 __global__ void __launch_bounds__(kEventThreads, kEventBlocksPerSm)
 event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_events, const uint8_t* pair,
                     uint32_t* touch, unsigned long long* packed, uint64_t n, unsigned long long* delta,
@@ -19,7 +19,7 @@ event_reduce_kernel(const uint32_t* ev_entry, const uint8_t* ev_hit, uint64_t n_
   const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
   EventVec first[kEventVecs];   // (together with *wide: one behind the other is a latency more)
   load_events(ev_entry, ev_hit, n_events / 4, 0, gtid, stride, first);
-  const uint32_t bad = reduce_events<PACKED, DEAL>(PACKED && *wide == 0u, first, ev_entry, ev_hit, n_events, pair, touch,
+  const uint32_t bad = reduce_events<PACKED>(PACKED && *wide == 0u, first, ev_entry, ev_hit, n_events, pair, touch,
                                                    packed, n, gtid, stride, s_cnt, delta);
   if (bad) atomicOr(status, bad);
 }
@@ -43,10 +43,7 @@ cudaError_t launch_event_reduce(const uint32_t* ev_entry, const uint8_t* ev_hit,
   unsigned long long* delta = ws.delta;
   uint32_t* status = ws.status;
   void* args[] = {&ev_entry, &ev_hit, &n_events, &pair, &touch, &packed, &n, &delta, &wide, &status};
-  const bool rounds = n_events / 4 > blocks * kEventThreads * kEventVecs;   // more than one of the grid: see reduce_events
-  const void* fn = !packed ? (const void*)event_reduce_kernel<false, false>
-                 : rounds  ? (const void*)event_reduce_kernel<true, true>
-                           : (const void*)event_reduce_kernel<true, false>;
+  const void* fn = packed ? (const void*)event_reduce_kernel<true> : (const void*)event_reduce_kernel<false>;
   const cudaError_t e = launch_scoring_kernel(fn, dim3((unsigned)blocks), dim3(kEventThreads), args, 0, s, false, ws,
                                               n_events <= kEventOverlapMax);
   count_launches(1);

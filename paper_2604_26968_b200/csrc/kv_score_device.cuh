@@ -44,7 +44,10 @@ namespace kvt {
 // consecutive entries (an aligned group of four ids): one 4-byte load then
 // fetches their pairs and FREE bits, and one atomic on a packed word, or two on the 32-bit
 // counts, counts the four touches.  Those two go out from neighbouring lanes of one instruction, so
-// that a 32-byte sector of counts is visited once and not twice.
+// that a 32-byte sector of counts is visited once and not twice.  (A warp's events dealt out again, neighbours to
+// neighbouring lanes, where vectors are no runs: 1 us less in 141 where single entries in order follow runs, but
+// 12 M events on 18.8 M entries 189 -> 239 us a pass with one broken vector a warp, blocks of two heads 207 -> 245,
+// 6 M single entries in order on 3.1 M 53.7 -> 59.8.)
 //
 // What bounds it: the latency of two dependent scattered reads (event, pair byte) and
 // the rate of the atomics.  The next vectors' events are on their way while the current
@@ -131,7 +134,7 @@ __host__ __device__ __forceinline__ bool is_run(const uint32_t id[4], uint32_t n
 // refused events.  nxt: the thread's first vectors, from load_events.  use_packed (PACKED only): where the
 // touches go; no second template, since a kernel with two copies of this takes longer to fetch (4,096 entries
 // 13.4 -> 13.9 us a pass).  Every thread of the block must call it.
-template <bool PACKED, bool DEAL>
+template <bool PACKED>
 __device__ __forceinline__ uint32_t reduce_events(bool use_packed, EventVec nxt[kEventVecs], const uint32_t* ev_entry, const uint8_t* ev_hit,
                                                   uint64_t n_events, const uint8_t* pair, uint32_t* touch,
                                                   unsigned long long* packed, uint64_t n, uint64_t gtid,
@@ -201,26 +204,6 @@ __device__ __forceinline__ uint32_t reduce_events(bool use_packed, EventVec nxt[
       uint32_t id[4];
       ids_of(cur[u], id);
       run[u] = is_run(id, n32, to_packed);
-      if constexpr (DEAL) {
-        // Where vectors are no runs (the slots that an epoch has filled again, in order of their ids), a
-        // warp's 128 events are dealt out again, neighbours to neighbouring lanes: a gather or an
-        // addition of 32 neighbours touches a third of the sectors (15.3 M events, 18.8 M entries 143.9 ->
-        // 142.7 us a pass).  Traces of one round are bound by its latency, to which the second reading
-        // of the ids adds (4,096 entries 12.4 -> 12.6).
-        const uint64_t v0 = (it * kEventVecs + u) * stride + gtid - lane;   // (the warp's first vector)
-        if (!__all_sync(0xFFFFFFFFu, run[u]) && v0 + 32u <= n4) {
-          const uint64_t e = 4u * v0 + lane;
-          uint32_t hit = 0;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            id[j] = ev_entry[e + 32u * j];
-            hit |= (uint32_t)ev_hit[e + 32u * j] << (8 * j);
-          }
-          cur[u].id = make_uint4(id[0], id[1], id[2], id[3]);
-          cur[u].hit = hit;
-          run[u] = false;
-        }
-      }
       pr4[u] = gather(id, run[u]);
     }
     if (it + 1 < iters) load_events(ev_entry, ev_hit, n4, it + 1, gtid, stride, nxt);

@@ -1,6 +1,6 @@
-"""Traces of several rounds whose warps' events are dealt out again where vectors are no runs: runs, broken
-runs, single entries, entries out of range and flags of any value mixed in one trace, around a round of
-the whole grid, against the oracle, bit for bit, with the status bits."""
+"""Traces of several rounds of the grid whose vectors are runs, broken runs, single entries and entries out of
+range, with flags of any value, mixed in one trace, around a round of the whole grid, against the oracle,
+bit for bit, with the status bits."""
 import numpy as np
 import pytest
 
