@@ -132,8 +132,9 @@ __host__ __device__ __forceinline__ bool is_run(const uint32_t id[4], uint32_t n
 // counts for pair p (events | hits << 16) since the last flush.  delta: the 32
 // global epoch counters (index 2 * pair + hit).  Returns the KV_DEV_* bits of
 // refused events.  nxt: the thread's first vectors, from load_events.  use_packed (PACKED only): where the
-// touches go; no second template, since a kernel with two copies of this takes longer to fetch (4,096 entries
-// 13.4 -> 13.9 us a pass).  Every thread of the block must call it.
+// touches go; looked at late, since it comes from memory, and no second template, since a kernel with two copies
+// of this takes longer to fetch (4,096 entries: without such a choice 13.05 us a pass, like this 13.2, with two
+// copies 13.5).  Every thread of the block must call it.
 template <bool PACKED>
 __device__ __forceinline__ uint32_t reduce_events(bool use_packed, EventVec nxt[kEventVecs], const uint32_t* ev_entry, const uint8_t* ev_hit,
                                                   uint64_t n_events, const uint8_t* pair, uint32_t* touch,
@@ -203,7 +204,7 @@ __device__ __forceinline__ uint32_t reduce_events(bool use_packed, EventVec nxt[
     for (uint32_t u = 0; u < kEventVecs; ++u) {  // all gathers before any is used
       uint32_t id[4];
       ids_of(cur[u], id);
-      run[u] = is_run(id, n32, to_packed);
+      run[u] = is_run(id, n32, PACKED);
       pr4[u] = gather(id, run[u]);
     }
     if (it + 1 < iters) load_events(ev_entry, ev_hit, n4, it + 1, gtid, stride, nxt);
@@ -212,7 +213,8 @@ __device__ __forceinline__ uint32_t reduce_events(bool use_packed, EventVec nxt[
       uint32_t id[4];
       ids_of(cur[u], id);
       const uint32_t pr = pr4[u], hit4 = nonzero_bytes(cur[u].hit);
-      const bool whole = run[u] && !(pr & 0x80808080u);   // four resident entries in a row
+      // four resident entries in a row (use_packed is looked at as late as this: it comes from memory)
+      const bool whole = run[u] && !(pr & 0x80808080u) && (to_packed || !(id[0] & 3u));
       if (to_packed && whole) {
         const uint32_t r = id[0] & 3u;
         atomicAdd(packed + (id[0] >> 2), packed_touches(0x01010101u << (8u * r)));
