@@ -20,9 +20,10 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 @pytest.fixture(scope="module")
 def copy(tmp_path_factory):
+    # (-Bsymbolic: other tests load the library itself for everybody, and its functions would be taken)
     so = str(tmp_path_factory.mktemp("refused") / "libkvtier_refused.so")
     subprocess.run([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), *kv_build.NVCC_FLAGS, "--threads", "8",
-                    "-Xlinker", "--wrap=cudaLaunchKernelExC", *[os.path.join(kv_build.CSRC, s) for s in kv_build.SOURCES],
+                    "-Xlinker", "--wrap=cudaLaunchKernelExC", "-Xlinker", "-Bsymbolic", *[os.path.join(kv_build.CSRC, s) for s in kv_build.SOURCES],
                     os.path.join(ROOT, "tests", "refused_launch.cu"), "-o", so], check=True)
     return so
 
