@@ -45,11 +45,11 @@ NCU_PACK_TRAFFIC_BYTES_PER_PAYLOAD_BYTE = 487.35 / 268.44
 PACK_KERNEL_NAME = "move_tma_kernel<true> (pack)"
 
 # DRAM traffic of the scoring + selection pass (event_reduce_kernel followed by
-# select_persistent_kernel<true>) from ncu, bytes per launch pair, keyed by pool number: captured
+# select_persistent_kernel<true, ...>) from ncu, bytes per launch pair, keyed by pool number: captured
 # at the pool's full entry count with --tiny-entries (these kernels never touch block payload).
 # None = no capture of the kernels as they stand.  (ncu flushes the caches before every kernel it
 # replays: the figures are those of a cold L2, without what kv_set_l2_residency keeps there.)
-NCU_SCORE_SELECT_TRAFFIC = {5: 465.0e6, 3: 352.0e6}
+NCU_SCORE_SELECT_TRAFFIC = {5: 538.9e6, 3: 398.1e6}
 
 
 def parse():
@@ -692,7 +692,8 @@ def main():
                    "promote_lists": w.promote_style + ("" if "runs" not in w.promote_style else " of %d slots" % w.max_run),
                    "fused_score_select": not (args.no_fused or dist_on),
                    "l2_residency": ("budget %d MiB: %s in the persisting part of the L2" % (
-                       args.l2_mb, "touch counts" if 4 * N <= (args.l2_mb << 20) else "pair bytes")) if l2_on else "off",
+                       args.l2_mb, "packed touch counts" if not (args.no_fused or dist_on) and (N + 3) // 4 * 8 <= (args.l2_mb << 20)
+                       else "touch counts" if 4 * N <= (args.l2_mb << 20) else "pair bytes")) if l2_on else "off",
                    "head_weights": bool(args.head_weights),
                    "ring_slots": [p.ring_slots for p in w.parts], "scale": scale,
                    "parallelism": "1 pool per GPU" + (", 256-byte all-reduce of pair counters" if dist_on else ""),
@@ -713,8 +714,8 @@ def main():
                                                      if timing["gather_launches"] else None),
         },
         "hostlink": link,
-        "roofline": {"kernel": ("event_reduce_kernel + select_persistent_kernel<true>" if fused else
-                                "event_reduce_kernel + entry_update_kernel + select_persistent_kernel<false>")
+        "roofline": {"kernel": ("event_reduce_kernel + select_persistent_kernel<true, ...>" if fused else
+                                "event_reduce_kernel + entry_update_kernel + select_persistent_kernel<false, ...>")
                                + " (the scoring + selection pass that `value` times)",
                      "bound": "hbm", "achieved": ss_gbs, "peak": peak, "peak_kind": "of " + peak_kind, "unit": "GB/s",
                      "frac": ss_gbs / peak, "traffic": ss_traffic,
