@@ -27,7 +27,7 @@
 //      chunks, and writes its own victims in ascending id order straight from the
 //      bitmaps.
 //
-// What bounds it: phase A streams 20 B an entry from HBM, its issue slots half busy; B to D are
+// What bounds it: phase A streams 24 B an entry from HBM, its issue slots half busy; B to D are
 // three exchanges between all CTAs (two histograms, one table of counts) of ~2.5 us each, latency of L2
 // and of the block barriers around them.  An exchange is a grid barrier (a counter that
 // every CTA increments and one of its threads polls).  (Tried for the third one: no
@@ -41,15 +41,15 @@
 // memory, so that a captured launch can be replayed.  The selection without caller's scratch
 // (SHARED = true) cannot rely on the launch before it: it clears its one set itself, while its
 // keys are read (a memset ahead of the launch took 3.0 us of a 21.9 us pass over 1,000,003 entries).
-// Measured, a pass with the event reduction: 4,096 entries 13.1 us, 0.9 M 26.8, 3.1 M 37.2, 18.8 M 149
+// Measured, a pass with the event reduction: 4,096 entries 13.7 us, 0.9 M 26.7, 3.1 M 38.5, 18.8 M 158
 // (notes per thread and whole chunks only, 32-bit touch counts: 32.5, 40.3, 59.9, 206).
 //
 // The same kernel also exists fused with the per-entry scoring pass (FUSED = true):
 // every CTA first updates the entries of its own rows (posterior, EMA, score), their
 // inputs streamed through shared-memory stages by asynchronous copies.  The touch counts are
-// the packed ones of reduce_events, two bytes an entry, beside the caller's (entry phase of 18.8 M entries 97 -> 83 us,
-// the event reduction ahead of it 40 -> 32; a pass 177 -> 152, of 3.1 M entries 41.1 -> 39.3, of
-// 0.9 M even), or, for a while after a trace that overflowed them, the caller's alone.  The event
+// the packed ones of reduce_events, two bytes an entry, beside the caller's (against the caller's alone the
+// event reduction of 18.8 M entries takes 32 us instead of 40, a pass 158 instead of 184, of 3.1 M
+// entries 38.1 instead of 41.3), or, for a while after a trace that overflowed them, the caller's alone.  The event
 // reduction stays a launch of its own ahead of it: its scattered gathers and atomics run slower
 // beside this kernel's shared memory (11.5 M entries 101 -> 111 us), and for small traces a
 // cooperative launch's own gap of ~3 us takes the place of the one saved (0.9 M 27.3 -> 27.5).
