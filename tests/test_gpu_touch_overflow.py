@@ -90,3 +90,18 @@ def test_captured_call_meets_hot_traces():
         assert rc == O.OK and np.array_equal(g.victims[:w.k].cpu().numpy().view(np.uint32), v), i
     del graph
     ls.close()
+
+
+def test_no_room_for_packed_counts():
+    """Under the LRU policy 25.1 M entries (42 rows) leave no room for packed counts in the stages: the call
+    counts in 32 bits, whatever the counts, and stays at two launches."""
+    from lockstep import Lockstep
+    w = W.Workload("wide", [W.gqa(3, 8, 8, 2, 4, 1_045_834, 64, "entry")], 0.02, 0.0, seed=7)
+    ls = Lockstep(w, payload=False, batch_bytes=1 << 20, policy=2)
+    g = ls.gpu
+    r = np.random.default_rng(5)
+    for e, hot in enumerate([False, True, False]):
+        before = g.pool.kv_get_stats()["kernel_launches"]
+        score_select(ls, e, *trace(w.N, hot, r, 400_001), True)
+        assert g.pool.kv_get_stats()["kernel_launches"] - before == 2
+    ls.close()
